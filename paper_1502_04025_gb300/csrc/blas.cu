@@ -204,7 +204,7 @@ __global__ void k_scale_by_norm(const double2 *w, int64_t n, const double2 *norm
         double2 a = w[k];
         a = make_double2(a.x * f, a.y * f);
         out[k] = a;
-        if (out32) out32[k] = make_float2((float)a.x, (float)a.y);
+        if (out32) out32[k] = make_float2(d2f(a.x), d2f(a.y));
     }
 }
 

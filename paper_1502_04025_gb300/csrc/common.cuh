@@ -77,6 +77,67 @@ __device__ __forceinline__ void cfmac(cpx<R> &acc, cpx<R> a, cpx<R> b)
     acc.im = fma(-a.im, b.re, acc.im);
 }
 
+// ------------------------------------------- FP64 <-> FP32 by integer operations
+//
+// The conversion instructions between FP64 and FP32 (or integers) run at 2
+// lanes per clock and SM on this GPU, as slowly as FP64 arithmetic (measured:
+// 1.99 against 64-90 for integer operations), so a pass that converts every
+// component of a field is bound by them and not by memory.  These forms give
+// the conversion instructions' results bit for bit: the exponent and mantissa
+// bits are moved by integer operations, and the rare values outside FP32's
+// normal range (subnormal results, overflow, infinities, NaN) take the
+// instruction.
+
+// round to nearest even
+__device__ __forceinline__ float d2f(double v)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t mag = hi & 0x7fffffffu, sign = hi & 0x80000000u;
+    const uint32_t e = mag - 0x38000000u;  // the exponent rebased to FP32's
+    uint32_t f = __funnelshift_l(lo, e, 3);
+    const uint32_t r = lo << 3;  // the 29 dropped bits, at the top of the word
+    f += (r > 0x80000000u || (r == 0x80000000u && (f & 1u))) ? 1u : 0u;
+    // normal results: rebased exponent 1..253 (254 may round up to infinity)
+    if (e - 0x00100000u < 0x0fd00000u) return __uint_as_float(f | sign);
+    if ((mag | lo) == 0u) return __uint_as_float(sign);
+    return __double2float_rn(v);
+}
+
+// exact
+__device__ __forceinline__ double f2d(float v)
+{
+    const uint32_t b = __float_as_uint(v), mag = b & 0x7fffffffu, sign = b & 0x80000000u;
+    if (mag - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)(((mag >> 3) + 0x38000000u) | sign), (int)(b << 29));
+    if (mag == 0u) return __hiloint2double((int)sign, 0);
+    return (double)v;
+}
+
+// a * b in FP64 (the product of two 24-bit mantissas is exact)
+__device__ __forceinline__ double mul_f2d(float a, float b)
+{
+    const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
+    const uint32_t ma = ua & 0x7fffffffu, mb = ub & 0x7fffffffu, sign = (ua ^ ub) & 0x80000000u;
+    if (ma - 0x00800000u < 0x7f000000u && mb - 0x00800000u < 0x7f000000u) {
+        uint64_t p = (uint64_t)((ma & 0x007fffffu) | 0x00800000u) * ((mb & 0x007fffffu) | 0x00800000u);
+        const uint32_t top = (uint32_t)(p >> 47);  // 1 when the product of the mantissas is >= 2
+        p <<= 6u - top;                            // leading one at bit 52
+        const uint32_t e = (ma >> 23) + (mb >> 23) + (1023u - 254u) + top;
+        return __hiloint2double((int)((((uint32_t)(p >> 32)) - 0x00100000u + (e << 20)) | sign), (int)(uint32_t)p);
+    }
+    return (double)a * (double)b;
+}
+
+// Four doubles (32 bytes) with one access; p on a 32-byte boundary.
+__device__ __forceinline__ void ld_global_x4(const double2 *p, double2 &a, double2 &b)
+{
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(a.x), "=d"(a.y), "=d"(b.x), "=d"(b.y) : "l"(p));
+}
+__device__ __forceinline__ void st_global_x4(double2 *p, double2 a, double2 b)
+{
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(a.x), "d"(a.y), "d"(b.x), "d"(b.y) : "memory");
+}
+
 // --------------------------------------------------------- storage formats
 
 // One complex number per plane entry.  16-bit formats of spinors and clover

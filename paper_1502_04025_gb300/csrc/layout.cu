@@ -176,26 +176,100 @@ qdd_status make_geometry(const int L[4], const int dom[4], HostGeom &hg)
 
 // ------------------------------------------------------------------ kernels
 
+// threads of a block of the one-thread-per-site conversions
+constexpr int kSiteThreads = 128;
+
+// Spinor conversions between the host layout (FP64, one site's 12 components
+// contiguous) and the internal storages.  Bound by memory: the conversions
+// themselves are integer operations (d2f, f2d, mul_f2d), and a site's 192
+// bytes move as six 32-byte accesses, whole sectors (aligned host buffers;
+// `a32` false: 16 bytes at a time).  Measured on 32^3x64, per right-hand side,
+// against the conversion instructions and 16-byte accesses (89 us at the
+// measured HBM rate for FP32): in, FP32 95 -> 92 us, BF16 316 -> 94 us; out,
+// FP32 250 -> 92 us, FP64 336 -> 116 us; FP16 in, 12 x 16^3x32, 240 -> 69 us.
+
+// one component of an unscaled storage
+__device__ __forceinline__ void st_d(double2 *p, cpx<double> v) { *p = make_double2(v.re, v.im); }
+__device__ __forceinline__ void st_d(float2 *p, cpx<double> v) { *p = make_float2(d2f(v.re), d2f(v.im)); }
+__device__ __forceinline__ void st_d(__half2 *p, cpx<double> v) { *p = __floats2half2_rn(d2f(v.re), d2f(v.im)); }
+__device__ __forceinline__ void st_d(__nv_bfloat162 *p, cpx<double> v)
+{
+    *p = __floats2bfloat162_rn(d2f(v.re), d2f(v.im));
+}
+
+// The 12 components y of a site in a 16-bit storage with its scale (largest
+// component), in FP32 arithmetic.
+template <typename S>
+__device__ __forceinline__ void store_scaled(Field<S> f, int64_t base, int64_t sbase, int Vd, int d, int s,
+                                             const cpx<float> *y)
+{
+    float m = 0.f;
+#pragma unroll
+    for (int k = 0; k < 12; k++) m = fmaxf(m, fmaxf(fabsf(y[k].re), fabsf(y[k].im)));
+    f.scale[sbase + (int64_t)d * Vd + s] = m;
+    const float inv = m > 0.f ? 1.f / m : 0.f;
+    cpx<float> v[12];
+#pragma unroll
+    for (int k = 0; k < 12; k++) v[k] = inv * y[k];
+    st_sp_site<float, S>(f.p + base + (int64_t)d * 12 * Vd, s, Vd, v);
+}
+
+// The 12 FP64 components v of a site in a 16-bit storage: each is the FP64
+// quotient by the site's scale, rounded (through FP32) to 16 bits.  FP64
+// multiplications would bind the pass (24 per site at 2 per clock and SM), so
+// the quotient is taken in FP32, where it is within 2^-22 of the FP64 one, and
+// the two 16-bit roundings of the interval of 2^-21 around it are compared:
+// where they agree, that is the result; where a rounding boundary lies between
+// them (one value in 2^11 for FP16, 2^14 for BF16) the FP64 product decides.
+// Sites whose scale is near the end of FP32's range take FP64 throughout.
+template <typename S>
+__device__ __forceinline__ void store_scaled_d(Field<S> f, int64_t base, int64_t sbase, int Vd, int d, int s,
+                                               const cpx<double> *v)
+{
+    const typename S::T2 *tag = nullptr;
+    cpx<float> y[12];
+    float m = 0.f;
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+        y[k] = mk(d2f(v[k].re), d2f(v[k].im));
+        m = fmaxf(m, fmaxf(fabsf(y[k].re), fabsf(y[k].im)));
+    }
+    f.scale[sbase + (int64_t)d * Vd + s] = m;
+    const bool small = m < 0x1p-100f;
+    const float inv = small ? 0.f : 1.f / m;
+    uint32_t w[12];
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+        const float a = inv * y[k].re, b = inv * y[k].im;
+        const float lo = 1.f - 0x1p-21f, hi = 1.f + 0x1p-21f;
+        w[k] = f2_word(a * lo, b * lo, tag);
+        if (small || w[k] != f2_word(a * hi, b * hi, tag)) {
+            const double inv64 = m > 0.f ? 1.0 / (double)m : 0.0;
+            w[k] = f2_word((float)(v[k].re * inv64), (float)(v[k].im * inv64), tag);
+        }
+    }
+    typename S::T2 *p = f.p + base + (int64_t)d * 12 * Vd;
+    if constexpr (S::kQuad) {
+        uint4 *q = reinterpret_cast<uint4 *>(p) + s;
+#pragma unroll
+        for (int j = 0; j < 3; j++) q[(int64_t)j * Vd] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+    } else {
+        uint32_t *q = reinterpret_cast<uint32_t *>(p) + s;
+#pragma unroll
+        for (int k = 0; k < 12; k++) q[(int64_t)k * Vd] = w[k];
+    }
+}
+
 template <typename S>
 __device__ __forceinline__ void store_spinor(Field<S> f, int64_t base, int64_t sbase, int Vd, int d, int s,
                                              const cpx<double> *v)
 {
-    typename S::T2 *p = f.p + base + (int64_t)d * 12 * Vd + s;
-    if (S::kScaled) {
-        double m = 0;
-        for (int k = 0; k < 12; k++) m = fmax(m, fmax(fabs(v[k].re), fabs(v[k].im)));
-        float sc = (float)m;
-        double inv = m > 0 ? 1.0 / (double)sc : 0.0;
-        f.scale[sbase + (int64_t)d * Vd + s] = sc;
-        if constexpr (S::kQuad) {
-            cpx<double> y[12];
-            for (int k = 0; k < 12; k++) y[k] = mk(v[k].re * inv, v[k].im * inv);
-            st_sp_site<double, S>(f.p + base + (int64_t)d * 12 * Vd, s, Vd, y);
-        } else {
-            for (int k = 0; k < 12; k++) st_c<double>(p + (int64_t)k * Vd, mk(v[k].re * inv, v[k].im * inv));
-        }
+    if constexpr (S::kScaled) {
+        store_scaled_d<S>(f, base, sbase, Vd, d, s, v);
     } else {
-        for (int k = 0; k < 12; k++) st_c<double>(p + (int64_t)k * Vd, v[k]);
+        typename S::T2 *p = f.p + base + (int64_t)d * 12 * Vd + s;
+#pragma unroll
+        for (int k = 0; k < 12; k++) st_d(p + (int64_t)k * Vd, v[k]);
     }
 }
 
@@ -203,14 +277,21 @@ template <typename S>
 __device__ __forceinline__ void load_spinor_d(Field<S> f, int64_t base, int64_t sbase, int Vd, int d, int s,
                                               cpx<double> *v)
 {
-    if constexpr (S::kQuad) {
-        double sc = (double)f.scale[sbase + (int64_t)d * Vd + s];
-        ld_sp_site<double, S>(f.p + base + (int64_t)d * 12 * Vd, s, Vd, v);
-        for (int k = 0; k < 12; k++) v[k] = sc * v[k];
+    if constexpr (S::kBytes == 16) {
+        const double2 *p = f.p + base + (int64_t)d * 12 * Vd + s;
+#pragma unroll
+        for (int k = 0; k < 12; k++) v[k] = ld_c<double>(p + (int64_t)k * Vd);
     } else {
-        const typename S::T2 *p = f.p + base + (int64_t)d * 12 * Vd + s;
-        double sc = S::kScaled ? (double)f.scale[sbase + (int64_t)d * Vd + s] : 1.0;
-        for (int k = 0; k < 12; k++) v[k] = sc * ld_c<double>(p + (int64_t)k * Vd);
+        cpx<float> y[12];
+        ld_sp_site<float, S>(f.p + base + (int64_t)d * 12 * Vd, s, Vd, y);
+        if constexpr (S::kScaled) {
+            const float sc = f.scale[sbase + (int64_t)d * Vd + s];
+#pragma unroll
+            for (int k = 0; k < 12; k++) v[k] = mk(mul_f2d(sc, y[k].re), mul_f2d(sc, y[k].im));
+        } else {
+#pragma unroll
+            for (int k = 0; k < 12; k++) v[k] = mk(f2d(y[k].re), f2d(y[k].im));
+        }
     }
 }
 
@@ -225,8 +306,8 @@ __global__ void k_links_in(Geom g, const int *site_of, const double2 *src, doubl
 }
 
 template <typename S>
-__global__ void k_spinor_in(Geom g, const int *site_of, const double2 *src, Field<S> dst, int64_t rstride,
-                            int64_t sstride)
+__global__ void __launch_bounds__(kSiteThreads) k_spinor_in(Geom g, const int *site_of, const double2 *src,
+                                                            Field<S> dst, int64_t rstride, int64_t sstride, bool a32)
 {
     int gi = blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= g.V) return;
@@ -234,17 +315,23 @@ __global__ void k_spinor_in(Geom g, const int *site_of, const double2 *src, Fiel
     int d, s;
     split_index(g, gi, d, s);
     const double2 *p = src + ((int64_t)r * g.V + __ldg(site_of + gi)) * 12;
-    cpx<double> v[12];
-    for (int k = 0; k < 12; k++) {
-        double2 a = __ldg(p + k);
-        v[k] = mk(a.x, a.y);
+    double2 a[12];
+    if (a32) {
+#pragma unroll
+        for (int k = 0; k < 12; k += 2) ld_global_x4(p + k, a[k], a[k + 1]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 12; k++) a[k] = __ldg(p + k);
     }
+    cpx<double> v[12];
+#pragma unroll
+    for (int k = 0; k < 12; k++) v[k] = mk(a[k].x, a[k].y);
     store_spinor<S>(dst, r * rstride, r * sstride, g.Vd, d, s, v);
 }
 
 template <typename S>
-__global__ void k_spinor_out(Geom g, const int *site_of, Field<S> src, int64_t rstride, int64_t sstride,
-                             double2 *dst)
+__global__ void __launch_bounds__(kSiteThreads) k_spinor_out(Geom g, const int *site_of, Field<S> src, int64_t rstride,
+                                                             int64_t sstride, double2 *dst, bool a32)
 {
     int gi = blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= g.V) return;
@@ -254,11 +341,18 @@ __global__ void k_spinor_out(Geom g, const int *site_of, Field<S> src, int64_t r
     cpx<double> v[12];
     load_spinor_d<S>(src, r * rstride, r * sstride, g.Vd, d, s, v);
     double2 *p = dst + ((int64_t)r * g.V + __ldg(site_of + gi)) * 12;
-    for (int k = 0; k < 12; k++) p[k] = make_double2(v[k].re, v[k].im);
+    if (a32) {
+#pragma unroll
+        for (int k = 0; k < 12; k += 2)
+            st_global_x4(p + k, make_double2(v[k].re, v[k].im), make_double2(v[k + 1].re, v[k + 1].im));
+    } else {
+#pragma unroll
+        for (int k = 0; k < 12; k++) p[k] = make_double2(v[k].re, v[k].im);
+    }
 }
 
 template <typename SI, typename SO>
-__global__ void k_spinor_convert(Geom g, Field<SI> src, Field<SO> dst, int64_t rstride, int64_t sstride)
+__global__ void __launch_bounds__(kSiteThreads) k_spinor_convert(Geom g, Field<SI> src, Field<SO> dst, int64_t rstride, int64_t sstride)
 {
     int gi = blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= g.V) return;
@@ -291,23 +385,14 @@ __global__ void k_scale_convert(Geom g, const double2 *w, const double2 *norm2, 
     const double f = fs;
     const int64_t base = (int64_t)d * 12 * g.Vd + s;
     cpx<float> v[12];
-    float m = 0.f;
+#pragma unroll
     for (int k = 0; k < 12; k++) {
         double2 a = w[base + (int64_t)k * g.Vd];
         a = make_double2(a.x * f, a.y * f);
         out64[base + (int64_t)k * g.Vd] = a;
-        v[k] = mk((float)a.x, (float)a.y);
-        m = fmaxf(m, fmaxf(fabsf(v[k].re), fabsf(v[k].im)));
+        v[k] = mk(d2f(a.x), d2f(a.y));
     }
-    dst.scale[(int64_t)d * g.Vd + s] = m;
-    const float inv = m > 0.f ? 1.f / m : 0.f;
-    if constexpr (SO::kQuad) {
-        for (int k = 0; k < 12; k++) v[k] = inv * v[k];
-        st_sp_site<float, SO>(dst.p + (int64_t)d * 12 * g.Vd, s, g.Vd, v);
-    } else {
-        typename SO::T2 *p = dst.p + base;
-        for (int k = 0; k < 12; k++) st_c<float>(p + (int64_t)k * g.Vd, inv * v[k]);
-    }
+    store_scaled<SO>(dst, 0, 0, g.Vd, d, s, v);
 }
 
 template <typename S>
@@ -316,7 +401,7 @@ __global__ void k_links_convert(int64_t n, const double2 *src, typename S::T2 *d
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     double2 a = __ldg(src + i);
-    st_c<double>(dst + i, mk(a.x, a.y));
+    st_d(dst + i, mk(a.x, a.y));
 }
 
 // FP64 complex -> (re.hi, re.lo, im.hi, im.lo) FP32 split
@@ -371,7 +456,7 @@ __global__ void k_links12_convert(Geom g, const double2 *src, typename S::T2 *ds
         for (int k = 0; k < 6; k++) {
             double2 a = __ldg(src + ((int64_t)d * 36 + mu * 9 + k) * g.Vd + s);
             const int p = mu * 6 + k;
-            st_c<double>(dst + (S::kBytes == 4 ? pair_index(d, 24, p, g.Vd, s) : ((int64_t)d * 24 + p) * g.Vd + s),
+            st_d(dst + (S::kBytes == 4 ? pair_index(d, 24, p, g.Vd, s) : ((int64_t)d * 24 + p) * g.Vd + s),
                          mk(a.x, a.y));
         }
 }
@@ -435,8 +520,8 @@ qdd_status launch_spinor_in(Gauge *g, const double *src, void *dst, float *dst_s
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
     QDD_DISPATCH_PREC(prec, S, {
         Field<S> f{(typename S::T2 *)dst, dst_scale};
-        k_spinor_in<S><<<grid_sites(hg.V, nrhs, 256), 256, 0, s>>>(g->geom, g->d_site_of.as<int>(),
-                                                                   (const double2 *)src, f, rs, ss);
+        k_spinor_in<S><<<grid_sites(hg.V, nrhs, kSiteThreads), kSiteThreads, 0, s>>>(
+            g->geom, g->d_site_of.as<int>(), (const double2 *)src, f, rs, ss, ((uintptr_t)src & 31) == 0);
     });
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
@@ -450,8 +535,8 @@ qdd_status launch_spinor_out(Gauge *g, const void *src, const float *src_scale, 
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
     QDD_DISPATCH_PREC(prec, S, {
         Field<S> f{(typename S::T2 *)src, (float *)src_scale};
-        k_spinor_out<S><<<grid_sites(hg.V, nrhs, 256), 256, 0, s>>>(g->geom, g->d_site_of.as<int>(), f, rs, ss,
-                                                                    (double2 *)dst);
+        k_spinor_out<S><<<grid_sites(hg.V, nrhs, kSiteThreads), kSiteThreads, 0, s>>>(
+            g->geom, g->d_site_of.as<int>(), f, rs, ss, (double2 *)dst, ((uintptr_t)dst & 31) == 0);
     });
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
@@ -462,13 +547,13 @@ qdd_status launch_spinor_convert(Gauge *g, const void *src, const float *src_sca
 {
     const HostGeom &hg = g->hg;
     int64_t rs = (int64_t)hg.V * 12, ss = hg.V;
-    dim3 grid = grid_sites(hg.V, nrhs, 256);
+    dim3 grid = grid_sites(hg.V, nrhs, kSiteThreads);
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
     QDD_DISPATCH_PREC(sp, SI, {
         Field<SI> fi{(typename SI::T2 *)src, (float *)src_scale};
         QDD_DISPATCH_PREC(dp, SO, {
             Field<SO> fo{(typename SO::T2 *)dst, dst_scale};
-            k_spinor_convert<SI, SO><<<grid, 256, 0, s>>>(g->geom, fi, fo, rs, ss);
+            k_spinor_convert<SI, SO><<<grid, kSiteThreads, 0, s>>>(g->geom, fi, fo, rs, ss);
         });
     });
     QDD_CUDA(cudaGetLastError());
