@@ -68,9 +68,10 @@ typedef enum {
     QDD_PREC_F32 = 1,
     QDD_PREC_F16S = 2,
     QDD_PREC_BF16S = 3,
-    QDD_PREC_DF64 = 4, /* operator only: FP64-class accuracy (about 2^-46) from
-                          pairs of FP32 numbers; links and clover split into
-                          hi + lo parts.  For qdd_apply_D and arnoldi_prec. */
+    QDD_PREC_DF64 = 4, /* operator only: FP64-class accuracy (57 bits below each
+                          site's largest component) from 64-bit fixed-point
+                          numbers in two 32-bit limbs, on a copy of links and
+                          clover in that form.  For qdd_apply_D and arnoldi_prec. */
     QDD_PREC_H16 = 5   /* the paper's half precision (Sec. 3.3): FP16 links and
                           clover (per-site scale), FP32 spinors, FP32 arithmetic */
 } qdd_prec;
@@ -331,8 +332,11 @@ qdd_status qdd_layout_faces(const int L[4], const int dom[4], int foff[8], uint3
 
 /*
  * out = D in for nrhs spinors (host layout), periodic boundary conditions.
- * prec = QDD_PREC_F64 computes in FP64; QDD_PREC_DF64 in double-float
- * (FP32 pairs, about 2^-46 relative); QDD_PREC_F32 converts links, clover
+ * prec = QDD_PREC_F64 and QDD_PREC_DF64 compute in 64-bit fixed point, to
+ * FP64's accuracy or better against the largest component of the sites
+ * involved; QDD_PREC_F64 falls back to FP64 arithmetic where the links have no
+ * fixed-point copy (not finite, above 2^64, or a copy that would fill the HBM
+ * budget past a half); QDD_PREC_F32 converts links, clover
  * and input to FP32 and computes in FP32 (1848 flop per site); F16S / BF16S
  * read 16-bit links/clover/spinor with FP32 arithmetic.
  */

@@ -40,7 +40,8 @@ def _stale(obj: str, src: str) -> bool:
     if not os.path.exists(obj):
         return True
     t = os.path.getmtime(obj)
-    deps = [src, os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "internal.h"),
+    deps = [src, os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "fixed.cuh"),
+            os.path.join(CSRC, "internal.h"),
             os.path.join(CSRC, "admission.h"), os.path.join(ROOT, "include", "qdd.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 

@@ -1,5 +1,6 @@
 // C ABI of libqdd: contexts, gauge fields, operator and preconditioner
 // entry points, and host-side helpers (arXiv:1502.04025, Sec. 3).
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdarg>
@@ -145,6 +146,9 @@ void DevMem::release()
 
 // -------------------------------------------------------- precision copies
 
+// link entries up to 2^64 have a fixed-point copy
+constexpr int kMaxFixedLinkExp = 64;
+
 static size_t elem_bytes(qdd_prec p)
 {
     switch (p) {
@@ -171,12 +175,14 @@ qdd_status ensure_copy(Gauge *g, qdd_prec prec, cudaStream_t s)
         return QDD_EINVAL;
     }
     if (prec == QDD_PREC_DF64) {
-        // links and clover split into hi + lo FP32 parts (the operator only)
+        if (g->link_exp > kMaxFixedLinkExp) return QDD_OK;  // FP64 arithmetic stands in
         const size_t n = (size_t)g->hg.V * 36;
-        QDD_TRY(c.links.ensure(g->ctx, n * sizeof(float4)));
-        QDD_TRY(c.clov.ensure(g->ctx, n * sizeof(float4)));
-        QDD_TRY(launch_split_convert(g, g->links64.as<double2>(), c.links.as<float4>(), (int64_t)n, s));
-        QDD_TRY(launch_split_convert(g, g->clov64.as<double2>(), c.clov.as<float4>(), (int64_t)n, s));
+        QDD_TRY(c.links.ensure(g->ctx, n * 16));
+        QDD_TRY(c.clov.ensure(g->ctx, n * 16));
+        QDD_TRY(c.clov_s.ensure(g->ctx, (size_t)g->hg.V * sizeof(int)));
+        QDD_TRY(launch_fields_fx(g, c, s));
+        // FP64 callers on other streams may take the copy from here on
+        QDD_CUDA(cudaStreamSynchronize(s));
         c.valid = true;
         return QDD_OK;
     }
@@ -193,6 +199,26 @@ qdd_status ensure_copy(Gauge *g, qdd_prec prec, cudaStream_t s)
     QDD_TRY(launch_clover_convert(g, g->clov64.as<double2>(), prec, c.clov.p, c.clov_s.as<float>(), s, true));
     QDD_TRY(launch_clover_convert(g, g->sclov64.as<double2>(), prec, c.sclov.p, c.sclov_s.as<float>(), s));
     c.valid = true;
+    return QDD_OK;
+}
+
+qdd_status ensure_fixed(Gauge *g, bool required, cudaStream_t s, bool *ok)
+{
+    *ok = false;
+    if (g->link_exp > kMaxFixedLinkExp) return QDD_OK;
+    if (!required) {
+        std::lock_guard<std::mutex> lk(g->copy_mu);
+        const size_t need = (size_t)g->hg.V * (2 * 36 * 16 + 4);
+        const PrecCopy &c = g->copies[QDD_PREC_DF64];
+        if (!c.valid && !c.links.p && g->ctx->used.load() + need > g->ctx->budget / 2) return QDD_OK;
+    }
+    qdd_status st = ensure_copy(g, QDD_PREC_DF64, s);
+    if (st != QDD_OK && !required && (st == QDD_EBUDGET || st == QDD_ENOMEM)) {
+        clear_error();
+        return QDD_OK;
+    }
+    QDD_TRY(st);
+    *ok = true;
     return QDD_OK;
 }
 
@@ -405,11 +431,12 @@ qdd_status qdd_create_gauge_field(qdd_ctx *ctx, const int L[4], const int dom[4]
     QDD_TRY(launch_links_to_internal(g.get(), src, 0));
     // SU(3) links (to rounding) let the full-lattice operator read two rows per link
     DevMem bad;
-    QDD_TRY(bad.alloc(ctx, sizeof(int)));
+    QDD_TRY(bad.alloc(ctx, 2 * sizeof(int)));
     QDD_TRY(launch_su3_check(g.get(), kSu3Tol, bad.as<int>(), 0));
-    int h_bad = 1;
-    QDD_CUDA(cudaMemcpy(&h_bad, bad.p, sizeof(int), cudaMemcpyDeviceToHost));
-    g->su3 = h_bad == 0;
+    int h_bad[2] = {1, 0};
+    QDD_CUDA(cudaMemcpy(h_bad, bad.p, sizeof(h_bad), cudaMemcpyDeviceToHost));
+    g->su3 = h_bad[0] == 0;
+    g->link_exp = h_bad[1] == 0x7ff ? 1 << 20 : std::max(h_bad[1] - 1022, -800);
     g->two_rows = g->su3;
     QDD_CUDA(cudaDeviceSynchronize());
     ctx->timer.resolve();
@@ -636,16 +663,27 @@ qdd_status qdd_apply_D(qdd_gauge *g, const double *in, double *out, int nrhs, qd
     double *dout = nullptr;
     QDD_TRY(stage_in(g, st->io, in, nrhs, on_device, s, &din));
     QDD_TRY(st->a.ensure(g->ctx, V * 12 * eb * nrhs));
-    QDD_TRY(st->b.ensure(g->ctx, V * 12 * eb * nrhs));
-    if (scaled) {
-        QDD_TRY(st->a_s.ensure(g->ctx, V * 4 * nrhs));
-        QDD_TRY(st->b_s.ensure(g->ctx, V * 4 * nrhs));
+    // FP64-class arithmetic in fixed point: the input is converted on its way
+    // in, the operator writes the host layout
+    bool fixed = false;
+    if (arith != QDD_PREC_F32) {
+        if (!g->have_clover) {
+            set_error("set_clover has not been called");
+            return QDD_EINVAL;
+        }
+        QDD_TRY(ensure_fixed(g, arith == QDD_PREC_DF64, s, &fixed));
     }
-    QDD_TRY(launch_spinor_in(g, din, st->a.p, st->a_s.as<float>(), prec, nrhs, s));
+    if (!fixed) QDD_TRY(st->b.ensure(g->ctx, V * 12 * eb * nrhs));
+    if (scaled || fixed) QDD_TRY(st->a_s.ensure(g->ctx, V * 4 * nrhs));
+    if (scaled) QDD_TRY(st->b_s.ensure(g->ctx, V * 4 * nrhs));
+    const FxField fxa{st->a.p, st->a_s.as<int>()};
+    if (fixed) QDD_TRY(launch_spinor_in_fx(g, din, fxa, nrhs, s));
+    else QDD_TRY(launch_spinor_in(g, din, st->a.p, st->a_s.as<float>(), prec, nrhs, s));
     // a sharded field: its boundary planes (FP64, host layout) move while the operator runs
     QDD_TRY(slab_dslash_begin(g, din, false, true, nrhs, s));
-    QDD_TRY(launch_dslash(g, arith, fp, st->a.p, st->a_s.as<float>(), prec, st->b.p, st->b_s.as<float>(), prec,
-                          nullptr, nrhs, s));
+    if (!fixed)
+        QDD_TRY(launch_dslash(g, arith, fp, st->a.p, st->a_s.as<float>(), prec, st->b.p, st->b_s.as<float>(), prec,
+                              nullptr, nrhs, s));
     // a sharded field corrects the output's boundary planes from the input
     // (FP64, host layout), so the host output must not reuse the input's staging
     DevMem &oio = g->slab ? st->c : st->io;
@@ -654,7 +692,8 @@ qdd_status qdd_apply_D(qdd_gauge *g, const double *in, double *out, int nrhs, qd
         return QDD_EINVAL;
     }
     QDD_TRY(stage_out(g, oio, out, nrhs, on_device, s, &dout));
-    QDD_TRY(launch_spinor_out(g, st->b.p, st->b_s.as<float>(), dout, prec, nrhs, s));
+    if (fixed) QDD_TRY(launch_dslash_fx(g, fxa, (double2 *)dout, true, nullptr, nrhs, s));
+    else QDD_TRY(launch_spinor_out(g, st->b.p, st->b_s.as<float>(), dout, prec, nrhs, s));
     QDD_TRY(slab_dslash_end(g, (double2 *)dout, false, nrhs, s));
     return finish_out(g, oio, out, nrhs, on_device, s);
 }

@@ -18,6 +18,7 @@
 // planes paired, one 8-byte load per two planes.
 #include <type_traits>
 
+#include "fixed.cuh"
 #include "internal.h"
 
 namespace qdd {
@@ -287,253 +288,373 @@ __global__ void __launch_bounds__(128, (dslash_min_blocks<R, SL>())) k_dslash(Ge
 }
 
 // ------------------------------------------------------------------------
-// Double-float operator: y = D x with every product and sum carried as a pair
-// of FP32 numbers (error-free transformations), from links and clover split
-// into hi + lo FP32 parts.  About 2^-46 relative accuracy at a fraction of the
-// cost of FP64 arithmetic on this GPU; used for w = D z_j in the Arnoldi step.
+// The FP64 operator (and the double-float precision's) in 64-bit fixed point
+// (fixed.cuh): y = D x, or b - D x, in FP64.  One thread per site; a hop's
+// colour products are three integer multiply-adds per real product, summed
+// exactly at the neighbour site's scale, rounded, and shifted to the largest
+// scale of the nine sites before the hops are added; the clover product keeps
+// the site's own scale; both are converted once and combined in FP64.
+//
+// Bound: integer multiply-adds 2520 per site (39 clocks of an SM at 64 lanes)
+// and about as many other integer operations, against 69 clocks for the
+// 1536 bytes per site at the measured HBM rate, where FP64 arithmetic takes 570
+// clocks (1140 instructions at 2 lanes).  TABLE_FX
+// The four directions are compiled once each, for both signs (a
+// runtime flag picks the transposed link and the signs): eight bodies would
+// not fit the instruction cache.
 
-__device__ __forceinline__ cdf ld_cdf(const float4 *p)
+__device__ __forceinline__ cfx ld_cfx(const int4 *p)
 {
-    float4 v = __ldg(p);
+    const int4 v = __ldg(p);
     return {{v.x, v.y}, {v.z, v.w}};
 }
 
-__device__ __forceinline__ cdf ld_in_df(const float2 *p)
-{
-    float2 v = __ldg(p);
-    return {{v.x, 0.f}, {v.y, 0.f}};
-}
-
-__device__ __forceinline__ cdf ld_in_df(const double2 *p)
-{
-    double2 v = __ldg(p);
-    return {df_from_double(v.x), df_from_double(v.y)};
-}
-
-// Spin structure of one hop in the chiral basis.  With u the upper and l the
-// lower two spins, (1 -+ gamma_mu) x projects to h = u -+ A l and the lower
-// spins of the result are -+ A^dagger (U h), where A is a 2x2 matrix of unit
-// complex numbers, anti-diagonal for x, y and diagonal for z, t:
-//   x: A = [[0, -i], [-i, 0]]   y: A = [[0, -1], [1, 0]]
-//   z: A = [[-i, 0], [0, i]]    t: A = 1
-// One direction and sign is therefore a swap flag, a rotate-by-i flag and
-// four signs.  The double-float operator runs one hop body driven by these
-// runtime values: eight inlined copies of its long double-float chains did
-// not fit the instruction cache.
-struct HopSpin {
-    bool swap, rot;
-    float p0, p1;  // h_0 = u_0 + p0 (rot ? i : 1) l_{swap}, h_1 = u_1 + p1 (rot ? i : 1) l_{1-swap}
-    float r0, r1;  // lower_0 += r0 (rot ? i : 1) w_{swap}, lower_1 += r1 (rot ? i : 1) w_{1-swap}
+// Fields of the fixed-point operator.
+struct FxArgs {
+    const int4 *U, *A, *x;    // links and clover in planes of 36, spinors in planes of 12
+    const int *ae, *xe;       // exponents: clover per site, spinors per right-hand side and site
+    int lsh;                  // scale of the links
+    const double2 *b;         // residual form: b - D x
+    double2 *out;             // internal planes, or (site_of) the host layout
+    const int *site_of;
+    bool a32;                 // host layout: out on a 32-byte boundary
 };
 
-__device__ __forceinline__ HopSpin hop_spin(int mu, int back)
+__device__ __forceinline__ double fx_unscale(fx v, int sh) { return ldexp((double)fx_join(v), -sh); }
+
+// A site that reads one kept in FP64 (non-finite or extreme values): D x of the
+// site in FP64 from the same fields.  Never on the ordinary path.
+__device__ __noinline__ void dslash_fx_raw(const Geom &g, const FxArgs &f, int64_t rbase, int64_t sbase, int d, int s,
+                                           double kappa, double2 *y)
 {
-    const bool swap = mu < 2, rot = (mu & 1) == 0;
-    const float s0 = mu == 3 ? 1.f : -1.f;  // A's row-0 entry = s0 (rot ? i : 1)
-    const float s1 = mu == 0 ? -1.f : 1.f;  // A's row-1 entry = s1 (rot ? i : 1)
-    const float t = back ? 1.f : -1.f;      // forward hop: h = u - A l; backward: h = u + A l
-    // rows of A^dagger: conjugate transpose; conjugation flips an imaginary unit
-    float d0 = swap ? s1 : s0, d1 = swap ? s0 : s1;
-    if (rot) {
-        d0 = -d0;
-        d1 = -d1;
-    }
-    return {swap, rot, t * s0, t * s1, t * d0, t * d1};
-}
-
-// sg * (rot ? i z : z), exact
-__device__ __forceinline__ cdf cdf_unit(bool rot, float sg, cdf z)
-{
-    df a = rot ? df_neg(z.im) : z.re;
-    df b = rot ? z.re : z.im;
-    return {{__fmul_rn(sg, a.hi), __fmul_rn(sg, a.lo)}, {__fmul_rn(sg, b.hi), __fmul_rn(sg, b.lo)}};
-}
-
-__device__ __forceinline__ cdf cdf_sel(bool c, cdf a, cdf b) { return c ? a : b; }
-
-// Two double-float multiply-accumulates at once, as the two lanes of paired
-// FP32 operations: each lane runs dfacc_mul_add's sequence of operations
-// (TwoProd by FMA, TwoSum, the error terms summed in the same order), so
-// each lane's result is the same bits as the scalar form.  Used for the two
-// spins of a half spinor, which share every link entry.
-struct dfacc2 {
-    float2 s, c;
-};
-
-__device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
-__device__ __forceinline__ float2 bc2(float v) { return make_float2(v, v); }
-
-__device__ __forceinline__ void dfacc2_mul_add(dfacc2 &acc, df x, float2 yhi, float2 ylo)
-{
-    const float2 xh = bc2(x.hi), xl = bc2(x.lo);
-    const float2 p = __fmul2_rn(xh, yhi);
-    float2 e = __ffma2_rn(xh, yhi, neg2(p));
-    e = __ffma2_rn(xh, ylo, e);
-    e = __ffma2_rn(xl, yhi, e);
-    // TwoSum(acc.s, p)
-    const float2 s = __fadd2_rn(acc.s, p);
-    const float2 bb = __fadd2_rn(s, neg2(acc.s));
-    const float2 t = __fadd2_rn(__fadd2_rn(acc.s, neg2(__fadd2_rn(s, neg2(bb)))), __fadd2_rn(p, neg2(bb)));
-    acc.s = s;
-    acc.c = __fadd2_rn(acc.c, __fadd2_rn(t, e));
-}
-
-// value of the pair's two accumulators (FastTwoSum per lane)
-__device__ __forceinline__ void dfacc2_value(const dfacc2 &a, df &v0, df &v1)
-{
-    const float2 s = __fadd2_rn(a.s, a.c);
-    const float2 e = __fadd2_rn(a.c, neg2(__fadd2_rn(s, neg2(a.s))));
-    v0 = {s.x, e.x};
-    v1 = {s.y, e.y};
-}
-
-// w = U h for both spins of the half spinor h (row-major U, the oriented
-// link), the two spins as the lanes of paired operations
-__device__ __forceinline__ void su3_mul_half_df2(const cdf *U, const cdf *h, cdf *w)
-{
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        dfacc2 re = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        dfacc2 im = re;
-#pragma unroll
-        for (int b = 0; b < 3; b++) {
-            const cdf u = U[a * 3 + b];
-            const cdf h0 = h[b], h1 = h[3 + b];
-            const float2 rhi = make_float2(h0.re.hi, h1.re.hi), rlo = make_float2(h0.re.lo, h1.re.lo);
-            const float2 ihi = make_float2(h0.im.hi, h1.im.hi), ilo = make_float2(h0.im.lo, h1.im.lo);
-            // cdfacc_mul_add<false>: re += u.re h.re, re += (-u.im) h.im, im += u.re h.im, im += u.im h.re
-            dfacc2_mul_add(re, u.re, rhi, rlo);
-            dfacc2_mul_add(re, df_neg(u.im), ihi, ilo);
-            dfacc2_mul_add(im, u.re, ihi, ilo);
-            dfacc2_mul_add(im, u.im, rhi, rlo);
+    cpx<double> acc[12], x[12], u[9];
+    for (int k = 0; k < 12; k++) acc[k] = mk(0.0, 0.0);
+    auto spinor = [&](int dd, int ss) {
+        const int e = f.xe[sbase + (int64_t)dd * g.Vd + ss];
+        for (int k = 0; k < 12; k++) {
+            const int4 w = f.x[rbase + ((int64_t)dd * 12 + k) * g.Vd + ss];
+            x[k] = e == kFxRaw ? mk(__hiloint2double(w.y, w.x), __hiloint2double(w.w, w.z))
+                               : mk(fx_unscale({w.x, w.y}, kFxSpinorBits - e), fx_unscale({w.z, w.w}, kFxSpinorBits - e));
         }
-        df r0, r1, i0, i1;
-        dfacc2_value(re, r0, r1);
-        dfacc2_value(im, i0, i1);
-        w[a] = {r0, i0};
-        w[3 + a] = {r1, i1};
-    }
-}
-
-// the double-float colour products with the two spins as paired lanes (the
-// 48^3x96 solve's operator class 44.41 -> 43.56 ms, the same solution bits)
-constexpr bool kPairedDf = true;
-
-// acc += hop contribution; U is the oriented link (U(n) for a forward hop,
-// U(n - mu)^dagger for a backward one), row-major
-__device__ __forceinline__ void hop_df_rt(const HopSpin &hs, const cdf *U, const cdf *x, cdfacc *acc)
-{
-    cdf h[6];
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        cdf l0 = x[6 + c], l1 = x[9 + c];
-        h[c] = cdf_add(x[c], cdf_unit(hs.rot, hs.p0, cdf_sel(hs.swap, l1, l0)));
-        h[3 + c] = cdf_add(x[3 + c], cdf_unit(hs.rot, hs.p1, cdf_sel(hs.swap, l0, l1)));
-    }
-    cdf w[6];
-    if constexpr (kPairedDf) {
-        su3_mul_half_df2(U, h, w);
-    } else {
-#pragma unroll
-        for (int sp = 0; sp < 2; sp++)
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                cdfacc t;
-                cdfacc_zero(t);
-#pragma unroll
-                for (int b = 0; b < 3; b++) cdfacc_mul_add<false>(t, U[a * 3 + b], h[sp * 3 + b]);
-                w[sp * 3 + a] = cdfacc_value(t);
-            }
-    }
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        cdf w0 = w[c], w1 = w[3 + c];
-        cdf b0 = cdf_unit(hs.rot, hs.r0, cdf_sel(hs.swap, w1, w0));
-        cdf b1 = cdf_unit(hs.rot, hs.r1, cdf_sel(hs.swap, w0, w1));
-        dfacc_add(acc[0 * 3 + c].re, w0.re); dfacc_add(acc[0 * 3 + c].im, w0.im);
-        dfacc_add(acc[1 * 3 + c].re, w1.re); dfacc_add(acc[1 * 3 + c].im, w1.im);
-        dfacc_add(acc[2 * 3 + c].re, b0.re); dfacc_add(acc[2 * 3 + c].im, b0.im);
-        dfacc_add(acc[3 * 3 + c].re, b1.re); dfacc_add(acc[3 * 3 + c].im, b1.im);
-    }
-}
-
-template <typename SI, int VD = 0>
-__global__ void __launch_bounds__(128, 4) k_dslash_df(Geom g0, const float4 *U, const float4 *A,
-                                                   const typename SI::T2 *in, double2 *out, df kappa)
-{
-    const Geom g = fixed_geom<VD>(g0);
-    int gi = blockIdx.x * blockDim.x + threadIdx.x;
-    if (gi >= g.V) return;
-    const int64_t rbase = (int64_t)blockIdx.y * g.V * 12;
-    int d, s;
-    lex_site(g, gi, d, s);
-    cdfacc acc[12];
-#pragma unroll
-    for (int k = 0; k < 12; k++) cdfacc_zero(acc[k]);
-#pragma unroll 1
+    };
     for (int dir = 0; dir < 8; dir++) {
         const int mu = dir >> 1, back = dir & 1;
-        uint16_t e = __ldg(g.nbl + s * 8 + dir);
-        int nd = (e & kCross) ? __ldg(g.nbd + d * 8 + dir) : d;
-        int ns = e & kSlotMask;
+        const uint16_t e = __ldg(g.nbl + s * 8 + dir);
+        const int nd = (e & kCross) ? __ldg(g.nbd + d * 8 + dir) : d, ns = e & kSlotMask;
         if (!(QDD_IN_RANGE(nd, 0, g.Nd) && QDD_IN_RANGE(ns, 0, g.Vd))) continue;
-        cdf x[12], u[9];
-        const typename SI::T2 *xp = in + rbase + (int64_t)nd * 12 * g.Vd + ns;
-#pragma unroll
-        for (int k = 0; k < 12; k++) x[k] = ld_in_df(xp + (int64_t)k * g.Vd);
-        const int ld = back ? nd : d, ls = back ? ns : s;
-        const float4 *up = U + ((int64_t)ld * 36 + mu * 9) * g.Vd + ls;
-#pragma unroll
+        spinor(nd, ns);
         for (int k = 0; k < 9; k++) {
-            // backward hop: element (a, b) of U^dagger is conj(U_ba)
-            const int src = back ? (k % 3) * 3 + k / 3 : k;
-            cdf v = ld_cdf(up + (int64_t)src * g.Vd);
-            u[k] = back ? cdf{v.re, df_neg(v.im)} : v;
+            const int4 w = f.U[((int64_t)(back ? nd : d) * 36 + mu * 9 + k) * g.Vd + (back ? ns : s)];
+            u[k] = mk(fx_unscale({w.x, w.y}, f.lsh), fx_unscale({w.z, w.w}, f.lsh));
         }
-        hop_df_rt(hop_spin(mu, back), u, x, acc);
+        switch (dir) {
+        case 0: hop<0, +1>(u, x, acc); break;
+        case 1: hop<0, -1>(u, x, acc); break;
+        case 2: hop<1, +1>(u, x, acc); break;
+        case 3: hop<1, -1>(u, x, acc); break;
+        case 4: hop<2, +1>(u, x, acc); break;
+        case 5: hop<2, -1>(u, x, acc); break;
+        case 6: hop<3, +1>(u, x, acc); break;
+        default: hop<3, -1>(u, x, acc); break;
+        }
     }
-    // y = A x - kappa * (hop sum), one chirality block per iteration; the
-    // block's hop sum is always hv[0..5] (the second block is shifted down)
-    cdf hv[12];
+    spinor(d, s);
+    const int a = f.ae[(int64_t)d * g.Vd + s];
+    cpx<double> m[18], z[6];
+    for (int blk = 0; blk < 2; blk++) {
+        for (int k = 0; k < 18; k++) {
+            const int4 w = f.A[((int64_t)d * 36 + blk * 18 + k) * g.Vd + s];
+            m[k] = mk(fx_unscale({w.x, w.y}, kFxCloverBits - a), fx_unscale({w.z, w.w}, kFxCloverBits - a));
+        }
+        herm6_mul(m, x + 6 * blk, z);
+        for (int k = 0; k < 6; k++)
+            y[6 * blk + k] = make_double2(fma(-kappa, acc[6 * blk + k].re, z[k].re), fma(-kappa, acc[6 * blk + k].im, z[k].im));
+    }
+}
+
+struct cfxsum {
+    int64_t re, im;
+};
+
+// lower spins += q a_mu^+ w for the product w of spin sp (q = -1 forward, +1
+// backward): the result's lower spin and unit factor of project()'s a_mu^+
+template <int MU>
+__device__ __forceinline__ void fx_lower(int sp, bool back, int64_t wr, int64_t wi, cfxsum &t)
+{
+    // a^+ w: x: (i w1, i w0); y: (w1, -w0); z: (i w0, -i w1); t: (w0, w1)
+    const bool rot = MU == 0 || MU == 2;
+    const bool neg = (MU == 1 && sp == 0) || (MU == 2 && sp == 1);
+    const int64_t br = rot ? -wi : wr, bi = rot ? wr : wi;
+    if (back != neg) { t.re += br; t.im += bi; }
+    else { t.re -= br; t.im -= bi; }
+}
+
+template <int MU>
+__device__ __forceinline__ void fx_hop_dir(const Geom &g, const FxArgs &f, int64_t rbase, int d, int s, int E,
+                                           const int *xe, cfxsum *acc)
+{
+#pragma unroll 1
+    for (int back = 0; back < 2; back++) {
+        const int dir = 2 * MU + back;
+        const uint16_t en = __ldg(g.nbl + s * 8 + dir);
+        const int nd = (en & kCross) ? __ldg(g.nbd + d * 8 + dir) : d, ns = en & kSlotMask;
+        if (!(QDD_IN_RANGE(nd, 0, g.Nd) && QDD_IN_RANGE(ns, 0, g.Vd))) continue;
+        const int sft = min(E - __ldg(xe + (int64_t)nd * g.Vd + ns), 63);
+        const int4 *xp = f.x + rbase + (int64_t)nd * 12 * g.Vd + ns;
+        // projection h = u + q (a_mu l), limb by limb (the limbs grow by one bit)
+        const int q = back ? 1 : -1;
+        cfx h[6];
 #pragma unroll
-    for (int k = 0; k < 12; k++) hv[k] = cdfacc_value(acc[k]);
-    const typename SI::T2 *xp = in + rbase + (int64_t)d * 12 * g.Vd + s;
-    const float4 *ap = A + (int64_t)d * 36 * g.Vd + s;
-    double2 *op = out + rbase + (int64_t)d * 12 * g.Vd + s;
-    const df mk_ = df_neg(kappa);
+        for (int c = 0; c < 3; c++) {
+            const cfx u0 = ld_cfx(xp + (int64_t)c * g.Vd), u1 = ld_cfx(xp + (int64_t)(3 + c) * g.Vd);
+            const cfx l0 = ld_cfx(xp + (int64_t)(6 + c) * g.Vd), l1 = ld_cfx(xp + (int64_t)(9 + c) * g.Vd);
+            auto add = [](fx a, int qq, fx b) -> fx { return {a.hi + qq * b.hi, a.lo + qq * b.lo}; };
+            auto tmi_ = [&](cfx u, cfx l, int qq) -> cfx { return {add(u.re, qq, l.im), add(u.im, -qq, l.re)}; };
+            if (MU == 0) { h[c] = tmi_(u0, l1, q); h[3 + c] = tmi_(u1, l0, q); }
+            else if (MU == 1) {
+                h[c] = {add(u0.re, -q, l1.re), add(u0.im, -q, l1.im)};
+                h[3 + c] = {add(u1.re, q, l0.re), add(u1.im, q, l0.im)};
+            } else if (MU == 2) { h[c] = tmi_(u0, l0, q); h[3 + c] = tmi_(u1, l1, -q); }
+            else {
+                h[c] = {add(u0.re, q, l0.re), add(u0.im, q, l0.im)};
+                h[3 + c] = {add(u1.re, q, l1.re), add(u1.im, q, l1.im)};
+            }
+        }
+        // forward: U h; backward: U^+ h (transposed link, the sign of its
+        // imaginary part moved to the half spinor)
+        const int4 *up = f.U + ((int64_t)(back ? nd : d) * 36 + MU * 9) * g.Vd + (back ? ns : s);
+        const int64_t sa = (back ? 1 : 3) * (int64_t)g.Vd, sb = (back ? 3 : 1) * (int64_t)g.Vd;
+        fx hr[6], hi[6];  // +-h.re (enters im), -+h.im (enters re)
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+            hr[k] = {h[k].re.hi * -q, h[k].re.lo * -q};
+            hi[k] = {h[k].im.hi * q, h[k].im.lo * q};
+        }
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            cfx u[3];
+#pragma unroll
+            for (int b = 0; b < 3; b++) u[b] = ld_cfx(up + a * sa + b * sb);
+#pragma unroll
+            for (int sp = 0; sp < 2; sp++) {
+                fxacc re = {0, 0}, im = {0, 0};
+#pragma unroll
+                for (int b = 0; b < 3; b++) {
+                    fx_mac(re, u[b].re, h[sp * 3 + b].re);
+                    fx_mac(re, u[b].im, hi[sp * 3 + b]);
+                    fx_mac(im, u[b].re, h[sp * 3 + b].im);
+                    fx_mac(im, u[b].im, hr[sp * 3 + b]);
+                }
+                const int64_t wr = fx_value(re) >> sft, wi = fx_value(im) >> sft;
+                acc[sp * 3 + a].re += wr;
+                acc[sp * 3 + a].im += wi;
+                // the lower spin fed by this one: the other for x, y; the same for z, t
+                const int lo = 6 + 3 * (MU < 2 ? 1 - sp : sp) + a;
+                fx_lower<MU>(sp, back != 0, wr, wi, acc[lo]);
+            }
+        }
+    }
+}
+
+template <bool RESID, bool HOST, int VD = 0>
+__global__ void __launch_bounds__(128, 3) k_dslash_fx(Geom g0, FxArgs f, double kappa)
+{
+    const Geom g = fixed_geom<VD>(g0);
+    const int gt = blockIdx.x * blockDim.x + threadIdx.x;
+    if (gt >= g.V) return;
+    const int64_t r = blockIdx.y, rbase = r * (int64_t)g.V * 12, sbase = r * (int64_t)g.V;
+    int d, s;
+    lex_site(g, gt, d, s);
+    const int gi = d * g.Vd + s;
+    const int *xe = f.xe + sbase;
+    // the common scale: the largest exponent of the site and its neighbours
+    const int e0 = __ldg(xe + gi);
+    int E = e0;
+#pragma unroll
+    for (int dir = 0; dir < 8; dir++) {
+        const uint16_t en = __ldg(g.nbl + s * 8 + dir);
+        const int nd = (en & kCross) ? __ldg(g.nbd + d * 8 + dir) : d, ns = en & kSlotMask;
+        if (QDD_IN_RANGE(nd, 0, g.Nd) && QDD_IN_RANGE(ns, 0, g.Vd)) E = max(E, __ldg(xe + (int64_t)nd * g.Vd + ns));
+    }
+    const double2 *bp = RESID ? f.b + rbase + (int64_t)d * 12 * g.Vd + s : nullptr;
+    double2 *op = HOST ? f.out + (r * g.V + __ldg(f.site_of + gi)) * 12 : f.out + rbase + (int64_t)d * 12 * g.Vd + s;
+    auto store6 = [&](int blk, double2 *y) {
+        if (RESID) {
+#pragma unroll
+            for (int k = 0; k < 6; k++) {
+                const double2 v = __ldg(bp + (int64_t)(6 * blk + k) * g.Vd);
+                y[k] = make_double2(v.x - y[k].x, v.y - y[k].y);
+            }
+        }
+        if (HOST && f.a32) {
+#pragma unroll
+            for (int k = 0; k < 6; k += 2) st_global_x4(op + 6 * blk + k, y[k], y[k + 1]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 6; k++) op[(int64_t)(6 * blk + k) * (HOST ? 1 : g.Vd)] = y[k];
+        }
+    };
+    if (E >= kFxRaw) {
+        double2 y[12];
+        dslash_fx_raw(g, f, rbase, sbase, d, s, kappa, y);
+        store6(0, y);
+        store6(1, y + 6);
+        return;
+    }
+    cfxsum acc[12];
+#pragma unroll
+    for (int k = 0; k < 12; k++) acc[k] = {0, 0};
+    fx_hop_dir<0>(g, f, rbase, d, s, E, xe, acc);
+    fx_hop_dir<1>(g, f, rbase, d, s, E, xe, acc);
+    fx_hop_dir<2>(g, f, rbase, d, s, E, xe, acc);
+    fx_hop_dir<3>(g, f, rbase, d, s, E, xe, acc);
+
+    const int ca = e0 + __ldg(f.ae + gi) + 2 * kFxLimb - kFxSpinorBits - kFxCloverBits;  // scale of the clover sums
+    const int ch = E + 2 * kFxLimb - kFxSpinorBits - f.lsh;  // scale of the hop sums
+    const int4 *xp = f.x + rbase + (int64_t)d * 12 * g.Vd + s;
+    const int4 *ap = f.A + (int64_t)d * 36 * g.Vd + s;
+    // one chirality block per iteration; the block's hop sum is acc[0..5] (the second is moved down)
 #pragma unroll 1
     for (int blk = 0; blk < 2; blk++) {
-        cdf x[6], m[18];
+        cfx x[6];
 #pragma unroll
-        for (int k = 0; k < 6; k++) x[k] = ld_in_df(xp + (int64_t)(6 * blk + k) * g.Vd);
-#pragma unroll
-        for (int k = 0; k < 18; k++) m[k] = ld_cdf(ap + (int64_t)(blk * 18 + k) * g.Vd);
-        cdfacc y[6];
-        df dg[6] = {m[0].re, m[0].im, m[1].re, m[1].im, m[2].re, m[2].im};
+        for (int k = 0; k < 6; k++) x[k] = ld_cfx(xp + (int64_t)(6 * blk + k) * g.Vd);
+        double2 y[6];
 #pragma unroll
         for (int i = 0; i < 6; i++) {
-            cdfacc_zero(y[i]);
-            dfacc_mul_add(y[i].re, dg[i], x[i].re);
-            dfacc_mul_add(y[i].im, dg[i], x[i].im);
-        }
-        int k = 3;
+            // row i: the diagonal, the upper entries b x_j, the lower ones conj(b) x_j
+            fxacc re = {0, 0}, im = {0, 0};
+            const cfx dd = ld_cfx(ap + (int64_t)(blk * 18 + (i >> 1)) * g.Vd);
+            const fx dg = (i & 1) ? dd.im : dd.re;
+            fx_mac(re, dg, x[i].re);
+            fx_mac(im, dg, x[i].im);
 #pragma unroll
-        for (int i = 0; i < 6; i++)
-#pragma unroll
-            for (int j = i + 1; j < 6; j++) {
-                cdfacc_mul_add<false>(y[i], m[k], x[j]);
-                cdfacc_mul_add<true>(y[j], m[k], x[i]);
-                k++;
+            for (int j = 0; j < 6; j++) {
+                if (j == i) continue;
+                const int lo = i < j ? i : j, up = i < j ? j : i;
+                const int k = 3 + lo * 5 - lo * (lo - 1) / 2 + (up - lo - 1);  // packed index of (lo, up)
+                const cfx m = ld_cfx(ap + (int64_t)(blk * 18 + k) * g.Vd);
+                const fx mi = j > i ? m.im : fx{-m.im.hi, -m.im.lo};
+                fx_mac(re, m.re, x[j].re);
+                fx_mac(im, m.re, x[j].im);
+                fx_mac(im, mi, x[j].re);
+                fx_mac(re, fx{-mi.hi, -mi.lo}, x[j].im);
             }
-#pragma unroll
-        for (int i = 0; i < 6; i++) {
-            dfacc_mul_add(y[i].re, mk_, hv[i].re);
-            dfacc_mul_add(y[i].im, mk_, hv[i].im);
-            cdf v = cdfacc_value(y[i]);
-            op[(int64_t)(6 * blk + i) * g.Vd] = make_double2(df_to_double(v.re), df_to_double(v.im));
-            hv[i] = hv[6 + i];
+            y[i] = make_double2(fma(-kappa, fx_to_double(acc[i].re, ch), fx_to_double(fx_value(re), ca)),
+                                fma(-kappa, fx_to_double(acc[i].im, ch), fx_to_double(fx_value(im), ca)));
         }
+        store6(blk, y);
+#pragma unroll
+        for (int i = 0; i < 6; i++) acc[i] = acc[6 + i];
     }
+}
+
+// A spinor field in internal planes (FP64 or FP32) into fixed point.
+template <typename SI>
+__global__ void __launch_bounds__(128) k_spinor_fx(Geom g, const typename SI::T2 *src, int4 *x, int *xe)
+{
+    const int gi = blockIdx.x * blockDim.x + threadIdx.x;
+    if (gi >= g.V) return;
+    const int64_t r = blockIdx.y, rbase = r * (int64_t)g.V * 12;
+    int d, s;
+    split_index(g, gi, d, s);
+    cpx<double> v[12];
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+        const typename SI::T2 a = __ldg(src + rbase + ((int64_t)d * 12 + k) * g.Vd + s);
+        if constexpr (SI::kBytes == 16) v[k] = mk((double)a.x, (double)a.y);
+        else v[k] = mk(f2d(a.x), f2d(a.y));
+    }
+    fx_store_site(x + rbase + (int64_t)d * 12 * g.Vd, s, g.Vd, xe + r * g.V + gi, v);
+}
+
+// Links (one scale) and clover (a scale per site) into fixed point.
+__global__ void k_links_fx(int64_t n, const double2 *src, int4 *dst, int lsh)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double2 a = __ldg(src + i);
+    // |U| < 2^(61 - lsh) here; rounded at 2^-lsh
+    auto conv = [&](double v) {
+        const int ex = fx_exponent(v);
+        const uint32_t hi = (uint32_t)__double2hiint(v);
+        const uint64_t m = ex ? ((uint64_t)((hi & 0x000fffffu) | 0x00100000u) << 32 | (uint32_t)__double2loint(v)) : 0;
+        const int sh = ex - 1075 + lsh;  // v 2^lsh = m 2^sh
+        const uint64_t x = sh >= 0 ? m << sh : (sh > -63 ? (m + (1ull << (-sh - 1))) >> -sh : 0);
+        return fx_split((int32_t)hi < 0 ? -(int64_t)x : (int64_t)x);
+    };
+    const fx re = conv(a.x), im = conv(a.y);
+    dst[i] = make_int4(re.hi, re.lo, im.hi, im.lo);
+}
+
+__global__ void __launch_bounds__(128) k_clover_fx(Geom g, const double2 *src, int4 *dst, int *ae)
+{
+    const int gi = blockIdx.x * blockDim.x + threadIdx.x;
+    if (gi >= g.V) return;
+    int d, s;
+    split_index(g, gi, d, s);
+    const double2 *p = src + (int64_t)d * 36 * g.Vd + s;
+    int emax = 1;
+    for (int k = 0; k < 36; k++) {
+        const double2 a = __ldg(p + (int64_t)k * g.Vd);
+        emax = max(emax, max(fx_exponent(a.x), fx_exponent(a.y)));
+    }
+    ae[gi] = emax - 1022;
+    int4 *q = dst + (int64_t)d * 36 * g.Vd + s;
+    for (int k = 0; k < 36; k++) {
+        const double2 a = __ldg(p + (int64_t)k * g.Vd);
+        const fx re = fx_from_double(a.x, emax, kFxCloverBits), im = fx_from_double(a.y, emax, kFxCloverBits);
+        q[(int64_t)k * g.Vd] = make_int4(re.hi, re.lo, im.hi, im.lo);
+    }
+}
+
+qdd_status launch_fields_fx(Gauge *g, PrecCopy &c, cudaStream_t s)
+{
+    const int64_t n = (int64_t)g->hg.V * 36;
+    LaunchScope ls(g->ctx->timer, K_OTHER, s);
+    k_links_fx<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, g->links64.as<double2>(), c.links.as<int4>(),
+                                                           fx_link_shift(g));
+    k_clover_fx<<<(g->hg.V + 127) / 128, 128, 0, s>>>(g->geom, g->clov64.as<double2>(), c.clov.as<int4>(),
+                                                      c.clov_s.as<int>());
+    QDD_CUDA(cudaGetLastError());
+    return QDD_OK;
+}
+
+qdd_status launch_spinor_fx(Gauge *g, const void *src, qdd_prec ip, const FxField &x, int nrhs, cudaStream_t s)
+{
+    const dim3 grid((g->hg.V + 127) / 128, nrhs);
+    LaunchScope ls(g->ctx->timer, K_DSLASH, s);
+    if (ip == QDD_PREC_F64) k_spinor_fx<StF64><<<grid, 128, 0, s>>>(g->geom, (const double2 *)src, (int4 *)x.x, x.e);
+    else if (ip == QDD_PREC_F32) k_spinor_fx<StF32><<<grid, 128, 0, s>>>(g->geom, (const float2 *)src, (int4 *)x.x, x.e);
+    else {
+        set_error("the fixed-point operator takes FP32 or FP64 spinors");
+        return QDD_EINVAL;
+    }
+    QDD_CUDA(cudaGetLastError());
+    return QDD_OK;
+}
+
+qdd_status launch_dslash_fx(Gauge *g, const FxField &x, double2 *out, bool host_layout, const double2 *b, int nrhs,
+                            cudaStream_t s)
+{
+    const PrecCopy &c = g->copies[QDD_PREC_DF64];
+    FxArgs f{c.links.as<int4>(), c.clov.as<int4>(), (const int4 *)x.x, c.clov_s.as<int>(), x.e, fx_link_shift(g), b,
+             out, host_layout ? g->d_site_of.as<int>() : nullptr, ((uintptr_t)out & 31) == 0};
+    const dim3 grid((g->hg.V + 127) / 128, nrhs);
+    LaunchScope ls(g->ctx->timer, K_DSLASH, s);
+    const bool v256 = g->hg.Vd == 256;  // 4^4 domains: the volume fixed at compile time
+    if (b) {
+        if (v256) k_dslash_fx<true, false, 256><<<grid, 128, 0, s>>>(g->geom, f, g->kappa);
+        else k_dslash_fx<true, false><<<grid, 128, 0, s>>>(g->geom, f, g->kappa);
+    } else if (host_layout) {
+        if (v256) k_dslash_fx<false, true, 256><<<grid, 128, 0, s>>>(g->geom, f, g->kappa);
+        else k_dslash_fx<false, true><<<grid, 128, 0, s>>>(g->geom, f, g->kappa);
+    } else {
+        if (v256) k_dslash_fx<false, false, 256><<<grid, 128, 0, s>>>(g->geom, f, g->kappa);
+        else k_dslash_fx<false, false><<<grid, 128, 0, s>>>(g->geom, f, g->kappa);
+    }
+    QDD_CUDA(cudaGetLastError());
+    return QDD_OK;
 }
 
 // out-of-range indices the kernels of this file have skipped (QDD_CHECK builds)
@@ -580,13 +701,25 @@ static qdd_status run_dslash_lowp(Gauge *g, qdd_prec fp, Field<SC> A, const void
 }
 
 qdd_status launch_dslash(Gauge *g, qdd_prec arith, qdd_prec fp, const void *in, const float *in_s, qdd_prec ip,
-                         void *out, float *out_s, qdd_prec op, const double2 *b, int nrhs, cudaStream_t s)
+                         void *out, float *out_s, qdd_prec op, const double2 *b, int nrhs, cudaStream_t s,
+                         const FxField *fxb)
 {
     if (!g->have_clover) {
         set_error("set_clover has not been called");
         return QDD_EINVAL;
     }
-    if (arith == QDD_PREC_F64) {
+    // FP64-class arithmetic: in fixed point when the caller has a fixed-point
+    // buffer and the fields have their fixed-point copy, else in FP64
+    if (arith == QDD_PREC_F64 || arith == QDD_PREC_DF64) {
+        if (fp == QDD_PREC_DF64) fp = QDD_PREC_F64;
+        if (fxb && op == QDD_PREC_F64 && (ip == QDD_PREC_F64 || ip == QDD_PREC_F32)) {
+            bool ok = false;
+            QDD_TRY(ensure_fixed(g, arith == QDD_PREC_DF64, s, &ok));
+            if (ok) {
+                QDD_TRY(launch_spinor_fx(g, in, ip, *fxb, nrhs, s));
+                return launch_dslash_fx(g, *fxb, (double2 *)out, false, b, nrhs, s);
+            }
+        }
         if (fp != QDD_PREC_F64 || op != QDD_PREC_F64) {
             set_error("FP64 operator needs FP64 fields and output");
             return QDD_EINVAL;
@@ -601,31 +734,6 @@ qdd_status launch_dslash(Gauge *g, qdd_prec arith, qdd_prec fp, const void *in, 
             return run_dslash<double, StF64, StF64, StF32, StF64, false>(g, U, A, in, in_s, out, out_s, b, nrhs, s);
         default: break;
         }
-    } else if (arith == QDD_PREC_DF64 && !b && op == QDD_PREC_F64) {
-        QDD_TRY(ensure_copy(g, QDD_PREC_DF64, s));
-        PrecCopy &c = g->copies[QDD_PREC_DF64];
-        dim3 grid((g->hg.V + 127) / 128, nrhs);
-        df kap = {(float)g->kappa, (float)(g->kappa - (double)(float)g->kappa)};
-        LaunchScope ls(g->ctx->timer, K_DSLASH, s);
-        const bool v256 = g->hg.Vd == 256;  // 4^4 domains: the volume fixed at compile time
-        if (ip == QDD_PREC_F32 && v256)
-            k_dslash_df<StF32, 256><<<grid, 128, 0, s>>>(g->geom, c.links.as<float4>(), c.clov.as<float4>(),
-                                                         (const float2 *)in, (double2 *)out, kap);
-        else if (ip == QDD_PREC_F32)
-            k_dslash_df<StF32><<<grid, 128, 0, s>>>(g->geom, c.links.as<float4>(), c.clov.as<float4>(),
-                                                    (const float2 *)in, (double2 *)out, kap);
-        else if (ip == QDD_PREC_F64 && v256)
-            k_dslash_df<StF64, 256><<<grid, 128, 0, s>>>(g->geom, c.links.as<float4>(), c.clov.as<float4>(),
-                                                         (const double2 *)in, (double2 *)out, kap);
-        else if (ip == QDD_PREC_F64)
-            k_dslash_df<StF64><<<grid, 128, 0, s>>>(g->geom, c.links.as<float4>(), c.clov.as<float4>(),
-                                                    (const double2 *)in, (double2 *)out, kap);
-        else {
-            set_error("double-float operator takes FP32 or FP64 input");
-            return QDD_EINVAL;
-        }
-        QDD_CUDA(cudaGetLastError());
-        return QDD_OK;
     } else if (arith == QDD_PREC_F32 && !b) {
         QDD_TRY(ensure_copy(g, fp, s));
         PrecCopy &c = g->copies[fp];

@@ -162,6 +162,8 @@ struct HostGeom {
 qdd_status make_geometry(const int L[4], const int dom[4], HostGeom &hg);
 
 // A lower-precision copy of the fields the operator and the preconditioner read.
+// The copy of QDD_PREC_DF64 holds links and clover in fixed point (fixed.cuh),
+// the clover's exponents in clov_s.
 struct PrecCopy {
     bool valid = false;
     DevMem links, clov, clov_s, sclov, sclov_s;
@@ -215,6 +217,7 @@ struct Gauge {
     DevMem d_nbl, d_nbd, d_site_of, d_block_slot, d_fcoord;
     DevMem links64;           // FP64 links, internal layout
     bool su3 = false;         // every link SU(3) to kSu3Tol
+    int link_exp = 1 << 20;   // every link entry below 2^link_exp in magnitude (huge when one is not finite)
     bool two_rows = false;    // the FP32/16-bit full-lattice operator reads two rows per link
     bool have_clover = false;
     int sap_variant = 0;      // Schwarz kernel form (qdd_set_schwarz_variant)
@@ -244,10 +247,18 @@ __host__ __device__ __forceinline__ int64_t pair_index(int64_t d, int P, int p, 
 }
 
 qdd_status ensure_copy(Gauge *g, qdd_prec prec, cudaStream_t s);
+// The fixed-point copy of links and clover (the copy of QDD_PREC_DF64).  *ok =
+// false, with QDD_OK, where FP64 arithmetic has to stand in: links that are not
+// finite or very large, or (required = false: the FP64 precision, which needs
+// no copy) an HBM budget that the copy would fill past a half.
+qdd_status ensure_fixed(Gauge *g, bool required, cudaStream_t s, bool *ok);
 // the two-row link copy of a storage precision (FP32, FP16, BF16)
 qdd_status ensure_links12(Gauge *g, qdd_prec prec, cudaStream_t s);
 // links whose unitarity and determinant deviate by more than this keep three rows
 constexpr double kSu3Tol = 1e-10;
+
+// scale of a field's fixed-point links (fixed.cuh)
+inline int fx_link_shift(const Gauge *g) { return g->su3 ? 60 : 58 - g->link_exp; }
 
 // storage of the spinors and of the links/clover copy a precision mode uses
 inline qdd_prec spinor_store(qdd_prec p) { return p == QDD_PREC_H16 ? QDD_PREC_F32 : p; }
@@ -259,8 +270,17 @@ inline bool is_sap_prec(qdd_prec p)
 
 // ------------------------------------------------------------- launchers
 
+// A spinor field in fixed point (fixed.cuh): x takes 16 bytes per complex
+// component (as FP64 does), e one exponent per site, of every right-hand side.
+struct FxField {
+    void *x;
+    int *e;
+};
+
 // layout.cu
 qdd_status launch_links_to_internal(Gauge *g, const double *links_host_layout_dev, cudaStream_t s);
+// host-layout FP64 spinors (device) -> fixed point
+qdd_status launch_spinor_in_fx(Gauge *g, const double *src, const FxField &x, int nrhs, cudaStream_t s);
 // host-layout FP64 spinors (device) <-> internal fields of storage prec
 qdd_status launch_spinor_in(Gauge *g, const double *src, void *dst, float *dst_scale, qdd_prec prec, int nrhs,
                             cudaStream_t s);
@@ -278,20 +298,28 @@ qdd_status launch_links_convert(Gauge *g, qdd_prec dp, void *dst, cudaStream_t s
 // paired: the full-lattice operator's copy (16-bit formats in paired-plane order)
 qdd_status launch_clover_convert(Gauge *g, const double2 *src, qdd_prec dp, void *dst, float *dst_scale,
                                  cudaStream_t s, bool paired = false);
-// *d_bad = 1 when some link is not SU(3) to tol; two-row copy of the links
-qdd_status launch_su3_check(Gauge *g, double tol, int *d_bad, cudaStream_t s);
+// d_out[0] = 1 when some link is not SU(3) to tol; d_out[1] = the largest FP64
+// exponent field of the link entries; two-row copy of the links
+qdd_status launch_su3_check(Gauge *g, double tol, int *d_out, cudaStream_t s);
 qdd_status launch_links12_convert(Gauge *g, qdd_prec dp, void *dst, cudaStream_t s);
-// FP64 complex -> double-float (hi, lo) pairs
-qdd_status launch_split_convert(Gauge *g, const double2 *src, float4 *dst, int64_t n, cudaStream_t s);
 
 // clover.cu
 qdd_status launch_clover_build(Gauge *g, double csw, double kappa, int *d_singular, cudaStream_t s);
 
-// dslash.cu: out = D in (or out = b - D in when b != NULL); arith F64 or F32;
-// in_prec/out_prec the storage of the spinors; link/clover storage = fields_prec.
+// dslash.cu: out = D in (or out = b - D in when b != NULL); arith F64, DF64 or
+// F32; in_prec/out_prec the storage of the spinors; link/clover storage =
+// fields_prec.  fxb: a buffer (not in, out or b) for the input in fixed point,
+// which the FP64-class arithmetics then use.
 qdd_status launch_dslash(Gauge *g, qdd_prec arith, qdd_prec fields_prec, const void *in, const float *in_s,
                          qdd_prec in_prec, void *out, float *out_s, qdd_prec out_prec, const double2 *b, int nrhs,
-                         cudaStream_t s);
+                         cudaStream_t s, const FxField *fxb = nullptr);
+// the parts of the fixed-point operator: the fields' copy, a spinor field in
+// internal FP64 or FP32 planes, the operator (out in internal planes or in the
+// host layout; b: residual form, internal planes only)
+qdd_status launch_fields_fx(Gauge *g, PrecCopy &c, cudaStream_t s);
+qdd_status launch_spinor_fx(Gauge *g, const void *src, qdd_prec ip, const FxField &x, int nrhs, cudaStream_t s);
+qdd_status launch_dslash_fx(Gauge *g, const FxField &x, double2 *out, bool host_layout, const double2 *b, int nrhs,
+                            cudaStream_t s);
 
 // sap.cu: one half-sweep over the domains of `colour`
 struct SapBuffers {

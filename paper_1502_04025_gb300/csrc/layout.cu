@@ -11,6 +11,7 @@
 #include <cstdio>
 #include <cstring>
 
+#include "fixed.cuh"
 #include "internal.h"
 
 namespace qdd {
@@ -305,6 +306,21 @@ __global__ void k_links_in(Geom g, const int *site_of, const double2 *src, doubl
     for (int k = 0; k < 36; k++) dst[((int64_t)d * 36 + k) * g.Vd + s] = __ldg(p + k);
 }
 
+// the 12 components of a site in the host layout
+__device__ __forceinline__ void ld_host_site(const double2 *p, bool a32, cpx<double> *v)
+{
+    double2 a[12];
+    if (a32) {
+#pragma unroll
+        for (int k = 0; k < 12; k += 2) ld_global_x4(p + k, a[k], a[k + 1]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 12; k++) a[k] = __ldg(p + k);
+    }
+#pragma unroll
+    for (int k = 0; k < 12; k++) v[k] = mk(a[k].x, a[k].y);
+}
+
 template <typename S>
 __global__ void __launch_bounds__(kSiteThreads) k_spinor_in(Geom g, const int *site_of, const double2 *src,
                                                             Field<S> dst, int64_t rstride, int64_t sstride, bool a32)
@@ -314,19 +330,23 @@ __global__ void __launch_bounds__(kSiteThreads) k_spinor_in(Geom g, const int *s
     int r = blockIdx.y;
     int d, s;
     split_index(g, gi, d, s);
-    const double2 *p = src + ((int64_t)r * g.V + __ldg(site_of + gi)) * 12;
-    double2 a[12];
-    if (a32) {
-#pragma unroll
-        for (int k = 0; k < 12; k += 2) ld_global_x4(p + k, a[k], a[k + 1]);
-    } else {
-#pragma unroll
-        for (int k = 0; k < 12; k++) a[k] = __ldg(p + k);
-    }
     cpx<double> v[12];
-#pragma unroll
-    for (int k = 0; k < 12; k++) v[k] = mk(a[k].x, a[k].y);
+    ld_host_site(src + ((int64_t)r * g.V + __ldg(site_of + gi)) * 12, a32, v);
     store_spinor<S>(dst, r * rstride, r * sstride, g.Vd, d, s, v);
+}
+
+// the same into fixed point
+__global__ void __launch_bounds__(kSiteThreads) k_spinor_in_fx(Geom g, const int *site_of, const double2 *src, int4 *x,
+                                                               int *xe, bool a32)
+{
+    int gi = blockIdx.x * blockDim.x + threadIdx.x;
+    if (gi >= g.V) return;
+    const int64_t r = blockIdx.y;
+    int d, s;
+    split_index(g, gi, d, s);
+    cpx<double> v[12];
+    ld_host_site(src + (r * g.V + __ldg(site_of + gi)) * 12, a32, v);
+    fx_store_site(x + (r * g.V + (int64_t)d * g.Vd) * 12, s, g.Vd, xe + r * g.V + gi, v);
 }
 
 template <typename S>
@@ -404,19 +424,10 @@ __global__ void k_links_convert(int64_t n, const double2 *src, typename S::T2 *d
     st_d(dst + i, mk(a.x, a.y));
 }
 
-// FP64 complex -> (re.hi, re.lo, im.hi, im.lo) FP32 split
-__global__ void k_split_convert(int64_t n, const double2 *src, float4 *dst)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double2 a = __ldg(src + i);
-    float rh = __double2float_rn(a.x), ih = __double2float_rn(a.y);
-    dst[i] = make_float4(rh, __double2float_rn(a.x - (double)rh), ih, __double2float_rn(a.y - (double)ih));
-}
-
-// Sets *bad when a link is not SU(3) to tol: max |(U U^+ - 1)_ij| or |det U - 1|.
+// Sets out[0] when a link is not SU(3) to tol: max |(U U^+ - 1)_ij| or
+// |det U - 1|; out[1] = the largest FP64 exponent field of the link entries.
 // One thread per link (domain d, direction mu, site s).
-__global__ void k_su3_check(Geom g, const double2 *U, double tol, int *bad)
+__global__ void k_su3_check(Geom g, const double2 *U, double tol, int *out)
 {
     const int64_t li = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (li >= (int64_t)g.V * 4) return;
@@ -438,7 +449,10 @@ __global__ void k_su3_check(Geom g, const double2 *U, double tol, int *bad)
     cpx<double> det = u[0] * (u[4] * u[8] - u[5] * u[7]) - u[1] * (u[3] * u[8] - u[5] * u[6]) +
                       u[2] * (u[3] * u[7] - u[4] * u[6]);
     dev = fmax(dev, fmax(fabs(det.re - 1.0), fabs(det.im)));
-    if (!(dev <= tol)) atomicOr(bad, 1);
+    if (!(dev <= tol)) atomicOr(out, 1);
+    int ex = 0;
+    for (int k = 0; k < 9; k++) ex = max(ex, max(fx_exponent(u[k].re), fx_exponent(u[k].im)));
+    if (ex > *(volatile int *)(out + 1)) atomicMax(out + 1, ex);
 }
 
 // The first two rows of every link: 24 planes per site, plane mu*6 + 3*row + col
@@ -527,6 +541,16 @@ qdd_status launch_spinor_in(Gauge *g, const double *src, void *dst, float *dst_s
     return QDD_OK;
 }
 
+qdd_status launch_spinor_in_fx(Gauge *g, const double *src, const FxField &x, int nrhs, cudaStream_t s)
+{
+    const HostGeom &hg = g->hg;
+    LaunchScope ls(g->ctx->timer, K_OTHER, s);
+    k_spinor_in_fx<<<grid_sites(hg.V, nrhs, kSiteThreads), kSiteThreads, 0, s>>>(
+        g->geom, g->d_site_of.as<int>(), (const double2 *)src, (int4 *)x.x, x.e, ((uintptr_t)src & 31) == 0);
+    QDD_CUDA(cudaGetLastError());
+    return QDD_OK;
+}
+
 qdd_status launch_spinor_out(Gauge *g, const void *src, const float *src_scale, double *dst, qdd_prec prec, int nrhs,
                              cudaStream_t s)
 {
@@ -592,12 +616,12 @@ qdd_status launch_links_convert(Gauge *g, qdd_prec dp, void *dst, cudaStream_t s
     return QDD_OK;
 }
 
-qdd_status launch_su3_check(Gauge *g, double tol, int *d_bad, cudaStream_t s)
+qdd_status launch_su3_check(Gauge *g, double tol, int *d_out, cudaStream_t s)
 {
     const int64_t n = (int64_t)g->hg.V * 4;
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
-    QDD_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), s));
-    k_su3_check<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g->geom, g->links64.as<double2>(), tol, d_bad);
+    QDD_CUDA(cudaMemsetAsync(d_out, 0, 2 * sizeof(int), s));
+    k_su3_check<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g->geom, g->links64.as<double2>(), tol, d_out);
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
 }
@@ -609,14 +633,6 @@ qdd_status launch_links12_convert(Gauge *g, qdd_prec dp, void *dst, cudaStream_t
         k_links12_convert<S><<<grid_sites(g->hg.V, 1, 256), 256, 0, s>>>(g->geom, g->links64.as<double2>(),
                                                                           (typename S::T2 *)dst);
     });
-    QDD_CUDA(cudaGetLastError());
-    return QDD_OK;
-}
-
-qdd_status launch_split_convert(Gauge *g, const double2 *src, float4 *dst, int64_t n, cudaStream_t s)
-{
-    LaunchScope ls(g->ctx->timer, K_OTHER, s);
-    k_split_convert<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, src, dst);
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
 }

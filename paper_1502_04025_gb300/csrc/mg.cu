@@ -720,7 +720,8 @@ static qdd_status mg_vcycle_with(Gauge *g, Multigrid &M, const double2 *v, void 
     if (M.p.post_ncy > 0) {
         // r = v - D z, then z += M_SAP r
         const qdd_prec ar = zp == QDD_PREC_F64 ? QDD_PREC_F64 : QDD_PREC_F32;
-        QDD_TRY(launch_dslash(g, ar, ar, z, nullptr, zp, M.t64.p, nullptr, QDD_PREC_F64, nullptr, 1, s));
+        const FxField fxb{M.r64.p, M.rho.as<int>()};  // both are written after the operator
+        QDD_TRY(launch_dslash(g, ar, ar, z, nullptr, zp, M.t64.p, nullptr, QDD_PREC_F64, nullptr, 1, s, &fxb));
         {
             LaunchScope ls(g->ctx->timer, K_SAP, s);
             k_mg_sub<<<(int)((nfine + 255) / 256), 256, 0, s>>>(v, M.t64.as<double2>(), M.r64.as<double2>(), nfine);

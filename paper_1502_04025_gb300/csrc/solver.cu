@@ -66,6 +66,7 @@ size_t workspace_bytes(const Gauge *g, int m, int B, qdd_prec sp, bool use_sap, 
         b += n * ebytes(spinor_store(sp)) * B + sap_face_bytes(g->hg, sp, B);
         if (sp == QDD_PREC_F16S || sp == QDD_PREC_BF16S) b += V * 4 * B;
     }
+    else b += V * 4 * B;  // the operator's exponents (ensure_ws)
     if (kdr > 0) b += n * 16 * B * (size_t)(3 * kdr + 1);
     return b + (1 << 20);
 }
@@ -109,6 +110,10 @@ static qdd_status ensure_ws(Gauge *g, Workspace &w, int m, int B, qdd_prec sp, b
     }
     ScalarMap sm{m, B};
     QDD_TRY(w.dev.ensure(c, sm.total() * sizeof(double2)));
+    // exponents of the operator's fixed-point input, whose components take the
+    // host-transfer buffer between the input and the output: the Schwarz
+    // method's residual, consumed by then, where there is one
+    if (!use_sap) QDD_TRY(w.rho.ensure(c, V * sizeof(int) * B));
     QDD_TRY(blas_scratch_ensure(c, w.scratch));
     QDD_TRY(w.err.ensure(c, sizeof(int)));
     if (w.host_elems < sm.total()) {
@@ -129,6 +134,8 @@ qdd_status solve_prepare(Gauge *g, Workspace *w, const qdd_solve_params *p, cuda
     QDD_TRY(ensure_ws(g, *w, p->restart_m, p->nrhs, sp, p->use_sap == 1, p->dr_k));
     if (p->use_sap) QDD_TRY(ensure_copy(g, sp, s));
     if (p->arnoldi_prec != QDD_PREC_F64) QDD_TRY(ensure_copy(g, p->arnoldi_prec, s));
+    bool fixed = false;  // the FP64 operator's optional fixed-point copy (the true residual is always FP64)
+    QDD_TRY(ensure_fixed(g, false, s, &fixed));
     if (p->relax_eta > 0 || p->arnoldi_prec == QDD_PREC_F32) {
         QDD_TRY(ensure_copy(g, QDD_PREC_F32, s));
         if (g->two_rows) QDD_TRY(ensure_links12(g, QDD_PREC_F32, s));
@@ -235,6 +242,7 @@ qdd_status solve_impl(Gauge *g, Workspace *wsp, const double *b_in, double *x_ou
     int iters = 0, restarts = 0, deflated = 0;
     bool converged = false;
     qdd_status status = QDD_OK;
+    const FxField fxb{w.io.p, w.rho.as<int>()};  // the operator's input in fixed point
     SapBuffers sb{w.rho.p, w.face.p, nullptr, w.rho_s.as<float>()};
     double2 *ZR = w.ZR.as<double2>();
 
@@ -245,7 +253,7 @@ qdd_status solve_impl(Gauge *g, Workspace *wsp, const double *b_in, double *x_ou
         else {
             QDD_TRY(slab_dslash_begin(g, X, false, false, B, s));  // sharded: boundary planes
             QDD_TRY(launch_dslash(g, QDD_PREC_F64, QDD_PREC_F64, X, nullptr, QDD_PREC_F64, pending_dr ? w.Vt.as<double2>() : V,
-                                  nullptr, QDD_PREC_F64, Bv, B, s));
+                                  nullptr, QDD_PREC_F64, Bv, B, s, &fxb));
             QDD_TRY(slab_dslash_end(g, V, true, B, s));
         }
         double2 *R0 = (cycle > 0 && pending_dr) ? w.Vt.as<double2>() : V;
@@ -435,7 +443,7 @@ qdd_status solve_impl(Gauge *g, Workspace *wsp, const double *b_in, double *x_ou
                                       QDD_PREC_F64, nullptr, B, s));
             else if (p->arnoldi_prec == QDD_PREC_F64 || p->arnoldi_prec == QDD_PREC_DF64)
                 QDD_TRY(launch_dslash(g, p->arnoldi_prec, p->arnoldi_prec, zj, nullptr, zp, wv, nullptr,
-                                      QDD_PREC_F64, nullptr, B, s));
+                                      QDD_PREC_F64, nullptr, B, s, &fxb));
             else
                 QDD_TRY(launch_dslash(g, QDD_PREC_F32, QDD_PREC_F32, zj, nullptr, QDD_PREC_F32, wv, nullptr,
                                       QDD_PREC_F64, nullptr, B, s));
