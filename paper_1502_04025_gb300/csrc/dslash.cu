@@ -376,17 +376,19 @@ struct cfxsum {
     int64_t re, im;
 };
 
-// lower spins += q a_mu^+ w for the product w of spin sp (q = -1 forward, +1
-// backward): the result's lower spin and unit factor of project()'s a_mu^+
+// t += a_mu^+ w, the part of the product w of spin sp, with project()'s a_mu
 template <int MU>
-__device__ __forceinline__ void fx_lower(int sp, bool back, int64_t wr, int64_t wi, cfxsum &t)
+__device__ __forceinline__ void fx_lower(int sp, int64_t wr, int64_t wi, cfxsum &t)
 {
     // a^+ w: x: (i w1, i w0); y: (w1, -w0); z: (i w0, -i w1); t: (w0, w1)
-    const bool rot = MU == 0 || MU == 2;
     const bool neg = (MU == 1 && sp == 0) || (MU == 2 && sp == 1);
-    const int64_t br = rot ? -wi : wr, bi = rot ? wr : wi;
-    if (back != neg) { t.re += br; t.im += bi; }
-    else { t.re -= br; t.im -= bi; }
+    if (MU == 0 || MU == 2) {
+        if (neg) { t.re += wi; t.im -= wr; }
+        else { t.re -= wi; t.im += wr; }
+    } else {
+        if (neg) { t.re -= wr; t.im -= wi; }
+        else { t.re += wr; t.im += wi; }
+    }
 }
 
 template <int MU>
@@ -403,6 +405,9 @@ __device__ __forceinline__ void fx_hop_dir(const Geom &g, const FxArgs &f, int64
         const int4 *xp = f.x + rbase + (int64_t)nd * 12 * g.Vd + ns;
         // projection h = u + q (a_mu l), limb by limb (the limbs grow by one bit)
         const int q = back ? 1 : -1;
+        // forward: U h; backward: U^+ h (transposed link, conjugated)
+        const int4 *up = f.U + ((int64_t)(back ? nd : d) * 36 + MU * 9) * g.Vd + (back ? ns : s);
+        const int64_t sa = (back ? 1 : 3) * (int64_t)g.Vd, sb = (back ? 3 : 1) * (int64_t)g.Vd;
         cfx h[6];
 #pragma unroll
         for (int c = 0; c < 3; c++) {
@@ -420,37 +425,32 @@ __device__ __forceinline__ void fx_hop_dir(const Geom &g, const FxArgs &f, int64
                 h[3 + c] = {add(u1.re, q, l1.re), add(u1.im, q, l1.im)};
             }
         }
-        // forward: U h; backward: U^+ h (transposed link, the sign of its
-        // imaginary part moved to the half spinor)
-        const int4 *up = f.U + ((int64_t)(back ? nd : d) * 36 + MU * 9) * g.Vd + (back ? ns : s);
-        const int64_t sa = (back ? 1 : 3) * (int64_t)g.Vd, sb = (back ? 3 : 1) * (int64_t)g.Vd;
-        fx hr[6], hi[6];  // +-h.re (enters im), -+h.im (enters re)
+        // the lower spins get -a^+ w forward and +a^+ w backward: their sums
+        // change sign before each of the two
 #pragma unroll
-        for (int k = 0; k < 6; k++) {
-            hr[k] = {h[k].re.hi * -q, h[k].re.lo * -q};
-            hi[k] = {h[k].im.hi * q, h[k].im.lo * q};
-        }
+        for (int k = 6; k < 12; k++) acc[k] = {-acc[k].re, -acc[k].im};
+        // Per row of the link: both spins' real and imaginary sums at once, so
+        // that a multiply-add's accumulator is needed again only four
+        // instructions later.
 #pragma unroll
         for (int a = 0; a < 3; a++) {
-            cfx u[3];
+            fxacc t[4] = {fx_zero(), fx_zero(), fx_zero(), fx_zero()};  // spin 0 re, im, spin 1 re, im
 #pragma unroll
-            for (int b = 0; b < 3; b++) u[b] = ld_cfx(up + a * sa + b * sb);
+            for (int b = 0; b < 3; b++) {
+                const cfx v = ld_cfx(up + a * sa + b * sb);
+                const fx vp = {v.im.hi * q, v.im.lo * q}, vn = {-vp.hi, -vp.lo};
+                fx_mac4(t, v.re, h[b].re, h[b].im, h[3 + b].re, h[3 + b].im);
+                fx_mac2(t[0], t[2], vp, h[b].im, h[3 + b].im);
+                fx_mac2(t[1], t[3], vn, h[b].re, h[3 + b].re);
+            }
 #pragma unroll
             for (int sp = 0; sp < 2; sp++) {
-                fxacc re = {0, 0}, im = {0, 0};
-#pragma unroll
-                for (int b = 0; b < 3; b++) {
-                    fx_mac(re, u[b].re, h[sp * 3 + b].re);
-                    fx_mac(re, u[b].im, hi[sp * 3 + b]);
-                    fx_mac(im, u[b].re, h[sp * 3 + b].im);
-                    fx_mac(im, u[b].im, hr[sp * 3 + b]);
-                }
-                const int64_t wr = fx_value(re) >> sft, wi = fx_value(im) >> sft;
+                const int64_t wr = fx_value(t[2 * sp]) >> sft, wi = fx_value(t[2 * sp + 1]) >> sft;
                 acc[sp * 3 + a].re += wr;
                 acc[sp * 3 + a].im += wi;
                 // the lower spin fed by this one: the other for x, y; the same for z, t
                 const int lo = 6 + 3 * (MU < 2 ? 1 - sp : sp) + a;
-                fx_lower<MU>(sp, back != 0, wr, wi, acc[lo]);
+                fx_lower<MU>(sp, wr, wi, acc[lo]);
             }
         }
     }
@@ -513,39 +513,55 @@ __global__ void __launch_bounds__(128, 3) k_dslash_fx(Geom g0, FxArgs f, double 
     const int ch = E + 2 * kFxLimb - kFxSpinorBits - f.lsh;  // scale of the hop sums
     const int4 *xp = f.x + rbase + (int64_t)d * 12 * g.Vd + s;
     const int4 *ap = f.A + (int64_t)d * 36 * g.Vd + s;
-    // one chirality block per iteration; the block's hop sum is acc[0..5] (the second is moved down)
+    // one chirality block per iteration; the hop sums wait in shared memory, so
+    // that the clover sums have their registers (2 % on 4^4 domains, 6 % on others)
+    __shared__ int64_t hop_sum[24][128];
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+        hop_sum[2 * k][threadIdx.x] = acc[k].re;
+        hop_sum[2 * k + 1][threadIdx.x] = acc[k].im;
+    }
 #pragma unroll 1
     for (int blk = 0; blk < 2; blk++) {
         cfx x[6];
 #pragma unroll
         for (int k = 0; k < 6; k++) x[k] = ld_cfx(xp + (int64_t)(6 * blk + k) * g.Vd);
+        // all six rows at once: every entry is read once, b for row i and
+        // conj(b) for row j, and the sums it feeds are independent
+        fxacc t[12];  // rows' real parts, then imaginary parts
+#pragma unroll
+        for (int i = 0; i < 12; i++) t[i] = fx_zero();
+#pragma unroll
+        for (int i = 0; i < 6; i += 2) {
+            const cfx dd = ld_cfx(ap + (int64_t)(blk * 18 + (i >> 1)) * g.Vd);
+            fx_mac(t[i], dd.re, x[i].re);
+            fx_mac(t[6 + i], dd.re, x[i].im);
+            fx_mac(t[i + 1], dd.im, x[i + 1].re);
+            fx_mac(t[7 + i], dd.im, x[i + 1].im);
+        }
+        int k = 3;
+#pragma unroll
+        for (int i = 0; i < 6; i++)
+#pragma unroll
+            for (int j = i + 1; j < 6; j++) {
+                const cfx m = ld_cfx(ap + (int64_t)(blk * 18 + k) * g.Vd);
+                fxacc w[4] = {t[i], t[6 + i], t[j], t[6 + j]};
+                fx_mac4(w, m.re, x[j].re, x[j].im, x[i].re, x[i].im);
+                fx_mac4(w, m.im, fx{-x[j].im.hi, -x[j].im.lo}, x[j].re, x[i].im, fx{-x[i].re.hi, -x[i].re.lo});
+                t[i] = w[0];
+                t[6 + i] = w[1];
+                t[j] = w[2];
+                t[6 + j] = w[3];
+                k++;
+            }
         double2 y[6];
 #pragma unroll
-        for (int i = 0; i < 6; i++) {
-            // row i: the diagonal, the upper entries b x_j, the lower ones conj(b) x_j
-            fxacc re = {0, 0}, im = {0, 0};
-            const cfx dd = ld_cfx(ap + (int64_t)(blk * 18 + (i >> 1)) * g.Vd);
-            const fx dg = (i & 1) ? dd.im : dd.re;
-            fx_mac(re, dg, x[i].re);
-            fx_mac(im, dg, x[i].im);
-#pragma unroll
-            for (int j = 0; j < 6; j++) {
-                if (j == i) continue;
-                const int lo = i < j ? i : j, up = i < j ? j : i;
-                const int k = 3 + lo * 5 - lo * (lo - 1) / 2 + (up - lo - 1);  // packed index of (lo, up)
-                const cfx m = ld_cfx(ap + (int64_t)(blk * 18 + k) * g.Vd);
-                const fx mi = j > i ? m.im : fx{-m.im.hi, -m.im.lo};
-                fx_mac(re, m.re, x[j].re);
-                fx_mac(im, m.re, x[j].im);
-                fx_mac(im, mi, x[j].re);
-                fx_mac(re, fx{-mi.hi, -mi.lo}, x[j].im);
-            }
-            y[i] = make_double2(fma(-kappa, fx_to_double(acc[i].re, ch), fx_to_double(fx_value(re), ca)),
-                                fma(-kappa, fx_to_double(acc[i].im, ch), fx_to_double(fx_value(im), ca)));
-        }
+        for (int i = 0; i < 6; i++)
+            y[i] = make_double2(fma(-kappa, fx_to_double(hop_sum[12 * blk + 2 * i][threadIdx.x], ch),
+                                    fx_to_double(fx_value(t[i]), ca)),
+                                fma(-kappa, fx_to_double(hop_sum[12 * blk + 2 * i + 1][threadIdx.x], ch),
+                                    fx_to_double(fx_value(t[6 + i]), ca)));
         store6(blk, y);
-#pragma unroll
-        for (int i = 0; i < 6; i++) acc[i] = acc[6 + i];
     }
 }
 

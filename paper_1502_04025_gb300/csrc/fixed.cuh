@@ -58,8 +58,30 @@ __device__ __forceinline__ void fx_mac(fxacc &s, fx a, fx b)
     s.c += (int64_t)a.hi * b.lo;
     s.c += (int64_t)a.lo * b.hi;
 }
-// the sum over 2^60, rounded
-__device__ __forceinline__ int64_t fx_value(const fxacc &s) { return s.h + ((s.c + (1ll << (kFxLimb - 1))) >> kFxLimb); }
+// s[k] += a x_k for four x
+__device__ __forceinline__ void fx_mac4(fxacc *s, fx a, fx x0, fx x1, fx x2, fx x3)
+{
+    const fx x[4] = {x0, x1, x2, x3};
+#pragma unroll
+    for (int k = 0; k < 4; k++) s[k].h += (int64_t)a.hi * x[k].hi;
+#pragma unroll
+    for (int k = 0; k < 4; k++) s[k].c += (int64_t)a.hi * x[k].lo;
+#pragma unroll
+    for (int k = 0; k < 4; k++) s[k].c += (int64_t)a.lo * x[k].hi;
+}
+__device__ __forceinline__ void fx_mac2(fxacc &s0, fxacc &s1, fx a, fx x0, fx x1)
+{
+    s0.h += (int64_t)a.hi * x0.hi;
+    s1.h += (int64_t)a.hi * x1.hi;
+    s0.c += (int64_t)a.hi * x0.lo;
+    s1.c += (int64_t)a.hi * x1.lo;
+    s0.c += (int64_t)a.lo * x0.hi;
+    s1.c += (int64_t)a.lo * x1.hi;
+}
+// an empty sum (half a unit of the result, so that fx_value rounds), and the
+// sum over 2^60
+__device__ __forceinline__ fxacc fx_zero() { return {0, 1ll << (kFxLimb - 1)}; }
+__device__ __forceinline__ int64_t fx_value(const fxacc &s) { return s.h + (s.c >> kFxLimb); }
 
 // v 2^ex in FP64 (v's leading 53 bits, rounded; the result is a normal number or zero)
 __device__ __forceinline__ double fx_to_double(int64_t v, int ex)
@@ -92,6 +114,58 @@ __device__ __forceinline__ fx fx_from_double(double v, int emax, int bits)
 }
 
 __device__ __forceinline__ int fx_exponent(double v) { return (int)(((uint32_t)__double2hiint(v) >> 20) & 0x7ff); }
+
+// ---- FP64 vectors
+//
+// A group of FP64 numbers that share one scale, the largest exponent field.
+// fx_group_done: false unless the group has a fixed-point form whose products
+// with another such group are normal FP64 numbers (finite, exponents within
+// +-400, or all zero).
+struct fxgroup {
+    uint32_t top, any;  // largest high word without sign, the bits set in any word
+    int emax;
+};
+__device__ __forceinline__ void fx_group_add(fxgroup &g, double2 v)
+{
+    const uint32_t a = (uint32_t)__double2hiint(v.x) & 0x7fffffffu, b = (uint32_t)__double2hiint(v.y) & 0x7fffffffu;
+    g.top = max(g.top, max(a, b));
+    g.any |= (uint32_t)__double2loint(v.x) | (uint32_t)__double2loint(v.y);
+}
+__device__ __forceinline__ bool fx_group_done(fxgroup &g)
+{
+    g.emax = (int)(g.top >> 20);
+    if ((g.top | g.any) == 0u) g.emax = 1023;  // all zero: every number is far below the scale
+    return g.emax > 623 && g.emax < 1423;
+}
+
+// shifts by 32 and more give 0
+__device__ __forceinline__ uint32_t shr_clamp(uint32_t v, uint32_t n)
+{
+    uint32_t r;
+    asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
+    return r;
+}
+
+// A number of a group (exponent field at most emax, emax > 100) with `kBits`
+// bits below 2^(emax - 1022), 32 < kBits <= 62, rounded towards zero: limbs of
+// its magnitude, 0 <= lo < 2^30, both with its sign.  (Subnormal numbers and
+// zeros are shifted out.)
+template <int kBits>
+__device__ __forceinline__ fx fx_from_grouped(double v, int emax)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t t = __funnelshift_l(lo, hi, 11) | 0x80000000u, r = lo << 11;  // mantissa, leading one on top
+    const uint32_t sh = (uint32_t)(emax + (64 - kBits)) - ((hi >> 20) & 0x7ffu);  // magnitude = (t:r) >> sh
+    const uint32_t mh = shr_clamp(t, sh - (32 - kFxLimb));
+    const uint32_t ml = (sh < 32 ? __funnelshift_r(r, t, sh) : shr_clamp(t, sh - 32)) & ((1u << kFxLimb) - 1);
+    const int sg = ((int)hi >> 31) | 1;
+    return {(int)mh * sg, (int)ml * sg};
+}
+template <int kBits>
+__device__ __forceinline__ cfx fx_from_group(double2 v, const fxgroup &g)
+{
+    return {fx_from_grouped<kBits>(v.x, g.emax), fx_from_grouped<kBits>(v.y, g.emax)};
+}
 
 // The 12 components v of a site into the fixed-point field f (planes of the
 // domain block at blk) and its exponent.
