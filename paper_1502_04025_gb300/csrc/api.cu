@@ -112,10 +112,41 @@ Timer::~Timer()
 
 // ------------------------------------------------------------------ memory
 
+// the gauge field whose fixed-point copy this thread is building (its lock is held)
+static thread_local const Gauge *fx_building = nullptr;
+
+static void fx_release(Gauge *g)
+{
+    FxCopy &f = g->fx;
+    if (!f.required) g->ctx->optional -= f.links.bytes + f.clov.bytes + f.clov_e.bytes;
+    f.links.release();
+    f.clov.release();
+    f.clov_e.release();
+    f.have_links = f.have_clov = f.required = false;
+}
+
+// Gives up optional fixed-point copies that nobody reads, until at least
+// `need` bytes have come back.
+static void fx_reclaim(Ctx *c, size_t need)
+{
+    if (c->optional.load() == 0) return;
+    std::lock_guard<std::mutex> lk(c->gauges_mu);
+    size_t got = 0;
+    for (Gauge *g : c->gauges) {
+        if (got >= need) break;
+        if (g == fx_building) continue;
+        std::unique_lock<std::shared_mutex> ul(g->fx.mu, std::try_to_lock);
+        if (!ul.owns_lock() || g->fx.required) continue;
+        got += g->fx.links.bytes + g->fx.clov.bytes + g->fx.clov_e.bytes;
+        fx_release(g);
+    }
+}
+
 qdd_status DevMem::alloc(Ctx *c, size_t n)
 {
     release();
     if (n == 0) return QDD_OK;
+    if (c->used.load() + n > c->budget) fx_reclaim(c, c->used.load() + n - c->budget);
     if (c->used.load() + n > c->budget) {
         set_error("allocation of %zu bytes exceeds the HBM budget (%zu of %zu bytes in use)", n, c->used.load(),
                   c->budget);
@@ -163,6 +194,10 @@ qdd_status ensure_copy(Gauge *g, qdd_prec prec, cudaStream_t s)
 {
     if (prec == QDD_PREC_F64) return QDD_OK;
     if (prec == QDD_PREC_H16) return ensure_copy(g, QDD_PREC_F16S, s);
+    if (prec == QDD_PREC_DF64) {
+        FxLock lk;
+        return fx_acquire(g, true, true, s, lk);
+    }
     if (prec < QDD_PREC_F64 || prec > QDD_PREC_DF64) {
         set_error("invalid precision %d", (int)prec);
         return QDD_EINVAL;
@@ -173,18 +208,6 @@ qdd_status ensure_copy(Gauge *g, qdd_prec prec, cudaStream_t s)
     if (!g->have_clover) {
         set_error("set_clover has not been called");
         return QDD_EINVAL;
-    }
-    if (prec == QDD_PREC_DF64) {
-        if (g->link_exp > kMaxFixedLinkExp) return QDD_OK;  // FP64 arithmetic stands in
-        const size_t n = (size_t)g->hg.V * 36;
-        QDD_TRY(c.links.ensure(g->ctx, n * 16));
-        QDD_TRY(c.clov.ensure(g->ctx, n * 16));
-        QDD_TRY(c.clov_s.ensure(g->ctx, (size_t)g->hg.V * sizeof(int)));
-        QDD_TRY(launch_fields_fx(g, c, s));
-        // FP64 callers on other streams may take the copy from here on
-        QDD_CUDA(cudaStreamSynchronize(s));
-        c.valid = true;
-        return QDD_OK;
     }
     const size_t V = g->hg.V, eb = elem_bytes(prec);
     const bool scaled = prec == QDD_PREC_F16S || prec == QDD_PREC_BF16S;
@@ -202,23 +225,55 @@ qdd_status ensure_copy(Gauge *g, qdd_prec prec, cudaStream_t s)
     return QDD_OK;
 }
 
-qdd_status ensure_fixed(Gauge *g, bool required, cudaStream_t s, bool *ok)
+static qdd_status fx_build(Gauge *g, bool required, bool clover, cudaStream_t s)
 {
-    *ok = false;
-    if (g->link_exp > kMaxFixedLinkExp) return QDD_OK;
-    if (!required) {
-        std::lock_guard<std::mutex> lk(g->copy_mu);
-        const size_t need = (size_t)g->hg.V * (2 * 36 * 16 + 4);
-        const PrecCopy &c = g->copies[QDD_PREC_DF64];
-        if (!c.valid && !c.links.p && g->ctx->used.load() + need > g->ctx->budget / 2) return QDD_OK;
+    FxCopy &f = g->fx;
+    Ctx *c = g->ctx;
+    const size_t n = (size_t)g->hg.V * 36 * 16, ne = (size_t)g->hg.V * sizeof(int);
+    if (!required && !f.required) {
+        const size_t more = (f.links.p ? 0 : n) + (clover && !f.clov.p ? n + ne : 0);
+        if (c->used.load() + more > c->budget / 2) return QDD_EBUDGET;
     }
-    qdd_status st = ensure_copy(g, QDD_PREC_DF64, s);
-    if (st != QDD_OK && !required && (st == QDD_EBUDGET || st == QDD_ENOMEM)) {
-        clear_error();
-        return QDD_OK;
-    }
+    const size_t before = f.links.bytes + f.clov.bytes + f.clov_e.bytes;
+    qdd_status st = f.links.ensure(c, n);
+    if (st == QDD_OK && clover) st = f.clov.ensure(c, n);
+    if (st == QDD_OK && clover) st = f.clov_e.ensure(c, ne);
+    if (!f.required) c->optional += f.links.bytes + f.clov.bytes + f.clov_e.bytes - before;
     QDD_TRY(st);
-    *ok = true;
+    if (!f.have_links) QDD_TRY(launch_links_fx(g, s));
+    if (clover && !f.have_clov) QDD_TRY(launch_clover_fx(g, s));
+    QDD_CUDA(cudaStreamSynchronize(s));  // other streams may read it from here on
+    f.have_links = true;
+    if (clover) f.have_clov = true;
+    if (required && !f.required) {
+        f.required = true;
+        c->optional -= f.links.bytes + f.clov.bytes + f.clov_e.bytes;
+    }
+    return QDD_OK;
+}
+
+qdd_status fx_acquire(Gauge *g, bool required, bool clover, cudaStream_t s, FxLock &lk)
+{
+    if (clover && !g->have_clover) {
+        set_error("set_clover has not been called");
+        return QDD_EINVAL;
+    }
+    if (g->link_exp > kMaxFixedLinkExp) return QDD_OK;
+    FxCopy &f = g->fx;
+    for (int turn = 0; turn < 3; turn++) {  // an optional copy may be given up between the two locks
+        lk = FxLock(f.mu);
+        if (f.have_links && (!clover || f.have_clov) && (!required || f.required)) return QDD_OK;
+        lk.unlock();
+        std::unique_lock<std::shared_mutex> ul(f.mu);
+        fx_building = g;
+        qdd_status st = fx_build(g, required, clover, s);
+        fx_building = nullptr;
+        if (st != QDD_OK && !required && (st == QDD_EBUDGET || st == QDD_ENOMEM)) {
+            clear_error();
+            return QDD_OK;
+        }
+        QDD_TRY(st);
+    }
     return QDD_OK;
 }
 
@@ -243,7 +298,19 @@ struct Staging {
     DevMem io, a, a_s, b, b_s, c, c_s, err;
 };
 
-Gauge::~Gauge() = default;
+Gauge::~Gauge()
+{
+    if (!ctx) return;
+    {
+        std::lock_guard<std::mutex> lk(ctx->gauges_mu);
+        for (size_t k = 0; k < ctx->gauges.size(); k++)
+            if (ctx->gauges[k] == this) {
+                ctx->gauges.erase(ctx->gauges.begin() + k);
+                break;
+            }
+    }
+    fx_release(this);
+}
 
 static qdd_status stage_in(Gauge *g, DevMem &io, const double *src, int nrhs, int on_device, cudaStream_t s,
                            const double **dev)
@@ -440,6 +507,10 @@ qdd_status qdd_create_gauge_field(qdd_ctx *ctx, const int L[4], const int dom[4]
     g->two_rows = g->su3;
     QDD_CUDA(cudaDeviceSynchronize());
     ctx->timer.resolve();
+    {
+        std::lock_guard<std::mutex> lk(ctx->gauges_mu);
+        ctx->gauges.push_back(g.get());
+    }
     *out = g.release();
     return QDD_OK;
 }
@@ -583,11 +654,17 @@ qdd_status qdd_set_clover(qdd_gauge *g, double c_sw, double kappa)
         DevMem flag;
         QDD_TRY(flag.alloc(g->ctx, sizeof(int)));
         QDD_CUDA(cudaMemset(flag.p, 0, sizeof(int)));
-        QDD_TRY(launch_clover_build(g, c_sw, kappa, flag.as<int>(), 0));
+        FxLock fl;
+        if (g->su3) QDD_TRY(fx_acquire(g, false, false, 0, fl));
+        QDD_TRY(launch_clover_build(g, c_sw, kappa, flag.as<int>(), fl.owns_lock(), 0));
         QDD_CUDA(cudaMemcpy(&singular, flag.p, sizeof(int), cudaMemcpyDeviceToHost));
     }
     g->ctx->timer.resolve();
-    for (int p = 0; p < 5; p++) g->copies[p].valid = false;
+    for (auto &c : g->copies) c.valid = false;
+    {
+        std::unique_lock<std::shared_mutex> ul(g->fx.mu);
+        g->fx.have_clov = false;
+    }
     g->have_clover = false;
     if (singular) {
         set_error("clover block singular on %d sites", singular);
@@ -663,27 +740,6 @@ qdd_status qdd_apply_D(qdd_gauge *g, const double *in, double *out, int nrhs, qd
     double *dout = nullptr;
     QDD_TRY(stage_in(g, st->io, in, nrhs, on_device, s, &din));
     QDD_TRY(st->a.ensure(g->ctx, V * 12 * eb * nrhs));
-    // FP64-class arithmetic in fixed point: the input is converted on its way
-    // in, the operator writes the host layout
-    bool fixed = false;
-    if (arith != QDD_PREC_F32) {
-        if (!g->have_clover) {
-            set_error("set_clover has not been called");
-            return QDD_EINVAL;
-        }
-        QDD_TRY(ensure_fixed(g, arith == QDD_PREC_DF64, s, &fixed));
-    }
-    if (!fixed) QDD_TRY(st->b.ensure(g->ctx, V * 12 * eb * nrhs));
-    if (scaled || fixed) QDD_TRY(st->a_s.ensure(g->ctx, V * 4 * nrhs));
-    if (scaled) QDD_TRY(st->b_s.ensure(g->ctx, V * 4 * nrhs));
-    const FxField fxa{st->a.p, st->a_s.as<int>()};
-    if (fixed) QDD_TRY(launch_spinor_in_fx(g, din, fxa, nrhs, s));
-    else QDD_TRY(launch_spinor_in(g, din, st->a.p, st->a_s.as<float>(), prec, nrhs, s));
-    // a sharded field: its boundary planes (FP64, host layout) move while the operator runs
-    QDD_TRY(slab_dslash_begin(g, din, false, true, nrhs, s));
-    if (!fixed)
-        QDD_TRY(launch_dslash(g, arith, fp, st->a.p, st->a_s.as<float>(), prec, st->b.p, st->b_s.as<float>(), prec,
-                              nullptr, nrhs, s));
     // a sharded field corrects the output's boundary planes from the input
     // (FP64, host layout), so the host output must not reuse the input's staging
     DevMem &oio = g->slab ? st->c : st->io;
@@ -692,6 +748,22 @@ qdd_status qdd_apply_D(qdd_gauge *g, const double *in, double *out, int nrhs, qd
         return QDD_EINVAL;
     }
     QDD_TRY(stage_out(g, oio, out, nrhs, on_device, s, &dout));
+    if (scaled || arith != QDD_PREC_F32) QDD_TRY(st->a_s.ensure(g->ctx, V * 4 * nrhs));
+    if (scaled) QDD_TRY(st->b_s.ensure(g->ctx, V * 4 * nrhs));
+    // FP64-class arithmetic in fixed point: the input is converted on its way
+    // in, the operator writes the host layout
+    FxLock fl;
+    if (arith != QDD_PREC_F32) QDD_TRY(fx_acquire(g, arith == QDD_PREC_DF64, true, s, fl));
+    const bool fixed = fl.owns_lock();
+    if (!fixed) QDD_TRY(st->b.ensure(g->ctx, V * 12 * eb * nrhs));
+    const FxField fxa{st->a.p, st->a_s.as<int>()};
+    if (fixed) QDD_TRY(launch_spinor_in_fx(g, din, fxa, nrhs, s));
+    else QDD_TRY(launch_spinor_in(g, din, st->a.p, st->a_s.as<float>(), prec, nrhs, s));
+    // a sharded field: its boundary planes (FP64, host layout) move while the operator runs
+    QDD_TRY(slab_dslash_begin(g, din, false, true, nrhs, s));
+    if (!fixed)
+        QDD_TRY(launch_dslash(g, arith, fp, st->a.p, st->a_s.as<float>(), prec, st->b.p, st->b_s.as<float>(), prec,
+                              nullptr, nrhs, s));
     if (fixed) QDD_TRY(launch_dslash_fx(g, fxa, (double2 *)dout, true, nullptr, nrhs, s));
     else QDD_TRY(launch_spinor_out(g, st->b.p, st->b_s.as<float>(), dout, prec, nrhs, s));
     QDD_TRY(slab_dslash_end(g, (double2 *)dout, false, nrhs, s));

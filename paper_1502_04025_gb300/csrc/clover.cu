@@ -10,6 +10,7 @@
 // upper block, - for the lower).  The even-odd domain solver also needs the
 // inverse blocks on odd sites (the Schwarz form keeps A on even sites and
 // A^{-1} on odd sites).  Built in FP64 once per (gauge, c_sw, kappa).
+#include "fixed.cuh"
 #include "internal.h"
 
 namespace qdd {
@@ -192,12 +193,324 @@ __global__ void k_clover_build(Geom g, const double2 *U, double csw, double kapp
     }
 }
 
-qdd_status launch_clover_build(Gauge *g, double csw, double kappa, int *d_singular, cudaStream_t s)
+// ------------------------------------------------------------------------
+// The same for SU(3) links, in 64-bit fixed point (fixed.cuh): the 72 matrix
+// products of a site's 24 leaves are integer multiply-adds on the links'
+// fixed-point copy (entries of SU(3) matrices stay below 1, so every product
+// keeps the links' scale 2^-60), the leaf sums, the anti-Hermitian and traceless
+// parts and the sums over planes are integers, and FP64 starts at the entries
+// of A.  In FP64 arithmetic the 7776 multiply-adds of the leaves take 3900 of
+// an SM's clocks per site (2 lanes per clock); as integer multiply-adds they take
+// about 360.  TABLE_CLOVER
+
+struct M3x {
+    cfx m[9];
+};
+
+__device__ __forceinline__ M3x load_link_fx(const Geom &g, const int4 *U, int gi, int mu)
+{
+    M3x r;
+    int d, s;
+    split_index(g, gi, d, s);
+    const int4 *p = U + ((int64_t)d * 36 + mu * 9) * g.Vd + s;
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        const int4 v = __ldg(p + (int64_t)k * g.Vd);
+        r.m[k] = {{v.x, v.y}, {v.z, v.w}};
+    }
+    return r;
+}
+
+// entry (i, j) of op(a) op(b), op the adjoint where DA, DB
+template <bool DA, bool DB>
+__device__ __forceinline__ void fx_mul_entry(const M3x &a, const M3x &b, int i, int j, fxacc &re, fxacc &im)
+{
+    re = fx_zero();
+    im = fx_zero();
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const cfx x = DA ? a.m[k * 3 + i] : a.m[i * 3 + k], y = DB ? b.m[j * 3 + k] : b.m[k * 3 + j];
+        const fx ny = {-y.im.hi, -y.im.lo};
+        // conjugation of x and y: the sign of their imaginary parts
+        fx_mac(re, x.re, y.re);
+        fx_mac(im, x.re, DB ? ny : y.im);
+        fx_mac(re, x.im, DA == DB ? ny : y.im);
+        const fx xi = {DA ? -x.im.hi : x.im.hi, DA ? -x.im.lo : x.im.lo};
+        fx_mac(im, xi, y.re);
+    }
+}
+
+template <bool DA, bool DB>
+__device__ __forceinline__ M3x fx_mul(const M3x &a, const M3x &b)
+{
+    M3x r;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            fxacc re, im;
+            fx_mul_entry<DA, DB>(a, b, i, j, re, im);
+            r.m[i * 3 + j] = {fx_split(fx_value(re)), fx_split(fx_value(im))};
+        }
+    return r;
+}
+
+// Q = sum of leaves / 8 (three bits dropped, so that the sums below keep their
+// headroom): scale 2^-57 per leaf
+struct M3q {
+    int64_t re[9], im[9];
+};
+template <bool DA, bool DB>
+__device__ __forceinline__ void fx_leaf_add(M3q &q, const M3x &a, const M3x &b)
+{
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            fxacc re, im;
+            fx_mul_entry<DA, DB>(a, b, i, j, re, im);
+            q.re[i * 3 + j] += fx_value(re) >> 3;
+            q.im[i * 3 + j] += fx_value(im) >> 3;
+        }
+}
+
+// the link of the step from n to m = n +- da: U_da(n) forward, U_da(m)^+ backward
+__device__ __forceinline__ M3x step_link_fx(const Geom &g, const int4 *U, int n, int m, int da, bool back)
+{
+    M3x u = load_link_fx(g, U, back ? m : n, da);
+    if (back) {
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+#pragma unroll
+            for (int j = i; j < 3; j++) {
+                const cfx x = u.m[i * 3 + j], y = u.m[j * 3 + i];
+                u.m[i * 3 + j] = {y.re, {-y.im.hi, -y.im.lo}};
+                u.m[j * 3 + i] = {x.re, {-x.im.hi, -x.im.lo}};
+            }
+    }
+    return u;
+}
+
+// 8 F_{mu nu} = traceless part of Q - Q^+ at gi, scale 2^-57, as nine integers:
+// the imaginary diagonal, then re and im of the entries (0,1), (0,2), (1,2)
+constexpr int kLeafBits = 57;
+__device__ __forceinline__ void field_strength_fx(const Geom &g, const int4 *U, int gi, int mu, int nu, int64_t *F)
+{
+    const int n_pm = nbr(g, gi, 2 * mu), n_mm = nbr(g, gi, 2 * mu + 1);
+    const int n_pn = nbr(g, gi, 2 * nu), n_mn = nbr(g, gi, 2 * nu + 1);
+    M3q q;
+#pragma unroll
+    for (int k = 0; k < 9; k++) q.re[k] = q.im[k] = 0;
+    // one leaf per iteration, each the product of two half paths X Y or X Y^+
+    // (one copy of the code: four would not fit the instruction cache):
+    //   0: U_mu(n) U_nu(n+mu) . (U_nu(n) U_mu(n+nu))^+
+    //   1: U_nu(n) U_mu^+(n-mu+nu) . (U_mu^+(n-mu) U_nu(n-mu))^+
+    //   2: U_mu^+(n-mu) U_nu^+(n-mu-nu) . (U_nu^+(n-nu) U_mu^+(n-mu-nu))^+
+    //   3: U_nu^+(n-nu) U_mu(n-nu) . (U_mu(n) U_nu^+(n+mu-nu))^+
+    // Read as forward or backward hops from n: every leaf is a first step along
+    // (dir a, dir b) and its mirror (dir b, dir a).
+#pragma unroll 1
+    for (int leaf = 0; leaf < 4; leaf++) {
+        // leaf runs from step a then b on one side, b then a on the other, with
+        // (a, b) = (+mu, +nu), (+nu, -mu), (-mu, -nu), (-nu, +mu)
+        const bool swap = leaf & 1;
+        const int da = swap ? nu : mu, db = swap ? mu : nu;
+        const bool ba = leaf >= 2, bb = leaf == 1 || leaf == 2;  // backward first / second step
+        const int na = swap ? (ba ? n_mn : n_pn) : (ba ? n_mm : n_pm);  // n + a
+        const int nb = swap ? (bb ? n_mm : n_pm) : (bb ? n_mn : n_pn);  // n + b
+        // X = link(n, a) link(n + a, b), Y = link(n, b) link(n + b, a); leaf = X Y^+
+        const M3x a0 = step_link_fx(g, U, gi, na, da, ba);
+        const int nab = nbr(g, na, 2 * db + (bb ? 1 : 0));
+        const M3x X = fx_mul<false, false>(a0, step_link_fx(g, U, na, nab, db, bb));
+        const M3x b0 = step_link_fx(g, U, gi, nb, db, bb);
+        const M3x Y = fx_mul<false, false>(b0, step_link_fx(g, U, nb, nab, da, ba));
+        fx_leaf_add<false, true>(q, X, Y);
+    }
+    const int64_t d0 = q.im[0], d1 = q.im[4], d2 = q.im[8], mean = (d0 + d1 + d2) / 3;
+    F[0] = 2 * (d0 - mean);
+    F[1] = 2 * (d1 - mean);
+    F[2] = 2 * (d2 - mean);
+    F[3] = q.re[1] - q.re[3];
+    F[4] = q.im[1] + q.im[3];
+    F[5] = q.re[2] - q.re[6];
+    F[6] = q.im[2] + q.im[6];
+    F[7] = q.re[5] - q.re[7];
+    F[8] = q.im[5] + q.im[7];
+}
+
+// Minus the inverse of a Hermitian 6x6 matrix by six symmetric sweeps without
+// pivoting, in place: dg the diagonal, u the upper triangle row by row (i < j).
+// False when a pivot is small against the matrix (the caller pivots instead).
+__device__ __forceinline__ bool sweep6(double *dg, zd *u)
+{
+    double big = 0;
+#pragma unroll
+    for (int i = 0; i < 6; i++) big = fmax(big, fabs(dg[i]));
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        auto at = [](int i, int j) { return i * 5 - i * (i - 1) / 2 + (j - i - 1); };  // i < j
+        ok = ok && fabs(dg[k]) > 0.02 * big;
+        const double p = 1.0 / dg[k];
+        zd col[6], row[6];  // a_ik, and a_ik / d
+#pragma unroll
+        for (int i = 0; i < 6; i++) {
+            if (i == k) continue;
+            col[i] = i < k ? u[at(i, k)] : conj(u[at(k, i)]);
+            row[i] = p * col[i];
+        }
+#pragma unroll
+        for (int i = 0; i < 6; i++) {
+            if (i == k) continue;
+            dg[i] = fma(-row[i].re, col[i].re, dg[i]);
+            dg[i] = fma(-row[i].im, col[i].im, dg[i]);
+#pragma unroll
+            for (int j = i + 1; j < 6; j++) {
+                if (j == k) continue;
+                zd &t = u[at(i, j)];  // a_ij -= a_ik conj(a_jk) / d
+                t.re = fma(-row[i].re, col[j].re, t.re);
+                t.re = fma(-row[i].im, col[j].im, t.re);
+                t.im = fma(-row[i].im, col[j].re, t.im);
+                t.im = fma(row[i].re, col[j].im, t.im);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 6; i++) {
+            if (i < k) u[at(i, k)] = row[i];
+            else if (i > k) u[at(k, i)] = conj(row[i]);
+        }
+        dg[k] = -p;
+    }
+    return ok;
+}
+
+// the inverse with pivoting, for blocks that sweep6 refuses
+__device__ __noinline__ bool invert6_packed(const double *dg, const zd *u, double *dgo, zd *uo)
+{
+    zd M[36], inv[36];
+    int k = 0;
+    for (int i = 0; i < 6; i++) {
+        M[i * 6 + i] = mk(dg[i], 0.0);
+        for (int j = i + 1; j < 6; j++) {
+            M[i * 6 + j] = u[k];
+            M[j * 6 + i] = conj(u[k]);
+            k++;
+        }
+    }
+    if (!invert6(M, inv)) return false;
+    k = 0;
+    for (int i = 0; i < 6; i++) {
+        dgo[i] = inv[i * 6 + i].re;
+        for (int j = i + 1; j < 6; j++) uo[k++] = 0.5 * (inv[i * 6 + j] + conj(inv[j * 6 + i]));
+    }
+    return true;
+}
+
+__device__ __forceinline__ void store_herm6(double2 *dst, int64_t stride, const double *dg, const zd *u)
+{
+#pragma unroll
+    for (int k = 0; k < 3; k++) dst[k * stride] = make_double2(dg[2 * k], dg[2 * k + 1]);
+#pragma unroll
+    for (int k = 0; k < 15; k++) dst[(3 + k) * stride] = make_double2(u[k].re, u[k].im);
+}
+
+constexpr int kCloverThreads = 64;
+
+__global__ void __launch_bounds__(kCloverThreads) k_clover_build_fx(Geom g, const int4 *U, double kc, double2 *A,
+                                                                    double2 *S, int *singular)
+{
+    __shared__ int64_t F[6][9][kCloverThreads];
+    const int gi = blockIdx.x * kCloverThreads + threadIdx.x, t = threadIdx.x;
+    if (gi >= g.V) return;
+    int d, s;
+    split_index(g, gi, d, s);
+#pragma unroll 1
+    for (int plane = 0; plane < 6; plane++) {  // xy, xz, xt, yz, yt, zt
+        const int mu = plane < 3 ? 0 : (plane < 5 ? 1 : 2), nu = plane < 3 ? plane + 1 : (plane < 5 ? plane - 1 : 3);
+        int64_t f[9];
+        field_strength_fx(g, U, gi, mu, nu, f);
+#pragma unroll
+        for (int k = 0; k < 9; k++) F[plane][k][t] = f[k];
+    }
+    const bool odd = s >= g.Vh;
+    constexpr int ex = -kLeafBits - 3;  // F is an eighth of its integers
+#pragma unroll 1
+    for (int ch = 0; ch < 2; ch++) {
+        const int se = ch == 0 ? 1 : -1;
+        // G_1 = -F_yz +- F_xt, G_2 = F_xz +- F_yt, G_3 = -F_xy +- F_zt
+        int64_t g1[9], g2[9], g3[9];
+#pragma unroll
+        for (int k = 0; k < 9; k++) {
+            g1[k] = se * F[2][k][t] - F[3][k][t];
+            g2[k] = F[1][k][t] + se * F[4][k][t];
+            g3[k] = se * F[5][k][t] - F[0][k][t];
+        }
+        // i G is Hermitian: diagonal -im, upper entry (a,b) (-im, re), lower its conjugate
+        auto her = [](const int64_t *gk, int a, int b, int64_t &re, int64_t &im) {
+            if (a == b) { re = -gk[a]; im = 0; return; }
+            const int lo = a < b ? a : b, k = lo == 0 ? (a + b == 1 ? 3 : 5) : 7;
+            re = -gk[k + 1];
+            im = a < b ? gk[k] : -gk[k];
+        };
+        double dg[6];
+        zd u[15];
+        int k = 0;
+#pragma unroll
+        for (int i = 0; i < 6; i++) {
+            const int a = i % 3;
+            int64_t re, im;
+            her(g3, a, a, re, im);
+            dg[i] = fma(i < 3 ? kc : -kc, fx_to_double(re, ex), 1.0);
+#pragma unroll
+            for (int j = i + 1; j < 6; j++) {
+                const int b = j % 3;
+                if ((i < 3) == (j < 3)) {  // +-kc i G_3
+                    her(g3, a, b, re, im);
+                    if (i >= 3) { re = -re; im = -im; }
+                } else {  // kc (i G_1 - i (i G_2))
+                    int64_t r2, i2;
+                    her(g1, a, b, re, im);
+                    her(g2, a, b, r2, i2);
+                    re += i2;
+                    im -= r2;
+                }
+                u[k++] = mk(kc * fx_to_double(re, ex), kc * fx_to_double(im, ex));
+            }
+        }
+        const int64_t base = ((int64_t)d * 36 + ch * 18) * g.Vd + s;
+        store_herm6(A + base, g.Vd, dg, u);
+        if (odd) {
+            double d0[6];
+            zd u0[15];
+#pragma unroll
+            for (int i = 0; i < 6; i++) d0[i] = dg[i];
+#pragma unroll
+            for (int i = 0; i < 15; i++) u0[i] = u[i];
+            if (sweep6(dg, u)) {
+#pragma unroll
+                for (int i = 0; i < 6; i++) dg[i] = -dg[i];
+#pragma unroll
+                for (int i = 0; i < 15; i++) u[i] = -u[i];
+            } else if (!invert6_packed(d0, u0, dg, u)) {
+                atomicAdd(singular, 1);
+                for (int i = 0; i < 6; i++) dg[i] = 0.0;
+                for (int i = 0; i < 15; i++) u[i] = mk(0.0, 0.0);
+            }
+        }
+        store_herm6(S + base, g.Vd, dg, u);
+    }
+}
+
+qdd_status launch_clover_build(Gauge *g, double csw, double kappa, int *d_singular, bool fixed, cudaStream_t s)
 {
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
-    k_clover_build<<<(g->hg.V + 127) / 128, 128, 0, s>>>(g->geom, g->links64.as<double2>(), csw, kappa,
-                                                        g->clov64.as<double2>(), g->sclov64.as<double2>(),
-                                                        d_singular);
+    if (fixed)
+        k_clover_build_fx<<<(g->hg.V + kCloverThreads - 1) / kCloverThreads, kCloverThreads, 0, s>>>(
+            g->geom, g->fx.links.as<int4>(), kappa * csw, g->clov64.as<double2>(), g->sclov64.as<double2>(), d_singular);
+    else
+        k_clover_build<<<(g->hg.V + 127) / 128, 128, 0, s>>>(g->geom, g->links64.as<double2>(), csw, kappa,
+                                                            g->clov64.as<double2>(), g->sclov64.as<double2>(),
+                                                            d_singular);
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
 }

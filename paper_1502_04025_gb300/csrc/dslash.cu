@@ -624,14 +624,21 @@ __global__ void __launch_bounds__(128) k_clover_fx(Geom g, const double2 *src, i
     }
 }
 
-qdd_status launch_fields_fx(Gauge *g, PrecCopy &c, cudaStream_t s)
+qdd_status launch_links_fx(Gauge *g, cudaStream_t s)
 {
     const int64_t n = (int64_t)g->hg.V * 36;
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
-    k_links_fx<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, g->links64.as<double2>(), c.links.as<int4>(),
+    k_links_fx<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, g->links64.as<double2>(), g->fx.links.as<int4>(),
                                                            fx_link_shift(g));
-    k_clover_fx<<<(g->hg.V + 127) / 128, 128, 0, s>>>(g->geom, g->clov64.as<double2>(), c.clov.as<int4>(),
-                                                      c.clov_s.as<int>());
+    QDD_CUDA(cudaGetLastError());
+    return QDD_OK;
+}
+
+qdd_status launch_clover_fx(Gauge *g, cudaStream_t s)
+{
+    LaunchScope ls(g->ctx->timer, K_OTHER, s);
+    k_clover_fx<<<(g->hg.V + 127) / 128, 128, 0, s>>>(g->geom, g->clov64.as<double2>(), g->fx.clov.as<int4>(),
+                                                      g->fx.clov_e.as<int>());
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
 }
@@ -653,8 +660,8 @@ qdd_status launch_spinor_fx(Gauge *g, const void *src, qdd_prec ip, const FxFiel
 qdd_status launch_dslash_fx(Gauge *g, const FxField &x, double2 *out, bool host_layout, const double2 *b, int nrhs,
                             cudaStream_t s)
 {
-    const PrecCopy &c = g->copies[QDD_PREC_DF64];
-    FxArgs f{c.links.as<int4>(), c.clov.as<int4>(), (const int4 *)x.x, c.clov_s.as<int>(), x.e, fx_link_shift(g), b,
+    const FxCopy &c = g->fx;
+    FxArgs f{c.links.as<int4>(), c.clov.as<int4>(), (const int4 *)x.x, c.clov_e.as<int>(), x.e, fx_link_shift(g), b,
              out, host_layout ? g->d_site_of.as<int>() : nullptr, ((uintptr_t)out & 31) == 0};
     const dim3 grid((g->hg.V + 127) / 128, nrhs);
     LaunchScope ls(g->ctx->timer, K_DSLASH, s);
@@ -729,9 +736,9 @@ qdd_status launch_dslash(Gauge *g, qdd_prec arith, qdd_prec fp, const void *in, 
     if (arith == QDD_PREC_F64 || arith == QDD_PREC_DF64) {
         if (fp == QDD_PREC_DF64) fp = QDD_PREC_F64;
         if (fxb && op == QDD_PREC_F64 && (ip == QDD_PREC_F64 || ip == QDD_PREC_F32)) {
-            bool ok = false;
-            QDD_TRY(ensure_fixed(g, arith == QDD_PREC_DF64, s, &ok));
-            if (ok) {
+            FxLock lk;
+            QDD_TRY(fx_acquire(g, arith == QDD_PREC_DF64, true, s, lk));
+            if (lk.owns_lock()) {
                 QDD_TRY(launch_spinor_fx(g, in, ip, *fxb, nrhs, s));
                 return launch_dslash_fx(g, *fxb, (double2 *)out, false, b, nrhs, s);
             }

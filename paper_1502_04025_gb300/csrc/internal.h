@@ -11,6 +11,7 @@
 #include <map>
 #include <memory>
 #include <mutex>
+#include <shared_mutex>
 #include <string>
 #include <thread>
 #include <vector>
@@ -127,6 +128,11 @@ struct Ctx {
     int nsm = 0;
     size_t budget = 0;
     std::atomic<size_t> used{0};
+    // of these, optional copies that an allocation may take back (fx_reclaim),
+    // and the gauge fields that may hold one
+    std::atomic<size_t> optional{0};
+    std::mutex gauges_mu;
+    std::vector<struct Gauge *> gauges;
     Timer timer;
     // scratch of the reductions (per-block partials), grown on demand
     DevMem red_scratch;
@@ -162,13 +168,24 @@ struct HostGeom {
 qdd_status make_geometry(const int L[4], const int dom[4], HostGeom &hg);
 
 // A lower-precision copy of the fields the operator and the preconditioner read.
-// The copy of QDD_PREC_DF64 holds links and clover in fixed point (fixed.cuh),
-// the clover's exponents in clov_s.
 struct PrecCopy {
     bool valid = false;
     DevMem links, clov, clov_s, sclov, sclov_s;
     bool valid12 = false;
     DevMem links12;  // first two rows of each link, for the full-lattice operator
+};
+
+// Links and clover in fixed point (fixed.cuh), for the FP64-class operator and
+// the clover build.  QDD_PREC_DF64 needs it (required); for QDD_PREC_F64 and the
+// clover build, which have FP64 arithmetic to fall back on, it is optional:
+// built while at most half of the HBM budget is in use, and given up when
+// another allocation would exceed the budget.  Readers hold mu shared from
+// fx_acquire until their kernels are launched (freeing device memory waits for
+// launched kernels); building and giving up hold it exclusively.
+struct FxCopy {
+    std::shared_mutex mu;
+    DevMem links, clov, clov_e;  // clov_e: one exponent per site
+    bool have_links = false, have_clov = false, required = false;
 };
 
 // Device and pinned host buffers of one solve (Krylov basis, preconditioner
@@ -223,7 +240,8 @@ struct Gauge {
     int sap_variant = 0;      // Schwarz kernel form (qdd_set_schwarz_variant)
     double csw = 0, kappa = 0;
     DevMem clov64, sclov64;   // FP64 clover A and Schwarz form (A even, A^-1 odd)
-    PrecCopy copies[5];       // index = qdd_prec; F64 entry aliases the masters
+    PrecCopy copies[6];       // index = qdd_prec; used for F32, F16S and BF16S
+    FxCopy fx;
     std::unique_ptr<Workspace> ws;  // workspace of the synchronous entry points
     std::unique_ptr<struct Staging> stage;  // buffers of apply_D / sap_apply, freed with the gauge
     std::shared_ptr<struct Multigrid> mg;  // two-level multigrid preconditioner (qdd_mg_setup)
@@ -247,11 +265,12 @@ __host__ __device__ __forceinline__ int64_t pair_index(int64_t d, int P, int p, 
 }
 
 qdd_status ensure_copy(Gauge *g, qdd_prec prec, cudaStream_t s);
-// The fixed-point copy of links and clover (the copy of QDD_PREC_DF64).  *ok =
-// false, with QDD_OK, where FP64 arithmetic has to stand in: links that are not
-// finite or very large, or (required = false: the FP64 precision, which needs
-// no copy) an HBM budget that the copy would fill past a half.
-qdd_status ensure_fixed(Gauge *g, bool required, cudaStream_t s, bool *ok);
+// The fixed-point copy of links and (clover) of the clover term, built where it
+// is missing.  lk holds it on return; where it does not, FP64 arithmetic has to
+// stand in: links that are not finite or very large, or no room for a copy that
+// is not required (which is no error).
+using FxLock = std::shared_lock<std::shared_mutex>;
+qdd_status fx_acquire(Gauge *g, bool required, bool clover, cudaStream_t s, FxLock &lk);
 // the two-row link copy of a storage precision (FP32, FP16, BF16)
 qdd_status ensure_links12(Gauge *g, qdd_prec prec, cudaStream_t s);
 // links whose unitarity and determinant deviate by more than this keep three rows
@@ -303,8 +322,8 @@ qdd_status launch_clover_convert(Gauge *g, const double2 *src, qdd_prec dp, void
 qdd_status launch_su3_check(Gauge *g, double tol, int *d_out, cudaStream_t s);
 qdd_status launch_links12_convert(Gauge *g, qdd_prec dp, void *dst, cudaStream_t s);
 
-// clover.cu
-qdd_status launch_clover_build(Gauge *g, double csw, double kappa, int *d_singular, cudaStream_t s);
+// clover.cu: fixed = from the links' fixed-point copy (SU(3) links only)
+qdd_status launch_clover_build(Gauge *g, double csw, double kappa, int *d_singular, bool fixed, cudaStream_t s);
 
 // dslash.cu: out = D in (or out = b - D in when b != NULL); arith F64, DF64 or
 // F32; in_prec/out_prec the storage of the spinors; link/clover storage =
@@ -313,10 +332,12 @@ qdd_status launch_clover_build(Gauge *g, double csw, double kappa, int *d_singul
 qdd_status launch_dslash(Gauge *g, qdd_prec arith, qdd_prec fields_prec, const void *in, const float *in_s,
                          qdd_prec in_prec, void *out, float *out_s, qdd_prec out_prec, const double2 *b, int nrhs,
                          cudaStream_t s, const FxField *fxb = nullptr);
-// the parts of the fixed-point operator: the fields' copy, a spinor field in
-// internal FP64 or FP32 planes, the operator (out in internal planes or in the
-// host layout; b: residual form, internal planes only)
-qdd_status launch_fields_fx(Gauge *g, PrecCopy &c, cudaStream_t s);
+// the parts of the fixed-point operator: the copies of links and clover, a
+// spinor field in internal FP64 or FP32 planes, the operator (out in internal
+// planes or in the host layout; b: residual form, internal planes only); the
+// caller of the operator holds the copy (fx_acquire)
+qdd_status launch_links_fx(Gauge *g, cudaStream_t s);
+qdd_status launch_clover_fx(Gauge *g, cudaStream_t s);
 qdd_status launch_spinor_fx(Gauge *g, const void *src, qdd_prec ip, const FxField &x, int nrhs, cudaStream_t s);
 qdd_status launch_dslash_fx(Gauge *g, const FxField &x, double2 *out, bool host_layout, const double2 *b, int nrhs,
                             cudaStream_t s);

@@ -105,7 +105,7 @@ static void worker_main(Ctx *ctx)
                         const size_t need = workspace_bytes(lead.g, pm.restart_m, total, pm.sap_prec,
                                                             pm.use_sap != 0, pm.dr_k);
                         // a workspace that cannot fit next to everything else is not tried
-                        const size_t held = workspace_held(ws.get()), used = ctx->used.load();
+                        const size_t held = workspace_held(ws.get()), used = ctx->used.load() - ctx->optional.load();
                         if ((used > held ? used - held : 0) + need > ctx->budget) return QDD_EBUDGET;
                         if (held > 2 * need) workspace_release(ws.get());
                         clear_error();

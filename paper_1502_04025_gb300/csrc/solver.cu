@@ -134,8 +134,8 @@ qdd_status solve_prepare(Gauge *g, Workspace *w, const qdd_solve_params *p, cuda
     QDD_TRY(ensure_ws(g, *w, p->restart_m, p->nrhs, sp, p->use_sap == 1, p->dr_k));
     if (p->use_sap) QDD_TRY(ensure_copy(g, sp, s));
     if (p->arnoldi_prec != QDD_PREC_F64) QDD_TRY(ensure_copy(g, p->arnoldi_prec, s));
-    bool fixed = false;  // the FP64 operator's optional fixed-point copy (the true residual is always FP64)
-    QDD_TRY(ensure_fixed(g, false, s, &fixed));
+    FxLock lk;  // the FP64 operator's optional fixed-point copy (the true residual is always FP64)
+    QDD_TRY(fx_acquire(g, false, true, s, lk));
     if (p->relax_eta > 0 || p->arnoldi_prec == QDD_PREC_F32) {
         QDD_TRY(ensure_copy(g, QDD_PREC_F32, s));
         if (g->two_rows) QDD_TRY(ensure_links12(g, QDD_PREC_F32, s));

@@ -149,3 +149,33 @@ def test_extreme_values_stay_where_they_are(q, ctx, ora, prec, value):
         # a hop keeps the two spins it does not touch: some components stay finite
         assert np.isfinite(got[near]).any()
     q.qdd_destroy_gauge(g)
+
+
+def test_optional_copies_give_way_to_a_tight_budget(q):
+    """What ran within a budget without the optional fixed-point copies still does: they are given up when an
+    allocation needs their room, and built again (or replaced by FP64 arithmetic) afterwards."""
+    L, dom = (16, 8, 8, 16), (4, 4, 4, 4)
+    V = int(np.prod(L))
+    U, b = inputs.gauge_field(L, 0.5, 1001), inputs.gaussian_source(L, 2001)
+
+    def steps(budget):
+        ctx = q.qdd_create(0, budget)
+        g = q.qdd_create_gauge_field(ctx, L, dom, U)
+        q.qdd_set_clover(g, 1.0, 0.12)
+        y = q.qdd_apply_D(g, b, "f64")
+        x, rep = q.qdd_solve(g, b, tol=1e-10, sap_prec="f32", arnoldi_prec="f32")
+        z = q.qdd_apply_D(g, x, "f64")
+        used = q.qdd_memory(ctx)[0]
+        q.qdd_destroy_gauge(g)
+        assert q.qdd_memory(ctx)[0] <= 1 << 20
+        q.qdd_destroy(ctx)
+        return y, x, z, used
+
+    y0, x0, z0, used = steps(0)
+    # without the copies, with the output buffer that FP64 arithmetic needs in their place
+    budget = used - V * (2 * 36 * 16 + 4) + V * 192
+    y1, x1, z1, used1 = steps(budget)
+    assert used1 <= budget
+    for a, c in ((y0, y1), (z0, z1)):
+        assert np.abs(a - c).max() <= 1e-13 * np.abs(a).max()
+    assert np.linalg.norm(x0 - x1) <= 1e-9 * np.linalg.norm(x0)
