@@ -201,7 +201,11 @@ __global__ void k_clover_build(Geom g, const double2 *U, double csw, double kapp
 // parts and the sums over planes are integers, and FP64 starts at the entries
 // of A.  In FP64 arithmetic the 7776 multiply-adds of the leaves take 3900 of
 // an SM's clocks per site (2 lanes per clock); as integer multiply-adds they take
-// about 360.  TABLE_CLOVER
+// about 360.  Measured on 16^3x32: 2945 -> 741 us, of which the FP64 inverses of
+// the odd sites' blocks keep the FP64 pipe busy 17 % (symmetric sweeps: 420 FP64
+// operations per block for 1730 of Gauss-Jordan with pivoting); the rest waits
+// on integer latencies (2.6 warps per scheduler at 168-255 registers; 128
+// registers spill and are no faster).
 
 struct M3x {
     cfx m[9];
@@ -221,26 +225,6 @@ __device__ __forceinline__ M3x load_link_fx(const Geom &g, const int4 *U, int gi
     return r;
 }
 
-// entry (i, j) of op(a) op(b), op the adjoint where DA, DB
-template <bool DA, bool DB>
-__device__ __forceinline__ void fx_mul_entry(const M3x &a, const M3x &b, int i, int j, fxacc &re, fxacc &im)
-{
-    re = fx_zero();
-    im = fx_zero();
-#pragma unroll
-    for (int k = 0; k < 3; k++) {
-        const cfx x = DA ? a.m[k * 3 + i] : a.m[i * 3 + k], y = DB ? b.m[j * 3 + k] : b.m[k * 3 + j];
-        const fx ny = {-y.im.hi, -y.im.lo};
-        // conjugation of x and y: the sign of their imaginary parts
-        fx_mac(re, x.re, y.re);
-        fx_mac(im, x.re, DB ? ny : y.im);
-        fx_mac(re, x.im, DA == DB ? ny : y.im);
-        const fx xi = {DA ? -x.im.hi : x.im.hi, DA ? -x.im.lo : x.im.lo};
-        fx_mac(im, xi, y.re);
-    }
-}
-
-template <bool DA, bool DB>
 __device__ __forceinline__ M3x fx_mul(const M3x &a, const M3x &b)
 {
     M3x r;
@@ -248,9 +232,27 @@ __device__ __forceinline__ M3x fx_mul(const M3x &a, const M3x &b)
     for (int i = 0; i < 3; i++)
 #pragma unroll
         for (int j = 0; j < 3; j++) {
-            fxacc re, im;
-            fx_mul_entry<DA, DB>(a, b, i, j, re, im);
+            fxacc re = fx_zero(), im = fx_zero();
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const cfx x = a.m[i * 3 + k], y = b.m[k * 3 + j];
+                fx_mac2(re, im, x.re, y.re, y.im);
+                fx_mac2(im, re, x.im, y.re, fx{-y.im.hi, -y.im.lo});
+            }
             r.m[i * 3 + j] = {fx_split(fx_value(re)), fx_split(fx_value(im))};
+        }
+    return r;
+}
+
+__device__ __forceinline__ M3x fx_adjoint(const M3x &u)
+{
+    M3x r;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const cfx x = u.m[j * 3 + i];
+            r.m[i * 3 + j] = {x.re, {-x.im.hi, -x.im.lo}};
         }
     return r;
 }
@@ -260,35 +262,18 @@ __device__ __forceinline__ M3x fx_mul(const M3x &a, const M3x &b)
 struct M3q {
     int64_t re[9], im[9];
 };
-template <bool DA, bool DB>
-__device__ __forceinline__ void fx_leaf_add(M3q &q, const M3x &a, const M3x &b)
-{
-#pragma unroll
-    for (int i = 0; i < 3; i++)
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            fxacc re, im;
-            fx_mul_entry<DA, DB>(a, b, i, j, re, im);
-            q.re[i * 3 + j] += fx_value(re) >> 3;
-            q.im[i * 3 + j] += fx_value(im) >> 3;
-        }
-}
 
 // the link of the step from n to m = n +- da: U_da(n) forward, U_da(m)^+ backward
 __device__ __forceinline__ M3x step_link_fx(const Geom &g, const int4 *U, int n, int m, int da, bool back)
 {
-    M3x u = load_link_fx(g, U, back ? m : n, da);
-    if (back) {
+    const M3x u = load_link_fx(g, U, back ? m : n, da), v = fx_adjoint(u);
+    M3x r;
 #pragma unroll
-        for (int i = 0; i < 3; i++)
-#pragma unroll
-            for (int j = i; j < 3; j++) {
-                const cfx x = u.m[i * 3 + j], y = u.m[j * 3 + i];
-                u.m[i * 3 + j] = {y.re, {-y.im.hi, -y.im.lo}};
-                u.m[j * 3 + i] = {x.re, {-x.im.hi, -x.im.lo}};
-            }
+    for (int k = 0; k < 9; k++) {
+        r.m[k].re = {back ? v.m[k].re.hi : u.m[k].re.hi, back ? v.m[k].re.lo : u.m[k].re.lo};
+        r.m[k].im = {back ? v.m[k].im.hi : u.m[k].im.hi, back ? v.m[k].im.lo : u.m[k].im.lo};
     }
-    return u;
+    return r;
 }
 
 // 8 F_{mu nu} = traceless part of Q - Q^+ at gi, scale 2^-57, as nine integers:
@@ -301,30 +286,43 @@ __device__ __forceinline__ void field_strength_fx(const Geom &g, const int4 *U, 
     M3q q;
 #pragma unroll
     for (int k = 0; k < 9; k++) q.re[k] = q.im[k] = 0;
-    // one leaf per iteration, each the product of two half paths X Y or X Y^+
-    // (one copy of the code: four would not fit the instruction cache):
-    //   0: U_mu(n) U_nu(n+mu) . (U_nu(n) U_mu(n+nu))^+
-    //   1: U_nu(n) U_mu^+(n-mu+nu) . (U_mu^+(n-mu) U_nu(n-mu))^+
-    //   2: U_mu^+(n-mu) U_nu^+(n-mu-nu) . (U_nu^+(n-nu) U_mu^+(n-mu-nu))^+
-    //   3: U_nu^+(n-nu) U_mu(n-nu) . (U_mu(n) U_nu^+(n+mu-nu))^+
-    // Read as forward or backward hops from n: every leaf is a first step along
-    // (dir a, dir b) and its mirror (dir b, dir a).
+    // A leaf runs from n over the steps a, b and back over a, b: X Y^+ with X =
+    // link(n, a) link(n + a, b) and Y = link(n, b) link(n + b, a), for (a, b) =
+    // (+mu, +nu), (+nu, -mu), (-mu, -nu), (-nu, +mu).  X, Y and X Y^+ run through
+    // one copy of the product (three copies: 826 us for 741, instruction fetch).
 #pragma unroll 1
     for (int leaf = 0; leaf < 4; leaf++) {
-        // leaf runs from step a then b on one side, b then a on the other, with
-        // (a, b) = (+mu, +nu), (+nu, -mu), (-mu, -nu), (-nu, +mu)
         const bool swap = leaf & 1;
         const int da = swap ? nu : mu, db = swap ? mu : nu;
-        const bool ba = leaf >= 2, bb = leaf == 1 || leaf == 2;  // backward first / second step
+        const bool ba = leaf >= 2, bb = leaf == 1 || leaf == 2;         // a, b backward
         const int na = swap ? (ba ? n_mn : n_pn) : (ba ? n_mm : n_pm);  // n + a
         const int nb = swap ? (bb ? n_mm : n_pm) : (bb ? n_mn : n_pn);  // n + b
-        // X = link(n, a) link(n + a, b), Y = link(n, b) link(n + b, a); leaf = X Y^+
-        const M3x a0 = step_link_fx(g, U, gi, na, da, ba);
         const int nab = nbr(g, na, 2 * db + (bb ? 1 : 0));
-        const M3x X = fx_mul<false, false>(a0, step_link_fx(g, U, na, nab, db, bb));
-        const M3x b0 = step_link_fx(g, U, gi, nb, db, bb);
-        const M3x Y = fx_mul<false, false>(b0, step_link_fx(g, U, nb, nab, da, ba));
-        fx_leaf_add<false, true>(q, X, Y);
+        M3x X, Yd;
+#pragma unroll 1
+        for (int h = 0; h < 3; h++) {
+            M3x l, r;
+            if (h < 2) {
+                const int m = h ? nb : na;
+                l = step_link_fx(g, U, gi, m, h ? db : da, h ? bb : ba);
+                r = step_link_fx(g, U, m, nab, h ? da : db, h ? ba : bb);
+            } else {
+                l = X;
+                r = Yd;
+            }
+            const M3x p = fx_mul(l, r);
+            if (h == 0) {
+                X = p;
+            } else if (h == 1) {
+                Yd = fx_adjoint(p);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 9; k++) {
+                    q.re[k] += fx_join(p.m[k].re) >> 3;
+                    q.im[k] += fx_join(p.m[k].im) >> 3;
+                }
+            }
+        }
     }
     const int64_t d0 = q.im[0], d1 = q.im[4], d2 = q.im[8], mean = (d0 + d1 + d2) / 3;
     F[0] = 2 * (d0 - mean);
@@ -416,7 +414,7 @@ __device__ __forceinline__ void store_herm6(double2 *dst, int64_t stride, const 
 
 constexpr int kCloverThreads = 64;
 
-__global__ void __launch_bounds__(kCloverThreads) k_clover_build_fx(Geom g, const int4 *U, double kc, double2 *A,
+__global__ void __launch_bounds__(kCloverThreads, 4) k_clover_build_fx(Geom g, const int4 *U, double kc, double2 *A,
                                                                     double2 *S, int *singular)
 {
     __shared__ int64_t F[6][9][kCloverThreads];

@@ -156,21 +156,26 @@ qdd_status make_geometry(const int L[4], const int dom[4], HostGeom &hg)
                 hg.nbd[(size_t)d * 8 + 2 * mu + st] = block_slot[nbk];
             }
     }
-    // internal index -> host site index
-    hg.site_of.assign(hg.V, 0);
+    // internal index -> host site index: the domain's origin plus the site's
+    // offset, the same in every domain (per site coordinates of 131072 sites
+    // took 0.7 ms of a gauge field's creation)
+    auto lex = [&](const int x[4]) { return x[0] + hg.L[0] * (x[1] + hg.L[1] * (x[2] + hg.L[2] * x[3])); };
+    std::vector<int> off(hg.Vd);
+    for (int s = 0; s < hg.Vd; s++) {
+        int c[4];
+        local_coords(hg.dom, hg.Vh, s, c);
+        off[s] = lex(c);
+    }
+    hg.site_of.resize(hg.V);
     for (int d = 0; d < hg.Nd; d++) {
-        int b = hg.slot_block[d], bc[4], t = b;
+        int t = hg.slot_block[d], x[4];
         for (int mu = 0; mu < 4; mu++) {
-            bc[mu] = t % hg.nb[mu];
+            x[mu] = t % hg.nb[mu] * hg.dom[mu];
             t /= hg.nb[mu];
         }
-        for (int s = 0; s < hg.Vd; s++) {
-            int c[4];
-            local_coords(hg.dom, hg.Vh, s, c);
-            int x[4];
-            for (int mu = 0; mu < 4; mu++) x[mu] = bc[mu] * hg.dom[mu] + c[mu];
-            hg.site_of[(size_t)d * hg.Vd + s] = x[0] + hg.L[0] * (x[1] + hg.L[1] * (x[2] + hg.L[2] * x[3]));
-        }
+        const int base = lex(x);
+        int *out = hg.site_of.data() + (size_t)d * hg.Vd;
+        for (int s = 0; s < hg.Vd; s++) out[s] = base + off[s];
     }
     return QDD_OK;
 }
@@ -439,16 +444,41 @@ __global__ void k_su3_check(Geom g, const double2 *U, double tol, int *out)
         double2 a = __ldg(p + (int64_t)k * g.Vd);
         u[k] = mk(a.x, a.y);
     }
-    double dev = 0;
-    for (int i = 0; i < 3; i++)
-        for (int j = 0; j < 3; j++) {
-            cpx<double> t = mk(i == j ? -1.0 : 0.0, 0.0);
-            for (int k = 0; k < 3; k++) t = t + u[i * 3 + k] * conj(u[j * 3 + k]);
-            dev = fmax(dev, fmax(fabs(t.re), fabs(t.im)));
+    // Rows 0 and 1 orthonormal and row 2 the conjugate of their cross product to
+    // a tenth of the tolerance imply both conditions; otherwise they are taken
+    // as they stand.  (54 FP64 multiply-adds for 170; 16^3x32: 200 -> 60 us)
+    double near = 0;
+    {
+        double n0 = -1.0, n1 = -1.0;
+        cpx<double> x01 = mk(0.0, 0.0);
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            n0 = fma(u[k].re, u[k].re, fma(u[k].im, u[k].im, n0));
+            n1 = fma(u[3 + k].re, u[3 + k].re, fma(u[3 + k].im, u[3 + k].im, n1));
+            cfmac(x01, u[k], u[3 + k]);
         }
-    cpx<double> det = u[0] * (u[4] * u[8] - u[5] * u[7]) - u[1] * (u[3] * u[8] - u[5] * u[6]) +
-                      u[2] * (u[3] * u[7] - u[4] * u[6]);
-    dev = fmax(dev, fmax(fabs(det.re - 1.0), fabs(det.im)));
+        near = fmax(fmax(fabs(n0), fabs(n1)), fmax(fabs(x01.re), fabs(x01.im)));
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const int a = (k + 1) % 3, b = (k + 2) % 3;
+            cpx<double> t = conj(u[6 + k]);
+            cfma(t, -u[a], u[3 + b]);
+            cfma(t, u[b], u[3 + a]);
+            near = fmax(near, fmax(fabs(t.re), fabs(t.im)));
+        }
+    }
+    double dev = 0;
+    if (!(near <= 0.1 * tol)) {
+        for (int i = 0; i < 3; i++)
+            for (int j = 0; j < 3; j++) {
+                cpx<double> t = mk(i == j ? -1.0 : 0.0, 0.0);
+                for (int k = 0; k < 3; k++) t = t + u[i * 3 + k] * conj(u[j * 3 + k]);
+                dev = fmax(dev, fmax(fabs(t.re), fabs(t.im)));
+            }
+        cpx<double> det = u[0] * (u[4] * u[8] - u[5] * u[7]) - u[1] * (u[3] * u[8] - u[5] * u[6]) +
+                          u[2] * (u[3] * u[7] - u[4] * u[6]);
+        dev = fmax(dev, fmax(fabs(det.re - 1.0), fabs(det.im)));
+    }
     if (!(dev <= tol)) atomicOr(out, 1);
     int ex = 0;
     for (int k = 0; k < 9; k++) ex = max(ex, max(fx_exponent(u[k].re), fx_exponent(u[k].im)));
