@@ -4,8 +4,8 @@
 //
 // One CTA per domain Lambda of the colour being swept, one thread per
 // even/odd site pair (k_sap), or two threads per site pair, each with two of
-// the four directions and one clover block (k_sap_pair, the form for FP32
-// links; see there).  The domain's links and Schwarz clover blocks (A on even
+// the four directions and one clover block (k_sap_pair, the form of most
+// domains; see there and dispatch_staging).  The domain's links and Schwarz clover blocks (A on even
 // sites, A^{-1} on odd sites) are staged into shared memory with bulk async
 // copies (cp.async.bulk, completion on an mbarrier) when they fit; Sec. 3.3
 // keeps each domain resident in a core's L2 for the same reason.  Then:
@@ -277,13 +277,18 @@ struct SapBlock {
     // components in (the paired-thread form's share of the clover)
     __device__ __forceinline__ void clover_blk(int s, int b, const cpx<R> *in, cpx<R> *out) const
     {
-        static_assert(STC, "the paired-thread form stages the clover");
         cpx<R> m[18];
+        if (STC) {
 #pragma unroll
-        for (int k = 0; k < 18; k++) m[k] = ld_s<R>(sC + (b * 18 + k) * Vd + s);
+            for (int k = 0; k < 18; k++) m[k] = ld_s<R>(sC + (b * 18 + k) * Vd + s);
+        } else {
+            const typename SC::T2 *p = a.C.p + ((int64_t)d * 36 + b * 18) * Vd + s;
+#pragma unroll
+            for (int k = 0; k < 18; k++) m[k] = ld_c<R>(p + (int64_t)k * Vd);
+        }
         herm6_mul(m, in, out);
         if (SC::kScaled) {
-            const R sc = (R)sCs[s];
+            const R sc = STC ? (R)sCs[s] : (R)__ldg(a.C.scale + (int64_t)d * Vd + s);
 #pragma unroll
             for (int k = 0; k < 6; k++) out[k] = sc * out[k];
         }
@@ -872,7 +877,8 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sap(const SapArgs<R, SL, SC, SS,
 // ------------------------------------------------- paired-thread form
 //
 // The same domain visit with two threads per even/odd site pair (FP32
-// arithmetic, links and clover staged, half-fields of whole warps).  The
+// arithmetic, links staged, clover staged (STC) or read through the cache,
+// half-fields of whole warps).  The
 // first Vh threads form half 0, the others half 1 (whole warps, so every
 // branch on the half is uniform in a warp).  Half hb owns clover block hb,
 // i.e. the six components of spins (2hb, 2hb+1) of every vector of the MR
@@ -889,12 +895,13 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sap(const SapArgs<R, SL, SC, SS,
 // executes more instructions per site (each thread's clover block in scalar
 // FMAs, the exchange).  With FP32 links, where the one-thread form holds a
 // single 4-warp CTA per SM, that pays (32^3x64: 0.647 against 0.927 ms per
-// half-sweep); with 16-bit links, two one-thread CTAs share an SM and the
-// paired form is not faster (48^3x96 BF16: 2.40 against 2.29 ms).  The two
+// half-sweep), as it does with 16-bit links on domains other than 4^4 (see
+// dispatch_staging); on 4^4 domains two one-thread CTAs of fixed shape share an
+// SM and the paired form is not faster (48^3x96 BF16: 2.40 against 2.29 ms).  The two
 // partial sums are added last, and the MR dot products run over six
 // components per thread, so results agree with the one-thread form to
 // rounding, not bit for bit.
-template <typename SL, typename SC, typename SS, typename SP, int MAXT, int MINB, int SHAPE>
+template <typename SL, typename SC, typename SS, typename SP, int MAXT, int MINB, int SHAPE, bool STC>
 __global__ void __launch_bounds__(MAXT, MINB) k_sap_pair(const SapArgs<float, SL, SC, SS, SP> a)
 {
     using R = float;
@@ -912,10 +919,13 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sap_pair(const SapArgs<float, SL
     unsigned char *ptr = smem;
     typename SL::T2 *sL = (typename SL::T2 *)ptr;
     ptr += align128((size_t)36 * Vd * sizeof(typename SL::T2));
-    typename SC::T2 *sC = (typename SC::T2 *)ptr;
-    ptr += align128((size_t)36 * Vd * sizeof(typename SC::T2));
+    typename SC::T2 *sC = nullptr;
     float *sCs = nullptr;
-    if (SC::kScaled) { sCs = (float *)ptr; ptr += align128((size_t)Vd * 4); }
+    if (STC) {
+        sC = (typename SC::T2 *)ptr;
+        ptr += align128((size_t)36 * Vd * sizeof(typename SC::T2));
+        if (SC::kScaled) { sCs = (float *)ptr; ptr += align128((size_t)Vd * 4); }
+    }
     cpx<R> *sR = (cpx<R> *)ptr;  ptr += align128((size_t)12 * Vh * sizeof(cpx<R>));  // even half-field
     cpx<R> *sT = (cpx<R> *)ptr;  ptr += align128((size_t)12 * Vh * sizeof(cpx<R>));  // odd half-field
     cpx<R> *sX = (cpx<R> *)ptr;  ptr += align128((size_t)12 * Vh * sizeof(cpx<R>));  // rho_o, then exchange
@@ -929,18 +939,22 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sap_pair(const SapArgs<float, SL
         mbar_init(bar, 1);
         mbar_init(bar + 1, 1);
         fence_mbar_init();
+        if (!STC) {  // the clover blocks, read from global memory
+            prefetch_l2(a.C.p + (int64_t)d * 36 * Vd, (uint32_t)(36 * Vd * sizeof(typename SC::T2)));
+            if (SC::kScaled) prefetch_l2(a.C.scale + (int64_t)d * Vd, (uint32_t)(Vd * 4));
+        }
         prefetch_l2(a.rho.p + (int64_t)d * 12 * Vd, (uint32_t)(12 * Vd * sizeof(typename SS::T2)));
         if (!a.first_psi) prefetch_l2(a.psi.p + (int64_t)d * 12 * Vd, (uint32_t)(12 * Vd * sizeof(typename SP::T2)));
     }
     __syncthreads();
     if (i == 0) {
         const uint32_t lb = (uint32_t)(36 * Vd * sizeof(typename SL::T2));
-        const uint32_t cb = (uint32_t)(36 * Vd * sizeof(typename SC::T2));
-        const uint32_t sb = SC::kScaled ? (uint32_t)(Vd * 4) : 0;
+        const uint32_t cb = STC ? (uint32_t)(36 * Vd * sizeof(typename SC::T2)) : 0;
+        const uint32_t sb = STC && SC::kScaled ? (uint32_t)(Vd * 4) : 0;
         mbar_arrive_expect_tx(bar, lb + cb + sb);
         bulk_g2s_chunked(sL, a.U.p + (int64_t)d * 36 * Vd, lb, bar);
-        bulk_g2s_chunked(sC, a.C.p + (int64_t)d * 36 * Vd, cb, bar);
-        if (SC::kScaled) bulk_g2s_chunked(sCs, a.C.scale + (int64_t)d * Vd, sb, bar);
+        if (STC) bulk_g2s_chunked(sC, a.C.p + (int64_t)d * 36 * Vd, cb, bar);
+        if (STC && SC::kScaled) bulk_g2s_chunked(sCs, a.C.scale + (int64_t)d * Vd, sb, bar);
     }
 
     // the neighbour entries of the two directions of this half, for the
@@ -954,7 +968,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sap_pair(const SapArgs<float, SL
     __shared__ int sNbd[8];
     if (i < 8) sNbd[i] = __ldg(g.nbd + d * 8 + i);
 
-    SapBlock<R, SL, SC, SS, SP, true, true, true> B{a, g, d, Vd, Vh, sL, sC, sCs};
+    SapBlock<R, SL, SC, SS, SP, true, STC, true> B{a, g, d, Vd, Vh, sL, sC, sCs};
     const R kappa = a.kappa;
     const int nwarps = 2 * Vh / 32;
     const int nphase = 3 + 2 * a.nmr;
@@ -1230,13 +1244,13 @@ static qdd_status run_sap(Gauge *g, const SapArgs<R, SL, SC, SS, SP> &a, cudaStr
     return QDD_OK;
 }
 
-template <typename SL, typename SC, typename SS, typename SP, int MAXT, int MINB, int SHAPE>
+template <typename SL, typename SC, typename SS, typename SP, int MAXT, int MINB, int SHAPE, bool STC = true>
 static qdd_status run_sap_pair(Gauge *g, const SapArgs<float, SL, SC, SS, SP> &a, cudaStream_t s, bool pdl,
                                bool timed)
 {
     const HostGeom &hg = g->hg;
-    size_t smem = sap_smem_layout<float, SL, SC>(hg.Vd, true, true);
-    auto kern = k_sap_pair<SL, SC, SS, SP, MAXT, MINB, SHAPE>;
+    size_t smem = sap_smem_layout<float, SL, SC>(hg.Vd, true, STC);
+    auto kern = k_sap_pair<SL, SC, SS, SP, MAXT, MINB, SHAPE, STC>;
     static thread_local size_t configured = 0;
     if (configured < smem) {
         QDD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1315,19 +1329,42 @@ static qdd_status dispatch_staging(Gauge *g, const SapArgs<R, SL, SC, SS, SP> &a
             3 * (sap_smem_layout<R, SL, SC>(Vd, true, false) + 1024) <= smem_per_sm())
             return run_sap<R, SL, SC, SS, SP, true, false, 128, 3>(g, a, s, pdl, timed);
     }
-    // the paired-thread form: FP32 arithmetic, links and clover staged,
-    // half-fields of whole warps, at most 512 threads.  The default with FP32
-    // links, where the one-thread form runs one CTA of Vh threads per SM (4^4
-    // domains, 32^3x64: 0.647 against 0.927 ms per half-sweep); with 16-bit
-    // links two one-thread CTAs share an SM and the paired form, with more
-    // instructions per site, is no faster (48^3x96 BF16: 2.40 against 2.29 ms).
+    // the paired-thread form: FP32 arithmetic, links staged, half-fields of
+    // whole warps, at most 512 threads.  The default wherever it measured faster
+    // (us per half-sweep, one-thread form against this one):
+    //   FP32 links, links and clover staged: one CTA of Vh threads per SM holds the
+    //     one-thread form back (4^4, 32^3x64: 927 against 647)
+    //   FP32 links, clover read through the cache (more than 256 sites): 6x4^3,
+    //     24x16x16x24: 95 against 84; not 8x4^3, whose one-thread form has its
+    //     shape fixed at compile time (16^3x32: 50.0 against 49.8)
+    //   FP16 links, 64 to 256 sites of a half-field: 6x4^3, 24x16x16x24 (H16) 84.6
+    //     against 69.5; 8x4^3, 32^4 (H16) 328 against 303; 4^3x6, 32x16x16x24 81.7
+    //     against 71.9; not 32-site half-fields (4x4x2x2, 32x32x16x16: 95.7 against
+    //     101), nor 4^4 domains, whose one-thread form has its shape fixed at
+    //     compile time and runs twice per SM (32^3x64, 12 sources: 5.28 against
+    //     5.51 ms)
+    //   not BF16 (6x4^3, 24x32^3: 291 against 261; 48^3x96, 4^4: 2.29 against 2.40
+    //     ms): its stored residual is so coarse that the forms' different rounding
+    //     moves single components of the result by up to 8e-4
+    // The choice depends on the domain's shape and the storage only, so that a
+    // sharded lattice runs the form of the whole one.
     if constexpr (sizeof(R) == 4) {
-        const bool pair = g->sap_variant == 3 || (g->sap_variant == 0 && std::is_same<SL, StF32>::value);
-        if (pair && hg.Vh % 32 == 0 && 2 * hg.Vh <= 512 && sap_smem_layout<R, SL, SC>(Vd, true, true) <= lim) {
+        constexpr bool f32_links = std::is_same<SL, StF32>::value;
+        const bool stc = sap_smem_layout<R, SL, SC>(Vd, true, true) <= lim;
+        const bool fits = hg.Vh % 32 == 0 && 2 * hg.Vh <= 512 && (stc || sap_smem_layout<R, SL, SC>(Vd, true, false) <= lim);
+        const bool faster = f32_links ? stc || shape != 2 : std::is_same<SL, StF16>::value && hg.Vh >= 64 && shape != 1;
+        if (fits && (g->sap_variant == 3 || (g->sap_variant == 0 && faster))) {
             constexpr int kMinb = sizeof(typename SL::T2) == 4 ? 2 : 1;  // 16-bit: two 4^4 domains per SM
-            if (shape == 1) return run_sap_pair<SL, SC, SS, SP, 256, kMinb, 1>(g, a, s, pdl, timed);
-            if (shape == 2) return run_sap_pair<SL, SC, SS, SP, 512, 1, 2>(g, a, s, pdl, timed);
-            return run_sap_pair<SL, SC, SS, SP, 512, 1, 0>(g, a, s, pdl, timed);
+            if (stc) {
+                if (shape == 1) return run_sap_pair<SL, SC, SS, SP, 256, kMinb, 1>(g, a, s, pdl, timed);
+                if constexpr (!f32_links)
+                    if (shape == 2) return run_sap_pair<SL, SC, SS, SP, 512, 1, 2>(g, a, s, pdl, timed);
+                return run_sap_pair<SL, SC, SS, SP, 512, 1, 0>(g, a, s, pdl, timed);
+            }
+            if constexpr (f32_links) {  // 16-bit links and clover fit up to 512 sites
+                if (shape == 2) return run_sap_pair<SL, SC, SS, SP, 512, 1, 2, false>(g, a, s, pdl, timed);
+                return run_sap_pair<SL, SC, SS, SP, 512, 1, 0, false>(g, a, s, pdl, timed);
+            }
         }
     }
     if (sap_smem_layout<R, SL, SC>(Vd, true, true) <= lim) {
