@@ -755,17 +755,27 @@ qdd_status qdd_apply_D(qdd_gauge *g, const double *in, double *out, int nrhs, qd
     FxLock fl;
     if (arith != QDD_PREC_F32) QDD_TRY(fx_acquire(g, arith == QDD_PREC_DF64, true, s, fl));
     const bool fixed = fl.owns_lock();
-    if (!fixed) QDD_TRY(st->b.ensure(g->ctx, V * 12 * eb * nrhs));
+    // FP32 spinors: the operator widens and writes the host layout too
+    const bool direct = arith == QDD_PREC_F32 && prec == QDD_PREC_F32;
+    if (!fixed && !direct) QDD_TRY(st->b.ensure(g->ctx, V * 12 * eb * nrhs));
     const FxField fxa{st->a.p, st->a_s.as<int>()};
     if (fixed) QDD_TRY(launch_spinor_in_fx(g, din, fxa, nrhs, s));
     else QDD_TRY(launch_spinor_in(g, din, st->a.p, st->a_s.as<float>(), prec, nrhs, s));
     // a sharded field: its boundary planes (FP64, host layout) move while the operator runs
     QDD_TRY(slab_dslash_begin(g, din, false, true, nrhs, s));
-    if (!fixed)
+    if (fixed) {
+        QDD_TRY(launch_dslash_fx(g, fxa, (double2 *)dout, true, nullptr, nrhs, s));
+    } else if (direct) {
+        if (!g->have_clover) {
+            set_error("set_clover has not been called");
+            return QDD_EINVAL;
+        }
+        QDD_TRY(launch_dslash_host(g, fp, st->a.p, (double2 *)dout, nrhs, s));
+    } else {
         QDD_TRY(launch_dslash(g, arith, fp, st->a.p, st->a_s.as<float>(), prec, st->b.p, st->b_s.as<float>(), prec,
                               nullptr, nrhs, s));
-    if (fixed) QDD_TRY(launch_dslash_fx(g, fxa, (double2 *)dout, true, nullptr, nrhs, s));
-    else QDD_TRY(launch_spinor_out(g, st->b.p, st->b_s.as<float>(), dout, prec, nrhs, s));
+        QDD_TRY(launch_spinor_out(g, st->b.p, st->b_s.as<float>(), dout, prec, nrhs, s));
+    }
     QDD_TRY(slab_dslash_end(g, (double2 *)dout, false, nrhs, s));
     return finish_out(g, oio, out, nrhs, on_device, s);
 }

@@ -187,6 +187,20 @@ __device__ __forceinline__ Geom fixed_geom(const Geom &g0)
     return g;
 }
 
+// Output in the host layout: FP64, a site's 12 components together (single
+// precision results of the operator entry point, which a separate pass would
+// read and widen again).
+struct StHost {
+    using T2 = double2;
+    static constexpr bool kScaled = false;
+    static constexpr int kBytes = 16;
+    static constexpr bool kQuad = false;
+};
+struct HostOut {
+    const int *site_of;  // host site index of an internal index
+    bool a32;            // the buffer starts on a 32-byte boundary
+};
+
 // CTAs per SM the register allocation aims at.  FP16 links: 4 (the lower
 // register cap of 5 costs more in the FP16 and H16 forms: on 32^3x64, FP16
 // 181.5 -> 175.0 us and H16 193.6 -> 190.1 us at 4; FP32 and BF16 are
@@ -199,7 +213,7 @@ constexpr int dslash_min_blocks()
 
 template <typename R, typename SL, typename SC, typename SI, typename SO, bool RESID, bool L12, int VD = 0>
 __global__ void __launch_bounds__(128, (dslash_min_blocks<R, SL>())) k_dslash(Geom g0, Field<SL> U, Field<SC> A, Field<SI> in, Field<SO> out,
-                                                const double2 *b, R kappa)
+                                                const double2 *b, R kappa, HostOut ho)
 {
     const Geom g = fixed_geom<VD>(g0);
     int gi = blockIdx.x * blockDim.x + threadIdx.x;
@@ -264,6 +278,20 @@ __global__ void __launch_bounds__(128, (dslash_min_blocks<R, SL>())) k_dslash(Ge
             double2 v = __ldg(bp + (int64_t)k * g.Vd);
             y[k] = mk<R>((R)v.x - y[k].re, (R)v.y - y[k].im);
         }
+    }
+    if constexpr (std::is_same<SO, StHost>::value) {
+        double2 *o = out.p + (r * g.V + __ldg(ho.site_of + gi)) * 12;
+        double2 v[12];
+#pragma unroll
+        for (int k = 0; k < 12; k++) v[k] = make_double2(f2d(y[k].re), f2d(y[k].im));
+        if (ho.a32) {
+#pragma unroll
+            for (int k = 0; k < 12; k += 2) st_global_x4(o + k, v[k], v[k + 1]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 12; k++) o[k] = v[k];
+        }
+        return;
     }
     typename SO::T2 *op = out.p + rbase + (int64_t)d * 12 * g.Vd + s;
     if (SO::kScaled) {
@@ -701,11 +729,12 @@ static qdd_status run_dslash(Gauge *g, Field<SL> U, Field<SC> A, const void *in,
     Field<SI> fi{(typename SI::T2 *)in, (float *)in_s};
     Field<SO> fo{(typename SO::T2 *)out, out_s};
     dim3 grid((g->hg.V + 127) / 128, nrhs);
+    const HostOut ho{g->d_site_of.as<int>(), ((uintptr_t)out & 31) == 0};
     LaunchScope ls(g->ctx->timer, K_DSLASH, s);
     if (g->hg.Vd == 256)  // 4^4 domains: the volume fixed at compile time
-        k_dslash<R, SL, SC, SI, SO, RESID, L12, 256><<<grid, 128, 0, s>>>(g->geom, U, A, fi, fo, b, (R)g->kappa);
+        k_dslash<R, SL, SC, SI, SO, RESID, L12, 256><<<grid, 128, 0, s>>>(g->geom, U, A, fi, fo, b, (R)g->kappa, ho);
     else
-        k_dslash<R, SL, SC, SI, SO, RESID, L12><<<grid, 128, 0, s>>>(g->geom, U, A, fi, fo, b, (R)g->kappa);
+        k_dslash<R, SL, SC, SI, SO, RESID, L12><<<grid, 128, 0, s>>>(g->geom, U, A, fi, fo, b, (R)g->kappa, ho);
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
 }
@@ -723,6 +752,20 @@ static qdd_status run_dslash_lowp(Gauge *g, qdd_prec fp, Field<SC> A, const void
     }
     Field<SL> U{(typename SL::T2 *)g->copies[fp].links.p, nullptr};
     return run_dslash<float, SL, SC, SI, SO, false, false>(g, U, A, in, in_s, out, out_s, nullptr, nrhs, s);
+}
+
+qdd_status launch_dslash_host(Gauge *g, qdd_prec fp, const void *in, double2 *out, int nrhs, cudaStream_t s)
+{
+    QDD_TRY(ensure_copy(g, fp, s));
+    PrecCopy &c = g->copies[fp];
+    if (fp == QDD_PREC_F32)
+        return run_dslash_lowp<StF32, StF32, StF32, StHost>(g, fp, Field<StF32>{c.clov.as<float2>(), nullptr}, in,
+                                                            nullptr, out, nullptr, nrhs, s);
+    if (fp == QDD_PREC_F16S)
+        return run_dslash_lowp<StF16, StF16, StF32, StHost>(
+            g, fp, Field<StF16>{c.clov.as<__half2>(), c.clov_s.as<float>()}, in, nullptr, out, nullptr, nrhs, s);
+    set_error("the operator writes the host layout for FP32 spinors only");
+    return QDD_EINVAL;
 }
 
 qdd_status launch_dslash(Gauge *g, qdd_prec arith, qdd_prec fp, const void *in, const float *in_s, qdd_prec ip,

@@ -332,6 +332,9 @@ qdd_status launch_clover_build(Gauge *g, double csw, double kappa, int *d_singul
 qdd_status launch_dslash(Gauge *g, qdd_prec arith, qdd_prec fields_prec, const void *in, const float *in_s,
                          qdd_prec in_prec, void *out, float *out_s, qdd_prec out_prec, const double2 *b, int nrhs,
                          cudaStream_t s, const FxField *fxb = nullptr);
+// out = D in for FP32 spinors (internal planes) with FP32 or FP16 links and
+// clover, out FP64 in the host layout
+qdd_status launch_dslash_host(Gauge *g, qdd_prec fields_prec, const void *in, double2 *out, int nrhs, cudaStream_t s);
 // the parts of the fixed-point operator: the copies of links and clover, a
 // spinor field in internal FP64 or FP32 planes, the operator (out in internal
 // planes or in the host layout; b: residual form, internal planes only); the

@@ -895,7 +895,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sap(const SapArgs<R, SL, SC, SS,
 // executes more instructions per site (each thread's clover block in scalar
 // FMAs, the exchange).  With FP32 links, where the one-thread form holds a
 // single 4-warp CTA per SM, that pays (32^3x64: 0.647 against 0.927 ms per
-// half-sweep), as it does with 16-bit links on domains other than 4^4 (see
+// half-sweep), as it does with FP16 links on domains other than 4^4 (see
 // dispatch_staging); on 4^4 domains two one-thread CTAs of fixed shape share an
 // SM and the paired form is not faster (48^3x96 BF16: 2.40 against 2.29 ms).  The two
 // partial sums are added last, and the MR dot products run over six
