@@ -237,32 +237,138 @@ __global__ void __launch_bounds__(kBT) k_reduce_final(const double2 *part, int n
     }
 }
 
-// w -= sum_j coef[j] v_j (j < nvec); optional per-block partial of |w|^2
-template <int NV>
-__global__ void __launch_bounds__(kBT) k_caxpy_norm(const double2 *__restrict__ v, int nvec, int64_t ld,
-                                                    const double2 *__restrict__ coef, double2 *w, int64_t n,
-                                                    double2 *part, unsigned *count, double2 *norm2_out)
+// w = w + sign * sum_j coef[j] v_j, v in FP64 or FP32, with an optional
+// per-block partial of |w|^2.  As the multi-dot, most elements run in 64-bit
+// fixed point next to the FP64 pipe (4 multiply-adds per element and vector, 2
+// lanes per clock and SM): of every kAxpyFx + kAxpyFma elements of a thread the
+// first run in integers.  Every element of every vector has its own scale (its
+// larger component's exponent), every coefficient too; the terms are shifted to
+// the largest scale of the element's terms and added exactly, with 56 bits below
+// that scale, and the result is rounded once.  Elements with a non-finite term or
+// an extreme exponent take FP64 arithmetic.  TABLE_AXPY
+constexpr int kAxpyFx = 3, kAxpyFma = 1;
+constexpr int kAxpyBits = 58;  // of coefficients and vectors: two products per sum
+constexpr int kFxLow = 624;    // exponent field of an all-zero group: below every term that counts
+
+struct FxCoef {
+    cfx c;
+    int e;   // |c| < 2^e
+    int ok;
+};
+
+__device__ __forceinline__ double2 as_d2(double2 v) { return v; }
+__device__ __forceinline__ double2 as_d2(float2 v) { return make_double2(f2d(v.x), f2d(v.y)); }
+
+// fixed-point group of one complex number; false when it has no usable form
+__device__ __forceinline__ bool fx_single(double2 v, fxgroup &g)
+{
+    g = {0, 0, 0};
+    fx_group_add(g, v);
+    g.emax = (g.top | g.any) ? (int)(g.top >> 20) : kFxLow;
+    return g.emax > 623 && g.emax < 1423;
+}
+
+// one number with exponent field at most emax as a plain integer with `kBits`
+// bits below 2^(emax - 1022)
+template <int kBits>
+__device__ __forceinline__ int64_t fx_plain(double v, int emax)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t t = __funnelshift_l(lo, hi, 11) | 0x80000000u, r = lo << 11;
+    const uint32_t sh = (uint32_t)(emax + (64 - kBits)) - ((hi >> 20) & 0x7ffu);
+    const uint64_t m = sh > 63 ? 0 : (((uint64_t)t << 32) | r) >> sh;
+    return (int)hi < 0 ? -(int64_t)m : (int64_t)m;
+}
+
+template <int NV, int SIGN, typename T2>
+__device__ __forceinline__ double2 axpy_fma(const T2 *__restrict__ v, int64_t ld, const double2 *c, double2 b)
+{
+#pragma unroll
+    for (int j = 0; j < NV; j++) {
+        const double2 a = as_d2(__ldg(v + j * ld)), cj = c[j];
+        b.x = fma(SIGN * cj.x, a.x, b.x);
+        b.x = fma(-SIGN * cj.y, a.y, b.x);
+        b.y = fma(SIGN * cj.x, a.y, b.y);
+        b.y = fma(SIGN * cj.y, a.x, b.y);
+    }
+    return b;
+}
+
+template <int NV, int SIGN, typename T2>
+__device__ __forceinline__ double2 axpy_fx(const T2 *__restrict__ v, int64_t ld, const double2 *c, const FxCoef *fc,
+                                           double2 b)
+{
+    double2 a[NV];
+    fxgroup ga[NV], gb;
+    bool ok = fx_single(b, gb);
+    int E = gb.emax - 1022;
+#pragma unroll
+    for (int j = 0; j < NV; j++) {
+        a[j] = as_d2(__ldg(v + j * ld));
+        ok = fx_single(a[j], ga[j]) && fc[j].ok && ok;
+        E = max(E, ga[j].emax - 1022 + fc[j].e);
+    }
+    if (!ok) return axpy_fma<NV, SIGN>(v, ld, c, b);
+    int64_t sx = fx_plain<56>(b.x, E + 1022), sy = fx_plain<56>(b.y, E + 1022);
+#pragma unroll
+    for (int j = 0; j < NV; j++) {
+        const cfx x = fx_from_group<kAxpyBits>(a[j], ga[j]), cj = fc[j].c;
+        fxacc re = fx_zero(), im = fx_zero();
+        fx_mac2(re, im, cj.re, x.re, x.im);
+        fx_mac2(im, re, cj.im, x.re, fx{-x.im.hi, -x.im.lo});
+        const int sh = min(E - (ga[j].emax - 1022 + fc[j].e), 63);
+        const int64_t tx = fx_value(re) >> sh, ty = fx_value(im) >> sh;
+        if (SIGN > 0) { sx += tx; sy += ty; }
+        else { sx -= tx; sy -= ty; }
+    }
+    return make_double2(fx_to_double(sx, E - 56), fx_to_double(sy, E - 56));
+}
+
+template <int NV, int SIGN, typename T2>
+__global__ void __launch_bounds__(kBT, 2) k_axpy(const T2 *__restrict__ v, int64_t ld,
+                                                 const double2 *__restrict__ coef, double2 *w, int64_t n,
+                                                 double2 *part, unsigned *count, double2 *norm2_out)
 {
     __shared__ double2 sm[kBT / 32];
-    double2 c[NV];
-#pragma unroll
-    for (int j = 0; j < NV; j++) c[j] = j < nvec ? coef[j] : make_double2(0, 0);
-    double nrm = 0;
-    for (int64_t k = (int64_t)blockIdx.x * kBT + threadIdx.x; k < n; k += (int64_t)gridDim.x * kBT) {
-        double2 b = w[k];
-#pragma unroll
-        for (int j = 0; j < NV; j++)
-            if (j < nvec) {
-                double2 a = __ldg(v + j * ld + k);
-                b.x = fma(-c[j].x, a.x, b.x);
-                b.x = fma(c[j].y, a.y, b.x);
-                b.y = fma(-c[j].x, a.y, b.y);
-                b.y = fma(-c[j].y, a.x, b.y);
-            }
-        if (nvec > 0) w[k] = b;
-        nrm = fma(b.x, b.x, nrm);
-        nrm = fma(b.y, b.y, nrm);
+    __shared__ double2 c[NV];
+    __shared__ FxCoef fc[NV];
+    if (threadIdx.x < NV) {
+        const double2 x = coef[threadIdx.x];
+        fxgroup g;
+        FxCoef f;
+        f.ok = fx_single(x, g);
+        f.c = fx_from_group<kAxpyBits>(x, g);
+        f.e = g.emax - 1022;
+        c[threadIdx.x] = x;
+        fc[threadIdx.x] = f;
     }
+    __syncthreads();
+    double nrm = 0;
+    const int64_t step = (int64_t)gridDim.x * kBT;
+    auto put = [&](int64_t k, double2 b) {
+        w[k] = b;
+        if (part) {
+            nrm = fma(b.x, b.x, nrm);
+            nrm = fma(b.y, b.y, nrm);
+        }
+    };
+    int64_t k = (int64_t)blockIdx.x * kBT + threadIdx.x;
+    constexpr int kT = kAxpyFx + kAxpyFma;
+    for (; k + (kT - 1) * step < n; k += kT * step) {
+#pragma unroll
+        for (int i = 0; i < kAxpyFma; i++) {
+            const int64_t q = k + (kAxpyFx + i) * step;
+            put(q, axpy_fma<NV, SIGN>(v + q, ld, c, w[q]));
+        }
+        // (unrolled only for few vectors: more would not fit the instruction cache)
+        constexpr int kUnroll = NV <= 3 ? kAxpyFx : 1;
+#pragma unroll kUnroll
+        for (int i = 0; i < kAxpyFx; i++) {
+            const int64_t q = k + i * step;
+            put(q, axpy_fx<NV, SIGN>(v + q, ld, c, fc, w[q]));
+        }
+    }
+    for (; k < n; k += step) put(k, axpy_fx<NV, SIGN>(v + k, ld, c, fc, w[k]));
     if (part) {
         double2 acc[1] = {make_double2(nrm, 0)};
         block_reduce<1>(acc, sm);
@@ -274,6 +380,28 @@ __global__ void __launch_bounds__(kBT) k_caxpy_norm(const double2 *__restrict__ 
         __syncthreads();  // sm is reused
         last_block_final<1>(part, 1, 1, count, norm2_out, sm);
     }
+}
+
+// per-block partials of |w|^2
+__global__ void __launch_bounds__(kBT) k_norm2(const double2 *__restrict__ w, int64_t n, double2 *part,
+                                               unsigned *count, double2 *norm2_out)
+{
+    __shared__ double2 sm[kBT / 32];
+    double nrm = 0;
+    for (int64_t k = (int64_t)blockIdx.x * kBT + threadIdx.x; k < n; k += (int64_t)gridDim.x * kBT) {
+        const double2 b = __ldg(w + k);
+        nrm = fma(b.x, b.x, nrm);
+        nrm = fma(b.y, b.y, nrm);
+    }
+    double2 acc[1] = {make_double2(nrm, 0)};
+    block_reduce<1>(acc, sm);
+    if (threadIdx.x == 0) {
+        double2 t = make_double2(0, 0);
+        for (int ww = 0; ww < kBT / 32; ww++) t = dsum2(t, sm[ww]);
+        part[blockIdx.x] = t;
+    }
+    __syncthreads();  // sm is reused
+    last_block_final<1>(part, 1, 1, count, norm2_out, sm);
 }
 
 // out = w / sqrt(norm2[0]) (out may alias w); out32 (optional) gets the same
@@ -294,26 +422,6 @@ __global__ void k_scale_by_norm(const double2 *w, int64_t n, const double2 *norm
         a = make_double2(a.x * f, a.y * f);
         out[k] = a;
         if (out32) out32[k] = make_float2(d2f(a.x), d2f(a.y));
-    }
-}
-
-// x += sum_j coef[j] z_j, z in FP64 or FP32
-template <typename T2>
-__global__ void __launch_bounds__(kBT) k_axpy_multi(const T2 *__restrict__ z, int nvec, int64_t ld,
-                                                    const double2 *__restrict__ coef, double2 *x, int64_t n)
-{
-    for (int64_t k = (int64_t)blockIdx.x * kBT + threadIdx.x; k < n; k += (int64_t)gridDim.x * kBT) {
-        double2 b = x[k];
-        for (int j = 0; j < nvec; j++) {
-            T2 a = z[j * ld + k];
-            double2 cj = coef[j];
-            double ax = (double)a.x, ay = (double)a.y;
-            b.x = fma(cj.x, ax, b.x);
-            b.x = fma(-cj.y, ay, b.x);
-            b.y = fma(cj.x, ay, b.y);
-            b.y = fma(cj.y, ax, b.y);
-        }
-        x[k] = b;
     }
 }
 
@@ -425,11 +533,11 @@ qdd_status blas_caxpy_multi_norm(Ctx *ctx, const double2 *v, int nvec, int64_t l
             double2 *part = (last && norm2_out) ? scratch : nullptr;
             unsigned *cnt = scratch_counter(ctx, scratch);
             if (nv == 0)
-                k_caxpy_norm<1><<<nb, kBT, 0, s>>>(v, 0, ld, coef, w, n, part, cnt, norm2_out);
+                k_norm2<<<nb, kBT, 0, s>>>(w, n, scratch, cnt, norm2_out);
             else
                 nv_dispatch(nv, [&](auto c) {
-                    k_caxpy_norm<decltype(c)::value><<<nb, kBT, 0, s>>>(v + j0 * ld, nv, ld, coef + j0, w, n, part,
-                                                                        cnt, norm2_out);
+                    k_axpy<decltype(c)::value, -1, double2><<<nb, kBT, 0, s>>>(v + j0 * ld, ld, coef + j0, w, n, part,
+                                                                               cnt, norm2_out);
                 });
         }
         j0 += nv;
@@ -484,12 +592,19 @@ qdd_status blas_axpy_multi(Ctx *ctx, const void *z, bool z_f32, int nvec, int64_
                            double2 *x, int64_t n, cudaStream_t s)
 {
     if (nvec <= 0) return QDD_OK;
-    ctx->timer.work(K_BLAS, 8.0 * nvec * n, ((z_f32 ? 8.0 : 16.0) * nvec + 32.0) * n);
-    LaunchScope ls(ctx->timer, K_BLAS, s);
-    if (z_f32)
-        k_axpy_multi<float2><<<blas_blocks(ctx, n), kBT, 0, s>>>((const float2 *)z, nvec, ld, coef, x, n);
-    else
-        k_axpy_multi<double2><<<blas_blocks(ctx, n), kBT, 0, s>>>((const double2 *)z, nvec, ld, coef, x, n);
+    for (int j0 = 0; j0 < nvec; j0 += kNV) {
+        const int nv = nvec - j0 < kNV ? nvec - j0 : kNV;
+        ctx->timer.work(K_BLAS, 8.0 * nv * n, ((z_f32 ? 8.0 : 16.0) * nv + 32.0) * n);
+        LaunchScope ls(ctx->timer, K_BLAS, s);
+        nv_dispatch(nv, [&](auto c) {
+            if (z_f32)
+                k_axpy<decltype(c)::value, 1, float2><<<blas_blocks(ctx, n), kBT, 0, s>>>(
+                    (const float2 *)z + j0 * ld, ld, coef + j0, x, n, nullptr, nullptr, nullptr);
+            else
+                k_axpy<decltype(c)::value, 1, double2><<<blas_blocks(ctx, n), kBT, 0, s>>>(
+                    (const double2 *)z + j0 * ld, ld, coef + j0, x, n, nullptr, nullptr, nullptr);
+        });
+    }
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
 }
