@@ -126,7 +126,7 @@ __device__ __forceinline__ void last_block_final(const double2 *part, int stride
 // Multi-dot.  In FP64 arithmetic it is bound by the FP64 pipe (4 multiply-adds
 // per element and vector at 2 lanes per clock and SM: 2 clocks, against 0.72
 // for the 16 bytes at the measured HBM rate), so the products run in 64-bit
-// fixed point (fixed.cuh) for two elements of three: a thread gives kDotTile
+// fixed point (fixed.cuh) for four elements of seven: a thread gives kDotTile
 // elements of w and of each vector a common scale (their largest exponent),
 // sums the products exactly with integer multiply-adds and adds one FP64 number
 // per tile, vector and component to its running sum; the kDotFma elements next
@@ -136,7 +136,7 @@ __device__ __forceinline__ void last_block_final(const double2 *part, int stride
 // Measured, us (event-timed): 5 vectors of 25.2 M elements 914 -> 507 (4768 GB/s; 646 all in
 // fixed point), 3 vectors 540 -> 309 (5218 GB/s), 16 vectors of 6.3 M 706 -> 469,
 // 5 vectors of 1.57 M 81 -> 52.
-constexpr int kDotTile = 4, kDotFma = 2;
+constexpr int kDotTile = 4, kDotFma = 3;
 constexpr int kDotNV = 8;     // vectors per launch: more would not fit the instruction cache
 constexpr int kDotBits = 58;  // of both factors: 8 products per sum, |cross| <= 8 * 2 * 2^28 2^30 < 2^63
 
@@ -245,8 +245,10 @@ __global__ void __launch_bounds__(kBT) k_reduce_final(const double2 *part, int n
 // larger component's exponent), every coefficient too; the terms are shifted to
 // the largest scale of the element's terms and added exactly, with 56 bits below
 // that scale, and the result is rounded once.  Elements with a non-finite term or
-// an extreme exponent take FP64 arithmetic.  TABLE_AXPY
-constexpr int kAxpyFx = 3, kAxpyFma = 1;
+// an extreme exponent take FP64 arithmetic.  Measured, 25.2 M elements: 5 vectors with
+// the norm 906 -> 637 us, 3 vectors 682 -> 453, 5 FP32 vectors (16 bytes of x and
+// 8 per vector) 1354 -> 1019; the shares 2:1 to 4:1 and 4:2 are within 2 %.
+constexpr int kAxpyFx = 2, kAxpyFma = 1;
 constexpr int kAxpyBits = 58;  // of coefficients and vectors: two products per sum
 constexpr int kFxLow = 624;    // exponent field of an all-zero group: below every term that counts
 
