@@ -302,6 +302,76 @@ __device__ __forceinline__ void st_sp_site(typename S::T2 *blk, int s, int Vd, c
     }
 }
 
+// The 9 entries of a link and the 18 of a clover block in the copies that the
+// Schwarz kernel stages, from the domain's planes blk (36 per site).  FP64 and
+// FP32 keep planes.  16-bit storage keeps entries of a site side by side, so that
+// one access brings several: a link's entries 0-3 and 4-7 as two quads (element
+// 4*Vd*q + 4*s + k%4 of its nine planes), entry 8 as a plane; a clover block's
+// entries 0-15 as four quads, 16 and 17 as a pair.  3 and 5 accesses for 9 and 18
+// (us per half-sweep, planes against this: H16, 6x4^3 domains on 24x16x16x24 69.5 ->
+// 65.0; BF16 on 24x32^3 291 -> 277; 4^4 domains on 32^4 within 0.3 %, and 165 -> 156 on
+// 24^3x48 with the three-CTA form, whose clover reads go through the cache).
+__host__ __device__ constexpr int clover_elem16(int k, int Vd, int s)
+{
+    return k < 16 ? (k / 4) * 4 * Vd + 4 * s + k % 4 : 16 * Vd + 2 * s + (k - 16);
+}
+
+// NC: through the read-only path (global memory); else a plain load
+template <typename T, bool NC>
+__device__ __forceinline__ T ld_as(const void *p)
+{
+    if (NC) return __ldg(reinterpret_cast<const T *>(p));
+    return *reinterpret_cast<const T *>(p);
+}
+template <typename R, typename T2>
+__device__ __forceinline__ cpx<R> word_c(uint32_t w)
+{
+    const float2 v = word_f2(w, (const T2 *)nullptr);
+    return {(R)v.x, (R)v.y};
+}
+template <typename R, typename S, bool NC>
+__device__ __forceinline__ void ld_link(const typename S::T2 *blk, int mu, int s, int Vd, cpx<R> *u)
+{
+    using T2 = typename S::T2;
+    const T2 *p = blk + mu * 9 * Vd;
+    if constexpr (S::kBytes == 4) {
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            const uint4 w = ld_as<uint4, NC>(p + q * 4 * Vd + 4 * s);
+            u[4 * q + 0] = word_c<R, T2>(w.x);
+            u[4 * q + 1] = word_c<R, T2>(w.y);
+            u[4 * q + 2] = word_c<R, T2>(w.z);
+            u[4 * q + 3] = word_c<R, T2>(w.w);
+        }
+        u[8] = word_c<R, T2>(ld_as<uint32_t, NC>(p + 8 * Vd + s));
+    } else {
+#pragma unroll
+        for (int k = 0; k < 9; k++) u[k] = NC ? ld_c<R>(p + k * Vd + s) : ld_s<R>(p + k * Vd + s);
+    }
+}
+template <typename R, typename S, bool NC>
+__device__ __forceinline__ void ld_clover_blk(const typename S::T2 *blk, int b, int s, int Vd, cpx<R> *m)
+{
+    using T2 = typename S::T2;
+    const T2 *p = blk + b * 18 * Vd;
+    if constexpr (S::kBytes == 4) {
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const uint4 w = ld_as<uint4, NC>(p + q * 4 * Vd + 4 * s);
+            m[4 * q + 0] = word_c<R, T2>(w.x);
+            m[4 * q + 1] = word_c<R, T2>(w.y);
+            m[4 * q + 2] = word_c<R, T2>(w.z);
+            m[4 * q + 3] = word_c<R, T2>(w.w);
+        }
+        const uint2 w = ld_as<uint2, NC>(p + 16 * Vd + 2 * s);
+        m[16] = word_c<R, T2>(w.x);
+        m[17] = word_c<R, T2>(w.y);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 18; k++) m[k] = NC ? ld_c<R>(p + k * Vd + s) : ld_s<R>(p + k * Vd + s);
+    }
+}
+
 // ------------------------------------------------------------------ geometry
 
 // Direction k = 2*mu + b: b = 0 the forward neighbour n+mu, b = 1 the backward n-mu.

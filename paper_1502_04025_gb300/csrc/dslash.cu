@@ -88,9 +88,7 @@ __device__ __forceinline__ void load_link(const Field<S> &U, int d, int s, int m
         u[7] = conj(u[2] * u[3] - u[0] * u[5]);
         u[8] = conj(u[0] * u[4] - u[1] * u[3]);
     } else {
-        const typename S::T2 *p = U.p + ((int64_t)d * 36 + mu * 9) * Vd + s;
-#pragma unroll
-        for (int k = 0; k < 9; k++) u[k] = ld_c<R>(p + (int64_t)k * Vd);
+        ld_link<R, S, true>(U.p + (int64_t)d * 36 * Vd, mu, s, Vd, u);
     }
 }
 

@@ -420,12 +420,21 @@ __global__ void k_scale_convert(Geom g, const double2 *w, const double2 *norm2, 
     store_scaled<SO>(dst, 0, 0, g.Vd, d, s, v);
 }
 
+// whole links in the order the Schwarz kernel stages (ld_link); i runs over the
+// destination, so that a warp writes consecutive elements
 template <typename S>
-__global__ void k_links_convert(int64_t n, const double2 *src, typename S::T2 *dst)
+__global__ void k_links_convert(int64_t n, int Vd, const double2 *src, typename S::T2 *dst)
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    double2 a = __ldg(src + i);
+    int64_t j = i;
+    if constexpr (S::kBytes == 4) {
+        const int64_t link = i / (9 * Vd);  // nine planes of one domain and direction
+        const int e = (int)(i - link * 9 * Vd);
+        const int k = e < 8 * Vd ? (e / (4 * Vd)) * 4 + e % 4 : 8, s = e < 8 * Vd ? e % (4 * Vd) / 4 : e - 8 * Vd;
+        j = link * 9 * Vd + (int64_t)k * Vd + s;
+    }
+    const double2 a = __ldg(src + j);
     st_d(dst + i, mk(a.x, a.y));
 }
 
@@ -506,7 +515,8 @@ __global__ void k_links12_convert(Geom g, const double2 *src, typename S::T2 *ds
 }
 
 // clover blocks: 36 planes per site; 16-bit formats get one scale per site
-// (paired: planes stored in pairs, for the full-lattice operator's copy)
+// (paired: planes stored in pairs, for the full-lattice operator's copy; else the
+// order the Schwarz kernel stages, ld_clover_blk)
 template <typename S>
 __global__ void k_clover_convert(Geom g, const double2 *src, Field<S> dst, int paired)
 {
@@ -529,7 +539,10 @@ __global__ void k_clover_convert(Geom g, const double2 *src, Field<S> dst, int p
     }
     for (int k = 0; k < 36; k++) {
         double2 a = __ldg(p + (int64_t)k * g.Vd);
-        typename S::T2 *o = paired ? dst.p + pair_index(d, 36, k, g.Vd, s) : q + (int64_t)k * g.Vd;
+        typename S::T2 *o = q + (int64_t)k * g.Vd;
+        if (S::kBytes == 4)
+            o = paired ? dst.p + pair_index(d, 36, k, g.Vd, s)
+                       : dst.p + ((int64_t)d * 36 + k / 18 * 18) * g.Vd + clover_elem16(k % 18, g.Vd, s);
         st_c<double>(o, mk(a.x * inv, a.y * inv));
     }
 }
@@ -639,7 +652,7 @@ qdd_status launch_links_convert(Gauge *g, qdd_prec dp, void *dst, cudaStream_t s
     int64_t n = (int64_t)g->hg.V * 36;
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
     QDD_DISPATCH_PREC(dp, S, {
-        k_links_convert<S><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, g->links64.as<double2>(),
+        k_links_convert<S><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, g->hg.Vd, g->links64.as<double2>(),
                                                                         (typename S::T2 *)dst);
     });
     QDD_CUDA(cudaGetLastError());

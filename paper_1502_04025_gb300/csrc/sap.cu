@@ -233,14 +233,8 @@ struct SapBlock {
 
     __device__ __forceinline__ void link(int dd, int s, int mu, cpx<R> *u) const
     {
-        if (STL && dd == d) {
-#pragma unroll
-            for (int k = 0; k < 9; k++) u[k] = ld_s<R>(sL + (mu * 9 + k) * Vd + s);
-        } else {
-            const typename SL::T2 *p = a.U.p + ((int64_t)dd * 36 + mu * 9) * Vd + s;
-#pragma unroll
-            for (int k = 0; k < 9; k++) u[k] = ld_c<R>(p + (int64_t)k * Vd);
-        }
+        if (STL && dd == d) ld_link<R, SL, false>(sL, mu, s, Vd, u);
+        else ld_link<R, SL, true>(a.U.p + (int64_t)dd * 36 * Vd, mu, s, Vd, u);
     }
 
     // out = C(s) in : the Schwarz clover of this domain's site s, both blocks;
@@ -251,14 +245,8 @@ struct SapBlock {
         cpx<R> m[2][18];
 #pragma unroll
         for (int blk = 0; blk < 2; blk++) {
-            if (STC) {
-#pragma unroll
-                for (int k = 0; k < 18; k++) m[blk][k] = ld_s<R>(sC + (blk * 18 + k) * Vd + s);
-            } else {
-                const typename SC::T2 *p = a.C.p + ((int64_t)d * 36 + blk * 18) * Vd + s;
-#pragma unroll
-                for (int k = 0; k < 18; k++) m[blk][k] = ld_c<R>(p + (int64_t)k * Vd);
-            }
+            if (STC) ld_clover_blk<R, SC, false>(sC, blk, s, Vd, m[blk]);
+            else ld_clover_blk<R, SC, true>(a.C.p + (int64_t)d * 36 * Vd, blk, s, Vd, m[blk]);
         }
         if constexpr (sizeof(R) == 4) {
             herm6_mul_x2(m[0], m[1], in, out);  // both blocks in paired FMAs
@@ -278,14 +266,8 @@ struct SapBlock {
     __device__ __forceinline__ void clover_blk(int s, int b, const cpx<R> *in, cpx<R> *out) const
     {
         cpx<R> m[18];
-        if (STC) {
-#pragma unroll
-            for (int k = 0; k < 18; k++) m[k] = ld_s<R>(sC + (b * 18 + k) * Vd + s);
-        } else {
-            const typename SC::T2 *p = a.C.p + ((int64_t)d * 36 + b * 18) * Vd + s;
-#pragma unroll
-            for (int k = 0; k < 18; k++) m[k] = ld_c<R>(p + (int64_t)k * Vd);
-        }
+        if (STC) ld_clover_blk<R, SC, false>(sC, b, s, Vd, m);
+        else ld_clover_blk<R, SC, true>(a.C.p + (int64_t)d * 36 * Vd, b, s, Vd, m);
         herm6_mul(m, in, out);
         if (SC::kScaled) {
             const R sc = STC ? (R)sCs[s] : (R)__ldg(a.C.scale + (int64_t)d * Vd + s);
@@ -1197,11 +1179,7 @@ __global__ void __launch_bounds__(128) k_sap_face_apply(const Geom g, const Fiel
         any |= (nb[k] & kCross) != 0;
     }
     if (!any) return;  // interior site: no hop enters from another domain
-    auto lnk = [&](int mu, cpx<R> *u) {
-        const typename SL::T2 *p = U.p + ((int64_t)d * 36 + mu * 9) * Vd + s;
-#pragma unroll
-        for (int k = 0; k < 9; k++) u[k] = ld_c<R>(p + (int64_t)k * Vd);
-    };
+    auto lnk = [&](int mu, cpx<R> *u) { ld_link<R, SL, true>(U.p + (int64_t)d * 36 * Vd, mu, s, Vd, u); };
     for (int rr = 0; rr < nrhs; rr++) {
         cpx<R> acc[12], v[12];
         face_in(g, nb, __ldg(g.fcoord + s), face + rr * fstride + (int64_t)d * 6 * g.nf, lnk, acc);
@@ -1323,11 +1301,26 @@ static qdd_status dispatch_staging(Gauge *g, const SapArgs<R, SL, SC, SS, SP> &a
         if (!same) shape = 0;
     }
     // the occupancy form: links staged, clover read through the cache, three
-    // CTAs per SM (FP32 arithmetic, domains of at most 256 sites)
+    // CTAs per SM (FP32 arithmetic, domains of at most 256 sites); the same bits
+    // as the one-thread form with two.  The default on 4^4 domains in 16 bits where
+    // the third CTA pays: when the colour's domains fit in one wave of three per
+    // SM but not of two (BF16, 384 domains on 152 SMs: 69.8 -> 53.1 us per
+    // half-sweep; 320: 59.3 -> 52.1), and for BF16 beyond four per SM (648: 95.8 -> 93.1,
+    // 864: 110.2 -> 104.5, 1024: 138 -> 134, 1296: 165 -> 156, 4096: 468 -> 452 us), but not
+    // between (512: 72.5 -> 82.4, 576: 73.9 -> 85.8) nor below (256: 36.5 -> 48.8);
+    // beyond four per SM F16S is faster with two (1024: 120 -> 125 us).
     if constexpr (sizeof(R) == 4) {
-        if (g->sap_variant == 1 && hg.Vh <= 128 && 3 * (sap_smem_layout<R, SL, SC>(Vd, true, false) + 128) <= 3 * lim &&
-            3 * (sap_smem_layout<R, SL, SC>(Vd, true, false) + 1024) <= smem_per_sm())
+        const int nsm = g->ctx->nsm;
+        constexpr bool bf16 = std::is_same<SL, StBF16>::value, bits16 = sizeof(typename SL::T2) == 4;
+        const bool third = bits16 && shape == 1 &&
+                           ((a.nblocks > 2 * nsm && a.nblocks <= 3 * nsm) || (bf16 && a.nblocks > 4 * nsm));
+        if ((g->sap_variant == 1 || (g->sap_variant == 0 && third)) && hg.Vh <= 128 &&
+            sap_smem_layout<R, SL, SC>(Vd, true, false) + 128 <= lim &&
+            3 * (sap_smem_layout<R, SL, SC>(Vd, true, false) + 1024) <= smem_per_sm()) {
+            if constexpr (bits16)
+                if (shape == 1) return run_sap<R, SL, SC, SS, SP, true, false, 128, 3, 1>(g, a, s, pdl, timed);
             return run_sap<R, SL, SC, SS, SP, true, false, 128, 3>(g, a, s, pdl, timed);
+        }
     }
     // the paired-thread form: FP32 arithmetic, links staged, half-fields of
     // whole warps, at most 512 threads.  The default wherever it measured faster
