@@ -212,14 +212,14 @@ qdd_status qdd_link_compression(qdd_gauge *g, int *two_rows, int *is_su3);
  * arithmetic, links staged, half a domain a multiple of 32 sites, at most 512
  * threads; otherwise the one-thread form runs); its partial sums are added in
  * another order, so it agrees with the one-thread form to rounding.  0
- * (default) runs form 3 where it applies and is the faster one: FP32 links on
- * all domains but 8x4^3, FP16 links on domains of 128 to 512 sites but 4^4; and
- * otherwise one thread per site pair, staging the domain's links and, when
- * it fits, its clover in shared memory, with the domain size fixed at compile
- * time for 4^4 domains in 16-bit storage and 8x4^3 domains in FP32.  1 stages
- * the links only, reads the clover through the cache and is compiled for three
- * CTAs per SM (FP32 arithmetic on domains of at most 256 sites; otherwise 0
- * runs); 2 is the one-thread form with the domain size always taken at run
+ * (default) runs form 3 where it applies and is the faster one: FP32 links, and
+ * FP16 links on domains of 128 to 512 sites but 4^4; otherwise form 1 on 4^4
+ * domains in 16-bit storage where a third CTA per SM pays (by the number of
+ * domains per colour); and otherwise one thread per site pair, staging the
+ * domain's links and, when it fits, its clover in shared memory, with the domain
+ * size fixed at compile time for 4^4 domains in 16-bit storage.  1 stages the
+ * links only, reads the clover through the cache and is compiled for three CTAs
+ * per SM (FP32 arithmetic on domains of at most 256 sites; otherwise 0 runs); 2 is the one-thread form with the domain size always taken at run
  * time.  Forms 1 and 2 give the same bits as the one-thread form.  The paper
  * sizes its domains to the cache (Sec. 3.3); on the GPU the choice trades
  * staged data and registers against the number of warps an SM holds.

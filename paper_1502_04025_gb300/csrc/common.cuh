@@ -303,17 +303,29 @@ __device__ __forceinline__ void st_sp_site(typename S::T2 *blk, int s, int Vd, c
 }
 
 // The 9 entries of a link and the 18 of a clover block in the copies that the
-// Schwarz kernel stages, from the domain's planes blk (36 per site).  FP64 and
-// FP32 keep planes.  16-bit storage keeps entries of a site side by side, so that
+// Schwarz kernel stages, from the domain's planes blk (36 per site).  FP64 keeps
+// planes.  FP32 keeps pairs (entries 2q and 2q+1 of a site side by side, element
+// 2*Vd*q + 2*s + k%2; a link's entry 8 a plane): one 16-byte access for two.
+// 16-bit storage keeps entries of a site side by side, so that
 // one access brings several: a link's entries 0-3 and 4-7 as two quads (element
 // 4*Vd*q + 4*s + k%4 of its nine planes), entry 8 as a plane; a clover block's
 // entries 0-15 as four quads, 16 and 17 as a pair.  3 and 5 accesses for 9 and 18
 // (us per half-sweep, planes against this: H16, 6x4^3 domains on 24x16x16x24 69.5 ->
 // 65.0; BF16 on 24x32^3 291 -> 277; 4^4 domains on 32^4 within 0.3 %, and 165 -> 156 on
 // 24^3x48 with the three-CTA form, whose clover reads go through the cache).
-__host__ __device__ constexpr int clover_elem16(int k, int Vd, int s)
+template <typename S>
+__host__ __device__ constexpr int link_elem(int k, int Vd, int s)
 {
-    return k < 16 ? (k / 4) * 4 * Vd + 4 * s + k % 4 : 16 * Vd + 2 * s + (k - 16);
+    return S::kBytes == 16 || k == 8 ? k * Vd + s
+           : S::kBytes == 8          ? (k / 2) * 2 * Vd + 2 * s + k % 2
+                                     : (k / 4) * 4 * Vd + 4 * s + k % 4;
+}
+template <typename S>
+__host__ __device__ constexpr int clover_elem(int k, int Vd, int s)
+{
+    return S::kBytes == 16                ? k * Vd + s
+           : S::kBytes == 8 || k >= 16    ? (k / 2) * 2 * Vd + 2 * s + k % 2
+                                          : (k / 4) * 4 * Vd + 4 * s + k % 4;
 }
 
 // NC: through the read-only path (global memory); else a plain load
@@ -344,6 +356,14 @@ __device__ __forceinline__ void ld_link(const typename S::T2 *blk, int mu, int s
             u[4 * q + 3] = word_c<R, T2>(w.w);
         }
         u[8] = word_c<R, T2>(ld_as<uint32_t, NC>(p + 8 * Vd + s));
+    } else if constexpr (S::kBytes == 8) {
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const float4 w = ld_as<float4, NC>(p + q * 2 * Vd + 2 * s);
+            u[2 * q] = {(R)w.x, (R)w.y};
+            u[2 * q + 1] = {(R)w.z, (R)w.w};
+        }
+        u[8] = NC ? ld_c<R>(p + 8 * Vd + s) : ld_s<R>(p + 8 * Vd + s);
     } else {
 #pragma unroll
         for (int k = 0; k < 9; k++) u[k] = NC ? ld_c<R>(p + k * Vd + s) : ld_s<R>(p + k * Vd + s);
@@ -366,6 +386,13 @@ __device__ __forceinline__ void ld_clover_blk(const typename S::T2 *blk, int b, 
         const uint2 w = ld_as<uint2, NC>(p + 16 * Vd + 2 * s);
         m[16] = word_c<R, T2>(w.x);
         m[17] = word_c<R, T2>(w.y);
+    } else if constexpr (S::kBytes == 8) {
+#pragma unroll
+        for (int q = 0; q < 9; q++) {
+            const float4 w = ld_as<float4, NC>(p + q * 2 * Vd + 2 * s);
+            m[2 * q] = {(R)w.x, (R)w.y};
+            m[2 * q + 1] = {(R)w.z, (R)w.w};
+        }
     } else {
 #pragma unroll
         for (int k = 0; k < 18; k++) m[k] = NC ? ld_c<R>(p + k * Vd + s) : ld_s<R>(p + k * Vd + s);

@@ -427,13 +427,11 @@ __global__ void k_links_convert(int64_t n, int Vd, const double2 *src, typename 
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    int64_t j = i;
-    if constexpr (S::kBytes == 4) {
-        const int64_t link = i / (9 * Vd);  // nine planes of one domain and direction
-        const int e = (int)(i - link * 9 * Vd);
-        const int k = e < 8 * Vd ? (e / (4 * Vd)) * 4 + e % 4 : 8, s = e < 8 * Vd ? e % (4 * Vd) / 4 : e - 8 * Vd;
-        j = link * 9 * Vd + (int64_t)k * Vd + s;
-    }
+    constexpr int W = 16 / S::kBytes;  // entries side by side
+    const int64_t link = i / (9 * Vd);  // nine planes of one domain and direction
+    const int e = (int)(i - link * 9 * Vd);
+    const int k = e < 8 * Vd ? (e / (W * Vd)) * W + e % W : 8, s = e < 8 * Vd ? e % (W * Vd) / W : e - 8 * Vd;
+    const int64_t j = link * 9 * Vd + (int64_t)k * Vd + s;
     const double2 a = __ldg(src + j);
     st_d(dst + i, mk(a.x, a.y));
 }
@@ -515,7 +513,7 @@ __global__ void k_links12_convert(Geom g, const double2 *src, typename S::T2 *ds
 }
 
 // clover blocks: 36 planes per site; 16-bit formats get one scale per site
-// (paired: planes stored in pairs, for the full-lattice operator's copy; else the
+// (paired: the full-lattice operator's copy, 16-bit planes in pairs; else the
 // order the Schwarz kernel stages, ld_clover_blk)
 template <typename S>
 __global__ void k_clover_convert(Geom g, const double2 *src, Field<S> dst, int paired)
@@ -540,9 +538,8 @@ __global__ void k_clover_convert(Geom g, const double2 *src, Field<S> dst, int p
     for (int k = 0; k < 36; k++) {
         double2 a = __ldg(p + (int64_t)k * g.Vd);
         typename S::T2 *o = q + (int64_t)k * g.Vd;
-        if (S::kBytes == 4)
-            o = paired ? dst.p + pair_index(d, 36, k, g.Vd, s)
-                       : dst.p + ((int64_t)d * 36 + k / 18 * 18) * g.Vd + clover_elem16(k % 18, g.Vd, s);
+        if (paired && S::kBytes == 4) o = dst.p + pair_index(d, 36, k, g.Vd, s);
+        else if (!paired) o = dst.p + ((int64_t)d * 36 + k / 18 * 18) * g.Vd + clover_elem<S>(k % 18, g.Vd, s);
         st_c<double>(o, mk(a.x * inv, a.y * inv));
     }
 }
@@ -686,8 +683,7 @@ qdd_status launch_clover_convert(Gauge *g, const double2 *src, qdd_prec dp, void
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
     QDD_DISPATCH_PREC(dp, S, {
         Field<S> f{(typename S::T2 *)dst, dst_scale};
-        k_clover_convert<S><<<grid_sites(g->hg.V, 1, 256), 256, 0, s>>>(g->geom, src, f,
-                                                                         paired && S::kBytes == 4 ? 1 : 0);
+        k_clover_convert<S><<<grid_sites(g->hg.V, 1, 256), 256, 0, s>>>(g->geom, src, f, paired ? 1 : 0);
     });
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;

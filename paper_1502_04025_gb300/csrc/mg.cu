@@ -151,12 +151,7 @@ __device__ __forceinline__ void mg_hops_dir(const Geom &g, const Field<StF32> &U
         if (!(QDD_IN_RANGE(nd, 0, g.Nd) && QDD_IN_RANGE(ns, 0, g.Vd))) continue;
         cpx<float> x[12], u[9];
         B.load(j, nd, ns, x);
-        const float2 *up = U.p + ((int64_t)(b ? nd : d) * 36 + MU * 9) * g.Vd + (b ? ns : s);
-#pragma unroll
-        for (int k = 0; k < 9; k++) {
-            float2 v = __ldg(up + (int64_t)k * g.Vd);
-            u[k] = mk<float>(v.x, v.y);
-        }
+        ld_link<float, StF32, true>(U.p + (int64_t)(b ? nd : d) * 36 * g.Vd, MU, b ? ns : s, g.Vd, u);
         if (b == 0) hop<MU, +1>(u, x, acc);
         else hop<MU, -1>(u, x, acc);
     }

@@ -1328,8 +1328,8 @@ static qdd_status dispatch_staging(Gauge *g, const SapArgs<R, SL, SC, SS, SP> &a
     //   FP32 links, links and clover staged: one CTA of Vh threads per SM holds the
     //     one-thread form back (4^4, 32^3x64: 927 against 647)
     //   FP32 links, clover read through the cache (more than 256 sites): 6x4^3,
-    //     24x16x16x24: 95 against 84; not 8x4^3, whose one-thread form has its
-    //     shape fixed at compile time (16^3x32: 50.0 against 49.8)
+    //     24x16x16x24: 92.4 against 77.2; 8x4^3, 16^3x32: 49.0 (its shape fixed at
+    //     compile time) against 46.8
     //   FP16 links, 64 to 256 sites of a half-field: 6x4^3, 24x16x16x24 (H16) 84.6
     //     against 69.5; 8x4^3, 32^4 (H16) 328 against 303; 4^3x6, 32x16x16x24 81.7
     //     against 71.9; not 32-site half-fields (4x4x2x2, 32x32x16x16: 95.7 against
@@ -1345,7 +1345,7 @@ static qdd_status dispatch_staging(Gauge *g, const SapArgs<R, SL, SC, SS, SP> &a
         constexpr bool f32_links = std::is_same<SL, StF32>::value;
         const bool stc = sap_smem_layout<R, SL, SC>(Vd, true, true) <= lim;
         const bool fits = hg.Vh % 32 == 0 && 2 * hg.Vh <= 512 && (stc || sap_smem_layout<R, SL, SC>(Vd, true, false) <= lim);
-        const bool faster = f32_links ? stc || shape != 2 : std::is_same<SL, StF16>::value && hg.Vh >= 64 && shape != 1;
+        const bool faster = f32_links || (std::is_same<SL, StF16>::value && hg.Vh >= 64 && shape != 1);
         if (fits && (g->sap_variant == 3 || (g->sap_variant == 0 && faster))) {
             constexpr int kMinb = sizeof(typename SL::T2) == 4 ? 2 : 1;  // 16-bit: two 4^4 domains per SM
             if (stc) {
@@ -1368,10 +1368,6 @@ static qdd_status dispatch_staging(Gauge *g, const SapArgs<R, SL, SC, SS, SP> &a
         return run_sap<R, SL, SC, SS, SP, true, true>(g, a, s, pdl, timed);
     }
     if (sap_smem_layout<R, SL, SC>(Vd, true, false) <= lim) {
-        // 8x4^3 domains with FP32 links (the clover does not fit): the shape fixed at compile time
-        if constexpr (sizeof(R) == 4 && std::is_same<SL, StF32>::value)
-            if (shape == 2 && g->sap_variant == 0)
-                return run_sap<R, SL, SC, SS, SP, true, false, 256, 1, 2>(g, a, s, pdl, timed);
         return run_sap<R, SL, SC, SS, SP, true, false>(g, a, s, pdl, timed);
     }
     if (sap_smem_layout<R, SL, SC>(Vd, false, false) <= lim)
