@@ -296,6 +296,11 @@ qdd_status ensure_links12(Gauge *g, qdd_prec prec, cudaStream_t s)
 // per-gauge staging buffers for the entry points that are not the solver
 struct Staging {
     DevMem io, a, a_s, b, b_s, c, c_s, err;
+    int *host_err = nullptr;  // page-locked copy of err, read after the call's last synchronisation
+    ~Staging()
+    {
+        if (host_err) cudaFreeHost(host_err);
+    }
 };
 
 Gauge::~Gauge()
@@ -804,6 +809,7 @@ qdd_status qdd_sap_apply(qdd_gauge *g, const double *eta, double *psi, double *r
     QDD_TRY(st->b.ensure(g->ctx, sap_face_bytes(g->hg, prec, nrhs)));   // face slots
     QDD_TRY(st->c.ensure(g->ctx, V * 12 * elem_bytes(pp) * nrhs));      // psi
     QDD_TRY(st->err.ensure(g->ctx, sizeof(int)));
+    if (!st->host_err) QDD_CUDA(cudaMallocHost((void **)&st->host_err, sizeof(int)));
     if (scaled) QDD_TRY(st->a_s.ensure(g->ctx, V * 4 * nrhs));
     QDD_CUDA(cudaMemsetAsync(st->err.p, 0, sizeof(int), s));
     QDD_TRY(launch_spinor_in(g, din, st->a.p, st->a_s.as<float>(), ssp, nrhs, s));
@@ -827,14 +833,14 @@ qdd_status qdd_sap_apply(qdd_gauge *g, const double *eta, double *psi, double *r
     double *dout = nullptr;
     QDD_TRY(stage_out(g, st->io, psi, nrhs, on_device, s, &dout));
     QDD_TRY(launch_spinor_out(g, st->c.p, nullptr, dout, pp, nrhs, s));
+    QDD_CUDA(cudaMemcpyAsync(st->host_err, st->err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     QDD_TRY(finish_out(g, st->io, psi, nrhs, on_device, s));
     if (rho) {
         QDD_TRY(stage_out(g, st->io, rho, nrhs, on_device, s, &dout));
         QDD_TRY(launch_spinor_out(g, st->a.p, st->a_s.as<float>(), dout, ssp, nrhs, s));
         QDD_TRY(finish_out(g, st->io, rho, nrhs, on_device, s));
     }
-    int err = 0;
-    QDD_CUDA(cudaMemcpy(&err, st->err.p, sizeof(int), cudaMemcpyDeviceToHost));
+    const int err = *st->host_err;
     if (err) {
         set_error("device wait ran out in the Schwarz kernel (flags %d)", err);
         return QDD_ETIMEOUT;
