@@ -274,7 +274,9 @@ __global__ void __launch_bounds__(128, (dslash_min_blocks<R, SL>())) k_dslash(Ge
 #pragma unroll
         for (int k = 0; k < 12; k++) {
             double2 v = __ldg(bp + (int64_t)k * g.Vd);
-            y[k] = mk<R>((R)v.x - y[k].re, (R)v.y - y[k].im);
+            // (FP32 arithmetic: the difference is FP64's, rounded once)
+            if constexpr (sizeof(R) == 4) y[k] = mk<R>(d2f(v.x - f2d(y[k].re)), d2f(v.y - f2d(y[k].im)));
+            else y[k] = mk<R>((R)v.x - y[k].re, (R)v.y - y[k].im);
         }
     }
     if constexpr (std::is_same<SO, StHost>::value) {
@@ -326,10 +328,10 @@ __global__ void __launch_bounds__(128, (dslash_min_blocks<R, SL>())) k_dslash(Ge
 // 1536 bytes per site at the measured HBM rate, where FP64 arithmetic takes 570
 // clocks (1140 instructions at 2 lanes).  Measured (32^4 sites, 4^4 domains): 540 us,
 // 152 clocks per site, against 2113 us in FP64 arithmetic; 24x16x12x32: 91 against
-// 312 us.  What is left is latency (12 warps per SM at 168 registers; 16 at 128
-// registers spill and are no faster).  The four directions are compiled once each, for both signs (a
-// runtime flag picks the transposed link and the signs): eight bodies would
-// not fit the instruction cache.
+// 312 us.  What is left is latency: 12 to 16 warps per SM at 168 or 128 registers.
+// The four directions are compiled once each, for both signs (a runtime flag
+// picks the transposed link and the signs): eight bodies would not fit the
+// instruction cache.
 
 __device__ __forceinline__ cfx ld_cfx(const int4 *p)
 {
@@ -484,8 +486,11 @@ __device__ __forceinline__ void fx_hop_dir(const Geom &g, const FxArgs &f, int64
     }
 }
 
+// CTAs per SM the register allocation aims at: 3 with the volume fixed at
+// compile time (540 against 561 us on 32^4), 4 without (16^3x32 in 8x4^3 domains 88.7
+// against 80.2, 24x16x12x32 in 6x4x2x4 91.0 against 89.5)
 template <bool RESID, bool HOST, int VD = 0>
-__global__ void __launch_bounds__(128, 3) k_dslash_fx(Geom g0, FxArgs f, double kappa)
+__global__ void __launch_bounds__(128, VD ? 3 : 4) k_dslash_fx(Geom g0, FxArgs f, double kappa)
 {
     const Geom g = fixed_geom<VD>(g0);
     const int gt = blockIdx.x * blockDim.x + threadIdx.x;
@@ -691,18 +696,19 @@ qdd_status launch_dslash_fx(Gauge *g, const FxField &x, double2 *out, bool host_
     const FxCopy &c = g->fx;
     FxArgs f{c.links.as<int4>(), c.clov.as<int4>(), (const int4 *)x.x, c.clov_e.as<int>(), x.e, fx_link_shift(g), b,
              out, host_layout ? g->d_site_of.as<int>() : nullptr, ((uintptr_t)out & 31) == 0};
-    const dim3 grid((g->hg.V + 127) / 128, nrhs);
+    const int bt = site_block(g, nrhs);
+    const dim3 grid((g->hg.V + bt - 1) / bt, nrhs);
     LaunchScope ls(g->ctx->timer, K_DSLASH, s);
     const bool v256 = g->hg.Vd == 256;  // 4^4 domains: the volume fixed at compile time
     if (b) {
-        if (v256) k_dslash_fx<true, false, 256><<<grid, 128, 0, s>>>(g->geom, f, g->kappa);
-        else k_dslash_fx<true, false><<<grid, 128, 0, s>>>(g->geom, f, g->kappa);
+        if (v256) k_dslash_fx<true, false, 256><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
+        else k_dslash_fx<true, false><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
     } else if (host_layout) {
-        if (v256) k_dslash_fx<false, true, 256><<<grid, 128, 0, s>>>(g->geom, f, g->kappa);
-        else k_dslash_fx<false, true><<<grid, 128, 0, s>>>(g->geom, f, g->kappa);
+        if (v256) k_dslash_fx<false, true, 256><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
+        else k_dslash_fx<false, true><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
     } else {
-        if (v256) k_dslash_fx<false, false, 256><<<grid, 128, 0, s>>>(g->geom, f, g->kappa);
-        else k_dslash_fx<false, false><<<grid, 128, 0, s>>>(g->geom, f, g->kappa);
+        if (v256) k_dslash_fx<false, false, 256><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
+        else k_dslash_fx<false, false><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
     }
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
@@ -726,30 +732,31 @@ static qdd_status run_dslash(Gauge *g, Field<SL> U, Field<SC> A, const void *in,
 {
     Field<SI> fi{(typename SI::T2 *)in, (float *)in_s};
     Field<SO> fo{(typename SO::T2 *)out, out_s};
-    dim3 grid((g->hg.V + 127) / 128, nrhs);
+    const int bt = site_block(g, nrhs);
+    dim3 grid((g->hg.V + bt - 1) / bt, nrhs);
     const HostOut ho{g->d_site_of.as<int>(), ((uintptr_t)out & 31) == 0};
     LaunchScope ls(g->ctx->timer, K_DSLASH, s);
     if (g->hg.Vd == 256)  // 4^4 domains: the volume fixed at compile time
-        k_dslash<R, SL, SC, SI, SO, RESID, L12, 256><<<grid, 128, 0, s>>>(g->geom, U, A, fi, fo, b, (R)g->kappa, ho);
+        k_dslash<R, SL, SC, SI, SO, RESID, L12, 256><<<grid, bt, 0, s>>>(g->geom, U, A, fi, fo, b, (R)g->kappa, ho);
     else
-        k_dslash<R, SL, SC, SI, SO, RESID, L12><<<grid, 128, 0, s>>>(g->geom, U, A, fi, fo, b, (R)g->kappa, ho);
+        k_dslash<R, SL, SC, SI, SO, RESID, L12><<<grid, bt, 0, s>>>(g->geom, U, A, fi, fo, b, (R)g->kappa, ho);
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
 }
 
 // FP32 arithmetic on links of storage SL: the two-row copy when the gauge
 // field allows it, else whole links
-template <typename SL, typename SC, typename SI, typename SO>
+template <typename SL, typename SC, typename SI, typename SO, bool RESID = false>
 static qdd_status run_dslash_lowp(Gauge *g, qdd_prec fp, Field<SC> A, const void *in, const float *in_s, void *out,
-                                  float *out_s, int nrhs, cudaStream_t s)
+                                  float *out_s, int nrhs, cudaStream_t s, const double2 *b = nullptr)
 {
     if (g->two_rows) {
         QDD_TRY(ensure_links12(g, fp, s));
         Field<SL> U{(typename SL::T2 *)g->copies[fp].links12.p, nullptr};
-        return run_dslash<float, SL, SC, SI, SO, false, true>(g, U, A, in, in_s, out, out_s, nullptr, nrhs, s);
+        return run_dslash<float, SL, SC, SI, SO, RESID, true>(g, U, A, in, in_s, out, out_s, b, nrhs, s);
     }
     Field<SL> U{(typename SL::T2 *)g->copies[fp].links.p, nullptr};
-    return run_dslash<float, SL, SC, SI, SO, false, false>(g, U, A, in, in_s, out, out_s, nullptr, nrhs, s);
+    return run_dslash<float, SL, SC, SI, SO, RESID, false>(g, U, A, in, in_s, out, out_s, b, nrhs, s);
 }
 
 qdd_status launch_dslash_host(Gauge *g, qdd_prec fp, const void *in, double2 *out, int nrhs, cudaStream_t s)
@@ -764,6 +771,13 @@ qdd_status launch_dslash_host(Gauge *g, qdd_prec fp, const void *in, double2 *ou
             g, fp, Field<StF16>{c.clov.as<__half2>(), c.clov_s.as<float>()}, in, nullptr, out, nullptr, nrhs, s);
     set_error("the operator writes the host layout for FP32 spinors only");
     return QDD_EINVAL;
+}
+
+qdd_status launch_dslash_residual32(Gauge *g, const void *in, const double2 *b, float2 *out, cudaStream_t s)
+{
+    QDD_TRY(ensure_copy(g, QDD_PREC_F32, s));
+    const Field<StF32> A{g->copies[QDD_PREC_F32].clov.as<float2>(), nullptr};
+    return run_dslash_lowp<StF32, StF32, StF32, StF32, true>(g, QDD_PREC_F32, A, in, nullptr, out, nullptr, 1, s, b);
 }
 
 qdd_status launch_dslash(Gauge *g, qdd_prec arith, qdd_prec fp, const void *in, const float *in_s, qdd_prec ip,

@@ -182,7 +182,7 @@ qdd_status make_geometry(const int L[4], const int dom[4], HostGeom &hg)
 
 // ------------------------------------------------------------------ kernels
 
-// threads of a block of the one-thread-per-site conversions
+// threads of a block of the one-thread-per-site conversions (at most)
 constexpr int kSiteThreads = 128;
 
 // Spinor conversions between the host layout (FP64, one site's 12 components
@@ -571,10 +571,11 @@ qdd_status launch_spinor_in(Gauge *g, const double *src, void *dst, float *dst_s
 {
     const HostGeom &hg = g->hg;
     int64_t rs = (int64_t)hg.V * 12, ss = hg.V;
+    const int bt = site_block(g, nrhs);
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
     QDD_DISPATCH_PREC(prec, S, {
         Field<S> f{(typename S::T2 *)dst, dst_scale};
-        k_spinor_in<S><<<grid_sites(hg.V, nrhs, kSiteThreads), kSiteThreads, 0, s>>>(
+        k_spinor_in<S><<<grid_sites(hg.V, nrhs, bt), bt, 0, s>>>(
             g->geom, g->d_site_of.as<int>(), (const double2 *)src, f, rs, ss, ((uintptr_t)src & 31) == 0);
     });
     QDD_CUDA(cudaGetLastError());
@@ -584,8 +585,9 @@ qdd_status launch_spinor_in(Gauge *g, const double *src, void *dst, float *dst_s
 qdd_status launch_spinor_in_fx(Gauge *g, const double *src, const FxField &x, int nrhs, cudaStream_t s)
 {
     const HostGeom &hg = g->hg;
+    const int bt = site_block(g, nrhs);
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
-    k_spinor_in_fx<<<grid_sites(hg.V, nrhs, kSiteThreads), kSiteThreads, 0, s>>>(
+    k_spinor_in_fx<<<grid_sites(hg.V, nrhs, bt), bt, 0, s>>>(
         g->geom, g->d_site_of.as<int>(), (const double2 *)src, (int4 *)x.x, x.e, ((uintptr_t)src & 31) == 0);
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
@@ -596,10 +598,11 @@ qdd_status launch_spinor_out(Gauge *g, const void *src, const float *src_scale, 
 {
     const HostGeom &hg = g->hg;
     int64_t rs = (int64_t)hg.V * 12, ss = hg.V;
+    const int bt = site_block(g, nrhs);
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
     QDD_DISPATCH_PREC(prec, S, {
         Field<S> f{(typename S::T2 *)src, (float *)src_scale};
-        k_spinor_out<S><<<grid_sites(hg.V, nrhs, kSiteThreads), kSiteThreads, 0, s>>>(
+        k_spinor_out<S><<<grid_sites(hg.V, nrhs, bt), bt, 0, s>>>(
             g->geom, g->d_site_of.as<int>(), f, rs, ss, (double2 *)dst, ((uintptr_t)dst & 31) == 0);
     });
     QDD_CUDA(cudaGetLastError());

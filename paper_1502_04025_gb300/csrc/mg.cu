@@ -254,6 +254,9 @@ __global__ void __launch_bounds__(kMgThreads) k_mg_coarse_build(Geom g, Field<St
 // rc[d][chi * nv + k] = <P_(d,chi,k), v>, one CTA per aggregate.  Each
 // thread reads its entries of v once and accumulates all NV products (v is
 // read once, P once); warp shuffles, then a fixed-order sum over the warps.
+__device__ __forceinline__ float to_f(double v) { return d2f(v); }
+__device__ __forceinline__ float to_f(float v) { return v; }
+
 template <int NV, typename T2>
 __global__ void __launch_bounds__(kMgThreads) k_mg_restrict(const float2 *P, int64_t stride, int Vd, const T2 *v,
                                                             float2 *rc)
@@ -268,7 +271,7 @@ __global__ void __launch_bounds__(kMgThreads) k_mg_restrict(const float2 *P, int
         for (int k = 0; k < NV; k++) px[k] = py[k] = 0.f;
         for (int e = threadIdx.x; e < n; e += blockDim.x) {
             const T2 b = v[base + e];
-            const float bx = (float)b.x, by = (float)b.y;
+            const float bx = to_f(b.x), by = to_f(b.y);
 #pragma unroll
             for (int k = 0; k < NV; k++) {
                 const float2 a = __ldg(P + k * stride + base + e);
@@ -635,12 +638,14 @@ struct Multigrid {
     }
 };
 
+// src64 NULL: M.rho already holds the source
 static qdd_status mg_sap(Gauge *g, Multigrid &M, qdd_prec sp, const double2 *src64, void *psi, bool accumulate,
                          int ncy, cudaStream_t s)
 {
     // rho = src in the smoother's storage, psi (+)= M_SAP rho
-    QDD_TRY(launch_spinor_convert(g, src64, nullptr, QDD_PREC_F64, M.rho.p, M.rho_s.as<float>(), spinor_store(sp), 1,
-                                  s));
+    if (src64)
+        QDD_TRY(launch_spinor_convert(g, src64, nullptr, QDD_PREC_F64, M.rho.p, M.rho_s.as<float>(), spinor_store(sp),
+                                      1, s));
     SapBuffers sb{M.rho.p, M.face.p, psi, M.rho_s.as<float>()};
     SeqScope seq(g->ctx->timer, K_SAP, s);
     for (int hs = 0; hs < 2 * ncy; hs++)
@@ -714,6 +719,12 @@ static qdd_status mg_vcycle_with(Gauge *g, Multigrid &M, const double2 *v, void 
     }
     if (M.p.post_ncy > 0) {
         // r = v - D z, then z += M_SAP r
+        if (zp == QDD_PREC_F32 && spinor_store(M.p.sap_prec) == QDD_PREC_F32) {
+            // the operator writes the smoother's FP32 residual itself (two FP64 passes
+            // over the field and a conversion less: 16^3x32 V-cycle 732 -> 722 us)
+            QDD_TRY(launch_dslash_residual32(g, z, v, M.rho.as<float2>(), s));
+            return mg_sap(g, M, M.p.sap_prec, nullptr, z, true, M.p.post_ncy, s);
+        }
         const qdd_prec ar = zp == QDD_PREC_F64 ? QDD_PREC_F64 : QDD_PREC_F32;
         const FxField fxb{M.r64.p, M.rho.as<int>()};  // both are written after the operator
         QDD_TRY(launch_dslash(g, ar, ar, z, nullptr, zp, M.t64.p, nullptr, QDD_PREC_F64, nullptr, 1, s, &fxb));
