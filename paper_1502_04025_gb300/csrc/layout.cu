@@ -220,6 +220,22 @@ __device__ __forceinline__ void store_scaled(Field<S> f, int64_t base, int64_t s
     st_sp_site<float, S>(f.p + base + (int64_t)d * 12 * Vd, s, Vd, v);
 }
 
+// FP64 (re, im) divided by the site's scale m, rounded through FP32 to 16 bits.
+// y: the same in FP32; inv = 1 / m in FP32 (0 and small = true where m is near
+// the end of its range).
+template <typename T2>
+__device__ __forceinline__ uint32_t scaled_word(double re, double im, cpx<float> y, float m, float inv, bool small)
+{
+    const T2 *tag = nullptr;
+    const float a = inv * y.re, b = inv * y.im;
+    const float lo = 1.f - 0x1p-21f, hi = 1.f + 0x1p-21f;
+    const uint32_t w = f2_word(a * lo, b * lo, tag);
+    if (!small && w == f2_word(a * hi, b * hi, tag)) return w;
+    asm volatile("" : "+f"(m));  // the FP64 division stays on this path (hoisted, it would run for every site)
+    const double inv64 = m > 0.f ? 1.0 / (double)m : 0.0;
+    return f2_word((float)(re * inv64), (float)(im * inv64), tag);
+}
+
 // The 12 FP64 components v of a site in a 16-bit storage: each is the FP64
 // quotient by the site's scale, rounded (through FP32) to 16 bits.  FP64
 // multiplications would bind the pass (24 per site at 2 per clock and SM), so
@@ -232,7 +248,6 @@ template <typename S>
 __device__ __forceinline__ void store_scaled_d(Field<S> f, int64_t base, int64_t sbase, int Vd, int d, int s,
                                                const cpx<double> *v)
 {
-    const typename S::T2 *tag = nullptr;
     cpx<float> y[12];
     float m = 0.f;
 #pragma unroll
@@ -245,15 +260,7 @@ __device__ __forceinline__ void store_scaled_d(Field<S> f, int64_t base, int64_t
     const float inv = small ? 0.f : 1.f / m;
     uint32_t w[12];
 #pragma unroll
-    for (int k = 0; k < 12; k++) {
-        const float a = inv * y[k].re, b = inv * y[k].im;
-        const float lo = 1.f - 0x1p-21f, hi = 1.f + 0x1p-21f;
-        w[k] = f2_word(a * lo, b * lo, tag);
-        if (small || w[k] != f2_word(a * hi, b * hi, tag)) {
-            const double inv64 = m > 0.f ? 1.0 / (double)m : 0.0;
-            w[k] = f2_word((float)(v[k].re * inv64), (float)(v[k].im * inv64), tag);
-        }
-    }
+    for (int k = 0; k < 12; k++) w[k] = scaled_word<typename S::T2>(v[k].re, v[k].im, y[k], m, inv, small);
     typename S::T2 *p = f.p + base + (int64_t)d * 12 * Vd;
     if constexpr (S::kQuad) {
         uint4 *q = reinterpret_cast<uint4 *>(p) + s;
@@ -512,7 +519,8 @@ __global__ void k_links12_convert(Geom g, const double2 *src, typename S::T2 *ds
         }
 }
 
-// clover blocks: 36 planes per site; 16-bit formats get one scale per site
+// clover blocks: 36 planes per site; 16-bit formats get one scale per site (32^3x64
+// BF16: FP64 maxima and products 868 us, this form 450)
 // (paired: the full-lattice operator's copy, 16-bit planes in pairs; else the
 // order the Schwarz kernel stages, ld_clover_blk)
 template <typename S>
@@ -524,23 +532,26 @@ __global__ void k_clover_convert(Geom g, const double2 *src, Field<S> dst, int p
     split_index(g, gi, d, s);
     const double2 *p = src + (int64_t)d * 36 * g.Vd + s;
     typename S::T2 *q = dst.p + (int64_t)d * 36 * g.Vd + s;
-    double inv = 1.0;
+    float m = 0.f;
     if (S::kScaled) {
-        double m = 0;
         for (int k = 0; k < 36; k++) {
             double2 a = __ldg(p + (int64_t)k * g.Vd);
-            m = fmax(m, fmax(fabs(a.x), fabs(a.y)));
+            m = fmaxf(m, fmaxf(fabsf(d2f(a.x)), fabsf(d2f(a.y))));
         }
-        float sc = (float)m;
-        dst.scale[gi] = sc;
-        inv = m > 0 ? 1.0 / (double)sc : 0.0;
+        dst.scale[gi] = m;
     }
+    const bool small = m < 0x1p-100f;
+    const float inv = small ? 0.f : 1.f / m;
     for (int k = 0; k < 36; k++) {
         double2 a = __ldg(p + (int64_t)k * g.Vd);
         typename S::T2 *o = q + (int64_t)k * g.Vd;
         if (paired && S::kBytes == 4) o = dst.p + pair_index(d, 36, k, g.Vd, s);
         else if (!paired) o = dst.p + ((int64_t)d * 36 + k / 18 * 18) * g.Vd + clover_elem<S>(k % 18, g.Vd, s);
-        st_c<double>(o, mk(a.x * inv, a.y * inv));
+        if constexpr (S::kScaled)
+            *reinterpret_cast<uint32_t *>(o) =
+                scaled_word<typename S::T2>(a.x, a.y, mk(d2f(a.x), d2f(a.y)), m, inv, small);
+        else
+            st_d(o, mk(a.x, a.y));
     }
 }
 
