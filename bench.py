@@ -63,7 +63,7 @@ CONFIGS = {
     2: dict(WL, source="gaussian", nrhs=1,
             name=("16^3x32 Wilson-clover, c_sw 1.0, kappa 0.125, eps 0.5 links; SAP-FGMRES(16), 8x4x4x4 domains, "
                   "nmr 4, ncy 4, FP32 preconditioner, FP64 outer (Gram-Schmidt, least squares, solution, true "
-                  "residual; double-float Arnoldi operator relaxed to FP32 below est 1e-5), tol 1e-10, "
+                  "residual; fixed-point Arnoldi operator relaxed to FP32 below est 1e-5), tol 1e-10, "
                   "1 Gaussian source")),
     3: dict(L=(32, 32, 32, 64), dom=(4, 4, 4, 4), eps=0.7, csw=1.5, kappa=0.1355, gauge_seed=1003, source_seed=2003,
             nmr=4, ncy=4, m=16, tol=1e-10, sap_prec="f16", arnoldi_prec="df64", relax_eta=1e-6, reorth=0,
@@ -74,7 +74,7 @@ CONFIGS = {
             source="z2", nrhs=1,
             name=("48^3x96 (10,616,832 sites), eps 0.7, c_sw 1.5, kappa 0.1355, 4^4 domains, nmr 4, ncy 4, "
                   "BF16-stored Schwarz preconditioner with FP32 arithmetic, FP64 FGMRES(16) (Gram-Schmidt, least "
-                  "squares, solution, true residual; double-float Arnoldi operator relaxed to FP32 below est "
+                  "squares, solution, true residual; fixed-point Arnoldi operator relaxed to FP32 below est "
                   "1e-5), tol 1e-10, one Z2 noise source")),
 }
 
@@ -132,7 +132,7 @@ def op_bytes_per_site(prec, three_rows=True):
     carry one FP32 scale per site."""
     rows = 3 if three_rows or prec in ("f64", "df64") else 2
     if prec in ("f64", "df64"):
-        return 4 * 9 * 16 + 36 * 16 + 2 * 12 * 16  # df64 splits FP64 values into FP32 pairs: the same bytes
+        return 4 * 9 * 16 + 36 * 16 + 2 * 12 * 16  # fixed point: two 32-bit limbs per real, the same bytes
     link = 4 * rows * 3 * (8 if prec == "f32" else 4)
     clover = 36 * 8 if prec == "f32" else 36 * 4 + 4
     spinor = 12 * 8 if prec in ("f32", "h16") else 12 * 4 + 4
@@ -928,7 +928,7 @@ SERVE_KAPPAS = [0.120, 0.125, 0.130, 0.135]
 def run_serve(args):
     """Poisson arrivals of solves on four lattice sizes with kappa in
     [0.120, 0.135] (four resident values) and 1-12 right-hand sides, FP32
-    preconditioner, double-float Arnoldi operator, tol 1e-10, admission by an
+    preconditioner, fixed-point Arnoldi operator, tol 1e-10, admission by an
     80% HBM budget; reports p50/p99 latency (submit to result) and solves/s."""
     from paper_1502_04025_gb300 import build
 

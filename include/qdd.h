@@ -200,7 +200,7 @@ void qdd_destroy_gauge(qdd_gauge *g);
  * and |det U - 1| <= 1e-10); when all pass, two-row storage is on.
  * qdd_set_link_compression(g, 0) switches it off; (g, 1) switches it back
  * on and returns QDD_EINVAL for a field that failed the check.  The FP64
- * and double-float operators and the Schwarz kernel read whole links.
+ * and DF64 operators and the Schwarz kernel read whole links.
  * qdd_link_compression reports the setting and the check's outcome.
  */
 qdd_status qdd_set_link_compression(qdd_gauge *g, int two_rows);
