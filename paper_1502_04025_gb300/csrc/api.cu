@@ -305,7 +305,7 @@ struct Staging {
 
 Gauge::~Gauge()
 {
-    if (!ctx) return;
+    if (!registered) return;
     {
         std::lock_guard<std::mutex> lk(ctx->gauges_mu);
         for (size_t k = 0; k < ctx->gauges.size(); k++)
@@ -515,6 +515,7 @@ qdd_status qdd_create_gauge_field(qdd_ctx *ctx, const int L[4], const int dom[4]
     {
         std::lock_guard<std::mutex> lk(ctx->gauges_mu);
         ctx->gauges.push_back(g.get());
+        g->registered = true;
     }
     *out = g.release();
     return QDD_OK;

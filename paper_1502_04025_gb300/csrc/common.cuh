@@ -314,13 +314,6 @@ __device__ __forceinline__ void st_sp_site(typename S::T2 *blk, int s, int Vd, c
 // 65.0; BF16 on 24x32^3 291 -> 277; 4^4 domains on 32^4 within 0.3 %, and 165 -> 156 on
 // 24^3x48 with the three-CTA form, whose clover reads go through the cache).
 template <typename S>
-__host__ __device__ constexpr int link_elem(int k, int Vd, int s)
-{
-    return S::kBytes == 16 || k == 8 ? k * Vd + s
-           : S::kBytes == 8          ? (k / 2) * 2 * Vd + 2 * s + k % 2
-                                     : (k / 4) * 4 * Vd + 4 * s + k % 4;
-}
-template <typename S>
 __host__ __device__ constexpr int clover_elem(int k, int Vd, int s)
 {
     return S::kBytes == 16                ? k * Vd + s

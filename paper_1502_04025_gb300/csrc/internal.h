@@ -228,6 +228,7 @@ struct Slab {
 
 struct Gauge {
     Ctx *ctx = nullptr;
+    bool registered = false;     // listed in ctx->gauges (until the context is destroyed)
     std::unique_ptr<Slab> slab;  // set for a field sharded in t
     HostGeom hg;
     Geom geom{};

@@ -209,6 +209,8 @@ Ctx::~Ctx()
     }
     q_cv.notify_all();
     for (auto &t : workers) t.join();
+    std::lock_guard<std::mutex> lk(gauges_mu);
+    for (Gauge *g : gauges) g->registered = false;  // fields that outlive their context leave it alone
 }
 
 }  // namespace qdd
