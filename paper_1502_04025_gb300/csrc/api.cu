@@ -177,8 +177,11 @@ void DevMem::release()
 
 // -------------------------------------------------------- precision copies
 
-// link entries up to 2^64 have a fixed-point copy
-constexpr int kMaxFixedLinkExp = 64;
+// Links have a fixed-point copy up to 2^64, and where their sizes differ by no
+// more than 2^4: the field has one scale, 58 bits below its largest entry, so
+// a link 2^4 smaller keeps the 53 bits of an FP64 number below its own largest.
+// SU(3) links (largest entries between 0.57 and 1) and unitary ones always do.
+constexpr int kMaxFixedLinkExp = 64, kMaxFixedLinkSpread = 4;
 
 static size_t elem_bytes(qdd_prec p)
 {
@@ -258,7 +261,7 @@ qdd_status fx_acquire(Gauge *g, bool required, bool clover, cudaStream_t s, FxLo
         set_error("set_clover has not been called");
         return QDD_EINVAL;
     }
-    if (g->link_exp > kMaxFixedLinkExp) return QDD_OK;
+    if (g->link_exp > kMaxFixedLinkExp || g->link_spread > kMaxFixedLinkSpread) return QDD_OK;
     FxCopy &f = g->fx;
     for (int turn = 0; turn < 3; turn++) {  // an optional copy may be given up between the two locks
         lk = FxLock(f.mu);
@@ -503,12 +506,13 @@ qdd_status qdd_create_gauge_field(qdd_ctx *ctx, const int L[4], const int dom[4]
     QDD_TRY(launch_links_to_internal(g.get(), src, 0));
     // SU(3) links (to rounding) let the full-lattice operator read two rows per link
     DevMem bad;
-    QDD_TRY(bad.alloc(ctx, 2 * sizeof(int)));
+    QDD_TRY(bad.alloc(ctx, 3 * sizeof(int)));
     QDD_TRY(launch_su3_check(g.get(), kSu3Tol, bad.as<int>(), 0));
-    int h_bad[2] = {1, 0};
+    int h_bad[3] = {1, 0, 0};
     QDD_CUDA(cudaMemcpy(h_bad, bad.p, sizeof(h_bad), cudaMemcpyDeviceToHost));
     g->su3 = h_bad[0] == 0;
     g->link_exp = h_bad[1] == 0x7ff ? 1 << 20 : std::max(h_bad[1] - 1022, -800);
+    g->link_spread = std::max(h_bad[1] - (0x7ff - h_bad[2]), 0);
     g->two_rows = g->su3;
     QDD_CUDA(cudaDeviceSynchronize());
     ctx->timer.resolve();

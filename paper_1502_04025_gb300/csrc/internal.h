@@ -236,6 +236,7 @@ struct Gauge {
     DevMem links64;           // FP64 links, internal layout
     bool su3 = false;         // every link SU(3) to kSu3Tol
     int link_exp = 1 << 20;   // every link entry below 2^link_exp in magnitude (huge when one is not finite)
+    int link_spread = 0;      // and the largest entry of every link (but zero ones) at least 2^(link_exp - 1 - this)
     bool two_rows = false;    // the FP32/16-bit full-lattice operator reads two rows per link
     bool have_clover = false;
     int sap_variant = 0;      // Schwarz kernel form (qdd_set_schwarz_variant)
@@ -328,7 +329,8 @@ qdd_status launch_links_convert(Gauge *g, qdd_prec dp, void *dst, cudaStream_t s
 qdd_status launch_clover_convert(Gauge *g, const double2 *src, qdd_prec dp, void *dst, float *dst_scale,
                                  cudaStream_t s, bool paired = false);
 // d_out[0] = 1 when some link is not SU(3) to tol; d_out[1] = the largest FP64
-// exponent field of the link entries; two-row copy of the links
+// exponent field of the link entries, d_out[2] = 0x7ff less the smallest of the
+// non-zero links' own largest ones; two-row copy of the links
 qdd_status launch_su3_check(Gauge *g, double tol, int *d_out, cudaStream_t s);
 qdd_status launch_links12_convert(Gauge *g, qdd_prec dp, void *dst, cudaStream_t s);
 

@@ -444,7 +444,9 @@ __global__ void k_links_convert(int64_t n, int Vd, const double2 *src, typename 
 }
 
 // Sets out[0] when a link is not SU(3) to tol: max |(U U^+ - 1)_ij| or
-// |det U - 1|; out[1] = the largest FP64 exponent field of the link entries.
+// |det U - 1|; out[1] = the largest FP64 exponent field of the link entries;
+// out[2] = 0x7ff less the smallest of the links' own largest exponent fields
+// (links of zeros left out).
 // One thread per link (domain d, direction mu, site s).
 __global__ void k_su3_check(Geom g, const double2 *U, double tol, int *out)
 {
@@ -495,8 +497,13 @@ __global__ void k_su3_check(Geom g, const double2 *U, double tol, int *out)
     }
     if (!(dev <= tol)) atomicOr(out, 1);
     int ex = 0;
-    for (int k = 0; k < 9; k++) ex = max(ex, max(fx_exponent(u[k].re), fx_exponent(u[k].im)));
+    bool zero = true;
+    for (int k = 0; k < 9; k++) {
+        ex = max(ex, max(fx_exponent(u[k].re), fx_exponent(u[k].im)));
+        zero = zero && u[k].re == 0 && u[k].im == 0;
+    }
     if (ex > *(volatile int *)(out + 1)) atomicMax(out + 1, ex);
+    if (!zero && 0x7ff - ex > *(volatile int *)(out + 2)) atomicMax(out + 2, 0x7ff - ex);
 }
 
 // The first two rows of every link: 24 planes per site, plane mu*6 + 3*row + col
@@ -674,7 +681,7 @@ qdd_status launch_su3_check(Gauge *g, double tol, int *d_out, cudaStream_t s)
 {
     const int64_t n = (int64_t)g->hg.V * 4;
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
-    QDD_CUDA(cudaMemsetAsync(d_out, 0, 2 * sizeof(int), s));
+    QDD_CUDA(cudaMemsetAsync(d_out, 0, 3 * sizeof(int), s));
     k_su3_check<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g->geom, g->links64.as<double2>(), tol, d_out);
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
