@@ -335,9 +335,10 @@ qdd_status qdd_layout_faces(const int L[4], const int dom[4], int foff[8], uint3
  * out = D in for nrhs spinors (host layout), periodic boundary conditions.
  * prec = QDD_PREC_F64 and QDD_PREC_DF64 compute in 64-bit fixed point, to
  * FP64's accuracy or better against the largest component of the sites
- * involved; both compute in FP64 arithmetic where the links have no
- * fixed-point copy (not finite, above 2^64, or of sizes that differ by more than
- * 2^4 from link to link), QDD_PREC_F64 also where a copy would fill the HBM
+ * involved; both compute in FP64 arithmetic where the fields have no
+ * fixed-point copy (links not finite, outside 2^-60..2^64, or of sizes that differ
+ * by more than 2^4 from link to link; a clover term whose largest entry lies
+ * outside 2^-60..2^60 at some site), QDD_PREC_F64 also where a copy would fill the HBM
  * budget past a half; QDD_PREC_F32 converts links, clover
  * and input to FP32 and computes in FP32 (1848 flop per site); F16S / BF16S
  * read 16-bit links/clover/spinor with FP32 arithmetic.

@@ -122,7 +122,7 @@ static void fx_release(Gauge *g)
     f.links.release();
     f.clov.release();
     f.clov_e.release();
-    f.have_links = f.have_clov = f.required = false;
+    f.have_links = f.have_clov = f.required = f.wide = false;
 }
 
 // Gives up optional fixed-point copies that nobody reads, until at least
@@ -177,11 +177,15 @@ void DevMem::release()
 
 // -------------------------------------------------------- precision copies
 
-// Links have a fixed-point copy up to 2^64, and where their sizes differ by no
-// more than 2^4: the field has one scale, 58 bits below its largest entry, so
+// Links have a fixed-point copy from 2^-60 to 2^64, and where their sizes differ
+// by no more than 2^4: the field has one scale, 58 bits below its largest entry, so
 // a link 2^4 smaller keeps the 53 bits of an FP64 number below its own largest.
 // SU(3) links (largest entries between 0.57 and 1) and unitary ones always do.
-constexpr int kMaxFixedLinkExp = 64, kMaxFixedLinkSpread = 4;
+constexpr int kMinFixedLinkExp = -60, kMaxFixedLinkExp = 64, kMaxFixedLinkSpread = 4;
+// A clover term has one where every site's largest entry lies within 2^+-60 (an
+// ordinary one's is near 1).  With spinors within 2^+-900 the scales of all
+// products then stay inside FP64's normal range, -1016 to 965 and 62 bits more.
+constexpr int kMaxFixedCloverExp = 60;
 
 static size_t elem_bytes(qdd_prec p)
 {
@@ -232,7 +236,7 @@ static qdd_status fx_build(Gauge *g, bool required, bool clover, cudaStream_t s)
 {
     FxCopy &f = g->fx;
     Ctx *c = g->ctx;
-    const size_t n = (size_t)g->hg.V * 36 * 16, ne = (size_t)g->hg.V * sizeof(int);
+    const size_t n = (size_t)g->hg.V * 36 * 16, ne = ((size_t)g->hg.V + 1) * sizeof(int);
     if (!required && !f.required) {
         const size_t more = (f.links.p ? 0 : n) + (clover && !f.clov.p ? n + ne : 0);
         if (c->used.load() + more > c->budget / 2) return QDD_EBUDGET;
@@ -245,9 +249,21 @@ static qdd_status fx_build(Gauge *g, bool required, bool clover, cudaStream_t s)
     QDD_TRY(st);
     if (!f.have_links) QDD_TRY(launch_links_fx(g, s));
     if (clover && !f.have_clov) QDD_TRY(launch_clover_fx(g, s));
+    int far = 0;
+    if (clover && !f.have_clov)
+        QDD_CUDA(cudaMemcpyAsync(&far, f.clov_e.as<int>() + g->hg.V, sizeof(int), cudaMemcpyDeviceToHost, s));
     QDD_CUDA(cudaStreamSynchronize(s));  // other streams may read it from here on
     f.have_links = true;
-    if (clover) f.have_clov = true;
+    if (clover && !f.have_clov) {
+        f.have_clov = true;
+        f.wide = far > kMaxFixedCloverExp;
+        if (f.wide) {  // FP64 arithmetic, until the next clover term: the room is not needed
+            if (!f.required) c->optional -= f.clov.bytes + f.clov_e.bytes;
+            f.clov.release();
+            f.clov_e.release();
+        }
+    }
+    if (f.wide) return QDD_OK;
     if (required && !f.required) {
         f.required = true;
         c->optional -= f.links.bytes + f.clov.bytes + f.clov_e.bytes;
@@ -261,10 +277,15 @@ qdd_status fx_acquire(Gauge *g, bool required, bool clover, cudaStream_t s, FxLo
         set_error("set_clover has not been called");
         return QDD_EINVAL;
     }
-    if (g->link_exp > kMaxFixedLinkExp || g->link_spread > kMaxFixedLinkSpread) return QDD_OK;
+    if (g->link_exp < kMinFixedLinkExp || g->link_exp > kMaxFixedLinkExp || g->link_spread > kMaxFixedLinkSpread)
+        return QDD_OK;
     FxCopy &f = g->fx;
     for (int turn = 0; turn < 3; turn++) {  // an optional copy may be given up between the two locks
         lk = FxLock(f.mu);
+        if (clover && f.have_clov && f.wide) {
+            lk.unlock();
+            return QDD_OK;
+        }
         if (f.have_links && (!clover || f.have_clov) && (!required || f.required)) return QDD_OK;
         lk.unlock();
         std::unique_lock<std::shared_mutex> ul(f.mu);
@@ -673,7 +694,7 @@ qdd_status qdd_set_clover(qdd_gauge *g, double c_sw, double kappa)
     for (auto &c : g->copies) c.valid = false;
     {
         std::unique_lock<std::shared_mutex> ul(g->fx.mu);
-        g->fx.have_clov = false;
+        g->fx.have_clov = g->fx.wide = false;
     }
     g->have_clover = false;
     if (singular) {

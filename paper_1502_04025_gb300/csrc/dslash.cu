@@ -636,6 +636,7 @@ __global__ void k_links_fx(int64_t n, const double2 *src, int4 *dst, int lsh)
     dst[i] = make_int4(re.hi, re.lo, im.hi, im.lo);
 }
 
+// ae[g.V] (zero at the launch) takes the largest exponent in magnitude.
 __global__ void __launch_bounds__(128) k_clover_fx(Geom g, const double2 *src, int4 *dst, int *ae)
 {
     const int gi = blockIdx.x * blockDim.x + threadIdx.x;
@@ -649,6 +650,8 @@ __global__ void __launch_bounds__(128) k_clover_fx(Geom g, const double2 *src, i
         emax = max(emax, max(fx_exponent(a.x), fx_exponent(a.y)));
     }
     ae[gi] = emax - 1022;
+    const int far = abs(emax - 1022);
+    if (far > *(volatile int *)(ae + g.V)) atomicMax(ae + g.V, far);
     int4 *q = dst + (int64_t)d * 36 * g.Vd + s;
     for (int k = 0; k < 36; k++) {
         const double2 a = __ldg(p + (int64_t)k * g.Vd);
@@ -670,6 +673,7 @@ qdd_status launch_links_fx(Gauge *g, cudaStream_t s)
 qdd_status launch_clover_fx(Gauge *g, cudaStream_t s)
 {
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
+    QDD_CUDA(cudaMemsetAsync(g->fx.clov_e.as<int>() + g->hg.V, 0, sizeof(int), s));
     k_clover_fx<<<(g->hg.V + 127) / 128, 128, 0, s>>>(g->geom, g->clov64.as<double2>(), g->fx.clov.as<int4>(),
                                                       g->fx.clov_e.as<int>());
     QDD_CUDA(cudaGetLastError());

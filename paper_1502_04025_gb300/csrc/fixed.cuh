@@ -83,7 +83,8 @@ __device__ __forceinline__ void fx_mac2(fxacc &s0, fxacc &s1, fx a, fx x0, fx x1
 __device__ __forceinline__ fxacc fx_zero() { return {0, 1ll << (kFxLimb - 1)}; }
 __device__ __forceinline__ int64_t fx_value(const fxacc &s) { return s.h + (s.c >> kFxLimb); }
 
-// v 2^ex in FP64 (v's leading 53 bits, rounded; the result is a normal number or zero)
+// v 2^ex in FP64 (v's leading 53 bits, rounded; the result is a normal number or
+// zero: -1022 <= ex <= 960, which the callers' ranges of scales ensure)
 __device__ __forceinline__ double fx_to_double(int64_t v, int ex)
 {
     if (v == 0) return 0.0;

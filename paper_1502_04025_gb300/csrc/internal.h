@@ -184,8 +184,9 @@ struct PrecCopy {
 // launched kernels); building and giving up hold it exclusively.
 struct FxCopy {
     std::shared_mutex mu;
-    DevMem links, clov, clov_e;  // clov_e: one exponent per site
+    DevMem links, clov, clov_e;  // clov_e: one exponent per site, then the largest in magnitude
     bool have_links = false, have_clov = false, required = false;
+    bool wide = false;           // have_clov: the term is out of the range that has a copy
 };
 
 // Device and pinned host buffers of one solve (Krylov basis, preconditioner
@@ -269,8 +270,8 @@ __host__ __device__ __forceinline__ int64_t pair_index(int64_t d, int P, int p, 
 qdd_status ensure_copy(Gauge *g, qdd_prec prec, cudaStream_t s);
 // The fixed-point copy of links and (clover) of the clover term, built where it
 // is missing.  lk holds it on return; where it does not, FP64 arithmetic has to
-// stand in: links that are not finite or very large, or no room for a copy that
-// is not required (which is no error).
+// stand in: links or a clover term out of range, links of different sizes, or no
+// room for a copy that is not required (which is no error).
 using FxLock = std::shared_lock<std::shared_mutex>;
 qdd_status fx_acquire(Gauge *g, bool required, bool clover, cudaStream_t s, FxLock &lk);
 // the two-row link copy of a storage precision (FP32, FP16, BF16)
