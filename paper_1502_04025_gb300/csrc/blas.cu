@@ -130,65 +130,99 @@ __device__ __forceinline__ void last_block_final(const double2 *part, int stride
 // elements of w and of each vector a common scale (their largest exponent),
 // sums the products exactly with integer multiply-adds and adds one FP64 number
 // per tile, vector and component to its running sum; the kDotFma elements next
-// to them run on the FP64 pipe meanwhile.  A tile with a non-finite element or
-// an extreme exponent takes FP64 arithmetic throughout.  Per tile the error
-// is about 2^-57 of its largest |v| |w|, below the rounding of the FP64 sums.
-// Measured, us (event-timed): 5 vectors of 25.2 M elements 914 -> 507 (4768 GB/s; 646 all in
-// fixed point), 3 vectors 540 -> 309 (5218 GB/s), 16 vectors of 6.3 M 706 -> 469,
-// 5 vectors of 1.57 M 81 -> 52.
+// to them run on the FP64 pipe meanwhile.
+//
+// The error of a tile's sum belongs to the scales A of v and B of w, not to its
+// products: 59 bits of each factor, truncated, give 8 products an error below
+// 8 2^-58 A B, the dropped products of the lower limbs (each at most 2^29) 8 2^-60,
+// and the last bit kept 2^-58: together below 2^-54.7 A B.  Eight FP64
+// multiply-adds round the tile's sum by up to 8 2^-53 S, S the sum of the products'
+// magnitudes.  So a tile is taken in fixed point where both components have
+// S >= A B / 16, which six leading bits of every factor show (four integer
+// multiply-adds for both sums of an element), and its error is then below 2^-50.7 S;
+// any other tile (elements of very different sizes, a part that is nearly zero
+// throughout, a non-finite element, an extreme exponent) takes FP64 arithmetic.
+// Of Gaussian tiles 1 in 8000 does.
+// Measured, us (event-timed), FP64 arithmetic against this: 5 vectors of 25.2 M
+// elements 914 -> 513 (4712 GB/s), 3 vectors 540 -> 333 (4838 GB/s), 16 vectors of
+// 6.3 M 706 -> 457, 5 vectors of 1.57 M 81 -> 53.  The magnitudes' check costs 0 to 6 %.
 constexpr int kDotTile = 4, kDotFma = 3;
-constexpr int kDotNV = 8;     // vectors per launch: more would not fit the instruction cache
-constexpr int kDotBits = 58;  // of both factors: 8 products per sum, |cross| <= 8 * 2 * 2^28 2^30 < 2^63
-
-// acc[j] += <v_j, w> over the kDotTile elements k, k + step, ... in fixed point
-// and the kDotFma after them in FP64 (all below n if FULL)
-template <int NV, bool FULL>
-__device__ __forceinline__ void dot_tile(const double2 *__restrict__ v, int64_t ld, const double2 *__restrict__ w,
-                                         int64_t k, int64_t step, int64_t n, double2 *acc)
+constexpr int kDotNV = 6;     // vectors per launch, at most: more spill registers (8: 16
+                              // vectors of 6.3 M 538 us, with 372 bytes of spills, against 457)
+// vectors of the next launch when `left` remain: as even as whole numbers allow
+static int dot_share(int left)
 {
-    constexpr int K = kDotTile, F = kDotFma;
+    const int launches = (left + kDotNV - 1) / kDotNV;
+    return (left + launches - 1) / launches;
+}
+constexpr int kDotBits = 59;  // of both factors: 8 products per sum, |cross| <= 8 * 2 * 2^29 2^29 = 2^62
+constexpr uint32_t kDotLow = 64 * 64 / 16;
+
+__device__ __forceinline__ void fma_dot(double2 &s, double2 a, double2 x)
+{
+    s.x = fma(a.x, x.x, s.x);
+    s.x = fma(a.y, x.y, s.x);
+    s.y = fma(a.x, x.y, s.y);
+    s.y = fma(-a.y, x.x, s.y);
+}
+
+// acc[j] += <v_j, w> over kDotTile elements k, k + step, ... in fixed point and
+// the F after them in FP64
+template <int NV, int F>
+__device__ __forceinline__ void dot_tile(const double2 *__restrict__ v, int64_t ld, const double2 *__restrict__ w,
+                                         int64_t k, int64_t step, double2 *acc)
+{
+    constexpr int K = kDotTile;
     double2 b[K + F];
     fxgroup gw = {0, 0, 0};
 #pragma unroll
-    for (int i = 0; i < K + F; i++) b[i] = FULL || k + i * step < n ? __ldg(w + k + i * step) : make_double2(0, 0);
+    for (int i = 0; i < K + F; i++) b[i] = __ldg(w + k + i * step);
 #pragma unroll
     for (int i = 0; i < K; i++) fx_group_add(gw, b[i]);
-    const bool okw = fx_group_done(gw);
+    const bool okw = fx_group_done(gw), zerow = fx_group_zero(gw);
     cfx fw[K];
+    uint32_t pw[K];  // leading bits of both parts
 #pragma unroll
-    for (int i = 0; i < K; i++) fw[i] = fx_from_group<kDotBits>(b[i], gw);
-    auto fma_dot = [&](double2 &s, double2 a, double2 x) {
-        s.x = fma(a.x, x.x, s.x);
-        s.x = fma(a.y, x.y, s.x);
-        s.y = fma(a.x, x.y, s.y);
-        s.y = fma(-a.y, x.x, s.y);
-    };
+    for (int i = 0; i < K; i++) {
+        uint32_t x, y;
+        fw[i] = {fx_centred<kDotBits>(b[i].x, gw.emax, x), fx_centred<kDotBits>(b[i].y, gw.emax, y)};
+        pw[i] = x | y << 16;
+    }
 #pragma unroll
     for (int j = 0; j < NV; j++) {
         const double2 *vj = v + j * ld + k;
         double2 a[K + F];
         fxgroup gv = {0, 0, 0};
 #pragma unroll
-        for (int i = 0; i < K + F; i++) a[i] = FULL || k + i * step < n ? __ldg(vj + i * step) : make_double2(0, 0);
+        for (int i = 0; i < K + F; i++) a[i] = __ldg(vj + i * step);
 #pragma unroll
         for (int i = 0; i < K; i++) fx_group_add(gv, a[i]);
 #pragma unroll
         for (int i = K; i < K + F; i++) fma_dot(acc[j], a[i], b[i]);
-        if (fx_group_done(gv) && okw) {
+        const bool okv = fx_group_done(gv);
+        cfx fa[K];
+        uint32_t px = 0, py = 0;  // sums of |Re v| (|Re w|, |Im w|) and |Im v| (|Re w|, |Im w|)
+#pragma unroll
+        for (int i = 0; i < K; i++) {
+            uint32_t x, y;
+            fa[i] = {fx_centred<kDotBits>(a[i].x, gv.emax, x), fx_centred<kDotBits>(a[i].y, gv.emax, y)};
+            px += x * pw[i];
+            py += y * pw[i];
+        }
+        const uint32_t low = min((px & 0xffffu) + (py >> 16), (px >> 16) + (py & 0xffffu));
+        if (okv && okw && (low >= kDotLow || zerow || fx_group_zero(gv))) {
             fxacc re = fx_zero(), im = fx_zero();
 #pragma unroll
             for (int i = 0; i < K; i++) {
-                const cfx fa = fx_from_group<kDotBits>(a[i], gv);
-                fx_mac2(re, im, fa.re, fw[i].re, fw[i].im);
-                fx_mac2(re, im, fa.im, fw[i].im, fx{-fw[i].re.hi, -fw[i].re.lo});
+                fx_mac2(re, im, fa[i].re, fw[i].re, fw[i].im);
+                fx_mac2(re, im, fa[i].im, fw[i].im, fx{-fw[i].re.hi, -fw[i].re.lo});
             }
             const int ex = gv.emax + gw.emax - 2 * 1022 + 2 * kFxLimb - 2 * kDotBits;
             acc[j].x += fx_to_double(fx_value(re), ex);
             acc[j].y += fx_to_double(fx_value(im), ex);
         } else {
 #pragma unroll
-            for (int i = 0; i < K; i++)
-                fma_dot(acc[j], a[i], FULL || k + i * step < n ? __ldg(w + k + i * step) : make_double2(0, 0));
+            for (int i = 0; i < K; i++) fma_dot(acc[j], a[i], __ldg(w + k + i * step));
         }
     }
 }
@@ -206,8 +240,12 @@ __global__ void __launch_bounds__(kBT, 2) k_cdot_partial(const double2 *__restri
     const int64_t step = (int64_t)gridDim.x * kBT;
     int64_t k = (int64_t)blockIdx.x * kBT + threadIdx.x;
     constexpr int kT = kDotTile + kDotFma;
-    for (; k + (kT - 1) * step < n; k += kT * step) dot_tile<NV, true>(v, ld, w, k, step, n, acc);
-    if (k < n) dot_tile<NV, false>(v, ld, w, k, step, n, acc);
+    for (; k + (kT - 1) * step < n; k += kT * step) dot_tile<NV, kDotFma>(v, ld, w, k, step, acc);
+    for (; k < n; k += step) {  // fewer than kT elements
+        const double2 b = __ldg(w + k);
+#pragma unroll
+        for (int j = 0; j < NV; j++) fma_dot(acc[j], __ldg(v + j * ld + k), b);
+    }
     block_reduce<NV>(acc, sm);
     if (threadIdx.x < NV) {
         double2 s = make_double2(0, 0);
@@ -495,9 +533,7 @@ static void dot_dispatch(int nv, F &&f)
     case 3: f(std::integral_constant<int, 3>{}); break;
     case 4: f(std::integral_constant<int, 4>{}); break;
     case 5: f(std::integral_constant<int, 5>{}); break;
-    case 6: f(std::integral_constant<int, 6>{}); break;
-    case 7: f(std::integral_constant<int, 7>{}); break;
-    default: f(std::integral_constant<int, 8>{}); break;
+    default: f(std::integral_constant<int, 6>{}); break;
     }
 }
 
@@ -506,8 +542,8 @@ qdd_status blas_cdot_multi(Ctx *ctx, const double2 *v, int nvec, int64_t ld, con
 {
     if (nvec <= 0) return QDD_OK;
     const int nb = blas_blocks(ctx, n);
-    for (int j0 = 0; j0 < nvec; j0 += kDotNV) {
-        int nv = nvec - j0 < kDotNV ? nvec - j0 : kDotNV;
+    for (int j0 = 0, nv; j0 < nvec; j0 += nv) {
+        nv = dot_share(nvec - j0);
         ctx->timer.work(K_BLAS, 8.0 * nv * n, 16.0 * (nv + 1) * n);
         LaunchScope ls(ctx->timer, K_BLAS, s);
         dot_dispatch(nv, [&](auto c) {
@@ -697,8 +733,8 @@ extern "C" qdd_status qdd_cdot_multi_noalloc(const double *v, int nvec, int64_t 
     double2 *O2 = (double2 *)out;
     // every block overwrites its own partials before the final sum reads them,
     // so nothing in the shared array has to start at zero
-    for (int j0 = 0; j0 < nvec; j0 += kDotNV) {
-        int nv = nvec - j0 < kDotNV ? nvec - j0 : kDotNV;
+    for (int j0 = 0, nv; j0 < nvec; j0 += nv) {
+        nv = dot_share(nvec - j0);
         dot_dispatch(nv, [&](auto c) {
             k_cdot_partial<decltype(c)::value><<<nb, kBT, 0, s>>>(V2 + j0 * ld, ld, W2, n, part);
         });

@@ -139,6 +139,8 @@ __device__ __forceinline__ bool fx_group_done(fxgroup &g)
     return g.emax > 623 && g.emax < 1423;
 }
 
+__device__ __forceinline__ bool fx_group_zero(const fxgroup &g) { return (g.top | g.any) == 0u; }
+
 // shifts by 32 and more give 0
 __device__ __forceinline__ uint32_t shr_clamp(uint32_t v, uint32_t n)
 {
@@ -166,6 +168,22 @@ template <int kBits>
 __device__ __forceinline__ cfx fx_from_group(double2 v, const fxgroup &g)
 {
     return {fx_from_grouped<kBits>(v.x, g.emax), fx_from_grouped<kBits>(v.y, g.emax)};
+}
+
+// The same with the limb below centred, |lo| <= 2^29 (and |hi| <= 2^(kBits - 30));
+// lead: the leading six bits below 2^(emax - 1022).
+template <int kBits>
+__device__ __forceinline__ fx fx_centred(double v, int emax, uint32_t &lead)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t t = __funnelshift_l(lo, hi, 11) | 0x80000000u, r = lo << 11;  // mantissa, leading one on top
+    const uint32_t sh = (uint32_t)(emax + (64 - kBits)) - ((hi >> 20) & 0x7ffu); // magnitude = (t:r) >> sh
+    const uint32_t mh = shr_clamp(t, sh - (32 - kFxLimb));
+    const uint32_t ml = (sh < 32 ? __funnelshift_r(r, t, sh) : shr_clamp(t, sh - 32)) & ((1u << kFxLimb) - 1);
+    const uint32_t up = ml >> (kFxLimb - 1);
+    lead = mh >> (kBits - kFxLimb - 6);
+    const int sg = ((int)hi >> 31) | 1;
+    return {(int)(mh + up) * sg, (int)(ml - (up << kFxLimb)) * sg};
 }
 
 // The 12 components v of a site into the fixed-point field f (planes of the
