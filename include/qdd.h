@@ -68,8 +68,7 @@ typedef enum {
     QDD_PREC_F32 = 1,
     QDD_PREC_F16S = 2,
     QDD_PREC_BF16S = 3,
-    QDD_PREC_DF64 = 4, /* operator only: FP64-class accuracy (57 bits below each
-                          site's largest component) from 64-bit fixed-point
+    QDD_PREC_DF64 = 4, /* operator only: FP64's accuracy from 64-bit fixed-point
                           numbers in two 32-bit limbs, on a copy of links and
                           clover in that form.  For qdd_apply_D and arnoldi_prec. */
     QDD_PREC_H16 = 5   /* the paper's half precision (Sec. 3.3): FP16 links and
@@ -333,13 +332,13 @@ qdd_status qdd_layout_faces(const int L[4], const int dom[4], int foff[8], uint3
 
 /*
  * out = D in for nrhs spinors (host layout), periodic boundary conditions.
- * prec = QDD_PREC_F64 and QDD_PREC_DF64 compute in 64-bit fixed point, to
- * FP64's accuracy or better against the largest component of the sites
- * involved; both compute in FP64 arithmetic where the fields have no
- * fixed-point copy (links not finite, outside 2^-60..2^64, or of sizes that differ
- * by more than 2^4 from link to link; a clover term whose largest entry lies
- * outside 2^-60..2^60 at some site), QDD_PREC_F64 also where a copy would fill the HBM
- * budget past a half; QDD_PREC_F32 converts links, clover
+ * prec = QDD_PREC_F64 and QDD_PREC_DF64: FP64's accuracy, component by component.
+ * Both compute in 64-bit fixed point, but in FP64 arithmetic the sites where a
+ * component is small against the scales involved, and every site where the fields
+ * have no fixed-point copy (|kappa| below 0.04; links not finite, outside
+ * 2^-60..2^64, or of sizes that differ by more than 2^4 from link to link; a clover
+ * term whose largest entry lies outside 2^-60..2^60 at some site), QDD_PREC_F64 also
+ * where a copy would fill the HBM budget past a half.  QDD_PREC_F32 converts links, clover
  * and input to FP32 and computes in FP32 (1848 flop per site); F16S / BF16S
  * read 16-bit links/clover/spinor with FP32 arithmetic.
  */

@@ -178,7 +178,7 @@ void DevMem::release()
 // -------------------------------------------------------- precision copies
 
 // Links have a fixed-point copy from 2^-60 to 2^64, and where their sizes differ
-// by no more than 2^4: the field has one scale, 58 bits below its largest entry, so
+// by no more than 2^4: the field has one scale, 60 bits below its largest entry, so
 // a link 2^4 smaller keeps the 53 bits of an FP64 number below its own largest.
 // SU(3) links (largest entries between 0.57 and 1) and unitary ones always do.
 constexpr int kMinFixedLinkExp = -60, kMaxFixedLinkExp = 64, kMaxFixedLinkSpread = 4;
@@ -186,6 +186,10 @@ constexpr int kMinFixedLinkExp = -60, kMaxFixedLinkExp = 64, kMaxFixedLinkSpread
 // ordinary one's is near 1).  With spinors within 2^+-900 the scales of all
 // products then stay inside FP64's normal range, -1016 to 965 and 62 bits more.
 constexpr int kMaxFixedCloverExp = 60;
+// The operator's fixed-point sums are as good as FP64's where the hops, times kappa, are
+// not far below the clover sum (fixed.cuh): with kappa at 0.04 the test leaves one
+// Gaussian site of 500 to FP64, at 0.12 none of 65536.
+constexpr double kMinFixedKappa = 0.04;
 
 static size_t elem_bytes(qdd_prec p)
 {
@@ -277,7 +281,8 @@ qdd_status fx_acquire(Gauge *g, bool required, bool clover, cudaStream_t s, FxLo
         set_error("set_clover has not been called");
         return QDD_EINVAL;
     }
-    if (g->link_exp < kMinFixedLinkExp || g->link_exp > kMaxFixedLinkExp || g->link_spread > kMaxFixedLinkSpread)
+    if (g->link_exp < kMinFixedLinkExp || g->link_exp > kMaxFixedLinkExp || g->link_spread > kMaxFixedLinkSpread ||
+        (clover && !(std::fabs(g->kappa) >= kMinFixedKappa)))
         return QDD_OK;
     FxCopy &f = g->fx;
     for (int turn = 0; turn < 3; turn++) {  // an optional copy may be given up between the two locks
@@ -534,6 +539,7 @@ qdd_status qdd_create_gauge_field(qdd_ctx *ctx, const int L[4], const int dom[4]
     g->su3 = h_bad[0] == 0;
     g->link_exp = h_bad[1] == 0x7ff ? 1 << 20 : std::max(h_bad[1] - 1022, -800);
     g->link_spread = std::max(h_bad[1] - (0x7ff - h_bad[2]), 0);
+    if (g->su3) g->link_exp = g->link_spread = 0;
     g->two_rows = g->su3;
     QDD_CUDA(cudaDeviceSynchronize());
     ctx->timer.resolve();
@@ -771,21 +777,30 @@ qdd_status qdd_apply_D(qdd_gauge *g, const double *in, double *out, int nrhs, qd
     double *dout = nullptr;
     QDD_TRY(stage_in(g, st->io, in, nrhs, on_device, s, &din));
     QDD_TRY(st->a.ensure(g->ctx, V * 12 * eb * nrhs));
-    // a sharded field corrects the output's boundary planes from the input
-    // (FP64, host layout), so the host output must not reuse the input's staging
-    DevMem &oio = g->slab ? st->c : st->io;
     if (g->slab && on_device && out == in) {
         set_error("a sharded field needs separate input and output buffers");
         return QDD_EINVAL;
     }
-    QDD_TRY(stage_out(g, oio, out, nrhs, on_device, s, &dout));
-    if (scaled || arith != QDD_PREC_F32) QDD_TRY(st->a_s.ensure(g->ctx, V * 4 * nrhs));
+    if (arith != QDD_PREC_F32) QDD_TRY(st->a_s.ensure(g->ctx, fx_exponent_bytes(V, nrhs)));
+    else if (scaled) QDD_TRY(st->a_s.ensure(g->ctx, V * 4 * nrhs));
     if (scaled) QDD_TRY(st->b_s.ensure(g->ctx, V * 4 * nrhs));
     // FP64-class arithmetic in fixed point: the input is converted on its way
     // in, the operator writes the host layout
     FxLock fl;
     if (arith != QDD_PREC_F32) QDD_TRY(fx_acquire(g, arith == QDD_PREC_DF64, true, s, fl));
     const bool fixed = fl.owns_lock();
+    // A sharded field corrects the output's boundary planes from the input (FP64,
+    // host layout), and the fixed-point operator goes back to it at single sites, so
+    // the host output must not reuse the input's staging; a device buffer that is
+    // both input and output is copied first.
+    DevMem &oio = g->slab || fixed ? st->c : st->io;
+    QDD_TRY(stage_out(g, oio, out, nrhs, on_device, s, &dout));
+    const size_t bytes = V * 12 * sizeof(double2) * nrhs;
+    if (fixed && (const char *)din < (const char *)dout + bytes && (const char *)dout < (const char *)din + bytes) {
+        QDD_TRY(st->b.ensure(g->ctx, bytes));
+        QDD_CUDA(cudaMemcpyAsync(st->b.p, din, bytes, cudaMemcpyDeviceToDevice, s));
+        din = st->b.as<double>();
+    }
     // FP32 spinors: the operator widens and writes the host layout too
     const bool direct = arith == QDD_PREC_F32 && prec == QDD_PREC_F32;
     if (!fixed && !direct) QDD_TRY(st->b.ensure(g->ctx, V * 12 * eb * nrhs));
@@ -795,7 +810,7 @@ qdd_status qdd_apply_D(qdd_gauge *g, const double *in, double *out, int nrhs, qd
     // a sharded field: its boundary planes (FP64, host layout) move while the operator runs
     QDD_TRY(slab_dslash_begin(g, din, false, true, nrhs, s));
     if (fixed) {
-        QDD_TRY(launch_dslash_fx(g, fxa, (double2 *)dout, true, nullptr, nrhs, s));
+        QDD_TRY(launch_dslash_fx(g, fxa, {din, kFxHost64}, (double2 *)dout, true, nullptr, nrhs, s));
     } else if (direct) {
         if (!g->have_clover) {
             set_error("set_clover has not been called");

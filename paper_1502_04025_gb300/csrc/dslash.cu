@@ -16,6 +16,8 @@
 // only the first two rows of each link and rebuild the third (96 fewer bytes
 // per site in FP32), and their 16-bit link and clover copies are stored with
 // planes paired, one 8-byte load per two planes.
+#include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "fixed.cuh"
@@ -316,19 +318,25 @@ __global__ void __launch_bounds__(128, (dslash_min_blocks<R, SL>())) k_dslash(Ge
 }
 
 // ------------------------------------------------------------------------
-// The FP64 operator (and the double-float precision's) in 64-bit fixed point
-// (fixed.cuh): y = D x, or b - D x, in FP64.  One thread per site; a hop's
+// The operator of the precisions F64 and DF64 in 64-bit fixed point (fixed.cuh):
+// y = D x, or b - D x, in FP64.  One thread per site; a hop's
 // colour products are three integer multiply-adds per real product, summed
 // exactly at the neighbour site's scale, rounded, and shifted to the largest
 // scale of the nine sites before the hops are added; the clover product keeps
-// the site's own scale; both are converted once and combined in FP64.
+// the site's own scale; both are converted once and combined in FP64.  Beside
+// them run sums of the products' magnitudes from the factors' leading bits, two
+// spins in one 32-bit word (81 multiply-adds per site): where one of the twelve is
+// small against the scales, the site goes on a list and k_dslash_list computes it
+// in FP64.
 //
 // Bound: integer multiply-adds 2520 per site (39 clocks of an SM at 64 lanes)
 // and about as many other integer operations, against 69 clocks for the
 // 1536 bytes per site at the measured HBM rate, where FP64 arithmetic takes 570
-// clocks (1140 instructions at 2 lanes).  Measured (32^4 sites, 4^4 domains): 540 us,
-// 152 clocks per site, against 2113 us in FP64 arithmetic; 24x16x12x32: 91 against
-// 312 us.  What is left is latency: 12 to 16 warps per SM at 168 or 128 registers.
+// clocks (1140 instructions at 2 lanes).  Measured, with the launch over an empty
+// list: 32^4 sites in 4^4 domains 556 us, 157 clocks per site, against 2113 us in FP64
+// arithmetic; 24x16x12x32 101 against 312 us.  The sums of magnitudes and that launch
+// are 20 and 12 us of it.
+// What is left is latency: 12 to 16 warps per SM at 168 or 128 registers.
 // The four directions are compiled once each, for both signs (a runtime flag
 // picks the transposed link and the signs): eight bodies would not fit the
 // instruction cache.
@@ -343,64 +351,17 @@ __device__ __forceinline__ cfx ld_cfx(const int4 *p)
 struct FxArgs {
     const int4 *U, *A, *x;    // links and clover in planes of 36, spinors in planes of 12
     const int *ae, *xe;       // exponents: clover per site, spinors per right-hand side and site
-    int lsh;                  // scale of the links
+    int *list;                // list[0] sites left to FP64 (r V + index) from list[1] on
+    int u;                    // exponent of the links
+    int ush;                  // a link entry's leading bits are its upper limb >> ush
+    float hop, clov;          // the test of the sums of magnitudes, in their units
     const double2 *b;         // residual form: b - D x
     double2 *out;             // internal planes, or (site_of) the host layout
     const int *site_of;
     bool a32;                 // host layout: out on a 32-byte boundary
+    FxInput src;              // what x was made from
+    const double2 *U64, *A64; // FP64 links and clover
 };
-
-__device__ __forceinline__ double fx_unscale(fx v, int sh) { return ldexp((double)fx_join(v), -sh); }
-
-// A site that reads one kept in FP64 (non-finite or extreme values): D x of the
-// site in FP64 from the same fields.  Never on the ordinary path.
-__device__ __noinline__ void dslash_fx_raw(const Geom &g, const FxArgs &f, int64_t rbase, int64_t sbase, int d, int s,
-                                           double kappa, double2 *y)
-{
-    cpx<double> acc[12], x[12], u[9];
-    for (int k = 0; k < 12; k++) acc[k] = mk(0.0, 0.0);
-    auto spinor = [&](int dd, int ss) {
-        const int e = f.xe[sbase + (int64_t)dd * g.Vd + ss];
-        for (int k = 0; k < 12; k++) {
-            const int4 w = f.x[rbase + ((int64_t)dd * 12 + k) * g.Vd + ss];
-            x[k] = e == kFxRaw ? mk(__hiloint2double(w.y, w.x), __hiloint2double(w.w, w.z))
-                               : mk(fx_unscale({w.x, w.y}, kFxSpinorBits - e), fx_unscale({w.z, w.w}, kFxSpinorBits - e));
-        }
-    };
-    for (int dir = 0; dir < 8; dir++) {
-        const int mu = dir >> 1, back = dir & 1;
-        const uint16_t e = __ldg(g.nbl + s * 8 + dir);
-        const int nd = (e & kCross) ? __ldg(g.nbd + d * 8 + dir) : d, ns = e & kSlotMask;
-        if (!(QDD_IN_RANGE(nd, 0, g.Nd) && QDD_IN_RANGE(ns, 0, g.Vd))) continue;
-        spinor(nd, ns);
-        for (int k = 0; k < 9; k++) {
-            const int4 w = f.U[((int64_t)(back ? nd : d) * 36 + mu * 9 + k) * g.Vd + (back ? ns : s)];
-            u[k] = mk(fx_unscale({w.x, w.y}, f.lsh), fx_unscale({w.z, w.w}, f.lsh));
-        }
-        switch (dir) {
-        case 0: hop<0, +1>(u, x, acc); break;
-        case 1: hop<0, -1>(u, x, acc); break;
-        case 2: hop<1, +1>(u, x, acc); break;
-        case 3: hop<1, -1>(u, x, acc); break;
-        case 4: hop<2, +1>(u, x, acc); break;
-        case 5: hop<2, -1>(u, x, acc); break;
-        case 6: hop<3, +1>(u, x, acc); break;
-        default: hop<3, -1>(u, x, acc); break;
-        }
-    }
-    spinor(d, s);
-    const int a = f.ae[(int64_t)d * g.Vd + s];
-    cpx<double> m[18], z[6];
-    for (int blk = 0; blk < 2; blk++) {
-        for (int k = 0; k < 18; k++) {
-            const int4 w = f.A[((int64_t)d * 36 + blk * 18 + k) * g.Vd + s];
-            m[k] = mk(fx_unscale({w.x, w.y}, kFxCloverBits - a), fx_unscale({w.z, w.w}, kFxCloverBits - a));
-        }
-        herm6_mul(m, x + 6 * blk, z);
-        for (int k = 0; k < 6; k++)
-            y[6 * blk + k] = make_double2(fma(-kappa, acc[6 * blk + k].re, z[k].re), fma(-kappa, acc[6 * blk + k].im, z[k].im));
-    }
-}
 
 struct cfxsum {
     int64_t re, im;
@@ -423,7 +384,7 @@ __device__ __forceinline__ void fx_lower(int sp, int64_t wr, int64_t wi, cfxsum 
 
 template <int MU>
 __device__ __forceinline__ void fx_hop_dir(const Geom &g, const FxArgs &f, int64_t rbase, int d, int s, int E,
-                                           const int *xe, cfxsum *acc)
+                                           const int *xe, cfxsum *acc, uint32_t *mag)
 {
 #pragma unroll 1
     for (int back = 0; back < 2; back++) {
@@ -455,6 +416,16 @@ __device__ __forceinline__ void fx_hop_dir(const Geom &g, const FxArgs &f, int64
                 h[3 + c] = {add(u1.re, q, l1.re), add(u1.im, q, l1.im)};
             }
         }
+        // Leading bits of the half spinor, 2^5 at the common scale (a component is
+        // below 2^6 of them), the two spins side by side; with a link's, 2^6 for 1 (5 for
+        // links that are not SU(3)), the sums of a row and of eight hops stay below
+        // 2^16: 2^6 sqrt(3) 2^6 8 (2^5 2.45 2^6 8).
+        uint32_t hp[3];
+        const int hsh = min(kFxSpinorBits - kFxLimb - 5 + sft, 31);
+#pragma unroll
+        for (int c = 0; c < 3; c++)
+            hp[c] = (uint32_t)max(abs(h[c].re.hi), abs(h[c].im.hi)) >> hsh |
+                    (uint32_t)max(abs(h[3 + c].re.hi), abs(h[3 + c].im.hi)) >> hsh << 16;
         // the lower spins get -a^+ w forward and +a^+ w backward: their sums
         // change sign before each of the two
 #pragma unroll
@@ -465,10 +436,12 @@ __device__ __forceinline__ void fx_hop_dir(const Geom &g, const FxArgs &f, int64
 #pragma unroll
         for (int a = 0; a < 3; a++) {
             fxacc t[4] = {fx_zero(), fx_zero(), fx_zero(), fx_zero()};  // spin 0 re, im, spin 1 re, im
+            uint32_t sum = 0;
 #pragma unroll
             for (int b = 0; b < 3; b++) {
                 const cfx v = ld_cfx(up + a * sa + b * sb);
                 const fx vp = {v.im.hi * q, v.im.lo * q}, vn = {-vp.hi, -vp.lo};
+                sum += ((uint32_t)max(abs(v.re.hi), abs(v.im.hi)) >> f.ush) * hp[b];
                 fx_mac4(t, v.re, h[b].re, h[b].im, h[3 + b].re, h[3 + b].im);
                 fx_mac2(t[0], t[2], vp, h[b].im, h[3 + b].im);
                 fx_mac2(t[1], t[3], vn, h[b].re, h[3 + b].re);
@@ -482,6 +455,8 @@ __device__ __forceinline__ void fx_hop_dir(const Geom &g, const FxArgs &f, int64
                 const int lo = 6 + 3 * (MU < 2 ? 1 - sp : sp) + a;
                 fx_lower<MU>(sp, wr, wi, acc[lo]);
             }
+            mag[a] += sum;
+            mag[3 + a] += MU < 2 ? sum << 16 | sum >> 16 : sum;
         }
     }
 }
@@ -527,23 +502,30 @@ __global__ void __launch_bounds__(128, VD ? 3 : 4) k_dslash_fx(Geom g0, FxArgs f
             for (int k = 0; k < 6; k++) op[(int64_t)(6 * blk + k) * (HOST ? 1 : g.Vd)] = y[k];
         }
     };
-    if (E >= kFxRaw) {
-        double2 y[12];
-        dslash_fx_raw(g, f, rbase, sbase, d, s, kappa, y);
-        store6(0, y);
-        store6(1, y + 6);
+    bool fp64 = E >= kFxRaw;
+    const int ae = __ldg(f.ae + gi);
+    cfxsum acc[12];
+    if (!fp64) {
+#pragma unroll
+        for (int k = 0; k < 12; k++) acc[k] = {0, 0};
+        uint32_t mag[6] = {0, 0, 0, 0, 0, 0};
+        fx_hop_dir<0>(g, f, rbase, d, s, E, xe, acc, mag);
+        fx_hop_dir<1>(g, f, rbase, d, s, E, xe, acc, mag);
+        fx_hop_dir<2>(g, f, rbase, d, s, E, xe, acc, mag);
+        fx_hop_dir<3>(g, f, rbase, d, s, E, xe, acc, mag);
+        uint32_t low = mag[0];
+#pragma unroll
+        for (int k = 0; k < 6; k++) low = min(low & 0xffffu, min(mag[k] & 0xffffu, mag[k] >> 16));
+        const int n = min(max(e0 + ae - E - f.u, -126), 127);
+        fp64 = E != kFxZero && !((float)low >= fmaf(f.clov, __int_as_float((n + 127) << 23), f.hop));
+    }
+    if (fp64) {
+        f.list[1 + atomicAdd(f.list, 1)] = (int)(r * g.V) + gi;
         return;
     }
-    cfxsum acc[12];
-#pragma unroll
-    for (int k = 0; k < 12; k++) acc[k] = {0, 0};
-    fx_hop_dir<0>(g, f, rbase, d, s, E, xe, acc);
-    fx_hop_dir<1>(g, f, rbase, d, s, E, xe, acc);
-    fx_hop_dir<2>(g, f, rbase, d, s, E, xe, acc);
-    fx_hop_dir<3>(g, f, rbase, d, s, E, xe, acc);
 
-    const int ca = e0 + __ldg(f.ae + gi) + 2 * kFxLimb - kFxSpinorBits - kFxCloverBits;  // scale of the clover sums
-    const int ch = E + 2 * kFxLimb - kFxSpinorBits - f.lsh;  // scale of the hop sums
+    const int ca = e0 + ae + 2 * kFxLimb - kFxSpinorBits - kFxCloverBits;    // scale of the clover sums
+    const int ch = E + f.u + 2 * kFxLimb - kFxSpinorBits - kFxLinkBits;      // scale of the hop sums
     const int4 *xp = f.x + rbase + (int64_t)d * 12 * g.Vd + s;
     const int4 *ap = f.A + (int64_t)d * 36 * g.Vd + s;
     // one chirality block per iteration; the hop sums wait in shared memory, so
@@ -598,6 +580,100 @@ __global__ void __launch_bounds__(128, VD ? 3 : 4) k_dslash_fx(Geom g0, FxArgs f
     }
 }
 
+// The listed sites in FP64, from the FP64 links and clover and the spinors as they
+// were before their conversion.  A warp per site: lane 6 mu + 3 sp + a takes
+// direction mu, both signs, spin sp of the half spinor, colour a of its product
+// (36 FP64 operations); lane k then adds component k of the hop sum, and lanes k
+// and 12 + k take three columns each of its clover row.  With one thread per site
+// the FP64 pipe (a warp's instruction takes 64 clocks of a quarter SM) would make
+// a list of one site 38 us long; about 70 instructions make it 3.  Few sites are
+// listed on ordinary fields, so the launch costs what an empty one does.
+template <bool RESID, bool HOST>
+__global__ void __launch_bounds__(128) k_dslash_list(Geom g, FxArgs f, double kappa)
+{
+    const int lane = threadIdx.x & 31, n = f.list[0];
+    const int mu = min(lane / 6, 3), k6 = lane % 6, sp = k6 / 3, a = k6 % 3;
+    const int ls = mu < 2 ? 1 - sp : sp;  // the lower spin that meets upper spin sp
+    auto spinor = [&](int64_t r, int dd, int ss, int k) -> cpx<double> {
+        if (f.src.kind == kFxPlanes32) {
+            const float2 v = __ldg((const float2 *)f.src.p + (r * g.V + (int64_t)dd * g.Vd) * 12 + (int64_t)k * g.Vd + ss);
+            return mk(f2d(v.x), f2d(v.y));
+        }
+        const double2 *p = (const double2 *)f.src.p;
+        const double2 v = f.src.kind == kFxHost64
+                              ? __ldg(p + (r * g.V + __ldg(f.site_of + dd * g.Vd + ss)) * 12 + k)
+                              : __ldg(p + (r * g.V + (int64_t)dd * g.Vd) * 12 + (int64_t)k * g.Vd + ss);
+        return mk(v.x, v.y);
+    };
+    for (int i = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; i < n; i += gridDim.x * (blockDim.x / 32)) {
+        const int at = f.list[1 + i], gi = at % g.V;
+        const int64_t r = at / g.V;
+        int d, s;
+        split_index(g, gi, d, s);
+        cpx<double> up = mk(0.0, 0.0), lo = mk(0.0, 0.0);
+#pragma unroll 1
+        for (int back = 0; back < 2; back++) {
+            const uint16_t e = __ldg(g.nbl + s * 8 + 2 * mu + back);
+            const int nd = (e & kCross) ? __ldg(g.nbd + d * 8 + 2 * mu + back) : d, ns = e & kSlotMask;
+            if (!(QDD_IN_RANGE(nd, 0, g.Nd) && QDD_IN_RANGE(ns, 0, g.Vd))) continue;
+            const double2 *U = f.U64 + ((int64_t)(back ? nd : d) * 36 + mu * 9) * g.Vd + (back ? ns : s);
+            // h = u + q A l, q = -1 forward and 1 backward; A: x (-i, -i), y (-1, 1), z (-i, i), t (1, 1)
+            const double q = ((mu == 1 && sp == 0) || (mu == 2 && sp == 1)) == (back == 1) ? -1.0 : 1.0;
+            cpx<double> w = mk(0.0, 0.0);
+#pragma unroll
+            for (int b = 0; b < 3; b++) {
+                const cpx<double> u = spinor(r, nd, ns, sp * 3 + b), l = spinor(r, nd, ns, 6 + ls * 3 + b);
+                const cpx<double> h = (mu & 1) == 0 ? mk(fma(q, l.im, u.re), fma(-q, l.re, u.im))
+                                                    : mk(fma(q, l.re, u.re), fma(q, l.im, u.im));
+                const double2 v = __ldg(U + (int64_t)(back ? b * 3 + a : a * 3 + b) * g.Vd);
+                cfma(w, mk(v.x, back ? -v.y : v.y), h);
+            }
+            up = up + w;
+            // q A^+ w: the conjugate phase
+            lo = lo + ((mu & 1) == 0 ? mk(-q * w.im, q * w.re) : mk(q * w.re, q * w.im));
+        }
+        const int k = lane % 12, blk = k / 6, row = k % 6;
+        cpx<double> hop = mk(0.0, 0.0);
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            // lower spin row / 3 comes from upper spin 1 - row / 3 in x and y
+            const int from = m * 6 + (blk && m < 2 ? (row + 3) % 6 : row);
+            const cpx<double> ua = mk(__shfl_sync(0xffffffffu, up.re, from), __shfl_sync(0xffffffffu, up.im, from));
+            const cpx<double> la = mk(__shfl_sync(0xffffffffu, lo.re, from), __shfl_sync(0xffffffffu, lo.im, from));
+            hop = hop + (blk ? la : ua);
+        }
+        cpx<double> y = mk(0.0, 0.0);
+        const double2 *A = f.A64 + ((int64_t)d * 36 + blk * 18) * g.Vd + s;
+        const int col0 = lane >= 12 && lane < 24 ? 3 : 0;
+#pragma unroll
+        for (int c = col0, m = 0; m < 3; m++, c++) {
+            const cpx<double> x = spinor(r, d, s, blk * 6 + c);
+            if (c == row) {
+                const double2 v = __ldg(A + (int64_t)(c >> 1) * g.Vd);
+                const double dg = c & 1 ? v.y : v.x;
+                y.re = fma(dg, x.re, y.re);
+                y.im = fma(dg, x.im, y.im);
+            } else {
+                const int p = min(row, c), t = max(row, c);
+                const double2 v = __ldg(A + (int64_t)(3 + p * 5 - p * (p - 1) / 2 + t - p - 1) * g.Vd);
+                cfma(y, mk(v.x, row < c ? v.y : -v.y), x);
+            }
+        }
+        y.re += __shfl_down_sync(0xffffffffu, y.re, 12);
+        y.im += __shfl_down_sync(0xffffffffu, y.im, 12);
+        if (lane < 12) {
+            double2 o = make_double2(fma(-kappa, hop.re, y.re), fma(-kappa, hop.im, y.im));
+            const int64_t plane = (r * g.V + (int64_t)d * g.Vd) * 12 + (int64_t)k * g.Vd + s;
+            if (RESID) {
+                const double2 v = __ldg(f.b + plane);
+                o = make_double2(v.x - o.x, v.y - o.y);
+            }
+            if (HOST) f.out[(r * g.V + __ldg(f.site_of + gi)) * 12 + k] = o;
+            else f.out[plane] = o;
+        }
+    }
+}
+
 // A spinor field in internal planes (FP64 or FP32) into fixed point.
 template <typename SI>
 __global__ void __launch_bounds__(128) k_spinor_fx(Geom g, const typename SI::T2 *src, int4 *x, int *xe)
@@ -605,6 +681,7 @@ __global__ void __launch_bounds__(128) k_spinor_fx(Geom g, const typename SI::T2
     const int gi = blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= g.V) return;
     const int64_t r = blockIdx.y, rbase = r * (int64_t)g.V * 12;
+    if (gi == 0 && r == 0) xe[(int64_t)g.V * gridDim.y] = 0;  // the operator's list is empty
     int d, s;
     split_index(g, gi, d, s);
     cpx<double> v[12];
@@ -623,7 +700,7 @@ __global__ void k_links_fx(int64_t n, const double2 *src, int4 *dst, int lsh)
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double2 a = __ldg(src + i);
-    // |U| < 2^(61 - lsh) here; rounded at 2^-lsh
+    // |U| <= 2^(60 - lsh) here; rounded at 2^-lsh
     auto conv = [&](double v) {
         const int ex = fx_exponent(v);
         const uint32_t hi = (uint32_t)__double2hiint(v);
@@ -645,10 +722,35 @@ __global__ void __launch_bounds__(128) k_clover_fx(Geom g, const double2 *src, i
     split_index(g, gi, d, s);
     const double2 *p = src + (int64_t)d * 36 * g.Vd + s;
     int emax = 1;
-    for (int k = 0; k < 36; k++) {
-        const double2 a = __ldg(p + (int64_t)k * g.Vd);
-        emax = max(emax, max(fx_exponent(a.x), fx_exponent(a.y)));
+    float big = 0.f;  // |Re| + |Im| summed over the rows of a block
+#pragma unroll 1
+    for (int blk = 0; blk < 2; blk++) {
+        float row[6];
+        auto entry = [&](int k) {
+            const double2 a = __ldg(p + (int64_t)(blk * 18 + k) * g.Vd);
+            emax = max(emax, max(fx_exponent(a.x), fx_exponent(a.y)));
+            return make_float2(fabsf(d2f(a.x)), fabsf(d2f(a.y)));
+        };
+#pragma unroll
+        for (int i = 0; i < 6; i += 2) {
+            const float2 v = entry(i / 2);
+            row[i] = v.x;
+            row[i + 1] = v.y;
+        }
+        int k = 3;
+#pragma unroll
+        for (int i = 0; i < 6; i++)
+#pragma unroll
+            for (int j = i + 1; j < 6; j++) {
+                const float2 v = entry(k++);
+                row[i] += v.x + v.y;
+                row[j] += v.x + v.y;
+            }
+#pragma unroll
+        for (int i = 0; i < 6; i++) big = fmaxf(big, row[i]);
     }
+    // (1 + 1e-6 for the FP32 sums; sites out of FP32's range have no copy)
+    if (big > 0x1p-80f && emax < 0x7ff) emax = max(emax, 1022 + fx_ceil_exponent(big * (1.000001f / kFxCloverRow)));
     ae[gi] = emax - 1022;
     const int far = abs(emax - 1022);
     if (far > *(volatile int *)(ae + g.V)) atomicMax(ae + g.V, far);
@@ -665,7 +767,7 @@ qdd_status launch_links_fx(Gauge *g, cudaStream_t s)
     const int64_t n = (int64_t)g->hg.V * 36;
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
     k_links_fx<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, g->links64.as<double2>(), g->fx.links.as<int4>(),
-                                                           fx_link_shift(g));
+                                                           kFxLinkBits - g->link_exp);
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
 }
@@ -694,26 +796,38 @@ qdd_status launch_spinor_fx(Gauge *g, const void *src, qdd_prec ip, const FxFiel
     return QDD_OK;
 }
 
-qdd_status launch_dslash_fx(Gauge *g, const FxField &x, double2 *out, bool host_layout, const double2 *b, int nrhs,
-                            cudaStream_t s)
+qdd_status launch_dslash_fx(Gauge *g, const FxField &x, const FxInput &src, double2 *out, bool host_layout,
+                            const double2 *b, int nrhs, cudaStream_t s)
 {
     const FxCopy &c = g->fx;
-    FxArgs f{c.links.as<int4>(), c.clov.as<int4>(), (const int4 *)x.x, c.clov_e.as<int>(), x.e, fx_link_shift(g), b,
-             out, host_layout ? g->d_site_of.as<int>() : nullptr, ((uintptr_t)out & 31) == 0};
+    const int ush = kFxLinkBits - kFxLimb - (g->su3 ? 6 : 5);
+    const float unit = (float)(1 << (kFxLinkBits - kFxLimb - ush + 5));  // of the sums of magnitudes, for 2^(E + u)
+    const FxArgs f{c.links.as<int4>(), c.clov.as<int4>(), (const int4 *)x.x, c.clov_e.as<int>(), x.e,
+                   x.e + (int64_t)g->hg.V * nrhs, g->link_exp, ush, unit * kFxHop,
+                   (float)(unit * kFxClover / std::fabs(g->kappa)), b, out, g->d_site_of.as<int>(),
+                   ((uintptr_t)out & 31) == 0, src, g->links64.as<double2>(), g->clov64.as<double2>()};
     const int bt = site_block(g, nrhs);
     const dim3 grid((g->hg.V + bt - 1) / bt, nrhs);
-    LaunchScope ls(g->ctx->timer, K_DSLASH, s);
     const bool v256 = g->hg.Vd == 256;  // 4^4 domains: the volume fixed at compile time
-    if (b) {
-        if (v256) k_dslash_fx<true, false, 256><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
-        else k_dslash_fx<true, false><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
-    } else if (host_layout) {
-        if (v256) k_dslash_fx<false, true, 256><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
-        else k_dslash_fx<false, true><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
-    } else {
-        if (v256) k_dslash_fx<false, false, 256><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
-        else k_dslash_fx<false, false><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
+    {
+        LaunchScope ls(g->ctx->timer, K_DSLASH, s);
+        if (b) {
+            if (v256) k_dslash_fx<true, false, 256><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
+            else k_dslash_fx<true, false><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
+        } else if (host_layout) {
+            if (v256) k_dslash_fx<false, true, 256><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
+            else k_dslash_fx<false, true><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
+        } else {
+            if (v256) k_dslash_fx<false, false, 256><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
+            else k_dslash_fx<false, false><<<grid, bt, 0, s>>>(g->geom, f, g->kappa);
+        }
     }
+    LaunchScope ls(g->ctx->timer, K_DSLASH, s);
+    const int nsm = g->ctx->nsm > 0 ? g->ctx->nsm : 148;
+    const int64_t blocks = std::min<int64_t>(4 * nsm, ((int64_t)g->hg.V * nrhs + 3) / 4);
+    if (b) k_dslash_list<true, false><<<(unsigned)blocks, 128, 0, s>>>(g->geom, f, g->kappa);
+    else if (host_layout) k_dslash_list<false, true><<<(unsigned)blocks, 128, 0, s>>>(g->geom, f, g->kappa);
+    else k_dslash_list<false, false><<<(unsigned)blocks, 128, 0, s>>>(g->geom, f, g->kappa);
     QDD_CUDA(cudaGetLastError());
     return QDD_OK;
 }
@@ -801,7 +915,8 @@ qdd_status launch_dslash(Gauge *g, qdd_prec arith, qdd_prec fp, const void *in, 
             QDD_TRY(fx_acquire(g, arith == QDD_PREC_DF64, true, s, lk));
             if (lk.owns_lock()) {
                 QDD_TRY(launch_spinor_fx(g, in, ip, *fxb, nrhs, s));
-                return launch_dslash_fx(g, *fxb, (double2 *)out, false, b, nrhs, s);
+                return launch_dslash_fx(g, *fxb, {in, ip == QDD_PREC_F64 ? kFxPlanes64 : kFxPlanes32}, (double2 *)out,
+                                        false, b, nrhs, s);
             }
         }
         if (fp != QDD_PREC_F64 || op != QDD_PREC_F64) {

@@ -9,21 +9,37 @@
 //
 // Scales are powers of two:
 //   spinor  x 2^(57 - e), e per site, |x| < 2^e for all 24 reals of the site
-//   links   U 2^lsh, one scale per field: 60 for SU(3) links (|U_ab| <= 1),
-//           58 - u for |U_ab| < 2^u otherwise
-//   clover  A 2^(60 - a), a per site, |A_ij| < 2^a
+//   links   U 2^(60 - u), u per field: |U_ab| < 2^u (u = 0, |U_ab| <= 1, for SU(3)),
+//           and |Re| + |Im| summed over a row or a column at most kFxLinkRow 2^u
+//           (sqrt 6 for a unitary one)
+//   clover  A 2^(60 - a), a per site: |A_ij| < 2^a, and |Re| + |Im| summed over a row
+//           at most kFxCloverRow 2^a
 // A spinor component thus keeps 57 bits below its site's largest one (FP64 keeps
 // 53 below itself).  A half spinor is the sum or difference of two components
 // limb by limb, so its limbs are one bit longer, |lo| <= 2^30, and may be
 // negated.  The sums stay below 2^63: per component of a colour product
 // |sum hi hi| <= 6 2^30 2^28 and |sum cross| <= sqrt(6) 2^30 2^30 + 6 2^29 2^28
-// < 3.3 2^60 for SU(3) rows (less for the other scale); the hop sum of eight
-// directions, each at most sqrt(6) 2^58, is below 19.6 2^58 < 2^62.3; the clover
-// sums of eleven products are below 11 (2^59 + 2^56) < 2^62.7.
+// < 3.3 2^60; the hop sum of eight directions, each at most sqrt(6) 2^58, is below
+// 19.6 2^58 < 2^62.3; the clover sums of eleven products are below
+// 11 (2^59 + 2^56) < 2^62.7.
+//
+// The error of a component y of D x belongs to these scales.  With E the largest
+// exponent of the nine sites and Q = 2^(E + u - 57), a hop's component is off by at
+// most 2 sqrt(6) Q (truncated spinors), 0.75 Q (rounded links), 3 Q (products of lower
+// limbs left out), 0.5 Q (rounding) and Q (shift to E): eight hops by 82 Q =
+// 2^(E + u - 50.65).  The clover sum, with q = 2^(e + a - 57): 1.25 q (spinors), 1.4 q
+// (A), 2.75 q (lower limbs), 0.5 q: 2^(e + a - 54.4).  FP64 arithmetic rounds a hop's
+// six multiply-adds, the projection before and the sum of eight after them, by up
+// to 15 2^-53 S, S the sum of the moduli of the products U h.  So a component is
+// as good as FP64's where
+//   S >= kFxHop 2^(E + u) + kFxClover 2^(e + a) / |kappa|,
+// which the leading bits of links and half spinors show (k_dslash_fx); a site with
+// any component below is computed in FP64.  Of 65536 sites with Gaussian spinors
+// the smallest S is 1.6 times that on links of eps = 0.5 and 0.7.
 //
 // A site with a non-finite component, or with its largest exponent near the
-// ends of FP64's range, keeps its FP64 components as they are (its exponent is
-// marked kFxRaw), and every site that reads one is computed in FP64.
+// ends of FP64's range, is marked kFxRaw in place of its exponent, and every site
+// that reads one is computed in FP64.
 #pragma once
 
 #include "common.cuh"
@@ -40,7 +56,16 @@ struct cfx {
 constexpr int kFxRaw = 1 << 20;     // exponent mark of a site kept in FP64
 constexpr int kFxZero = -900;       // exponent of an all-zero site
 constexpr int kFxLimb = 30;         // bits of the lower limb
-constexpr int kFxSpinorBits = 57, kFxCloverBits = 60;
+constexpr int kFxSpinorBits = 57, kFxCloverBits = 60, kFxLinkBits = 60;
+constexpr float kFxLinkRow = 2.4495f, kFxCloverRow = 1.25f;
+constexpr float kFxHop = 0.35f, kFxClover = 0.025f;
+
+// the smallest e with v <= 2^e (v >= 0; infinity and NaN give 128 and more)
+__device__ __forceinline__ int fx_ceil_exponent(float v)
+{
+    const uint32_t b = __float_as_uint(v);
+    return (int)(b >> 23) - 127 + ((b & 0x007fffffu) ? 1 : 0);
+}
 
 __device__ __forceinline__ fx fx_split(int64_t v)
 {
@@ -187,7 +212,7 @@ __device__ __forceinline__ fx fx_centred(double v, int emax, uint32_t &lead)
 }
 
 // The 12 components v of a site into the fixed-point field f (planes of the
-// domain block at blk) and its exponent.
+// domain block at blk) and its exponent (a raw site's components are not read).
 __device__ __forceinline__ void fx_store_site(int4 *blk, int s, int Vd, int *e_out, const cpx<double> *v)
 {
     int emax = 0;
@@ -203,15 +228,8 @@ __device__ __forceinline__ void fx_store_site(int4 *blk, int s, int Vd, int *e_o
     *e_out = zero ? kFxZero : (raw ? kFxRaw : emax - 1022);
 #pragma unroll
     for (int k = 0; k < 12; k++) {
-        int4 w;
-        if (raw) {
-            w = make_int4(__double2loint(v[k].re), __double2hiint(v[k].re), __double2loint(v[k].im),
-                          __double2hiint(v[k].im));
-        } else {
-            const fx a = fx_from_double(v[k].re, emax, kFxSpinorBits), b = fx_from_double(v[k].im, emax, kFxSpinorBits);
-            w = make_int4(a.hi, a.lo, b.hi, b.lo);
-        }
-        blk[(int64_t)k * Vd + s] = w;
+        const fx a = fx_from_double(v[k].re, emax, kFxSpinorBits), b = fx_from_double(v[k].im, emax, kFxSpinorBits);
+        blk[(int64_t)k * Vd + s] = make_int4(a.hi, a.lo, b.hi, b.lo);
     }
 }
 

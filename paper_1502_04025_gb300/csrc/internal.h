@@ -236,8 +236,8 @@ struct Gauge {
     DevMem d_nbl, d_nbd, d_site_of, d_block_slot, d_fcoord;
     DevMem links64;           // FP64 links, internal layout
     bool su3 = false;         // every link SU(3) to kSu3Tol
-    int link_exp = 1 << 20;   // every link entry below 2^link_exp in magnitude (huge when one is not finite)
-    int link_spread = 0;      // and the largest entry of every link (but zero ones) at least 2^(link_exp - 1 - this)
+    int link_exp = 1 << 20;   // the links' fixed-point exponent u (fixed.cuh; huge when one is not finite)
+    int link_spread = 0;      // the exponents of single links (but zero ones) go down to link_exp - link_spread
     bool two_rows = false;    // the FP32/16-bit full-lattice operator reads two rows per link
     bool have_clover = false;
     int sap_variant = 0;      // Schwarz kernel form (qdd_set_schwarz_variant)
@@ -279,9 +279,6 @@ qdd_status ensure_links12(Gauge *g, qdd_prec prec, cudaStream_t s);
 // links whose unitarity and determinant deviate by more than this keep three rows
 constexpr double kSu3Tol = 1e-10;
 
-// scale of a field's fixed-point links (fixed.cuh)
-inline int fx_link_shift(const Gauge *g) { return g->su3 ? 60 : 58 - g->link_exp; }
-
 // storage of the spinors and of the links/clover copy a precision mode uses
 inline qdd_prec spinor_store(qdd_prec p) { return p == QDD_PREC_H16 ? QDD_PREC_F32 : p; }
 inline qdd_prec field_store(qdd_prec p) { return p == QDD_PREC_H16 ? QDD_PREC_F16S : p; }
@@ -302,10 +299,21 @@ inline int site_block(const Gauge *g, int nrhs)
 }
 
 // A spinor field in fixed point (fixed.cuh): x takes 16 bytes per complex
-// component (as FP64 does), e one exponent per site, of every right-hand side.
+// component (as FP64 does); e one exponent per site, of every right-hand side,
+// then the number and the list of the sites that the operator leaves to FP64
+// arithmetic.
 struct FxField {
     void *x;
     int *e;
+};
+inline size_t fx_exponent_bytes(size_t V, int nrhs) { return (2 * V * nrhs + 1) * sizeof(int); }
+
+// The same field as the caller has it, for those sites: FP64 or FP32 in internal
+// planes, or FP64 in the host layout.
+enum FxSource { kFxPlanes64 = 0, kFxPlanes32 = 1, kFxHost64 = 2 };
+struct FxInput {
+    const void *p;
+    FxSource kind;
 };
 
 // layout.cu
@@ -329,9 +337,9 @@ qdd_status launch_links_convert(Gauge *g, qdd_prec dp, void *dst, cudaStream_t s
 // paired: the full-lattice operator's copy (16-bit formats in paired-plane order)
 qdd_status launch_clover_convert(Gauge *g, const double2 *src, qdd_prec dp, void *dst, float *dst_scale,
                                  cudaStream_t s, bool paired = false);
-// d_out[0] = 1 when some link is not SU(3) to tol; d_out[1] = the largest FP64
-// exponent field of the link entries, d_out[2] = 0x7ff less the smallest of the
-// non-zero links' own largest ones; two-row copy of the links
+// d_out[0] = 1 when some link is not SU(3) to tol; d_out[1] = 1022 + the largest
+// exponent of a link, d_out[2] = 0x7ff less the smallest such value of a non-zero
+// link; two-row copy of the links
 qdd_status launch_su3_check(Gauge *g, double tol, int *d_out, cudaStream_t s);
 qdd_status launch_links12_convert(Gauge *g, qdd_prec dp, void *dst, cudaStream_t s);
 
@@ -353,13 +361,14 @@ qdd_status launch_dslash_host(Gauge *g, qdd_prec fields_prec, const void *in, do
 qdd_status launch_dslash_residual32(Gauge *g, const void *in, const double2 *b, float2 *out, cudaStream_t s);
 // the parts of the fixed-point operator: the copies of links and clover, a
 // spinor field in internal FP64 or FP32 planes, the operator (out in internal
-// planes or in the host layout; b: residual form, internal planes only); the
-// caller of the operator holds the copy (fx_acquire)
+// planes or in the host layout; b: residual form, internal planes only; src: what x
+// was made from, which must not overlap out); the caller of the operator holds
+// the copy (fx_acquire)
 qdd_status launch_links_fx(Gauge *g, cudaStream_t s);
 qdd_status launch_clover_fx(Gauge *g, cudaStream_t s);
 qdd_status launch_spinor_fx(Gauge *g, const void *src, qdd_prec ip, const FxField &x, int nrhs, cudaStream_t s);
-qdd_status launch_dslash_fx(Gauge *g, const FxField &x, double2 *out, bool host_layout, const double2 *b, int nrhs,
-                            cudaStream_t s);
+qdd_status launch_dslash_fx(Gauge *g, const FxField &x, const FxInput &src, double2 *out, bool host_layout,
+                            const double2 *b, int nrhs, cudaStream_t s);
 
 // sap.cu: one half-sweep over the domains of `colour`
 struct SapBuffers {

@@ -354,6 +354,7 @@ __global__ void __launch_bounds__(kSiteThreads) k_spinor_in_fx(Geom g, const int
     int gi = blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= g.V) return;
     const int64_t r = blockIdx.y;
+    if (gi == 0 && r == 0) xe[(int64_t)g.V * gridDim.y] = 0;  // the operator's list is empty
     int d, s;
     split_index(g, gi, d, s);
     cpx<double> v[12];
@@ -444,9 +445,9 @@ __global__ void k_links_convert(int64_t n, int Vd, const double2 *src, typename 
 }
 
 // Sets out[0] when a link is not SU(3) to tol: max |(U U^+ - 1)_ij| or
-// |det U - 1|; out[1] = the largest FP64 exponent field of the link entries;
-// out[2] = 0x7ff less the smallest of the links' own largest exponent fields
-// (links of zeros left out).
+// |det U - 1|; out[1] = 1022 + the largest of the links' exponents u (fixed.cuh; 0x7ff
+// and more with a non-finite entry); out[2] = 0x7ff less the smallest such value of a
+// link that is not zero.
 // One thread per link (domain d, direction mu, site s).
 __global__ void k_su3_check(Geom g, const double2 *U, double tol, int *out)
 {
@@ -498,10 +499,18 @@ __global__ void k_su3_check(Geom g, const double2 *U, double tol, int *out)
     if (!(dev <= tol)) atomicOr(out, 1);
     int ex = 0;
     bool zero = true;
+    float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
+#pragma unroll
     for (int k = 0; k < 9; k++) {
         ex = max(ex, max(fx_exponent(u[k].re), fx_exponent(u[k].im)));
         zero = zero && u[k].re == 0 && u[k].im == 0;
+        const float m = fabsf(d2f(u[k].re)) + fabsf(d2f(u[k].im));
+        row[k / 3] += m;
+        col[k % 3] += m;
     }
+    const float l1 = fmaxf(fmaxf(fmaxf(row[0], row[1]), fmaxf(row[2], col[0])), fmaxf(col[1], col[2]));
+    // (within 2^60 only: other fields keep FP64 arithmetic; 1 + 1e-6 for the FP32 sums)
+    if (l1 > 0x1p-80f && ex < 0x7ff) ex = max(ex, 1022 + fx_ceil_exponent(l1 * (1.000001f / kFxLinkRow)));
     if (ex > *(volatile int *)(out + 1)) atomicMax(out + 1, ex);
     if (!zero && 0x7ff - ex > *(volatile int *)(out + 2)) atomicMax(out + 2, 0x7ff - ex);
 }

@@ -66,7 +66,7 @@ size_t workspace_bytes(const Gauge *g, int m, int B, qdd_prec sp, bool use_sap, 
         b += n * ebytes(spinor_store(sp)) * B + sap_face_bytes(g->hg, sp, B);
         if (sp == QDD_PREC_F16S || sp == QDD_PREC_BF16S) b += V * 4 * B;
     }
-    else b += V * 4 * B;  // the operator's exponents (ensure_ws)
+    else b += fx_exponent_bytes(V, B);  // of the operator's input (ensure_ws)
     if (kdr > 0) b += n * 16 * B * (size_t)(3 * kdr + 1);
     return b + (1 << 20);
 }
@@ -113,7 +113,7 @@ static qdd_status ensure_ws(Gauge *g, Workspace &w, int m, int B, qdd_prec sp, b
     // exponents of the operator's fixed-point input, whose components take the
     // host-transfer buffer between the input and the output: the Schwarz
     // method's residual, consumed by then, where there is one
-    if (!use_sap) QDD_TRY(w.rho.ensure(c, V * sizeof(int) * B));
+    if (!use_sap) QDD_TRY(w.rho.ensure(c, fx_exponent_bytes(V, B)));
     QDD_TRY(blas_scratch_ensure(c, w.scratch));
     QDD_TRY(w.err.ensure(c, sizeof(int)));
     if (w.host_elems < sm.total()) {
