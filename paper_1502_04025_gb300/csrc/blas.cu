@@ -19,7 +19,18 @@
 namespace qdd {
 
 constexpr int kBT = 256;       // threads per block
-constexpr int kNV = 16;        // basis vectors per pass
+constexpr int kNV = 16;        // vectors per pass of k_combine and places of a block's partials
+// Vectors per launch of the multi-dot and the updates, at most: more spill
+// registers (dots at 8: 372 bytes, 16 vectors of 6.3 M elements 538 us against 457;
+// updates at 8 and 16: 200 and 1200).
+constexpr int kPassNV = 6;
+// vectors of the next launch when `left` remain: as even as whole numbers allow
+static int pass_share(int left)
+{
+    if (left <= 0) return 0;
+    const int launches = (left + kPassNV - 1) / kPassNV;
+    return (left + launches - 1) / launches;
+}
 
 int blas_blocks(const Ctx *ctx, int64_t n)
 {
@@ -147,14 +158,6 @@ __device__ __forceinline__ void last_block_final(const double2 *part, int stride
 // elements 914 -> 513 (4712 GB/s), 3 vectors 540 -> 333 (4838 GB/s), 16 vectors of
 // 6.3 M 706 -> 457, 5 vectors of 1.57 M 81 -> 53.  The magnitudes' check costs 0 to 6 %.
 constexpr int kDotTile = 4, kDotFma = 3;
-constexpr int kDotNV = 6;     // vectors per launch, at most: more spill registers (8: 16
-                              // vectors of 6.3 M 538 us, with 372 bytes of spills, against 457)
-// vectors of the next launch when `left` remain: as even as whole numbers allow
-static int dot_share(int left)
-{
-    const int launches = (left + kDotNV - 1) / kDotNV;
-    return (left + launches - 1) / launches;
-}
 constexpr int kDotBits = 59;  // of both factors: 8 products per sum, |cross| <= 8 * 2 * 2^29 2^29 = 2^62
 constexpr uint32_t kDotLow = 64 * 64 / 16;
 
@@ -279,45 +282,77 @@ __global__ void __launch_bounds__(kBT) k_reduce_final(const double2 *part, int n
 // per-block partial of |w|^2.  As the multi-dot, most elements run in 64-bit
 // fixed point next to the FP64 pipe (4 multiply-adds per element and vector, 2
 // lanes per clock and SM): of every kAxpyFx + kAxpyFma elements of a thread the
-// first run in integers.  Every element of every vector has its own scale (its
-// larger component's exponent), every coefficient too; the terms are shifted to
-// the largest scale of the element's terms and added exactly, with 56 bits below
-// that scale, and the result is rounded once.  Elements with a non-finite term or
-// an extreme exponent take FP64 arithmetic.  Measured, 25.2 M elements: 5 vectors with
-// the norm 906 -> 637 us, 3 vectors 682 -> 453, 5 FP32 vectors (16 bytes of x and
-// 8 per vector) 1354 -> 1019; the shares 2:1 to 4:1 and 4:2 are within 2 %.
-constexpr int kAxpyFx = 2, kAxpyFma = 1;
-constexpr int kAxpyBits = 58;  // of coefficients and vectors: two products per sum
-constexpr int kFxLow = 624;    // exponent field of an all-zero group: below every term that counts
+// first run in integers.  Every real product is formed from the two 53-bit
+// mantissas (64 bits of it, below 2^-61 off) with its own exponent, shifted to the
+// largest exponent of the products and the old value that make up its sum, real and
+// imaginary parts apart, and added there; the sum keeps at least 55 bits below the
+// largest of its terms' scales (2 NV + 1 terms, 62 bits less their carry) and is
+// rounded once.  So the error is a fraction of the largest term, as FP64's is,
+// whatever the other part or the other elements are.  Elements with a non-finite
+// term or a sum near the ends of the range take FP64 arithmetic.  Measured, us, 25.2 M
+// elements, FP64 arithmetic against this: 5 vectors with the norm 906 -> 596, 3
+// vectors 682 -> 456, 5 FP32 vectors (16 bytes of x and 8 per vector) 1354 -> 1029.
+// All vector kernels of the 32^3x64 BF16 solve at shares 1:1, 3:2, 2:1, 3:1 and all in
+// integers: 6.26, 6.36, 6.46, 6.58, 7.00 ms.
+constexpr int kAxpyFx = 1, kAxpyFma = 1;
 
-struct FxCoef {
-    cfx c;
-    int e;   // |c| < 2^e
-    int ok;
+// |x| = (t:r) 2^(e - 1086), t with its leading bit set (t = r = 0, e = kFxNone for
+// zeros and subnormal numbers); s the sign in its leading bit
+constexpr int kFxNone = -8192;
+struct FxReal {
+    uint32_t t, r;
+    int e;
+    uint32_t s;
 };
+__device__ __forceinline__ FxReal fx_real(double v)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const int e = (int)((hi >> 20) & 0x7ffu);
+    FxReal x;
+    x.t = e ? __funnelshift_l(lo, hi, 11) | 0x80000000u : 0u;
+    x.r = e ? lo << 11 : 0u;
+    x.e = e ? e : kFxNone;
+    x.s = hi;
+    return x;
+}
 
 __device__ __forceinline__ double2 as_d2(double2 v) { return v; }
 __device__ __forceinline__ double2 as_d2(float2 v) { return make_double2(f2d(v.x), f2d(v.y)); }
 
-// fixed-point group of one complex number; false when it has no usable form
-__device__ __forceinline__ bool fx_single(double2 v, fxgroup &g)
+// a coefficient's parts; those of the fixed-point path are below 2^300, so that
+// nothing is lost with subnormal numbers (below 2^-722 in sums above 2^-646)
+struct FxCoef {
+    FxReal x, y;
+};
+__device__ __forceinline__ bool fx_coef_ok(double v)
 {
-    g = {0, 0, 0};
-    fx_group_add(g, v);
-    g.emax = (g.top | g.any) ? (int)(g.top >> 20) : kFxLow;
-    return g.emax > 623 && g.emax < 1423;
+    const int e = fx_exponent(v);
+    return e < 1323 && (e > 0 || v == 0);
 }
 
-// one number with exponent field at most emax as a plain integer with `kBits`
-// bits below 2^(emax - 1022)
-template <int kBits>
-__device__ __forceinline__ int64_t fx_plain(double v, int emax)
+// bits above a sum of n terms below 2^64 so that it stays below 2^63
+template <int N>
+__host__ __device__ constexpr int fx_carry()
 {
-    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
-    const uint32_t t = __funnelshift_l(lo, hi, 11) | 0x80000000u, r = lo << 11;
-    const uint32_t sh = (uint32_t)(emax + (64 - kBits)) - ((hi >> 20) & 0x7ffu);
-    const uint64_t m = sh > 63 ? 0 : (((uint64_t)t << 32) | r) >> sh;
-    return (int)hi < 0 ? -(int64_t)m : (int64_t)m;
+    int g = 1;
+    while ((1 << (g - 1)) < N) g++;
+    return g;
+}
+
+// acc += +-(the 64-bit magnitude m >> sh), the sign in the leading bit of s; one
+// unit short for a negative term (the sums start with that made up for, and with the
+// half unit that truncation takes on average)
+__device__ __forceinline__ void fx_add(int64_t &acc, uint64_t m, int sh, uint32_t s)
+{
+    const int64_t x = (int64_t)(m >> min(sh, 63)), sg = (int64_t)((int32_t)s >> 31);
+    acc += x ^ sg;
+}
+// acc += +-|a||c|, at 2^(top - 2108 + G) per unit
+template <int G>
+__device__ __forceinline__ void fx_add_product(int64_t &acc, const FxReal &a, const FxReal &c, int top, uint32_t flip)
+{
+    const uint64_t m = (uint64_t)a.t * c.t + __umulhi(a.t, c.r) + __umulhi(a.r, c.t);
+    fx_add(acc, m, top - (a.e + c.e) + G, a.s ^ c.s ^ flip);
 }
 
 template <int NV, int SIGN, typename T2>
@@ -336,32 +371,36 @@ __device__ __forceinline__ double2 axpy_fma(const T2 *__restrict__ v, int64_t ld
 
 template <int NV, int SIGN, typename T2>
 __device__ __forceinline__ double2 axpy_fx(const T2 *__restrict__ v, int64_t ld, const double2 *c, const FxCoef *fc,
-                                           double2 b)
+                                           bool coefs, double2 b)
 {
+    constexpr int G = fx_carry<2 * NV + 1>();
     double2 a[NV];
-    fxgroup ga[NV], gb;
-    bool ok = fx_single(b, gb);
-    int E = gb.emax - 1022;
+    const FxReal bx = fx_real(b.x), by = fx_real(b.y);
+    // exponents of the products, e_a + e_c; the old value's as a product with 1
+    int tx = bx.e + 1023, ty = by.e + 1023, any = max(bx.e, by.e);
 #pragma unroll
     for (int j = 0; j < NV; j++) {
         a[j] = as_d2(__ldg(v + j * ld));
-        ok = fx_single(a[j], ga[j]) && fc[j].ok && ok;
-        E = max(E, ga[j].emax - 1022 + fc[j].e);
+        const int ex = fx_real(a[j].x).e, ey = fx_real(a[j].y).e, cx = fc[j].x.e, cy = fc[j].y.e;
+        any = max(any, max(ex, ey));
+        tx = max(tx, max(ex + cx, ey + cy));
+        ty = max(ty, max(ey + cx, ex + cy));
     }
-    if (!ok) return axpy_fma<NV, SIGN>(v, ld, c, b);
-    int64_t sx = fx_plain<56>(b.x, E + 1022), sy = fx_plain<56>(b.y, E + 1022);
+    // sums between 2^-646 and 2^1000, no term infinite or NaN
+    if (!(coefs && any < 0x7ff && min(tx, ty) >= 1400 && max(tx, ty) <= 3040)) return axpy_fma<NV, SIGN>(v, ld, c, b);
+    int64_t sx = NV, sy = NV;
+    fx_add(sx, ((uint64_t)bx.t << 32) | bx.r, tx - (bx.e + 1023) + G + 1, bx.s);
+    fx_add(sy, ((uint64_t)by.t << 32) | by.r, ty - (by.e + 1023) + G + 1, by.s);
+    constexpr uint32_t kNeg = SIGN < 0 ? 0x80000000u : 0u;
 #pragma unroll
     for (int j = 0; j < NV; j++) {
-        const cfx x = fx_from_group<kAxpyBits>(a[j], ga[j]), cj = fc[j].c;
-        fxacc re = fx_zero(), im = fx_zero();
-        fx_mac2(re, im, cj.re, x.re, x.im);
-        fx_mac2(im, re, cj.im, x.re, fx{-x.im.hi, -x.im.lo});
-        const int sh = min(E - (ga[j].emax - 1022 + fc[j].e), 63);
-        const int64_t tx = fx_value(re) >> sh, ty = fx_value(im) >> sh;
-        if (SIGN > 0) { sx += tx; sy += ty; }
-        else { sx -= tx; sy -= ty; }
+        const FxReal x = fx_real(a[j].x), y = fx_real(a[j].y), cx = fc[j].x, cy = fc[j].y;
+        fx_add_product<G>(sx, x, cx, tx, kNeg);
+        fx_add_product<G>(sx, y, cy, tx, kNeg ^ 0x80000000u);
+        fx_add_product<G>(sy, y, cx, ty, kNeg);
+        fx_add_product<G>(sy, x, cy, ty, kNeg);
     }
-    return make_double2(fx_to_double(sx, E - 56), fx_to_double(sy, E - 56));
+    return make_double2(fx_to_double(sx, tx - 2108 + G), fx_to_double(sy, ty - 2108 + G));
 }
 
 template <int NV, int SIGN, typename T2>
@@ -372,17 +411,14 @@ __global__ void __launch_bounds__(kBT, 2) k_axpy(const T2 *__restrict__ v, int64
     __shared__ double2 sm[kBT / 32];
     __shared__ double2 c[NV];
     __shared__ FxCoef fc[NV];
+    int mine = 1;
     if (threadIdx.x < NV) {
         const double2 x = coef[threadIdx.x];
-        fxgroup g;
-        FxCoef f;
-        f.ok = fx_single(x, g);
-        f.c = fx_from_group<kAxpyBits>(x, g);
-        f.e = g.emax - 1022;
         c[threadIdx.x] = x;
-        fc[threadIdx.x] = f;
+        fc[threadIdx.x] = {fx_real(x.x), fx_real(x.y)};
+        mine = fx_coef_ok(x.x) && fx_coef_ok(x.y);
     }
-    __syncthreads();
+    const bool coefs = __syncthreads_and(mine);
     double nrm = 0;
     const int64_t step = (int64_t)gridDim.x * kBT;
     auto put = [&](int64_t k, double2 b) {
@@ -400,15 +436,13 @@ __global__ void __launch_bounds__(kBT, 2) k_axpy(const T2 *__restrict__ v, int64
             const int64_t q = k + (kAxpyFx + i) * step;
             put(q, axpy_fma<NV, SIGN>(v + q, ld, c, w[q]));
         }
-        // (unrolled only for few vectors: more would not fit the instruction cache)
-        constexpr int kUnroll = NV <= 3 ? kAxpyFx : 1;
-#pragma unroll kUnroll
+#pragma unroll
         for (int i = 0; i < kAxpyFx; i++) {
             const int64_t q = k + i * step;
-            put(q, axpy_fx<NV, SIGN>(v + q, ld, c, fc, w[q]));
+            put(q, axpy_fx<NV, SIGN>(v + q, ld, c, fc, coefs, w[q]));
         }
     }
-    for (; k < n; k += step) put(k, axpy_fx<NV, SIGN>(v + k, ld, c, fc, w[k]));
+    for (; k < n; k += step) put(k, axpy_fx<NV, SIGN>(v + k, ld, c, fc, coefs, w[k]));
     if (part) {
         double2 acc[1] = {make_double2(nrm, 0)};
         block_reduce<1>(acc, sm);
@@ -523,9 +557,9 @@ static void nv_dispatch(int nv, F &&f)
     }
 }
 
-// the same for the multi-dot, nv = 1..kDotNV
+// the same for the multi-dot and the updates, nv = 1..kPassNV
 template <typename F>
-static void dot_dispatch(int nv, F &&f)
+static void pass_dispatch(int nv, F &&f)
 {
     switch (nv) {
     case 1: f(std::integral_constant<int, 1>{}); break;
@@ -543,10 +577,10 @@ qdd_status blas_cdot_multi(Ctx *ctx, const double2 *v, int nvec, int64_t ld, con
     if (nvec <= 0) return QDD_OK;
     const int nb = blas_blocks(ctx, n);
     for (int j0 = 0, nv; j0 < nvec; j0 += nv) {
-        nv = dot_share(nvec - j0);
+        nv = pass_share(nvec - j0);
         ctx->timer.work(K_BLAS, 8.0 * nv * n, 16.0 * (nv + 1) * n);
         LaunchScope ls(ctx->timer, K_BLAS, s);
-        dot_dispatch(nv, [&](auto c) {
+        pass_dispatch(nv, [&](auto c) {
             k_cdot_partial<decltype(c)::value><<<nb, kBT, 0, s>>>(v + j0 * ld, ld, w, n, scratch,
                                                                   scratch_counter(ctx, scratch), out + j0);
         });
@@ -561,7 +595,7 @@ qdd_status blas_caxpy_multi_norm(Ctx *ctx, const double2 *v, int nvec, int64_t l
     const int nb = blas_blocks(ctx, n);
     int j0 = 0;
     do {
-        int nv = nvec - j0 < kNV ? nvec - j0 : kNV;
+        const int nv = pass_share(nvec - j0);
         bool last = j0 + nv >= nvec;
         // v read, w read and (when updated) written; |w|^2 on the last pass
         ctx->timer.work(K_BLAS, 8.0 * nv * n + ((last && norm2_out) ? 4.0 * n : 0.0),
@@ -573,7 +607,7 @@ qdd_status blas_caxpy_multi_norm(Ctx *ctx, const double2 *v, int nvec, int64_t l
             if (nv == 0)
                 k_norm2<<<nb, kBT, 0, s>>>(w, n, scratch, cnt, norm2_out);
             else
-                nv_dispatch(nv, [&](auto c) {
+                pass_dispatch(nv, [&](auto c) {
                     k_axpy<decltype(c)::value, -1, double2><<<nb, kBT, 0, s>>>(v + j0 * ld, ld, coef + j0, w, n, part,
                                                                                cnt, norm2_out);
                 });
@@ -630,11 +664,11 @@ qdd_status blas_axpy_multi(Ctx *ctx, const void *z, bool z_f32, int nvec, int64_
                            double2 *x, int64_t n, cudaStream_t s)
 {
     if (nvec <= 0) return QDD_OK;
-    for (int j0 = 0; j0 < nvec; j0 += kNV) {
-        const int nv = nvec - j0 < kNV ? nvec - j0 : kNV;
+    for (int j0 = 0, nv; j0 < nvec; j0 += nv) {
+        nv = pass_share(nvec - j0);
         ctx->timer.work(K_BLAS, 8.0 * nv * n, ((z_f32 ? 8.0 : 16.0) * nv + 32.0) * n);
         LaunchScope ls(ctx->timer, K_BLAS, s);
-        nv_dispatch(nv, [&](auto c) {
+        pass_dispatch(nv, [&](auto c) {
             if (z_f32)
                 k_axpy<decltype(c)::value, 1, float2><<<blas_blocks(ctx, n), kBT, 0, s>>>(
                     (const float2 *)z + j0 * ld, ld, coef + j0, x, n, nullptr, nullptr, nullptr);
@@ -734,8 +768,8 @@ extern "C" qdd_status qdd_cdot_multi_noalloc(const double *v, int nvec, int64_t 
     // every block overwrites its own partials before the final sum reads them,
     // so nothing in the shared array has to start at zero
     for (int j0 = 0, nv; j0 < nvec; j0 += nv) {
-        nv = dot_share(nvec - j0);
-        dot_dispatch(nv, [&](auto c) {
+        nv = pass_share(nvec - j0);
+        pass_dispatch(nv, [&](auto c) {
             k_cdot_partial<decltype(c)::value><<<nb, kBT, 0, s>>>(V2 + j0 * ld, ld, W2, n, part);
         });
         k_reduce_final<<<nv, kBT, 0, s>>>(part, nb, kNV, O2 + j0, 0);

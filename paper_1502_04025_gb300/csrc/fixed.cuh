@@ -174,29 +174,10 @@ __device__ __forceinline__ uint32_t shr_clamp(uint32_t v, uint32_t n)
     return r;
 }
 
-// A number of a group (exponent field at most emax, emax > 100) with `kBits`
-// bits below 2^(emax - 1022), 32 < kBits <= 62, rounded towards zero: limbs of
-// its magnitude, 0 <= lo < 2^30, both with its sign.  (Subnormal numbers and
-// zeros are shifted out.)
-template <int kBits>
-__device__ __forceinline__ fx fx_from_grouped(double v, int emax)
-{
-    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
-    const uint32_t t = __funnelshift_l(lo, hi, 11) | 0x80000000u, r = lo << 11;  // mantissa, leading one on top
-    const uint32_t sh = (uint32_t)(emax + (64 - kBits)) - ((hi >> 20) & 0x7ffu);  // magnitude = (t:r) >> sh
-    const uint32_t mh = shr_clamp(t, sh - (32 - kFxLimb));
-    const uint32_t ml = (sh < 32 ? __funnelshift_r(r, t, sh) : shr_clamp(t, sh - 32)) & ((1u << kFxLimb) - 1);
-    const int sg = ((int)hi >> 31) | 1;
-    return {(int)mh * sg, (int)ml * sg};
-}
-template <int kBits>
-__device__ __forceinline__ cfx fx_from_group(double2 v, const fxgroup &g)
-{
-    return {fx_from_grouped<kBits>(v.x, g.emax), fx_from_grouped<kBits>(v.y, g.emax)};
-}
-
-// The same with the limb below centred, |lo| <= 2^29 (and |hi| <= 2^(kBits - 30));
-// lead: the leading six bits below 2^(emax - 1022).
+// A number of a group (exponent field at most emax, emax > 600) with `kBits`
+// bits below 2^(emax - 1022), 36 < kBits <= 60, rounded towards zero, the limb below
+// centred, |lo| <= 2^29 (and |hi| <= 2^(kBits - 30)); lead: its leading six bits.
+// (Subnormal numbers and zeros are shifted out.)
 template <int kBits>
 __device__ __forceinline__ fx fx_centred(double v, int emax, uint32_t &lead)
 {
