@@ -338,17 +338,30 @@ __device__ __forceinline__ void field_strength_fx(const Geom &g, const int4 *U, 
 
 // Minus the inverse of a Hermitian 6x6 matrix by six symmetric sweeps without
 // pivoting, in place: dg the diagonal, u the upper triangle row by row (i < j).
-// False when a pivot is small against the matrix (the caller pivots instead).
+// False (the caller pivots instead) unless every pivot is as large as either part of
+// the entries below it when its turn comes, so that a sweep at most doubles the
+// rest as partial pivoting does, and no smaller than the largest entry of the
+// matrix by 2^6 or more (and not NaN or infinite).  Ordinary terms pass: all blocks at
+// kappa c_sw up to 0.4 on links of eps = 0.7, 96 % at 0.6, 22 % at 1, with the
+// errors of partial pivoting.  The comparisons are of the numbers' high words: in
+// FP64 they would take the FP64 pipe.
 __device__ __forceinline__ bool sweep6(double *dg, zd *u)
 {
-    double big = 0;
+    auto word = [](double v) { return (uint32_t)__double2hiint(v) & 0x7fffffffu; };
+    uint32_t big = 0;
 #pragma unroll
-    for (int i = 0; i < 6; i++) big = fmax(big, fabs(dg[i]));
+    for (int i = 0; i < 6; i++) big = max(big, word(dg[i]));
+#pragma unroll
+    for (int i = 0; i < 15; i++) big = max(big, max(word(u[i].re), word(u[i].im)));
     bool ok = true;
 #pragma unroll
     for (int k = 0; k < 6; k++) {
         auto at = [](int i, int j) { return i * 5 - i * (i - 1) / 2 + (j - i - 1); };  // i < j
-        ok = ok && fabs(dg[k]) > 0.02 * big;
+        uint32_t below = 0;
+#pragma unroll
+        for (int i = k + 1; i < 6; i++) below = max(below, max(word(u[at(k, i)].re), word(u[at(k, i)].im)));
+        const uint32_t piv = word(dg[k]);
+        ok = ok && piv >= below && piv + (6u << 20) >= big && piv < 0x7ff00000u;
         const double p = 1.0 / dg[k];
         zd col[6], row[6];  // a_ik, and a_ik / d
 #pragma unroll
