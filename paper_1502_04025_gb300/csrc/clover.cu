@@ -144,11 +144,10 @@ __device__ __forceinline__ void pack_herm6(const zd *M, double2 *dst, int64_t st
         }
 }
 
-__global__ void k_clover_build(Geom g, const double2 *U, double csw, double kappa, double2 *A, double2 *S,
-                               int *singular)
+// the term of site gi in FP64
+__device__ __noinline__ void clover_site(const Geom &g, const double2 *U, int gi, double kc, double2 *A, double2 *S,
+                                         int *singular)
 {
-    int gi = blockIdx.x * blockDim.x + threadIdx.x;
-    if (gi >= g.V) return;
     int d, s;
     split_index(g, gi, d, s);
     // F in the order (xy, xz, xt, yz, yt, zt)
@@ -156,7 +155,6 @@ __global__ void k_clover_build(Geom g, const double2 *U, double csw, double kapp
     M3 Fxt = field_strength(g, U, gi, 0, 3), Fyz = field_strength(g, U, gi, 1, 2);
     M3 Fyt = field_strength(g, U, gi, 1, 3), Fzt = field_strength(g, U, gi, 2, 3);
     bool odd = s >= g.Vh;
-    const double kc = kappa * csw;
     for (int ch = 0; ch < 2; ch++) {
         double se = ch == 0 ? 1.0 : -1.0;
         zd G1[9], G2[9], G3[9];
@@ -193,6 +191,12 @@ __global__ void k_clover_build(Geom g, const double2 *U, double csw, double kapp
     }
 }
 
+__global__ void k_clover_build(Geom g, const double2 *U, double kc, double2 *A, double2 *S, int *singular)
+{
+    const int gi = blockIdx.x * blockDim.x + threadIdx.x;
+    if (gi < g.V) clover_site(g, U, gi, kc, A, S, singular);
+}
+
 // ------------------------------------------------------------------------
 // The same for SU(3) links, in 64-bit fixed point (fixed.cuh): the 72 matrix
 // products of a site's 24 leaves are integer multiply-adds on the links'
@@ -206,6 +210,15 @@ __global__ void k_clover_build(Geom g, const double2 *U, double csw, double kapp
 // operations per block for 1730 of Gauss-Jordan with pivoting); the rest waits
 // on integer latencies (2.6 warps per scheduler at 168-255 registers; 128
 // registers spill and are no faster).
+//
+// An entry of a leaf is off by at most 10 2^-60: the links' rounding, each product's
+// left-out lower limbs (six of at most 1/4) and rounding, through three products.
+// FP64 arithmetic rounds it by up to 18 2^-53 S, S the sum of the magnitudes of the
+// last product's terms, and by about 2^-53 S on average.  So a plane's four leaves are
+// as good as FP64's where S, added over them, is at least 4 2^-6 for each of the nine
+// entries, which the factors' leading six bits show; a site with a smaller one in
+// any plane (a field that is nearly the unit field, whose field strength lies that
+// far below the leaves' entries) is computed in FP64.
 
 struct M3x {
     cfx m[9];
@@ -279,13 +292,21 @@ __device__ __forceinline__ M3x step_link_fx(const Geom &g, const int4 *U, int n,
 // 8 F_{mu nu} = traceless part of Q - Q^+ at gi, scale 2^-57, as nine integers:
 // the imaginary diagonal, then re and im of the entries (0,1), (0,2), (1,2)
 constexpr int kLeafBits = 57;
-__device__ __forceinline__ void field_strength_fx(const Geom &g, const int4 *U, int gi, int mu, int nu, int64_t *F)
+constexpr uint32_t kLeafLow = 4 * 64 * 64 >> 6;
+__device__ __forceinline__ uint32_t lead6(const cfx &x)
+{
+    return (uint32_t)max(abs(x.re.hi), abs(x.im.hi)) >> (kFxLinkBits - kFxLimb - 6);
+}
+// low: lowered to the plane's smallest sum of magnitudes, 64^2 for 1
+__device__ __forceinline__ void field_strength_fx(const Geom &g, const int4 *U, int gi, int mu, int nu, int64_t *F,
+                                                  uint32_t &low)
 {
     const int n_pm = nbr(g, gi, 2 * mu), n_mm = nbr(g, gi, 2 * mu + 1);
     const int n_pn = nbr(g, gi, 2 * nu), n_mn = nbr(g, gi, 2 * nu + 1);
     M3q q;
 #pragma unroll
     for (int k = 0; k < 9; k++) q.re[k] = q.im[k] = 0;
+    uint32_t mag[5] = {0, 0, 0, 0, 0};  // two entries a word: at most 4 3 64^2 < 2^16
     // A leaf runs from n over the steps a, b and back over a, b: X Y^+ with X =
     // link(n, a) link(n + a, b) and Y = link(n, b) link(n + b, a), for (a, b) =
     // (+mu, +nu), (+nu, -mu), (-mu, -nu), (-nu, +mu).  X, Y and X Y^+ run through
@@ -321,9 +342,19 @@ __device__ __forceinline__ void field_strength_fx(const Geom &g, const int4 *U, 
                     q.re[k] += fx_join(p.m[k].re) >> 3;
                     q.im[k] += fx_join(p.m[k].im) >> 3;
                 }
+#pragma unroll
+                for (int i = 0; i < 3; i++)
+#pragma unroll
+                    for (int j = 0; j < 3; j++)
+                        mag[(i * 3 + j) / 2] +=
+                            (lead6(l.m[i * 3]) * lead6(r.m[j]) + lead6(l.m[i * 3 + 1]) * lead6(r.m[3 + j]) +
+                             lead6(l.m[i * 3 + 2]) * lead6(r.m[6 + j]))
+                            << ((i * 3 + j) % 2 * 16);
             }
         }
     }
+#pragma unroll
+    for (int k = 0; k < 9; k++) low = min(low, k % 2 ? mag[k / 2] >> 16 : mag[k / 2] & 0xffffu);
     const int64_t d0 = q.im[0], d1 = q.im[4], d2 = q.im[8], mean = (d0 + d1 + d2) / 3;
     F[0] = 2 * (d0 - mean);
     F[1] = 2 * (d1 - mean);
@@ -427,21 +458,26 @@ __device__ __forceinline__ void store_herm6(double2 *dst, int64_t stride, const 
 
 constexpr int kCloverThreads = 64;
 
-__global__ void __launch_bounds__(kCloverThreads, 4) k_clover_build_fx(Geom g, const int4 *U, double kc, double2 *A,
-                                                                    double2 *S, int *singular)
+__global__ void __launch_bounds__(kCloverThreads, 4) k_clover_build_fx(Geom g, const int4 *U, const double2 *U64,
+                                                                    double kc, double2 *A, double2 *S, int *singular)
 {
     __shared__ int64_t F[6][9][kCloverThreads];
     const int gi = blockIdx.x * kCloverThreads + threadIdx.x, t = threadIdx.x;
     if (gi >= g.V) return;
     int d, s;
     split_index(g, gi, d, s);
+    uint32_t low = ~0u;
 #pragma unroll 1
     for (int plane = 0; plane < 6; plane++) {  // xy, xz, xt, yz, yt, zt
         const int mu = plane < 3 ? 0 : (plane < 5 ? 1 : 2), nu = plane < 3 ? plane + 1 : (plane < 5 ? plane - 1 : 3);
         int64_t f[9];
-        field_strength_fx(g, U, gi, mu, nu, f);
+        field_strength_fx(g, U, gi, mu, nu, f, low);
 #pragma unroll
         for (int k = 0; k < 9; k++) F[plane][k][t] = f[k];
+    }
+    if (low < kLeafLow) {
+        clover_site(g, U64, gi, kc, A, S, singular);
+        return;
     }
     const bool odd = s >= g.Vh;
     constexpr int ex = -kLeafBits - 3;  // F is an eighth of its integers
@@ -517,9 +553,10 @@ qdd_status launch_clover_build(Gauge *g, double csw, double kappa, int *d_singul
     LaunchScope ls(g->ctx->timer, K_OTHER, s);
     if (fixed)
         k_clover_build_fx<<<(g->hg.V + kCloverThreads - 1) / kCloverThreads, kCloverThreads, 0, s>>>(
-            g->geom, g->fx.links.as<int4>(), kappa * csw, g->clov64.as<double2>(), g->sclov64.as<double2>(), d_singular);
+            g->geom, g->fx.links.as<int4>(), g->links64.as<double2>(), kappa * csw, g->clov64.as<double2>(),
+            g->sclov64.as<double2>(), d_singular);
     else
-        k_clover_build<<<(g->hg.V + 127) / 128, 128, 0, s>>>(g->geom, g->links64.as<double2>(), csw, kappa,
+        k_clover_build<<<(g->hg.V + 127) / 128, 128, 0, s>>>(g->geom, g->links64.as<double2>(), kappa * csw,
                                                             g->clov64.as<double2>(), g->sclov64.as<double2>(),
                                                             d_singular);
     QDD_CUDA(cudaGetLastError());
