@@ -461,6 +461,9 @@ __global__ void k_su3_check(Geom g, const double2 *U, double tol, int *out)
         double2 a = __ldg(p + (int64_t)k * g.Vd);
         u[k] = mk(a.x, a.y);
     }
+    int ex = 0;
+#pragma unroll
+    for (int k = 0; k < 9; k++) ex = max(ex, max(fx_exponent(u[k].re), fx_exponent(u[k].im)));
     // Rows 0 and 1 orthonormal and row 2 the conjugate of their cross product to
     // a tenth of the tolerance imply both conditions; otherwise they are taken
     // as they stand.  (54 FP64 multiply-adds for 170; 16^3x32: 200 -> 60 us)
@@ -484,8 +487,9 @@ __global__ void k_su3_check(Geom g, const double2 *U, double tol, int *out)
             near = fmax(near, fmax(fabs(t.re), fabs(t.im)));
         }
     }
+    const bool su3 = near <= 0.1 * tol && ex < 0x7ff;  // (fmax passes NaN over)
     double dev = 0;
-    if (!(near <= 0.1 * tol)) {
+    if (!su3) {
         for (int i = 0; i < 3; i++)
             for (int j = 0; j < 3; j++) {
                 cpx<double> t = mk(i == j ? -1.0 : 0.0, 0.0);
@@ -496,13 +500,16 @@ __global__ void k_su3_check(Geom g, const double2 *U, double tol, int *out)
                           u[2] * (u[3] * u[7] - u[4] * u[6]);
         dev = fmax(dev, fmax(fabs(det.re - 1.0), fabs(det.im)));
     }
-    if (!(dev <= tol)) atomicOr(out, 1);
-    int ex = 0;
+    if (!(dev <= tol) || ex == 0x7ff) atomicOr(out, 1);
+    if (su3) {  // u = 0
+        if (*(volatile int *)(out + 1) < 1022) atomicMax(out + 1, 1022);
+        if (*(volatile int *)(out + 2) < 0x7ff - 1022) atomicMax(out + 2, 0x7ff - 1022);
+        return;
+    }
     bool zero = true;
     float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int k = 0; k < 9; k++) {
-        ex = max(ex, max(fx_exponent(u[k].re), fx_exponent(u[k].im)));
         zero = zero && u[k].re == 0 && u[k].im == 0;
         const float m = fabsf(d2f(u[k].re)) + fabsf(d2f(u[k].im));
         row[k / 3] += m;
