@@ -125,20 +125,33 @@ static void fx_release(Gauge *g)
     f.have_links = f.have_clov = f.required = f.wide = false;
 }
 
-// Gives up optional fixed-point copies that nobody reads, until at least
-// `need` bytes have come back.
+// Gives up optional fixed-point copies, until at least `need` bytes have come
+// back.  Another thread holds a copy while it launches the operator or builds the
+// copy, so one that is held is tried again for up to a second (two threads that build
+// copies may each want the other's).  This thread holds none but the one it builds:
+// whoever acquires a copy has made its own allocations before.
 static void fx_reclaim(Ctx *c, size_t need)
 {
-    if (c->optional.load() == 0) return;
-    std::lock_guard<std::mutex> lk(c->gauges_mu);
     size_t got = 0;
-    for (Gauge *g : c->gauges) {
-        if (got >= need) break;
-        if (g == fx_building) continue;
-        std::unique_lock<std::shared_mutex> ul(g->fx.mu, std::try_to_lock);
-        if (!ul.owns_lock() || g->fx.required) continue;
-        got += g->fx.links.bytes + g->fx.clov.bytes + g->fx.clov_e.bytes;
-        fx_release(g);
+    for (int turn = 0; turn < 10000 && c->optional.load() != 0; turn++) {
+        bool held = false;
+        {
+            std::lock_guard<std::mutex> lk(c->gauges_mu);
+            for (Gauge *g : c->gauges) {
+                if (got >= need) return;
+                if (g == fx_building) continue;
+                std::unique_lock<std::shared_mutex> ul(g->fx.mu, std::try_to_lock);
+                if (!ul.owns_lock()) {
+                    held = true;
+                    continue;
+                }
+                if (g->fx.required) continue;
+                got += g->fx.links.bytes + g->fx.clov.bytes + g->fx.clov_e.bytes;
+                fx_release(g);
+            }
+        }
+        if (!held || got >= need) return;
+        std::this_thread::sleep_for(std::chrono::microseconds(100));
     }
 }
 
@@ -163,6 +176,14 @@ qdd_status DevMem::alloc(Ctx *c, size_t n)
     bytes = n;
     c->used += n;
     return QDD_OK;
+}
+
+qdd_status optional_room(DevMem &m, Ctx *c, size_t n)
+{
+    const qdd_status st = m.ensure(c, n);
+    if (st != QDD_EBUDGET && st != QDD_ENOMEM) return st;
+    clear_error();
+    return QDD_EBUDGET;
 }
 
 void DevMem::release()
@@ -781,34 +802,41 @@ qdd_status qdd_apply_D(qdd_gauge *g, const double *in, double *out, int nrhs, qd
         set_error("a sharded field needs separate input and output buffers");
         return QDD_EINVAL;
     }
-    if (arith != QDD_PREC_F32) QDD_TRY(st->a_s.ensure(g->ctx, fx_exponent_bytes(V, nrhs)));
-    else if (scaled) QDD_TRY(st->a_s.ensure(g->ctx, V * 4 * nrhs));
-    if (scaled) QDD_TRY(st->b_s.ensure(g->ctx, V * 4 * nrhs));
-    // FP64-class arithmetic in fixed point: the input is converted on its way
-    // in, the operator writes the host layout
-    FxLock fl;
-    if (arith != QDD_PREC_F32) QDD_TRY(fx_acquire(g, arith == QDD_PREC_DF64, true, s, fl));
-    const bool fixed = fl.owns_lock();
-    // A sharded field corrects the output's boundary planes from the input (FP64,
-    // host layout), and the fixed-point operator goes back to it at single sites, so
-    // the host output must not reuse the input's staging; a device buffer that is
-    // both input and output is copied first.
-    DevMem &oio = g->slab || fixed ? st->c : st->io;
-    QDD_TRY(stage_out(g, oio, out, nrhs, on_device, s, &dout));
+    if (scaled) {
+        QDD_TRY(st->a_s.ensure(g->ctx, V * 4 * nrhs));
+        QDD_TRY(st->b_s.ensure(g->ctx, V * 4 * nrhs));
+    }
+    // a sharded field: its boundary planes (FP64, host layout) move while the operator runs
+    QDD_TRY(slab_dslash_begin(g, din, false, true, nrhs, s));
+    // FP32 spinors: the operator widens and writes the host layout
+    const bool direct = arith == QDD_PREC_F32 && prec == QDD_PREC_F32;
+    // FP64-class arithmetic in fixed point: the input is converted on its way in, the
+    // operator writes the host layout and goes back to the input at single sites, so
+    // the output must not reuse the input's staging, and a device buffer that is both
+    // is copied first.  FP64 arithmetic has its result in the same buffer b, which
+    // is there before the copy is acquired: nothing is allocated under its lock.
     const size_t bytes = V * 12 * sizeof(double2) * nrhs;
-    if (fixed && (const char *)din < (const char *)dout + bytes && (const char *)dout < (const char *)din + bytes) {
-        QDD_TRY(st->b.ensure(g->ctx, bytes));
+    const bool overlap = on_device && (const char *)in < (const char *)out + bytes && (const char *)out < (const char *)in + bytes;
+    FxLock fl;
+    if (arith != QDD_PREC_F32) {
+        if (!on_device || overlap) QDD_TRY(st->b.ensure(g->ctx, bytes));
+        if (g->slab && !on_device) QDD_TRY(st->c.ensure(g->ctx, bytes));
+        const qdd_status room = optional_room(st->a_s, g->ctx, fx_exponent_bytes(V, nrhs));
+        if (room == QDD_OK) QDD_TRY(fx_acquire(g, arith == QDD_PREC_DF64, true, s, fl));
+        else if (room != QDD_EBUDGET) return room;
+    }
+    const bool fixed = fl.owns_lock();
+    if (!fixed && !direct) QDD_TRY(st->b.ensure(g->ctx, V * 12 * eb * nrhs));
+    // (a sharded field corrects the output's boundary planes from the input)
+    DevMem &oio = g->slab ? st->c : fixed ? st->b : st->io;
+    QDD_TRY(stage_out(g, oio, out, nrhs, on_device, s, &dout));
+    if (fixed && overlap) {
         QDD_CUDA(cudaMemcpyAsync(st->b.p, din, bytes, cudaMemcpyDeviceToDevice, s));
         din = st->b.as<double>();
     }
-    // FP32 spinors: the operator widens and writes the host layout too
-    const bool direct = arith == QDD_PREC_F32 && prec == QDD_PREC_F32;
-    if (!fixed && !direct) QDD_TRY(st->b.ensure(g->ctx, V * 12 * eb * nrhs));
     const FxField fxa{st->a.p, st->a_s.as<int>()};
     if (fixed) QDD_TRY(launch_spinor_in_fx(g, din, fxa, nrhs, s));
     else QDD_TRY(launch_spinor_in(g, din, st->a.p, st->a_s.as<float>(), prec, nrhs, s));
-    // a sharded field: its boundary planes (FP64, host layout) move while the operator runs
-    QDD_TRY(slab_dslash_begin(g, din, false, true, nrhs, s));
     if (fixed) {
         QDD_TRY(launch_dslash_fx(g, fxa, {din, kFxHost64}, (double2 *)dout, true, nullptr, nrhs, s));
     } else if (direct) {

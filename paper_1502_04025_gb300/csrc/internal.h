@@ -268,10 +268,13 @@ __host__ __device__ __forceinline__ int64_t pair_index(int64_t d, int P, int p, 
 }
 
 qdd_status ensure_copy(Gauge *g, qdd_prec prec, cudaStream_t s);
+// room that a call can do without: QDD_EBUDGET, with no error message, where there is none
+qdd_status optional_room(DevMem &m, Ctx *c, size_t n);
 // The fixed-point copy of links and (clover) of the clover term, built where it
 // is missing.  lk holds it on return; where it does not, FP64 arithmetic has to
 // stand in: links or a clover term out of range, links of different sizes, or no
-// room for a copy that is not required (which is no error).
+// room for a copy that is not required (which is no error).  While it holds a copy a
+// thread allocates nothing: an allocation may have to take optional copies back.
 using FxLock = std::shared_lock<std::shared_mutex>;
 qdd_status fx_acquire(Gauge *g, bool required, bool clover, cudaStream_t s, FxLock &lk);
 // the two-row link copy of a storage precision (FP32, FP16, BF16)

@@ -66,7 +66,6 @@ size_t workspace_bytes(const Gauge *g, int m, int B, qdd_prec sp, bool use_sap, 
         b += n * ebytes(spinor_store(sp)) * B + sap_face_bytes(g->hg, sp, B);
         if (sp == QDD_PREC_F16S || sp == QDD_PREC_BF16S) b += V * 4 * B;
     }
-    else b += fx_exponent_bytes(V, B);  // of the operator's input (ensure_ws)
     if (kdr > 0) b += n * 16 * B * (size_t)(3 * kdr + 1);
     return b + (1 << 20);
 }
@@ -112,8 +111,12 @@ static qdd_status ensure_ws(Gauge *g, Workspace &w, int m, int B, qdd_prec sp, b
     QDD_TRY(w.dev.ensure(c, sm.total() * sizeof(double2)));
     // exponents of the operator's fixed-point input, whose components take the
     // host-transfer buffer between the input and the output: the Schwarz
-    // method's residual, consumed by then, where there is one
-    if (!use_sap) QDD_TRY(w.rho.ensure(c, fx_exponent_bytes(V, B)));
+    // method's residual, consumed by then, where there is one (else optional: without
+    // them the operator runs in FP64 arithmetic)
+    if (!use_sap) {
+        const qdd_status room = optional_room(w.rho, c, fx_exponent_bytes(V, B));
+        if (room != QDD_OK && room != QDD_EBUDGET) return room;
+    }
     QDD_TRY(blas_scratch_ensure(c, w.scratch));
     QDD_TRY(w.err.ensure(c, sizeof(int)));
     if (w.host_elems < sm.total()) {
@@ -134,13 +137,12 @@ qdd_status solve_prepare(Gauge *g, Workspace *w, const qdd_solve_params *p, cuda
     QDD_TRY(ensure_ws(g, *w, p->restart_m, p->nrhs, sp, p->use_sap == 1, p->dr_k));
     if (p->use_sap) QDD_TRY(ensure_copy(g, sp, s));
     if (p->arnoldi_prec != QDD_PREC_F64) QDD_TRY(ensure_copy(g, p->arnoldi_prec, s));
-    FxLock lk;  // the FP64 operator's optional fixed-point copy (the true residual is always FP64)
-    QDD_TRY(fx_acquire(g, false, true, s, lk));
     if (p->relax_eta > 0 || p->arnoldi_prec == QDD_PREC_F32) {
         QDD_TRY(ensure_copy(g, QDD_PREC_F32, s));
         if (g->two_rows) QDD_TRY(ensure_links12(g, QDD_PREC_F32, s));
     }
-    return QDD_OK;
+    FxLock lk;  // last, the FP64 operator's optional fixed-point copy (the true residual is always FP64)
+    return fx_acquire(g, false, true, s, lk);
 }
 
 qdd_status solve_impl(Gauge *g, Workspace *wsp, const double *b_in, double *x_out, int on_device,
@@ -242,7 +244,9 @@ qdd_status solve_impl(Gauge *g, Workspace *wsp, const double *b_in, double *x_ou
     int iters = 0, restarts = 0, deflated = 0;
     bool converged = false;
     qdd_status status = QDD_OK;
-    const FxField fxb{w.io.p, w.rho.as<int>()};  // the operator's input in fixed point
+    // the operator's input in fixed point
+    const FxField fxw{w.io.p, w.rho.as<int>()};
+    const FxField *fxb = w.rho.bytes >= fx_exponent_bytes(g->hg.V, B) ? &fxw : nullptr;
     SapBuffers sb{w.rho.p, w.face.p, nullptr, w.rho_s.as<float>()};
     double2 *ZR = w.ZR.as<double2>();
 
@@ -253,7 +257,7 @@ qdd_status solve_impl(Gauge *g, Workspace *wsp, const double *b_in, double *x_ou
         else {
             QDD_TRY(slab_dslash_begin(g, X, false, false, B, s));  // sharded: boundary planes
             QDD_TRY(launch_dslash(g, QDD_PREC_F64, QDD_PREC_F64, X, nullptr, QDD_PREC_F64, pending_dr ? w.Vt.as<double2>() : V,
-                                  nullptr, QDD_PREC_F64, Bv, B, s, &fxb));
+                                  nullptr, QDD_PREC_F64, Bv, B, s, fxb));
             QDD_TRY(slab_dslash_end(g, V, true, B, s));
         }
         double2 *R0 = (cycle > 0 && pending_dr) ? w.Vt.as<double2>() : V;
@@ -443,7 +447,7 @@ qdd_status solve_impl(Gauge *g, Workspace *wsp, const double *b_in, double *x_ou
                                       QDD_PREC_F64, nullptr, B, s));
             else if (p->arnoldi_prec == QDD_PREC_F64 || p->arnoldi_prec == QDD_PREC_DF64)
                 QDD_TRY(launch_dslash(g, p->arnoldi_prec, p->arnoldi_prec, zj, nullptr, zp, wv, nullptr,
-                                      QDD_PREC_F64, nullptr, B, s, &fxb));
+                                      QDD_PREC_F64, nullptr, B, s, fxb));
             else
                 QDD_TRY(launch_dslash(g, QDD_PREC_F32, QDD_PREC_F32, zj, nullptr, QDD_PREC_F32, wv, nullptr,
                                       QDD_PREC_F64, nullptr, B, s));
