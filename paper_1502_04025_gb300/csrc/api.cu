@@ -114,6 +114,8 @@ Timer::~Timer()
 
 // the gauge field whose fixed-point copy this thread is building (its lock is held)
 static thread_local const Gauge *fx_building = nullptr;
+// this thread asks for memory that it can do without: it takes no copies back for it
+static thread_local bool fx_optional = false;
 
 static void fx_release(Gauge *g)
 {
@@ -159,13 +161,19 @@ qdd_status DevMem::alloc(Ctx *c, size_t n)
 {
     release();
     if (n == 0) return QDD_OK;
-    if (c->used.load() + n > c->budget) fx_reclaim(c, c->used.load() + n - c->budget);
+    if (c->used.load() + n > c->budget && !fx_optional) fx_reclaim(c, c->used.load() + n - c->budget);
     if (c->used.load() + n > c->budget) {
         set_error("allocation of %zu bytes exceeds the HBM budget (%zu of %zu bytes in use)", n, c->used.load(),
                   c->budget);
         return QDD_EBUDGET;
     }
     cudaError_t e = cudaMalloc(&p, n);
+    if (e == cudaErrorMemoryAllocation && !fx_optional && c->optional.load() != 0) {
+        // the device is full below the budget (another library, another process)
+        cudaGetLastError();
+        fx_reclaim(c, n);
+        e = cudaMalloc(&p, n);
+    }
     if (e != cudaSuccess) {
         p = nullptr;
         cudaGetLastError();
@@ -180,7 +188,9 @@ qdd_status DevMem::alloc(Ctx *c, size_t n)
 
 qdd_status optional_room(DevMem &m, Ctx *c, size_t n)
 {
+    fx_optional = true;
     const qdd_status st = m.ensure(c, n);
+    fx_optional = false;
     if (st != QDD_EBUDGET && st != QDD_ENOMEM) return st;
     clear_error();
     return QDD_EBUDGET;
@@ -190,7 +200,10 @@ void DevMem::release()
 {
     if (p) {
         cudaFree(p);
-        if (ctx) ctx->used -= bytes;
+        if (ctx) {
+            ctx->used -= bytes;
+            ctx->frees++;
+        }
     }
     p = nullptr;
     bytes = 0;
@@ -264,12 +277,15 @@ static qdd_status fx_build(Gauge *g, bool required, bool clover, cudaStream_t s)
     const size_t n = (size_t)g->hg.V * 36 * 16, ne = ((size_t)g->hg.V + 1) * sizeof(int);
     if (!required && !f.required) {
         const size_t more = (f.links.p ? 0 : n) + (clover && !f.clov.p ? n + ne : 0);
-        if (c->used.load() + more > c->budget / 2) return QDD_EBUDGET;
+        if (c->used.load() + more > c->budget / 2 || f.no_room == c->frees.load()) return QDD_EBUDGET;
     }
     const size_t before = f.links.bytes + f.clov.bytes + f.clov_e.bytes;
+    fx_optional = !required;
     qdd_status st = f.links.ensure(c, n);
     if (st == QDD_OK && clover) st = f.clov.ensure(c, n);
     if (st == QDD_OK && clover) st = f.clov_e.ensure(c, ne);
+    fx_optional = false;
+    f.no_room = st == QDD_ENOMEM ? c->frees.load() : ~0ull;
     if (!f.required) c->optional += f.links.bytes + f.clov.bytes + f.clov_e.bytes - before;
     QDD_TRY(st);
     if (!f.have_links) QDD_TRY(launch_links_fx(g, s));

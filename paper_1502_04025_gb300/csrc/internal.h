@@ -128,6 +128,7 @@ struct Ctx {
     int nsm = 0;
     size_t budget = 0;
     std::atomic<size_t> used{0};
+    std::atomic<unsigned long long> frees{0};  // buffers given back so far
     // of these, optional copies that an allocation may take back (fx_reclaim),
     // and the gauge fields that may hold one
     std::atomic<size_t> optional{0};
@@ -179,7 +180,7 @@ struct PrecCopy {
 // the clover build.  QDD_PREC_DF64 needs it (required); for QDD_PREC_F64 and the
 // clover build, which have FP64 arithmetic to fall back on, it is optional:
 // built while at most half of the HBM budget is in use, and given up when
-// another allocation would exceed the budget.  Readers hold mu shared from
+// another allocation would exceed the budget or the device's memory.  Readers hold mu shared from
 // fx_acquire until their kernels are launched (freeing device memory waits for
 // launched kernels); building and giving up hold it exclusively.
 struct FxCopy {
@@ -187,6 +188,9 @@ struct FxCopy {
     DevMem links, clov, clov_e;  // clov_e: one exponent per site, then the largest in magnitude
     bool have_links = false, have_clov = false, required = false;
     bool wide = false;           // have_clov: the term is out of the range that has a copy
+    // the device had no room for the copy when this many buffers had been given back
+    // (not tried again before the next one is)
+    unsigned long long no_room = ~0ull;
 };
 
 // Device and pinned host buffers of one solve (Krylov basis, preconditioner
