@@ -139,6 +139,12 @@ def op_bytes_per_site(prec, three_rows=True):
     return link + clover + 2 * spinor
 
 
+def apply_bytes_per_site(prec, three_rows=True):
+    """op_bytes_per_site of the operator inside qdd_apply_D, which writes FP32
+    and H16 results as FP64 in the host layout (192 bytes of output for 96)."""
+    return op_bytes_per_site(prec, three_rows) + (12 * 8 if prec in ("f32", "h16") else 0)
+
+
 def crossing_hops_per_site(dom):
     """Average number of hops per site that leave a domain: 2 faces per
     direction, each holding Vd/dom[mu] sites."""
@@ -574,12 +580,12 @@ def run_qdd(args):
                 "flop_per_launch": flop,
                 "peak_source": f"{sm_count} SMs x 128 FP32 lanes x 2 flop x {pk.get('sm_max_mhz', 2070.0):.0f} MHz"}
     elif dom_cls == "dslash":
-        ms_launch = kt["dslash"][0] / kt["dslash"][1]
+        ms_launch = kt["dslash"][0] / kt["dslash"][1] * 3  # an application: conversion, operator, listed sites
         bytes_site = 576 + 576 + 96 + 192  # FP64-width links + clover, FP32 input, FP64 output
         achieved = nrhs * V * bytes_site / (ms_launch * 1e-3) / 1e9
         roof = {"kernel": "k_dslash (operator in the Arnoldi step)", "bound": "hbm", "achieved": achieved,
                 "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": achieved / pk["hbm_gbs"], "traffic": None,
-                "ms_per_launch": ms_launch, "launches": kt["dslash"][1]}
+                "ms_per_launch": ms_launch, "launches": kt["dslash"][1] // 3}
     else:
         ms_launch = kt["blas"][0] / kt["blas"][1]
         roof = {"kernel": "FP64 vector kernels", "bound": "hbm", "achieved": None, "peak": pk["hbm_gbs"],
@@ -672,7 +678,7 @@ def run_qdd(args):
             prec = name.split("_")[0]
             rows3 = name.endswith("three_rows") or not two_rows
             qdd.qdd_set_link_compression(gd, not rows3)
-            bps = op_bytes_per_site(prec, rows3)
+            bps = apply_bytes_per_site(prec, rows3)
             for _ in range(3):
                 qdd.qdd_apply_D(gd, xs, prec, out=ys)
             qdd.qdd_set_profiling(ctx, qdd.QDD_PROF_DSLASH)
@@ -681,7 +687,7 @@ def run_qdd(args):
                 qdd.qdd_apply_D(gd, xs, prec, out=ys)
             kd = qdd.qdd_get_kernel_times(ctx, reset=True)
             qdd.qdd_set_profiling(ctx, 0)
-            ms = kd["dslash"][0] / kd["dslash"][1]
+            ms = kd["dslash"][0] / 20  # per apply, all its launches
             dslash[name] = {"ms": ms, "gflops": 1848 * Vl / (ms * 1e-3) / 1e9,
                             "gbs": bps * Vl / (ms * 1e-3) / 1e9,
                             "frac_hbm": bps * Vl / (ms * 1e-3) / 1e9 / pk["hbm_gbs"],
@@ -784,8 +790,8 @@ def run_op_bench(args):
             qdd.qdd_apply_D(g, xs, prec, out=ys)
         kd = qdd.qdd_get_kernel_times(ctx, reset=True)
         qdd.qdd_set_profiling(ctx, 0)
-        ms = kd["dslash"][0] / kd["dslash"][1]
-        bps = op_bytes_per_site(prec, rows3)
+        ms = kd["dslash"][0] / args.op_iters  # per apply, all its launches
+        bps = apply_bytes_per_site(prec, rows3)
         out[name] = {"ms": ms, "gflops": 1848 * Vl / (ms * 1e-3) / 1e9, "gbs": bps * Vl / (ms * 1e-3) / 1e9,
                      "frac_hbm": bps * Vl / (ms * 1e-3) / 1e9 / pk["hbm_gbs"], "bytes_per_site": bps}
     print(json.dumps(out), flush=True)
