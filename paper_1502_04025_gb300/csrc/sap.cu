@@ -1304,10 +1304,11 @@ static qdd_status dispatch_staging(Gauge *g, const SapArgs<R, SL, SC, SS, SP> &a
     // CTAs per SM (FP32 arithmetic, domains of at most 256 sites); the same bits
     // as the one-thread form with two.  The default on 4^4 domains in 16 bits where
     // the third CTA pays: when the colour's domains fit in one wave of three per
-    // SM but not of two (BF16, 384 domains on 152 SMs: 69.8 -> 53.1 us per
-    // half-sweep; 320: 59.3 -> 52.1), and for BF16 beyond four per SM (648: 95.8 -> 93.1,
+    // SM but not of two (us per half-sweep on 152 SMs, 320, 384 and 448 domains: BF16
+    // 59.0 -> 51.7, 69.4 -> 52.7, 71.3 -> 54.1; FP16 55.4 -> 52.0, 56.9 -> 53.1, 58.3 -> 54.0; H16
+    // 59.6 -> 55.8, 62.1 -> 57.1, 64.0 -> 59.0), and for BF16 beyond four per SM (648: 95.8 -> 93.1,
     // 864: 110.2 -> 104.5, 1024: 138 -> 134, 1296: 165 -> 156, 4096: 468 -> 452 us), but not
-    // between (512: 72.5 -> 82.4, 576: 73.9 -> 85.8) nor below (256: 36.5 -> 48.8);
+    // between (BF16, 512: 72.5 -> 82.4, 576: 73.9 -> 85.8) nor below (256: 36.5 -> 48.8);
     // beyond four per SM F16S is faster with two (1024: 120 -> 125 us).
     if constexpr (sizeof(R) == 4) {
         const int nsm = g->ctx->nsm;
@@ -1326,19 +1327,19 @@ static qdd_status dispatch_staging(Gauge *g, const SapArgs<R, SL, SC, SS, SP> &a
     // whole warps, at most 512 threads.  The default wherever it measured faster
     // (us per half-sweep, one-thread form against this one):
     //   FP32 links, links and clover staged: one CTA of Vh threads per SM holds the
-    //     one-thread form back (4^4, 32^3x64: 927 against 647)
+    //     one-thread form back (4^4, 32^3x64: 913 against 651)
     //   FP32 links, clover read through the cache (more than 256 sites): 6x4^3,
-    //     24x16x16x24: 92.4 against 77.2; 8x4^3, 16^3x32: 49.0 (its shape fixed at
-    //     compile time) against 46.8
-    //   FP16 links, 64 to 256 sites of a half-field: 6x4^3, 24x16x16x24 (H16) 84.6
-    //     against 69.5; 8x4^3, 32^4 (H16) 328 against 303; 4^3x6, 32x16x16x24 81.7
+    //     24x16x16x24: 92.3 against 76.9; 8x4^3, 16^3x32: 49.0 (its shape fixed at
+    //     compile time) against 45.9
+    //   FP16 links, 64 to 256 sites of a half-field: 6x4^3, 24x16x16x24 (H16) 79.5
+    //     against 64.9; 8x4^3, 32^4 (H16) 313 against 292; 4^3x6, 32x16x16x24 81.7
     //     against 71.9; not 32-site half-fields (4x4x2x2, 32x32x16x16: 95.7 against
     //     101), nor 4^4 domains, whose one-thread form has its shape fixed at
     //     compile time and runs twice per SM (32^3x64, 12 sources: 5.28 against
     //     5.51 ms)
-    //   not BF16 (6x4^3, 24x32^3: 291 against 261; 48^3x96, 4^4: 2.29 against 2.40
+    //   not BF16 (6x4^3, 24x32^3: 281 against 257; 48^3x96, 4^4: 2.29 against 2.40
     //     ms): its stored residual is so coarse that the forms' different rounding
-    //     moves single components of the result by up to 8e-4
+    //     moves single components of the result by up to 1.1e-3
     // The choice depends on the domain's shape and the storage only, so that a
     // sharded lattice runs the form of the whole one.
     if constexpr (sizeof(R) == 4) {
