@@ -221,8 +221,8 @@ constexpr int kMinFixedLinkExp = -60, kMaxFixedLinkExp = 64, kMaxFixedLinkSpread
 // products then stay inside FP64's normal range, -1016 to 965 and 62 bits more.
 constexpr int kMaxFixedCloverExp = 60;
 // The operator's fixed-point sums are as good as FP64's where the hops, times kappa, are
-// not far below the clover sum (fixed.cuh): with kappa at 0.04 the test leaves one
-// Gaussian site of 500 to FP64, at 0.12 none of 65536.
+// not far below the clover sum (fixed.cuh): with kappa at 0.04 the test leaves two
+// Gaussian sites of 65536 to FP64, below that soon many.
 constexpr double kMinFixedKappa = 0.04;
 
 static size_t elem_bytes(qdd_prec p)

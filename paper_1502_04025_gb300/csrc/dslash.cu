@@ -611,7 +611,7 @@ __global__ void __launch_bounds__(128) k_dslash_list(Geom g, FxArgs f, double ka
         int d, s;
         split_index(g, gi, d, s);
         cpx<double> up = mk(0.0, 0.0), lo = mk(0.0, 0.0);
-#pragma unroll 1
+#pragma unroll
         for (int back = 0; back < 2; back++) {
             const uint16_t e = __ldg(g.nbl + s * 8 + 2 * mu + back);
             const int nd = (e & kCross) ? __ldg(g.nbd + d * 8 + 2 * mu + back) : d, ns = e & kSlotMask;

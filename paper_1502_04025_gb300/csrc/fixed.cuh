@@ -25,17 +25,18 @@
 //
 // The error of a component y of D x belongs to these scales.  With E the largest
 // exponent of the nine sites and Q = 2^(E + u - 57), a hop's component is off by at
-// most 2 sqrt(6) Q (truncated spinors), 0.75 Q (rounded links), 3 Q (products of lower
-// limbs left out), 0.5 Q (rounding) and Q (shift to E): eight hops by 82 Q =
-// 2^(E + u - 50.65).  The clover sum, with q = 2^(e + a - 57): 1.25 q (spinors), 1.4 q
-// (A), 2.75 q (lower limbs), 0.5 q: 2^(e + a - 54.4).  FP64 arithmetic rounds a hop's
+// most sqrt(6) Q (rounded spinors), 0.75 Q (rounded links), 3 Q (products of lower
+// limbs left out), 0.5 Q (rounding) and Q (shift to E): eight hops by 62 Q =
+// 2^(E + u - 51.05).  The clover sum, with q = 2^(e + a - 57): 0.6 q (spinors), 0.7 q
+// (A), 2.75 q (lower limbs), 0.5 q: 2^(e + a - 54.8).  FP64 arithmetic rounds a hop's
 // six multiply-adds, the projection before and the sum of eight after them, by up
 // to 15 2^-53 S, S the sum of the moduli of the products U h.  So a component is
 // as good as FP64's where
 //   S >= kFxHop 2^(E + u) + kFxClover 2^(e + a) / |kappa|,
 // which the leading bits of links and half spinors show (k_dslash_fx); a site with
-// any component below is computed in FP64.  Of 65536 sites with Gaussian spinors
-// the smallest S is 1.6 times that on links of eps = 0.5 and 0.7.
+// any component below is computed in FP64.  Of 65536 sites the smallest S is 2.1
+// times that with Gaussian spinors, and 1.4 times with the Schwarz method's second
+// direction, on links of eps = 0.5 and 0.7.
 //
 // A site with a non-finite component, or with its largest exponent near the
 // ends of FP64's range, is marked kFxRaw in place of its exponent, and every site
@@ -58,7 +59,7 @@ constexpr int kFxZero = -900;       // exponent of an all-zero site
 constexpr int kFxLimb = 30;         // bits of the lower limb
 constexpr int kFxSpinorBits = 57, kFxCloverBits = 60, kFxLinkBits = 60;
 constexpr float kFxLinkRow = 2.4495f, kFxCloverRow = 1.25f;
-constexpr float kFxHop = 0.35f, kFxClover = 0.025f;
+constexpr float kFxHop = 0.26f, kFxClover = 0.02f;
 
 // the smallest e with v <= 2^e (v >= 0; infinity and NaN give 128 and more)
 __device__ __forceinline__ int fx_ceil_exponent(float v)
@@ -123,14 +124,14 @@ __device__ __forceinline__ double fx_to_double(int64_t v, int ex)
 }
 
 // the FP64 number with bits (hi, lo) as an integer with `bits` bits below
-// 2^(emax - 1022), emax an exponent field at least its own
+// 2^(emax - 1022), rounded, emax an exponent field at least its own
 __device__ __forceinline__ int64_t fx_from_bits(uint32_t hi, uint32_t lo, int emax, int bits)
 {
     const int ex = (int)((hi >> 20) & 0x7ff);
     // 53-bit mantissa (subnormal numbers, far below any site's scale here, count as zero)
     const uint64_t m = ex ? ((uint64_t)((hi & 0x000fffffu) | 0x00100000u) << 32 | lo) : 0;
     const int d = emax - ex;
-    const uint64_t x = d > 63 ? 0 : (m << (bits - 53)) >> d;
+    const uint64_t x = d > 63 ? 0 : ((m << (bits - 53)) + ((1ull << d) >> 1)) >> d;  // (bits <= 60: no carry lost)
     return (int32_t)hi < 0 ? -(int64_t)x : (int64_t)x;
 }
 
