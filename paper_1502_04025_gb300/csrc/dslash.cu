@@ -580,31 +580,110 @@ __global__ void __launch_bounds__(128, VD ? 3 : 4) k_dslash_fx(Geom g0, FxArgs f
     }
 }
 
+// component k of site ss of domain dd as the caller has it
+__device__ __forceinline__ cpx<double> fx_source(const Geom &g, const FxArgs &f, int64_t r, int dd, int ss, int k)
+{
+    if (f.src.kind == kFxPlanes32) {
+        const float2 v = __ldg((const float2 *)f.src.p + (r * g.V + (int64_t)dd * g.Vd) * 12 + (int64_t)k * g.Vd + ss);
+        return mk(f2d(v.x), f2d(v.y));
+    }
+    const double2 *p = (const double2 *)f.src.p;
+    const double2 v = f.src.kind == kFxHost64 ? __ldg(p + (r * g.V + __ldg(f.site_of + dd * g.Vd + ss)) * 12 + k)
+                                              : __ldg(p + (r * g.V + (int64_t)dd * g.Vd) * 12 + (int64_t)k * g.Vd + ss);
+    return mk(v.x, v.y);
+}
+
+template <bool RESID, bool HOST>
+__device__ __forceinline__ void fx_store64(const Geom &g, const FxArgs &f, int64_t r, int d, int s, int k, double2 y)
+{
+    const int64_t plane = (r * g.V + (int64_t)d * g.Vd) * 12 + (int64_t)k * g.Vd + s;
+    if (RESID) {
+        const double2 v = __ldg(f.b + plane);
+        y = make_double2(v.x - y.x, v.y - y.y);
+    }
+    if (HOST) f.out[(r * g.V + __ldg(f.site_of + d * g.Vd + s)) * 12 + k] = y;
+    else f.out[plane] = y;
+}
+
+// one site by one thread
+template <bool RESID, bool HOST>
+__device__ __noinline__ void dslash_site64(const Geom &g, const FxArgs &f, int64_t r, int d, int s, double kappa)
+{
+    cpx<double> acc[12], x[12], u[9];
+#pragma unroll
+    for (int k = 0; k < 12; k++) acc[k] = mk(0.0, 0.0);
+    auto load = [&](int dir) {
+        const int back = dir & 1;
+        const uint16_t e = __ldg(g.nbl + s * 8 + dir);
+        const int nd = (e & kCross) ? __ldg(g.nbd + d * 8 + dir) : d, ns = e & kSlotMask;
+        if (!(QDD_IN_RANGE(nd, 0, g.Nd) && QDD_IN_RANGE(ns, 0, g.Vd))) return false;
+#pragma unroll
+        for (int k = 0; k < 12; k++) x[k] = fx_source(g, f, r, nd, ns, k);
+        const double2 *U = f.U64 + ((int64_t)(back ? nd : d) * 36 + (dir >> 1) * 9) * g.Vd + (back ? ns : s);
+#pragma unroll
+        for (int k = 0; k < 9; k++) {
+            const double2 v = __ldg(U + (int64_t)k * g.Vd);
+            u[k] = mk(v.x, v.y);
+        }
+        return true;
+    };
+    if (load(0)) hop<0, +1>(u, x, acc);
+    if (load(1)) hop<0, -1>(u, x, acc);
+    if (load(2)) hop<1, +1>(u, x, acc);
+    if (load(3)) hop<1, -1>(u, x, acc);
+    if (load(4)) hop<2, +1>(u, x, acc);
+    if (load(5)) hop<2, -1>(u, x, acc);
+    if (load(6)) hop<3, +1>(u, x, acc);
+    if (load(7)) hop<3, -1>(u, x, acc);
+#pragma unroll
+    for (int blk = 0; blk < 2; blk++) {
+        cpx<double> m[18], z[6];
+#pragma unroll
+        for (int k = 0; k < 18; k++) {
+            const double2 v = __ldg(f.A64 + ((int64_t)d * 36 + blk * 18 + k) * g.Vd + s);
+            m[k] = mk(v.x, v.y);
+        }
+#pragma unroll
+        for (int k = 0; k < 6; k++) x[k] = fx_source(g, f, r, d, s, 6 * blk + k);
+        herm6_mul(m, x, z);
+#pragma unroll
+        for (int k = 0; k < 6; k++)
+            fx_store64<RESID, HOST>(g, f, r, d, s, 6 * blk + k,
+                                    make_double2(fma(-kappa, acc[6 * blk + k].re, z[k].re),
+                                                 fma(-kappa, acc[6 * blk + k].im, z[k].im)));
+    }
+}
+
 // The listed sites in FP64, from the FP64 links and clover and the spinors as they
-// were before their conversion.  A warp per site: lane 6 mu + 3 sp + a takes
-// direction mu, both signs, spin sp of the half spinor, colour a of its product
+// were before their conversion.  A short list by a warp per site: lane 6 mu + 3 sp + a
+// takes direction mu, both signs, spin sp of the half spinor, colour a of its product
 // (36 FP64 operations); lane k then adds component k of the hop sum, and lanes k
 // and 12 + k take three columns each of its clover row.  With one thread per site
 // the FP64 pipe (a warp's instruction takes 64 clocks of a quarter SM) would make
-// a list of one site 38 us long; about 70 instructions make it 3.  Few sites are
-// listed on ordinary fields, so the launch costs what an empty one does.
+// a list of one site 38 us long; about 70 instructions make it 3.  But 70 are also
+// twice a site's share of 1140 (5.2 against 2.7 ns per site), so a list of more than 16
+// sites per warp of the grid, where both take about 200 us (one thread per site waits
+// on its scattered loads that long), goes by one thread per site.  Few sites are
+// listed on ordinary fields, and an empty list takes 2.4 us.
+// Measured, 24x16x12x32 with the fixed-point kernel (no site listed 101 us, FP64
+// arithmetic 316): a point source 107, a time slice 111, one colour 171 (a tenth of the
+// sites), even sites only 317 (half of them; 502 by warps), one colour on a nearly unit
+// field 507 (all; 874 by warps).
 template <bool RESID, bool HOST>
 __global__ void __launch_bounds__(128) k_dslash_list(Geom g, FxArgs f, double kappa)
 {
     const int lane = threadIdx.x & 31, n = f.list[0];
+    if (n > 16 * (int)(gridDim.x * (blockDim.x / 32))) {
+        for (int i = ((threadIdx.x / 32) * gridDim.x + blockIdx.x) * 32 + lane; i < n; i += gridDim.x * blockDim.x) {
+            const int at = f.list[1 + i];
+            int d, s;
+            split_index(g, at % g.V, d, s);
+            dslash_site64<RESID, HOST>(g, f, at / g.V, d, s, kappa);
+        }
+        return;
+    }
     const int mu = min(lane / 6, 3), k6 = lane % 6, sp = k6 / 3, a = k6 % 3;
     const int ls = mu < 2 ? 1 - sp : sp;  // the lower spin that meets upper spin sp
-    auto spinor = [&](int64_t r, int dd, int ss, int k) -> cpx<double> {
-        if (f.src.kind == kFxPlanes32) {
-            const float2 v = __ldg((const float2 *)f.src.p + (r * g.V + (int64_t)dd * g.Vd) * 12 + (int64_t)k * g.Vd + ss);
-            return mk(f2d(v.x), f2d(v.y));
-        }
-        const double2 *p = (const double2 *)f.src.p;
-        const double2 v = f.src.kind == kFxHost64
-                              ? __ldg(p + (r * g.V + __ldg(f.site_of + dd * g.Vd + ss)) * 12 + k)
-                              : __ldg(p + (r * g.V + (int64_t)dd * g.Vd) * 12 + (int64_t)k * g.Vd + ss);
-        return mk(v.x, v.y);
-    };
     for (int i = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; i < n; i += gridDim.x * (blockDim.x / 32)) {
         const int at = f.list[1 + i], gi = at % g.V;
         const int64_t r = at / g.V;
@@ -622,7 +701,7 @@ __global__ void __launch_bounds__(128) k_dslash_list(Geom g, FxArgs f, double ka
             cpx<double> w = mk(0.0, 0.0);
 #pragma unroll
             for (int b = 0; b < 3; b++) {
-                const cpx<double> u = spinor(r, nd, ns, sp * 3 + b), l = spinor(r, nd, ns, 6 + ls * 3 + b);
+                const cpx<double> u = fx_source(g, f, r, nd, ns, sp * 3 + b), l = fx_source(g, f, r, nd, ns, 6 + ls * 3 + b);
                 const cpx<double> h = (mu & 1) == 0 ? mk(fma(q, l.im, u.re), fma(-q, l.re, u.im))
                                                     : mk(fma(q, l.re, u.re), fma(q, l.im, u.im));
                 const double2 v = __ldg(U + (int64_t)(back ? b * 3 + a : a * 3 + b) * g.Vd);
@@ -647,7 +726,7 @@ __global__ void __launch_bounds__(128) k_dslash_list(Geom g, FxArgs f, double ka
         const int col0 = lane >= 12 && lane < 24 ? 3 : 0;
 #pragma unroll
         for (int c = col0, m = 0; m < 3; m++, c++) {
-            const cpx<double> x = spinor(r, d, s, blk * 6 + c);
+            const cpx<double> x = fx_source(g, f, r, d, s, blk * 6 + c);
             if (c == row) {
                 const double2 v = __ldg(A + (int64_t)(c >> 1) * g.Vd);
                 const double dg = c & 1 ? v.y : v.x;
@@ -661,16 +740,8 @@ __global__ void __launch_bounds__(128) k_dslash_list(Geom g, FxArgs f, double ka
         }
         y.re += __shfl_down_sync(0xffffffffu, y.re, 12);
         y.im += __shfl_down_sync(0xffffffffu, y.im, 12);
-        if (lane < 12) {
-            double2 o = make_double2(fma(-kappa, hop.re, y.re), fma(-kappa, hop.im, y.im));
-            const int64_t plane = (r * g.V + (int64_t)d * g.Vd) * 12 + (int64_t)k * g.Vd + s;
-            if (RESID) {
-                const double2 v = __ldg(f.b + plane);
-                o = make_double2(v.x - o.x, v.y - o.y);
-            }
-            if (HOST) f.out[(r * g.V + __ldg(f.site_of + gi)) * 12 + k] = o;
-            else f.out[plane] = o;
-        }
+        if (lane < 12)
+            fx_store64<RESID, HOST>(g, f, r, d, s, k, make_double2(fma(-kappa, hop.re, y.re), fma(-kappa, hop.im, y.im)));
     }
 }
 

@@ -154,3 +154,32 @@ def test_solve_of_a_point_source(env, ora, arnoldi, sap):
     for k in range(12):
         r = b[k] - ora.apply_D(L, U, A, 0.12, np.ascontiguousarray(x[k]))
         assert np.linalg.norm(r) <= 1.01e-11 * np.linalg.norm(b[k])
+
+
+@pytest.mark.parametrize("nrhs", [1, 2])
+@pytest.mark.parametrize("sites", ["one", "few", "most"])
+def test_lists_of_every_length(env, sites, nrhs):
+    """Sites left to FP64 arithmetic, from a single one (a warp per site) to more than the kernel's
+    warps take (a thread per site), in host layout and planes: a solve's residual and directions too."""
+    qdd, c = env
+    L, dom = (24, 16, 12, 16), (6, 4, 2, 4)
+    rng = np.random.default_rng(13)
+    U = inputs.gauge_field(L, 0.7, 1003)
+    V = int(np.prod(L))
+    x = np.stack([inputs.gaussian_source(L, 2003 + k) for k in range(nrhs)])
+    at = {"one": [V // 2], "few": rng.choice(V, 300, replace=False), "most": np.arange(V)}[sites]
+    x[:, at] *= 10.0 ** rng.uniform(-18, 0, (nrhs, len(at), 4, 3))
+    x[:, at, :, 1:] *= 1e-18
+    csw, kappa = 1.5, 0.1355
+    g = qdd.qdd_create_gauge_field(c, L, dom, U)
+    qdd.qdd_set_clover(g, csw, kappa)
+    blocks = qdd.qdd_get_clover(g, V)
+    y = qdd.qdd_apply_D(g, x if nrhs > 1 else x[0], "f64", nrhs=nrhs).reshape(nrhs, V, 4, 3)
+    _, rep = qdd.qdd_solve(g, x if nrhs > 1 else x[0], nrhs=nrhs, tol=1e-10, sap_prec="f32", arnoldi_prec="f64")
+    qdd.qdd_destroy_gauge(g)
+    A = np.zeros((V, 12, 12), np.complex128)
+    A[:, :6, :6], A[:, 6:, 6:] = blocks[:, 0], blocks[:, 1]
+    for k in range(nrhs):
+        err = np.abs(y[k] - apply_extended(L, U, A, kappa, x[k]))
+        assert (err <= 64 * 2.0 ** -53 * magnitudes(L, U, A, kappa, x[k])).all()
+    assert rep["converged"] and rep["true_rel_res"] <= 1e-10
