@@ -218,10 +218,11 @@ qdd_status qdd_link_compression(qdd_gauge *g, int *two_rows, int *is_su3);
  * domain's links and, when it fits, its clover in shared memory, with the domain
  * size fixed at compile time for 4^4 domains in 16-bit storage.  1 stages the
  * links only, reads the clover through the cache and is compiled for three CTAs
- * per SM (FP32 arithmetic on domains of at most 256 sites; otherwise 0 runs); 2 is the one-thread form with the domain size always taken at run
- * time.  Forms 1 and 2 give the same bits as the one-thread form.  The paper
- * sizes its domains to the cache (Sec. 3.3); on the GPU the choice trades
- * staged data and registers against the number of warps an SM holds.
+ * per SM (FP32 arithmetic on domains of at most 256 sites; otherwise 0 runs); 2 is
+ * the one-thread form with the domain size always taken at run time.  Forms 1 and
+ * 2 give the same bits as the one-thread form.  The paper sizes its domains to the
+ * cache (Sec. 3.3); on the GPU the choice trades staged data and registers against
+ * the number of warps an SM holds.
  * Returns QDD_EINVAL for a null field or a form outside 0..3.
  */
 qdd_status qdd_set_schwarz_variant(qdd_gauge *g, int variant);
@@ -338,7 +339,9 @@ qdd_status qdd_layout_faces(const int L[4], const int dom[4], int foff[8], uint3
  * have no fixed-point copy (|kappa| below 0.04; links not finite, outside
  * 2^-60..2^64, or of sizes that differ by more than 2^4 from link to link; a clover
  * term whose largest entry lies outside 2^-60..2^60 at some site), QDD_PREC_F64 also
- * where a copy would fill the HBM budget past a half.  QDD_PREC_F32 converts links, clover
+ * where a copy would fill the HBM budget past a half or the device has no room for
+ * it: the last bits of an FP64 result, and of a solve with FP64 operators, may depend
+ * on the memory in use, its accuracy does not.  QDD_PREC_F32 converts links, clover
  * and input to FP32 and computes in FP32 (1848 flop per site); F16S / BF16S
  * read 16-bit links/clover/spinor with FP32 arithmetic.
  */
@@ -436,6 +439,8 @@ qdd_status qdd_mg_get_basis(qdd_gauge *g, double *out);
  * multi-dot of the Gram-Schmidt step of FGMRES (Sec. 3.1).  v: nvec complex
  * FP64 vectors of n elements at stride ld elements; w: n elements;
  * out: nvec complex (device).  All device pointers; n <= 2^40, nvec <= 64.
+ * Each part of a result is as accurate as FP64 arithmetic makes it, against the
+ * sum of its products' magnitudes (most products run in 64-bit fixed point).
  * Uses library-owned device scratch for the per-block partial sums.
  */
 qdd_status qdd_cdot_multi(qdd_ctx *ctx, const double *v, int nvec, int64_t ld, const double *w, int64_t n,
