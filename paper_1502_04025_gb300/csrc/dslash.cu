@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(128, (dslash_min_blocks<R, SL>())) k_dslash(Ge
 // scale of the nine sites before the hops are added; the clover product keeps
 // the site's own scale; both are converted once and combined in FP64.  Beside
 // them run sums of the products' magnitudes from the factors' leading bits, two
-// spins in one 32-bit word (81 multiply-adds per site): where one of the twelve is
+// spins in one 32-bit word (72 multiply-adds per site): where one of the twelve is
 // small against the scales, the site goes on a list and k_dslash_list computes it
 // in FP64.
 //
