@@ -157,12 +157,29 @@ static void fx_reclaim(Ctx *c, size_t need)
     }
 }
 
+// n bytes of the budget, if they are there (threads allocate side by side)
+static bool reserve(Ctx *c, size_t n)
+{
+    size_t u = c->used.load();
+    do {
+        if (u + n > c->budget) return false;
+    } while (!c->used.compare_exchange_weak(u, u + n));
+    return true;
+}
+
 qdd_status DevMem::alloc(Ctx *c, size_t n)
 {
     release();
     if (n == 0) return QDD_OK;
-    if (c->used.load() + n > c->budget && !fx_optional) fx_reclaim(c, c->used.load() + n - c->budget);
-    if (c->used.load() + n > c->budget) {
+    // (another thread may build a copy anew between the two, so more than once)
+    bool room = reserve(c, n);
+    for (int turn = 0; !room && !fx_optional && turn < 8; turn++) {
+        const size_t u = c->used.load();
+        if (c->optional.load() == 0) break;
+        if (u + n > c->budget) fx_reclaim(c, u + n - c->budget);
+        room = reserve(c, n);
+    }
+    if (!room) {
         set_error("allocation of %zu bytes exceeds the HBM budget (%zu of %zu bytes in use)", n, c->used.load(),
                   c->budget);
         return QDD_EBUDGET;
@@ -176,13 +193,13 @@ qdd_status DevMem::alloc(Ctx *c, size_t n)
     }
     if (e != cudaSuccess) {
         p = nullptr;
+        c->used -= n;
         cudaGetLastError();
         set_error("cudaMalloc(%zu) failed: %s", n, cudaGetErrorString(e));
         return QDD_ENOMEM;
     }
     ctx = c;
     bytes = n;
-    c->used += n;
     return QDD_OK;
 }
 
